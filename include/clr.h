@@ -549,15 +549,12 @@ int clr_probe_peaks(int32_t reps, void* stream, clr_peaks* out);
  *          D (output, may be NULL) N pivots; K must not overlap x or D
  *   dyn_hits (output, device int, may be NULL): pivots replaced
  *   stream cudaStream_t as void* (NULL: legacy default stream)
- * No device memory is allocated or freed: the working matrix lives in one
- * static device array of CLR_NOALLOC_MAX_N^2 doubles (128 KiB) that every GPU
- * loading the library keeps until the process exits.  N > CLR_NOALLOC_MAX_N
- * gives CLR_E_UNSUPPORTED; N < 0 or a NULL required pointer CLR_E_INVALID.
- * The first call on a device resolves that array's address with
- * cudaGetSymbolAddress (with the device current); make the first call on each
- * device before any stream capture.  All calls on a device share the array:
- * calls whose kernels overlap on the GPU (different streams without ordering)
- * race on it.  Asynchronous: the results are ready when the stream is. */
+ * No device memory is allocated or freed: the factorization works in registers
+ * and shared memory.  N > CLR_NOALLOC_MAX_N gives CLR_E_UNSUPPORTED; N < 0 or a
+ * NULL required pointer CLR_E_INVALID.  The first call on a device sets kernel
+ * attributes (with the device current); make it before any stream capture.
+ * Calls share nothing, so they may overlap on the GPU.  Asynchronous: the results
+ * are ready when the stream is. */
 int clr_dense_ldl_solve_noalloc(const double* K, const double* signs, int32_t N, const double* rhs, double* x,
                                 double* D, double dyn_reg_eps, double dyn_reg_delta, int32_t* dyn_hits,
                                 void* stream);

@@ -1350,6 +1350,206 @@ __global__ void __launch_bounds__(128) k_step_psd_thread(ConeDev cd, const int32
   }
 }
 
+// The same step with KM lanes (4, 8 or 16) per cone side, lane r holding row r, for
+// lists too short to fill the GPU a thread per cone.  The thread version's time is
+// one cone's serial FP64 chain (a warp instruction holds its FP64 pipe 64 clocks
+// whatever its active lanes): 1.86 ms for four cones of orders 10 and 16.  Here the
+// rows of each step run side by side, the scalars are computed once on all lanes,
+// and the bisection tests the 2^LV - 1 points of its next LV levels at once (heap
+// node t on lane t, node 1 the first midpoint) and then walks down them, so every
+// accepted bound is the one the serial bisection takes: the same operations in the
+// same order per entry, hence the same bits, and the choice between the two may
+// depend on the length of the list.  On a GB300, 256 cones of
+// order 4 / 8 / 10 / 16: 0.07 / 0.10 / 0.12 / 0.19 ms (a thread per cone: 0.22 / 0.50 / 0.72 / 1.7).
+template <int KM>
+__global__ void __launch_bounds__(128) k_step_psd_lane(ConeDev cd, const int32_t* __restrict__ list, int64_t nlist,
+                                                       const double* __restrict__ s, const double* __restrict__ ds,
+                                                       const double* __restrict__ z, const double* __restrict__ dz,
+                                                       IterScal* sc, const int* skip) {
+  if (skip && *skip) return;
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int LD = KM + 1, MAT = KM * LD, PER = 2 * MAT + 4 * KM + 1;
+  constexpr int LV = KM == 16 ? 4 : (KM == 8 ? 3 : 2);  // bisection levels per pass
+  __shared__ double sm[(128 / KM) * PER];
+  const int r = threadIdx.x % KM;
+  const int64_t slot = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / KM;  // 2 cone + side
+  const bool live = slot < 2 * nlist;
+  const int64_t cone = live ? list[slot >> 1] : 0;
+  const int k = live ? cd.psd_ck[cone] : 0;
+  const int64_t row = live ? cd.psd_crow[cone] : 0;
+  const double* v = ((slot & 1) ? z : s) + row;
+  const double* dv = ((slot & 1) ? dz : ds) + row;
+  double* L = sm + (threadIdx.x / KM) * PER;
+  double* W = L + MAT;
+  double* u = W + MAT;
+  double* pv = u + KM;
+  double* av = pv + KM;  // tridiagonal matrix: diagonal, squared subdiagonal
+  double* bq = av + KM;
+  int kw = k;  // the warp's largest order
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) kw = max(kw, __shfl_xor_sync(FULL, kw, o));
+  const int shift = (threadIdx.x & 31) & ~(KM - 1);
+  const unsigned seg = (KM == 32 ? FULL : ((1u << KM) - 1u)) << shift;  // my side's lanes
+  const bool in = r < k;
+  for (int c = 0; c < KM; ++c) {
+    double x = 0.0, y = 0.0;
+    if (in && c < k) {
+      const int a = min(r, c), b = max(r, c);
+      x = v[b * (b + 1) / 2 + a];
+      y = dv[b * (b + 1) / 2 + a];
+      if (r != c) {
+        x /= kPsdSqrt2;
+        y /= kPsdSqrt2;
+      }
+    }
+    L[r * LD + c] = x;
+    W[r * LD + c] = y;
+  }
+  __syncwarp();
+  // Cholesky S = L L' (by columns, left-looking); u keeps the reciprocals of its diagonal
+  bool fail = false;
+  for (int j = 0; j < kw; ++j) {
+    double a = 1.0;
+    if (in && r >= j) {
+      a = L[r * LD + j];
+      for (int l = 0; l < j; ++l) a = fma(-L[r * LD + l], L[j * LD + l], a);
+    }
+    double d = __shfl_sync(FULL, a, j & (KM - 1), KM);
+    if (j < k && !(d > 0)) {
+      fail = true;
+      d = 1.0;
+    }
+    const double ljj = sqrt(d), rl = 1.0 / ljj;
+    if (in && r >= j) L[r * LD + j] = (r == j) ? ljj : a * rl;
+    if (r == j && in) u[j] = rl;
+    __syncwarp();
+  }
+  // W = L^{-1} dS (lane: a column), then X = W L^{-T} (lane: a row, lower part)
+  for (int i = 0; i < k; ++i) {
+    if (!in) break;
+    double a = W[i * LD + r];
+    for (int l = 0; l < i; ++l) a = fma(-L[i * LD + l], W[l * LD + r], a);
+    W[i * LD + r] = a * u[i];
+  }
+  __syncwarp();
+  if (in)
+    for (int j = 0; j <= r; ++j) {
+      double a = W[r * LD + j];
+      for (int l = 0; l < j; ++l) a = fma(-W[r * LD + l], L[j * LD + l], a);
+      W[r * LD + j] = a * u[j];
+    }
+  __syncwarp();
+  // Householder tridiagonalisation of X
+  double bown = 0.0;  // subdiagonal entry r (between rows r and r + 1)
+  for (int j = 0; j + 2 < kw; ++j) {
+    bool act = j + 2 < k;
+    double x0 = 0.0, ar = 0.0;
+    if (act) {
+      x0 = W[(j + 1) * LD + j];
+      for (int i = j + 2; i < k; ++i) ar = fma(W[i * LD + j], W[i * LD + j], ar);
+      if (r == j) bown = x0;
+      if (ar <= 0.0) act = false;  // the column is already tridiagonal
+    }
+    const double nrm = sqrt(fma(x0, x0, ar));
+    const double be = x0 >= 0.0 ? -nrm : nrm;
+    const double tau = (be - x0) / be;
+    const double sc1 = 1.0 / (x0 - be);
+    const bool mine = act && in && r > j;
+    double ui = 0.0;
+    if (mine) {
+      ui = (r == j + 1) ? 1.0 : W[r * LD + j] * sc1;
+      u[r] = ui;
+    }
+    __syncwarp();
+    double pi = 0.0;
+    if (mine) {
+      double acc = 0.0;
+      for (int l = j + 1; l < k; ++l) acc = fma(r >= l ? W[r * LD + l] : W[l * LD + r], u[l], acc);
+      pi = tau * acc;
+      pv[r] = pi;
+    }
+    __syncwarp();
+    double pu = 0.0;
+    if (act)
+      for (int i = j + 1; i < k; ++i) pu = fma(pv[i], u[i], pu);
+    __syncwarp();
+    if (mine) {
+      const double h = 0.5 * tau * pu;
+      pi = fma(-h, ui, pi);
+      pv[r] = pi;
+    }
+    __syncwarp();
+    if (mine)
+      for (int l = j + 1; l <= r; ++l) W[r * LD + l] = fma(-ui, pv[l], fma(-pi, u[l], W[r * LD + l]));
+    if (act && r == j) bown = be;
+    __syncwarp();
+  }
+  const double aown = in ? W[r * LD + r] : 0.0;
+  if (k >= 2 && r == k - 2) bown = W[(k - 1) * LD + (k - 2)];
+  if (r + 1 >= k) bown = 0.0;
+  av[r] = aown;
+  bq[r] = bown * bown;
+  fail = fail || (__ballot_sync(FULL, !isfinite(aown) || !isfinite(bown)) & seg) != 0;
+  const double bup = __shfl_up_sync(FULL, bown, 1, KM);
+  double lo = INFINITY;  // the Gershgorin bound
+  if (in) lo = aown - (r > 0 ? fabs(bup) : 0.0) - (r + 1 < k ? fabs(bown) : 0.0);
+#pragma unroll
+  for (int o = KM / 2; o > 0; o >>= 1) lo = fmin(lo, __shfl_xor_sync(FULL, lo, o, KM));
+  __syncwarp();
+  auto below = [&](double x) {
+    int cnt = 0;
+    double d = 1.0;
+    for (int i = 0; i < k; ++i) {
+      double t = av[i] - x;
+      if (i > 0) t = fma(-bq[i - 1], psd_rcp(d), t);
+      if (t == 0.0) t = -1e-300;
+      cnt += t < 0.0;
+      d = t;
+    }
+    return cnt;
+  };
+  const bool search = live && !fail && below(0.0) != 0;
+  double hi = 0.0;
+  bool run = search;
+  int it = 0;
+  while (__any_sync(FULL, run)) {
+    // my node's midpoint (heap index r; lane 0 idles), then its count
+    double lt = lo, ht = hi;
+    if (r > 0) {
+      const int depth = 31 - __clz(r);
+      for (int q = depth - 1; q >= 0; --q) {
+        const double m = 0.5 * (lt + ht);
+        if ((r >> q) & 1) lt = m;
+        else ht = m;
+      }
+    }
+    const bool pos = run && r > 0 && below(0.5 * (lt + ht)) > 0;
+    const unsigned bits = __ballot_sync(FULL, pos) >> shift;
+    int node = 1;
+    for (int q = 0; q < LV && run; ++q) {
+      const double mid = 0.5 * (lo + hi);
+      if (!(it < 80 && hi - lo > 1e-14 * fabs(lo)) || mid <= lo || mid >= hi) {
+        run = false;
+        break;
+      }
+      if ((bits >> node) & 1u) {
+        hi = mid;
+        node = 2 * node;
+      } else {
+        lo = mid;
+        node = 2 * node + 1;
+      }
+      ++it;
+    }
+  }
+  if (live && r == 0) {
+    double a = INFINITY;
+    if (fail) a = 0.0;
+    else if (search) a = -1.0 / (0.5 * (lo + hi));
+    if (a < INFINITY) atomicMin(&sc[cd.row_pid[row]].amin_bits, dbits(a));
+  }
+}
+
 __global__ void k_step_psd(ConeDev cd, const int32_t* __restrict__ list, const double* __restrict__ s,
                            const double* __restrict__ ds, const double* __restrict__ z, const double* __restrict__ dz,
                            IterScal* sc, const int* skip) {
@@ -1400,6 +1600,23 @@ __global__ void k_step_psd(ConeDev cd, const int32_t* __restrict__ list, const d
   if (threadIdx.x == 0 && amax < INFINITY) atomicMin(&sc[cd.row_pid[row]].amin_bits, dbits(amax));
 }
 
+// PSD cones of one order class: KM lanes per cone side up to kPsdLaneCones cones, a
+// thread per cone beyond (the same bits either way).  At 4096
+// cones of order 4 / 8 / 10 / 16 the lanes take 0.12 / 0.34 / 0.72 / 1.2 ms, the threads 0.22 / 0.50 /
+// 0.72 / 1.7 ms; the lanes' time grows with the list from ~1000 cones on, the threads' only from ~20 000.
+constexpr int64_t kPsdLaneCones = 4096;
+template <int KM>
+static void step_psd_small(cudaStream_t st, const ConeDev& cd, int cls, const double* s, const double* ds,
+                           const double* z, const double* dz, IterScal* sc, const int* skip) {
+  const int64_t n = cd.psd_nlist[cls];
+  if (n <= 0) return;
+  if (n <= kPsdLaneCones)
+    k_step_psd_lane<KM><<<grid_for(2 * n * KM, 128, 1 << 30), 128, 0, st>>>(cd, cd.psd_list[cls], n, s, ds, z, dz, sc,
+                                                                         skip);
+  else
+    k_step_psd_thread<KM><<<grid_for(n, 128, 1 << 30), 128, 0, st>>>(cd, cd.psd_list[cls], n, s, ds, z, dz, sc, skip);
+}
+
 int cones_step_symmetric(cudaStream_t st, const ConeDev& cd, const double* s, const double* ds, const double* z,
                          const double* dz, IterScal* sc, const int* skip) {
   if (cd.m_nonneg > 0) k_step_nonneg<<<grid_for(cd.m_nonneg, 256), 256, 0, st>>>(cd, s, ds, z, dz, sc, skip);
@@ -1408,20 +1625,11 @@ int cones_step_symmetric(cudaStream_t st, const ConeDev& cd, const double* s, co
     if (cd.soc_nsmall < cd.n_soc) k_step_soc<32><<<soc_grid(cd, 32), 256, 0, st>>>(cd, s, ds, z, dz, sc, skip);
   }
   if (cd.n_psd > 0) {
-    // orders up to 16: a thread per cone (tridiagonalisation and Sturm bisection);
-    // larger: a block per cone (two-sided Jacobi)
-    if (cd.psd_nlist[0] > 0)
-      k_step_psd_thread<4><<<grid_for(cd.psd_nlist[0], 128, 1 << 30), 128, 0, st>>>(cd, cd.psd_list[0],
-                                                                                   cd.psd_nlist[0], s, ds, z, dz, sc,
-                                                                                   skip);
-    if (cd.psd_nlist[1] > 0)
-      k_step_psd_thread<8><<<grid_for(cd.psd_nlist[1], 128, 1 << 30), 128, 0, st>>>(cd, cd.psd_list[1],
-                                                                                   cd.psd_nlist[1], s, ds, z, dz, sc,
-                                                                                   skip);
-    if (cd.psd_nlist[2] > 0)
-      k_step_psd_thread<16><<<grid_for(cd.psd_nlist[2], 128, 1 << 30), 128, 0, st>>>(cd, cd.psd_list[2],
-                                                                                    cd.psd_nlist[2], s, ds, z, dz, sc,
-                                                                                    skip);
+    // orders up to 16: tridiagonalisation and Sturm bisection; larger: a block per cone
+    // (two-sided Jacobi)
+    step_psd_small<4>(st, cd, 0, s, ds, z, dz, sc, skip);
+    step_psd_small<8>(st, cd, 1, s, ds, z, dz, sc, skip);
+    step_psd_small<16>(st, cd, 2, s, ds, z, dz, sc, skip);
     if (cd.psd_nlist[3] > 0) {
       const int threads = std::max(64, 32 * ((cd.psd_kmax + 1) / 2));
       k_step_psd<<<(unsigned)cd.psd_nlist[3], threads, 0, st>>>(cd, cd.psd_list[3], s, ds, z, dz, sc, skip);

@@ -46,3 +46,34 @@ def test_dense_ldl_tile_edges(N):
     xref = ldl_solve(L, Dref, rhs)
     assert np.abs(K @ x - rhs).max() <= N * 2.2e-16 * 1e3 * max(1.0, np.abs(xref).max())
     assert int(hits.item()) == 0
+
+
+# PSD step length: lanes per cone for short lists, a thread per cone for long ones; same bits
+@pytest.mark.parametrize("orders", [(1, 2, 3, 4), (5, 6, 7, 8), (9, 12, 15, 16)])
+def test_psd_step_lane_equals_thread(orders):
+    rng = np.random.default_rng(sum(orders))
+    cones, s, z, ds, dz = [], [], [], [], []
+    for rep in range(5):
+        for k in orders:
+            cones.append((OC.PSD, k * (k + 1) // 2, 0.0))
+            for out in (s, z):
+                M = rng.standard_normal((k, k))
+                out.append(OC.svec(M @ M.T / k + 0.3 * np.eye(k)))
+            for out in (ds, dz):
+                T = rng.standard_normal((k, k))
+                out.append(OC.svec(T + T.T) if rep else OC.svec(np.diag(rng.uniform(0.1, 1.0, k))))
+    ref = []
+    for i in range(len(cones)):  # every cone on its own, against the oracle
+        a = clr.clr_cones_step_length([cones[i]], s[i], z[i], ds[i], dz[i], 1e6)
+        o = min(1e6, OC.step_length_symmetric(OC.PSD, s[i], ds[i]), OC.step_length_symmetric(OC.PSD, z[i], dz[i]))
+        assert a == pytest.approx(o, rel=1e-10)
+        ref.append(a)
+    reps = 4096 // len(cones) + 1  # longer than the list length up to which lanes are used
+    for i in (0, len(cones) - 1, int(np.argmin(ref))):
+        many = clr.clr_cones_step_length([cones[i]] * (4097), np.tile(s[i], 4097), np.tile(z[i], 4097),
+                                         np.tile(ds[i], 4097), np.tile(dz[i], 4097), 1e6)
+        assert many == ref[i]
+    cat = lambda v, r: np.tile(np.concatenate(v), r)
+    few = clr.clr_cones_step_length(cones, *[cat(v, 1) for v in (s, z, ds, dz)], 1e6)
+    many = clr.clr_cones_step_length(cones * reps, *[cat(v, reps) for v in (s, z, ds, dz)], 1e6)
+    assert few == many == min(ref)

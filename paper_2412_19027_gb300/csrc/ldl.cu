@@ -38,15 +38,74 @@ __global__ void k_add_reg(T* __restrict__ F, const int64_t* __restrict__ diag_po
     F[diag_pos[k]] += (T)(dsign[k] * sc[pos_pid[k]].delta);
 }
 
+// Longest source list a single thread sums (k_pull_long beyond), and the longest that
+// a warp sums: the factor's lists are as many as a front's entries, the solves' as its
+// rows, so those go to a CTA earlier.
+constexpr int64_t kPullShort = 48, kFaWarp = 8192, kSvWarp = 512;
+
 template <typename T>
 __global__ void k_pull(T* __restrict__ X, const int64_t* __restrict__ tgt, const int64_t* __restrict__ ptr,
                        const int64_t* __restrict__ src, int64_t t0, int64_t t1, const int* skip) {
   if (skip && *skip) return;
   for (int64_t t = t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < t1; t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t q0 = ptr[t], q1 = ptr[t + 1];
+    if (q1 - q0 > kPullShort) continue;  // k_pull_long
     T acc = X[tgt[t]];
-    for (int64_t q = ptr[t]; q < ptr[t + 1]; ++q) acc += X[src[q]];
+    for (int64_t q = q0; q < q1; ++q) acc += X[src[q]];
     X[tgt[t]] = acc;
   }
+}
+
+// Targets with more than kPullShort sources, G threads (32 or 256) per target: a
+// thread's serial gather is one dependent L2 access after another (5000 sources: the
+// forward sweep of the portfolio n = 5000 root spent 384 us per solve in it, now 7; its
+// extend-add of 1.6e8 sources 1.5 -> 1.2 ms) and its
+// neighbours' lists start far apart; here consecutive threads read consecutive list
+// entries, four gathers in flight each.  The sum's order depends on the list's length
+// alone: entry q goes to partial q mod 4 G, partials added in fixed trees.
+template <typename T, int G>
+__global__ void __launch_bounds__(256) k_pull_long(T* __restrict__ X, const int64_t* __restrict__ tgt,
+                                                   const int64_t* __restrict__ ptr, const int64_t* __restrict__ src,
+                                                   const int64_t* __restrict__ ids, int64_t n, const int* skip) {
+  if (skip && *skip) return;
+  __shared__ T sh[8];
+  const int lane = threadIdx.x % G;
+  for (int64_t i = (blockIdx.x * (int64_t)256 + threadIdx.x) / G; i < n; i += (int64_t)gridDim.x * (256 / G)) {
+    const int64_t t = ids[i], q1 = ptr[t + 1];
+    T a[4] = {(T)0, (T)0, (T)0, (T)0};
+    int64_t q = ptr[t] + lane;
+    for (; q + 3 * G < q1; q += 4 * G) {
+      int64_t s[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s[u] = src[q + G * u];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] += X[s[u]];
+    }
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (q + G * u < q1) a[u] += X[src[q + G * u]];
+    T v = warp_sum((a[0] + a[1]) + (a[2] + a[3]));
+    if constexpr (G == 256) {
+      if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        v = sh[0];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) v += sh[w];
+      }
+      __syncthreads();
+    }
+    if (lane == 0) X[tgt[t]] += v;
+  }
+}
+
+// One level's pulls.
+template <typename T>
+static void pull_level(cudaStream_t stm, T* X, const int64_t* tgt, const int64_t* ptr, const int64_t* src, int64_t t0,
+                       int64_t t1, const LdlStructure::List& wl, const LdlStructure::List& cl, const int* skip) {
+  if (t1 - t0 > wl.n + cl.n) k_pull<T><<<grid_for(t1 - t0, 256), 256, 0, stm>>>(X, tgt, ptr, src, t0, t1, skip);
+  if (wl.n > 0) k_pull_long<T, 32><<<grid_for(wl.n * 32, 256), 256, 0, stm>>>(X, tgt, ptr, src, wl.id, wl.n, skip);
+  if (cl.n > 0) k_pull_long<T, 256><<<grid_for(cl.n * 256, 256), 256, 0, stm>>>(X, tgt, ptr, src, cl.id, cl.n, skip);
 }
 
 // Extend-add of large update blocks by relative indices, one child per front per
@@ -96,7 +155,7 @@ __device__ __forceinline__ T regularise(T d, int sgn, T eps, T delta, bool* hit)
 template <typename T>
 __global__ void k_factor_small(T* __restrict__ F, T* __restrict__ Dp, const int64_t* __restrict__ fronts,
                                const int64_t* __restrict__ sn_ptr, const int64_t* __restrict__ row_ptr,
-                               const int64_t* __restrict__ front_off, const int8_t* __restrict__ dsign, int small_max,
+                               const int64_t* __restrict__ front_off, const int8_t* __restrict__ dsign,
                                double eps_d, double delta_d, int* dyn_hits, const int* skip) {
   if (skip && *skip) return;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -105,7 +164,6 @@ __global__ void k_factor_small(T* __restrict__ F, T* __restrict__ Dp, const int6
   const int64_t J = fronts[blockIdx.x];
   const int c = (int)(sn_ptr[J + 1] - sn_ptr[J]);
   const int f = (int)(row_ptr[J + 1] - row_ptr[J]);
-  if (f > small_max) return;
   T* G = F + front_off[J];
   const int64_t k0 = sn_ptr[J];
   const T eps = (T)eps_d, delta = (T)delta_d;
@@ -134,6 +192,80 @@ __global__ void k_factor_small(T* __restrict__ F, T* __restrict__ Dp, const int6
   for (int q = threadIdx.x; q < f * f; q += blockDim.x) G[q] = S[q];
 }
 
+// One CTA per thin front (ldl_thin_front): its c columns in shared memory as they are
+// (P = L D) and scaled (L), then the trailing lower triangle F -= L P^T in 64 x 64 tiles,
+// a lane per row and eight columns per warp, so that every store is a full line.  LEAF:
+// no child has added to the trailing part, which is zero and not read.  Bound by the
+// stores of the update matrix (f^2 / 2 values) in FP32, by the FMAs in FP64 from c ~ 4 on.
+template <typename T, bool LEAF>
+__global__ void __launch_bounds__(256) k_factor_thin(T* __restrict__ F, T* __restrict__ Dp,
+                                                     const int64_t* __restrict__ fronts,
+                                                     const int64_t* __restrict__ sn_ptr,
+                                                     const int64_t* __restrict__ row_ptr,
+                                                     const int64_t* __restrict__ front_off,
+                                                     const int8_t* __restrict__ dsign, double eps_d, double delta_d,
+                                                     int* dyn_hits, const int* skip) {
+  if (skip && *skip) return;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ T s_inv;
+  const int64_t J = fronts[blockIdx.x];
+  const int c = (int)(sn_ptr[J + 1] - sn_ptr[J]);
+  const int f = (int)(row_ptr[J + 1] - row_ptr[J]);
+  T* P = reinterpret_cast<T*>(smraw);  // column t at t f; rows above the diagonal unused
+  T* L = P + f * c;
+  T* G = F + front_off[J];
+  const int64_t k0 = sn_ptr[J];
+  const T eps = (T)eps_d, delta = (T)delta_d;
+  const int tid = threadIdx.x;
+  for (int q = tid; q < f * c; q += 256) P[q] = G[q];
+  __syncthreads();
+  for (int t = 0; t < c; ++t) {
+    if (tid == 0) {
+      bool hit;
+      const T d = regularise(P[t + t * f], (int)dsign[k0 + t], eps, delta, &hit);
+      if (hit) atomicAdd(dyn_hits, 1);
+      Dp[k0 + t] = d;
+      G[t + (int64_t)t * f] = d;
+      s_inv = (T)1 / d;
+    }
+    __syncthreads();
+    const T inv = s_inv;
+    for (int i = t + 1 + tid; i < f; i += 256) {
+      const T l = P[i + t * f] * inv;
+      L[i + t * f] = l;
+      G[i + (int64_t)t * f] = l;
+      for (int s = t + 1; s < c && s <= i; ++s) P[i + s * f] -= l * P[s + t * f];
+    }
+    __syncthreads();
+  }
+  const int lane = tid & 31, w = tid >> 5;
+  for (int j0 = c; j0 < f; j0 += 64)
+    for (int i0 = j0; i0 < f; i0 += 64) {
+      const int r0 = i0 + lane, r1 = r0 + 32, cb = j0 + 8 * w;
+      if (cb >= f) continue;
+      T acc[2][8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc[0][q] = acc[1][q] = (T)0;
+      const int x0 = min(r0, f - 1), x1 = min(r1, f - 1);
+      for (int t = 0; t < c; ++t) {
+        const T l0 = L[x0 + t * f], l1 = L[x1 + t * f];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const T pv = P[min(cb + q, f - 1) + t * f];
+          acc[0][q] += l0 * pv;
+          acc[1][q] += l1 * pv;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int col = cb + q;
+        T* g = G + (int64_t)col * f;
+        if (r0 < f && r0 >= col && col < f) g[r0] = (LEAF ? (T)0 : g[r0]) - acc[0][q];
+        if (r1 < f && r1 >= col && col < f) g[r1] = (LEAF ? (T)0 : g[r1]) - acc[1][q];
+      }
+    }
+}
+
 // ------------------------------------------------------------------ solve
 template <typename T>
 __global__ void k_init_w(T* __restrict__ w, const int32_t* __restrict__ w_init, const double* __restrict__ rhs,
@@ -151,13 +283,12 @@ template <typename T>
 __global__ void k_fwd_front(const T* __restrict__ F, T* __restrict__ w, const int64_t* __restrict__ fronts,
                             const int64_t* __restrict__ sn_ptr, const int64_t* __restrict__ row_ptr,
                             const int64_t* __restrict__ front_off, const int64_t* __restrict__ upd_off,
-                            int small_max, const int* skip) {
+                            const int* skip) {
   if (skip && *skip) return;
   __shared__ T xb[32];
   const int64_t J = fronts[blockIdx.x];
   const int64_t c = sn_ptr[J + 1] - sn_ptr[J];
   const int64_t f = row_ptr[J + 1] - row_ptr[J];
-  if (f > small_max) return;
   const T* G = F + front_off[J];
   T* wj = w + upd_off[J];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -191,12 +322,11 @@ __global__ void k_bwd_front(const T* __restrict__ F, const T* __restrict__ Dp, T
                             const int64_t* __restrict__ fronts, const int64_t* __restrict__ sn_ptr,
                             const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ front_off,
                             const int64_t* __restrict__ upd_off, const int32_t* __restrict__ rows_kkt,
-                            int small_max, const int* skip) {
+                            const int* skip) {
   if (skip && *skip) return;
   const int64_t J = fronts[blockIdx.x];
   const int64_t c = sn_ptr[J + 1] - sn_ptr[J];
   const int64_t f = row_ptr[J + 1] - row_ptr[J];
-  if (f > small_max) return;
   const T* G = F + front_off[J];
   T* X = w + upd_off[J];
   const int32_t* rk = rows_kkt + row_ptr[J];
@@ -470,14 +600,64 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
     if ((!mp.rel.empty() && !st.rel) || !st.rel_off || !st.sn_parent) return CLR_E_OOM;
   }
   st.lev_small_maxf.assign(sy.nlev, 0);
+  st.lev_thin_smem.assign(sy.nlev, 0);
   st.lev_big.assign(sy.nlev, {});
-  for (int64_t l = 0; l < sy.nlev; ++l)
-    for (int64_t t = sy.lev_ptr[l]; t < sy.lev_ptr[l + 1]; ++t) {
-      const int64_t J = sy.lev_sn[t];
-      const int64_t f = sy.row_ptr[J + 1] - sy.row_ptr[J];
-      if (f > small_max) st.lev_big[l].push_back(J);
-      else st.lev_small_maxf[l] = std::max(st.lev_small_maxf[l], (int)f);
+  {
+    using List = LdlStructure::List;
+    std::vector<int64_t> buf;
+    std::vector<std::pair<List*, size_t>> where;
+    auto add = [&](std::vector<List>& lists, int64_t l, const std::vector<int64_t>& ids) {
+      if (lists.empty()) lists.assign(sy.nlev, List());
+      if (ids.empty()) return;
+      lists[l].n = (int64_t)ids.size();
+      where.emplace_back(&lists[l], buf.size());
+      buf.insert(buf.end(), ids.begin(), ids.end());
+    };
+    std::vector<char> has_child(sy.nsn, 0);
+    for (int64_t J = 0; J < sy.nsn; ++J)
+      if (sy.sn_parent[J] >= 0) has_child[sy.sn_parent[J]] = 1;
+    auto longs = [&](const std::vector<int64_t>& ptr, int64_t t0, int64_t t1, int64_t warp_max, std::vector<List>& wl,
+                     std::vector<List>& cl, int64_t l) {
+      std::vector<int64_t> w, c;
+      for (int64_t t = t0; t < t1; ++t) {
+        const int64_t n = ptr[t + 1] - ptr[t];
+        if (n > kPullShort) (n > warp_max ? c : w).push_back(t);
+      }
+      add(wl, l, w);
+      add(cl, l, c);
+    };
+    std::vector<int64_t> small, leaf, thin, both;
+    for (int64_t l = 0; l < sy.nlev; ++l) {
+      small.clear();
+      leaf.clear();
+      thin.clear();
+      both.clear();
+      for (int64_t t = sy.lev_ptr[l]; t < sy.lev_ptr[l + 1]; ++t) {
+        const int64_t J = sy.lev_sn[t];
+        const int64_t f = sy.row_ptr[J + 1] - sy.row_ptr[J], c = sy.sn_ptr[J + 1] - sy.sn_ptr[J];
+        if (f <= small_max) {
+          small.push_back(J);
+          st.lev_small_maxf[l] = std::max(st.lev_small_maxf[l], (int)f);
+        } else if (ldl_thin_front(f, c, small_max)) {
+          (has_child[J] ? thin : leaf).push_back(J);
+          st.lev_thin_smem[l] = std::max(st.lev_thin_smem[l], f * c);
+        } else {
+          st.lev_big[l].push_back(J);
+          continue;
+        }
+        both.push_back(J);
+      }
+      add(st.lev_small, l, small);
+      add(st.lev_thin_leaf, l, leaf);
+      add(st.lev_thin, l, thin);
+      add(st.lev_cta, l, both);
+      longs(mp.fa_ptr, mp.fa_lev_ptr[l], mp.fa_lev_ptr[l + 1], kFaWarp, st.fa_warp, st.fa_cta, l);
+      longs(mp.sv_ptr, mp.sv_lev_ptr[l], mp.sv_lev_ptr[l + 1], kSvWarp, st.sv_warp, st.sv_cta, l);
     }
+    int64_t* dbuf = buf.empty() ? nullptr : ar.upload(buf.data(), (int64_t)buf.size());
+    if (!buf.empty() && !dbuf) return CLR_E_OOM;
+    for (auto& [li, off] : where) li->id = dbuf + off;
+  }
   // ---- big fronts: arrays, E / y pools, launch plans per level ----
   {
     std::vector<int64_t> bf_f, bf_c, bf_goff, bf_eoff, bf_k0, bf_woff, bf_yoff, bf_rk, bf_pk;
@@ -769,6 +949,8 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
   static bool attr_set = false;
   if (!attr_set) {
     cudaFuncSetAttribute(k_factor_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_factor_thin<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+    cudaFuncSetAttribute(k_factor_thin<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
     attr_set = true;
   }
   return CLR_OK;
@@ -787,21 +969,26 @@ int LdlFactor<T>::factor(cudaStream_t stm, const double* kval, const IterScal* s
   k_add_reg<T><<<grid_for(S.N, 256), 256, 0, stm>>>(F, S.diag_pos, S.dsign, S.pos_pid, S.N, sc, skip);
   CLR_CHECK_LAUNCH();
   for (int64_t l = 0; l < S.nlev; ++l) {
-    const int64_t t0 = S.h_fa_lev_ptr[l], t1 = S.h_fa_lev_ptr[l + 1];
-    if (t1 > t0) k_pull<T><<<grid_for(t1 - t0, 256), 256, 0, stm>>>(F, S.fa_tgt, S.fa_ptr, S.fa_src, t0, t1, skip);
+    pull_level<T>(stm, F, S.fa_tgt, S.fa_ptr, S.fa_src, S.h_fa_lev_ptr[l], S.h_fa_lev_ptr[l + 1], S.fa_warp[l],
+                  S.fa_cta[l], skip);
     for (const WorkList& wl : S.push_rounds[l])
       if (wl.nblocks > 0)
         k_push<T><<<(unsigned)wl.nblocks, 256, 0, stm>>>(F, wl, S.sn_ptr, S.row_ptr, S.front_off, S.sn_parent,
                                                           S.rel_off, S.rel, skip);
-    const int64_t nf = S.h_lev_ptr[l + 1] - S.h_lev_ptr[l];
-    if ((int64_t)S.lev_big[l].size() < nf) {
+    if (S.lev_small[l].n > 0) {
       const int mf = S.lev_small_maxf[l];
       const size_t smem = sizeof(T) * (size_t)mf * (size_t)mf;
       const int threads = mf <= 16 ? 64 : (mf <= 48 ? 128 : 256);
-      k_factor_small<T><<<(unsigned)nf, threads, smem, stm>>>(F, Dp, S.lev_sn + S.h_lev_ptr[l], S.sn_ptr, S.row_ptr,
-                                                               S.front_off, S.dsign, S.small_max, dyn_eps, dyn_delta,
-                                                               dyn_hits, skip);
+      k_factor_small<T><<<(unsigned)S.lev_small[l].n, threads, smem, stm>>>(
+          F, Dp, S.lev_small[l].id, S.sn_ptr, S.row_ptr, S.front_off, S.dsign, dyn_eps, dyn_delta, dyn_hits, skip);
     }
+    const size_t tsm = 2 * sizeof(T) * (size_t)S.lev_thin_smem[l];
+    if (S.lev_thin_leaf[l].n > 0)
+      k_factor_thin<T, true><<<(unsigned)S.lev_thin_leaf[l].n, 256, tsm, stm>>>(
+          F, Dp, S.lev_thin_leaf[l].id, S.sn_ptr, S.row_ptr, S.front_off, S.dsign, dyn_eps, dyn_delta, dyn_hits, skip);
+    if (S.lev_thin[l].n > 0)
+      k_factor_thin<T, false><<<(unsigned)S.lev_thin[l].n, 256, tsm, stm>>>(
+          F, Dp, S.lev_thin[l].id, S.sn_ptr, S.row_ptr, S.front_off, S.dsign, dyn_eps, dyn_delta, dyn_hits, skip);
     if (!S.lev_big[l].empty()) {
       // FP64: the table with the split chain task; FP32: the fused one
       const bool f64 = sizeof(T) == 8;
@@ -827,22 +1014,20 @@ int LdlFactor<T>::solve(cudaStream_t stm, const double* rhs, const int* skip) co
   const LdlStructure& S = *s;
   k_init_w<T><<<grid_for(S.wtot, 256), 256, 0, stm>>>(w, S.w_init, rhs, S.wtot, skip);
   for (int64_t l = 0; l < S.nlev; ++l) {
-    const int64_t t0 = S.h_sv_lev_ptr[l], t1 = S.h_sv_lev_ptr[l + 1];
-    if (t1 > t0) k_pull<T><<<grid_for(t1 - t0, 256), 256, 0, stm>>>(w, S.sv_tgt, S.sv_ptr, S.sv_src, t0, t1, skip);
-    const int64_t nf = S.h_lev_ptr[l + 1] - S.h_lev_ptr[l];
-    if ((int64_t)S.lev_big[l].size() < nf)
-      k_fwd_front<T><<<(unsigned)nf, 256, 0, stm>>>(F, w, S.lev_sn + S.h_lev_ptr[l], S.sn_ptr, S.row_ptr,
-                                                     S.front_off, S.upd_off, S.small_max, skip);
+    pull_level<T>(stm, w, S.sv_tgt, S.sv_ptr, S.sv_src, S.h_sv_lev_ptr[l], S.h_sv_lev_ptr[l + 1], S.sv_warp[l],
+                  S.sv_cta[l], skip);
+    if (S.lev_cta[l].n > 0)
+      k_fwd_front<T><<<(unsigned)S.lev_cta[l].n, 256, 0, stm>>>(F, w, S.lev_cta[l].id, S.sn_ptr, S.row_ptr,
+                                                                 S.front_off, S.upd_off, skip);
     if (!S.lev_big[l].empty()) {
       int rc = BigFrontOps<T>::fwd(stm, S.bfd, S.bplans[l].fwd, E, Dp, w, ybuf, skip);
       if (rc) return rc;
     }
   }
   for (int64_t l = S.nlev - 1; l >= 0; --l) {
-    const int64_t nf = S.h_lev_ptr[l + 1] - S.h_lev_ptr[l];
-    if ((int64_t)S.lev_big[l].size() < nf)
-      k_bwd_front<T><<<(unsigned)nf, 256, 0, stm>>>(F, Dp, w, xs, S.lev_sn + S.h_lev_ptr[l], S.sn_ptr, S.row_ptr,
-                                                    S.front_off, S.upd_off, S.rows_kkt, S.small_max, skip);
+    if (S.lev_cta[l].n > 0)
+      k_bwd_front<T><<<(unsigned)S.lev_cta[l].n, 256, 0, stm>>>(F, Dp, w, xs, S.lev_cta[l].id, S.sn_ptr, S.row_ptr,
+                                                                 S.front_off, S.upd_off, S.rows_kkt, skip);
     if (!S.lev_big[l].empty()) {
       int rc = BigFrontOps<T>::bwd(stm, S.bfd, S.bplans[l].bwd, E, Dp, ybuf, xs, S.rows_kkt, skip);
       if (rc) return rc;

@@ -29,6 +29,17 @@ struct LdlStructure {
   std::vector<int64_t> h_lev_ptr, h_lev_sn, h_fa_lev_ptr, h_sv_lev_ptr;
   std::vector<int64_t> h_sn_ptr, h_row_ptr, h_front_off;
   std::vector<int> lev_small_maxf;               // largest small front of each level
+  // fronts by kernel, per level (device lists): small ones (one CTA each in shared
+  // memory), thin ones without and with children (ldl_thin_front), and both kinds
+  // together (the solves' one CTA per front)
+  struct List {
+    const int64_t* id = nullptr;
+    int64_t n = 0;
+  };
+  std::vector<List> lev_small, lev_thin_leaf, lev_thin, lev_cta;
+  std::vector<int64_t> lev_thin_smem;            // largest f c of a level's thin fronts
+  // pull targets with long source lists (indices into fa_tgt, sv_tgt): a warp each, a CTA each
+  std::vector<List> fa_warp, fa_cta, sv_warp, sv_cta;
   std::vector<std::vector<int64_t>> lev_big;     // big fronts of each level
   BigFrontDev bfd;                               // big-front arrays (device)
   std::vector<BigLevelPlan> bplans;              // per level
@@ -55,6 +66,21 @@ struct LdlStructure {
   int small_max = 0;
   int64_t max_front = 0;
 };
+
+// A front of more rows than small_max with few pivots: the arrow columns of a dense
+// row block (portfolio, Huber, entropy problems have thousands with 1 .. 5 pivots and
+// hundreds of rows).  Its update matrix is a rank-c product that one CTA streams out
+// (k_factor_thin); cut into 64 x 64 tile tasks of the dataflow launch, a task did
+// 1/64 .. 1/16 of a tile's work for the same loads, stores and waits (portfolio
+// n = 5000, FP32: 5000 fronts of ~250 rows 3.0 -> 0.20 ms), and the forward sweep
+// gave each front f / 32 CTAs of 512 threads for one or two columns (100 -> 9 us).
+// The line: f^2 c / 2 FMAs on one SM are 0.3 ms in FP64 at 2^21, about what the tile
+// tasks of one such front take end to end; the rule looks at the front alone, so a
+// problem's arithmetic does not depend on its cohort.
+constexpr int64_t kThinPivots = 16, kThinWork = (int64_t)1 << 21;
+inline bool ldl_thin_front(int64_t f, int64_t c, int small_max) {
+  return f > small_max && c <= kThinPivots && f * f * c <= kThinWork;
+}
 
 // pos_pid: problem of each elimination position (null: one problem).
 int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<int8_t>& dsign,

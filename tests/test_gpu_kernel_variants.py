@@ -77,3 +77,37 @@ def test_psd_step_lane_equals_thread(orders):
     few = clr.clr_cones_step_length(cones, *[cat(v, 1) for v in (s, z, ds, dz)], 1e6)
     many = clr.clr_cones_step_length(cones * reps, *[cat(v, reps) for v in (s, z, ds, dz)], 1e6)
     assert few == many == min(ref)
+
+
+# fronts of few pivots and many rows (k_factor_thin) and long pull lists: an arrow matrix
+# of `leaves` cliques of c pivots on r of the m root rows (leaf fronts of c + r rows)
+@pytest.mark.parametrize("bits", [64, 32])
+@pytest.mark.parametrize("leaves,c,r,m,extra", [
+    (3, 1, 130, 140, 0), (60, 2, 129, 200, 0), (60, 3, 192, 260, 4), (700, 1, 191, 193, 0),
+    (49, 16, 300, 330, 0), (20, 5, 256, 300, 9), (9000, 1, 128, 129, 0), (6, 17, 140, 160, 0)])
+def test_thin_fronts_and_long_pulls(bits, leaves, c, r, m, extra):
+    import scipy.sparse as sp
+    rng = np.random.default_rng(leaves + r)
+    N = leaves * (c + extra) + m
+    R, Cc, V = [], [], []
+    root = N - m
+    # with extra: a first clique of `extra` pivots under each leaf, so that the thin front has a child
+    for q in range(leaves):
+        p0 = q * (c + extra)
+        piv = np.arange(p0, p0 + extra + c)
+        for a in piv:
+            low = piv[piv > a]
+            R += list(low); Cc += [a] * len(low); V += list(0.1 * rng.standard_normal(len(low)))
+        rows = root + np.sort(rng.choice(m, r, replace=False))
+        for a in piv[extra:]:
+            R += list(rows); Cc += [a] * r; V += list(rng.standard_normal(r) / np.sqrt(leaves * r))
+    K = sp.csc_matrix((V, (R, Cc)), shape=(N, N))
+    sgn = np.where(np.arange(N) < root, 1.0, -1.0)
+    K = sp.tril(K, -1) + sp.diags(sgn * (2.0 + rng.random(N)))
+    rhs = rng.standard_normal(N)
+    x, D, hits = clr.clr_ldl_solve(K, sgn, rhs, order=np.arange(N), factor_bits=bits)
+    Kf = K + sp.tril(K, -1).T
+    # diagonally dominant quasi-definite blocks, growth < 10: backward error of the order of (sources + rows) eps
+    eps = 2.2e-16 if bits == 64 else 1.2e-7
+    assert np.abs(Kf @ x - rhs).max() <= 10 * np.sqrt(N) * eps * max(1.0, np.abs(x).max()) * 10
+    assert hits == 0 and np.all(sgn * D > 0)

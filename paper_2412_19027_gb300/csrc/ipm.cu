@@ -24,15 +24,13 @@
 #include <mutex>
 
 #include "ipm.cuh"
+#include "kmv.cuh"
 
 namespace clr {
 
 // ------------------------------------------------------------------ slots
 enum SumSlot { S_XPX = 0, S_QX, S_BZ, S_SZ, S_D0, S_D1, S_D2, S_NSLOT };
 enum MaxSlot { M_RD = 0, M_X, M_RP, M_S, M_Z, M_ATZ, M_PX, M_AXS, M_GS, M_NMAX };
-
-__device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
-__device__ __forceinline__ double bitsd(unsigned long long b) { return __longlong_as_double((long long)b); }
 
 // Launch geometry of the chunked kernels: one block per chunk, x chunks first.
 struct ChunkGrid {
@@ -74,7 +72,6 @@ __global__ void k_kmv(int mode, int64_t r0, int64_t r1, int64_t n, const int64_t
                       const double* __restrict__ rhs, double* __restrict__ out, const int32_t* __restrict__ pid,
                       IterScal* sc, const int* skip) {
   if (skip && *skip) return;
-  constexpr int NU = 32 / G;  // partial sums per lane: t = lane + G u
   const int lane = threadIdx.x % G;
   // the G lanes of a row group share its trip count: shuffles name only their own group
   const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
@@ -82,61 +79,20 @@ __global__ void k_kmv(int mode, int64_t r0, int64_t r1, int64_t n, const int64_t
   const int64_t gstride = ((int64_t)gridDim.x * blockDim.x) / G;
   RunExt<true> mx;
   for (int64_t i = r0 + gid; i < r1; i += gstride) {
-    double a[NU], b[NU];
-#pragma unroll
-    for (int u = 0; u < NU; ++u) a[u] = b[u] = 0.0;
     const int64_t p0 = kptr[i], p1 = kptr[i + 1];
     if (p1 - p0 > kLongRow) continue;  // k_kmv_long (the whole G-lane group skips)
-    // four 32-entry steps per pass: all loads of the pass issued before the adds,
-    // which keep the order of the plain one-step loop (partial t sums entries
-    // p = p0 + t (mod 32) in increasing p)
-    for (int64_t base = p0; base < p1; base += 128) {
-      double tv[4][NU];
-      bool tx[4][NU];
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int u = 0; u < NU; ++u) {
-          const int64_t p = base + 32 * k + lane + G * u;
-          tv[k][u] = 0.0;
-          tx[k][u] = true;
-          if (p < p1) {
-            const int32_t c = kcol[p];
-            tv[k][u] = (i < n ? kfv[p] : kval[kvi[p]]) * v[c];
-            tx[k][u] = c < n;
-          }
-        }
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int u = 0; u < NU; ++u) {
-          if (base + 32 * k + lane + G * u >= p1) continue;
-          if (tx[k][u]) a[u] += tv[k][u];
-          else b[u] += tv[k][u];
-        }
-    }
-#pragma unroll
-    for (int off = 16; off >= G; off >>= 1)
-#pragma unroll
-      for (int u = 0; u < off / G; ++u) {
-        a[u] += a[u + off / G];
-        b[u] += b[u + off / G];
-      }
-#pragma unroll
-    for (int off = (G == 32 ? 16 : G / 2); off > 0; off >>= 1) {
-      a[0] += __shfl_xor_sync(gmask, a[0], off, G);
-      b[0] += __shfl_xor_sync(gmask, b[0], off, G);
-    }
+    double a, b;
+    kmv_row<G>(i, p0, p1, n, kcol, kvi, kval, kfv, v, lane, gmask, a, b);
     if (lane == 0) {
       if (mode == 0) {
-        lo[i] = a[0];
-        hi[i] = b[0];
+        lo[i] = a;
+        hi[i] = b;
       } else if (mode == 1) {
-        const double r = rhs[i] - (a[0] + b[0]);
+        const double r = rhs[i] - (a + b);
         out[i] = r;
         mx.add(sc, &IterScal::rnorm_bits, pid[i], dbits(fabs(r)));
       } else {
-        out[i - n] = -rhs[i - n] + b[0];
+        out[i - n] = -rhs[i - n] + b;
       }
     }
   }
@@ -478,42 +434,6 @@ __global__ void k_set_from(ChunkGrid g, double* __restrict__ dst, const T* __res
   if (add && sc[pid].ir_skip) return;
   for (int64_t i = i0 + threadIdx.x; i < i0 + len; i += blockDim.x)
     dst[i] = add ? dst[i] + (double)src[i] : (double)src[i];
-}
-
-// Refinement test of one problem (Sec. 3.6): stop at the tolerance, or after
-// max_steps steps, or, when stop_ratio > 0 and ||r||_inf is already below the
-// acceptance bar fail_tol = 1e-4 max(1, ||rhs||_inf), as soon as a step has
-// reduced ||r||_inf by less than stop_ratio (the last correction is kept).  A
-// step that made ||r||_inf larger is undone (k_ir_revert) and ends the
-// refinement: the regularised factor is not a contraction for K there.
-// A refinement that ends above fail_tol marks the iteration (ir_fail = 1; 2 if
-// the residual is not finite): with a low-precision factor it is then redone in
-// FP64; in FP64 a non-finite solve stops the solve at the current iterate.
-__device__ bool ir_step_due(IterScal& q, double abstol, double reltol, double stop_ratio, int max_steps) {
-  const double r = bitsd(q.rnorm_bits);
-  q.rnorm_bits = 0ull;
-  q.ir_revert = 0;
-  if (q.ir_skip) return false;
-  const double fail_tol = 1e-4 * fmax(1.0, q.rhs_norm);
-  const double tol = abstol + reltol * q.rhs_norm;
-  if (r > q.ir_prev) {
-    q.ir_revert = 1;
-    q.ir_skip = 1;
-    if (!(q.ir_prev <= fail_tol)) q.ir_fail = max(q.ir_fail, isfinite(q.ir_prev) ? 1 : 2);
-    if (q.ir_prev > tol) q.ir_worst = fmax(q.ir_worst, q.ir_prev);
-    return false;
-  }
-  const bool stalled = stop_ratio > 0 && r <= fail_tol && !(r * stop_ratio < q.ir_prev);
-  q.ir_prev = r;
-  if (!(r > tol) || stalled || q.ir_cur >= max_steps) {  // NaN also stops
-    q.ir_skip = 1;
-    if (!(r <= fail_tol)) q.ir_fail = max(q.ir_fail, isfinite(r) ? 1 : 2);  // 2: a non-finite solve
-    if (r > tol) q.ir_worst = fmax(q.ir_worst, r);
-    return false;
-  }
-  q.ir_cur += 1;
-  q.ir_total += 1;
-  return true;
 }
 
 // Undo the last correction of the problems whose residual it made larger.
@@ -1087,6 +1007,34 @@ int Solver::upload() {
       if (!fv.empty() && !v_.kfv) return CLR_E_OOM;
     }
     const double avg = N ? (double)cnt[N] / (double)N : 1.0;
+    // one CTA per problem: rows summed by lane groups only, and a bounded number of entries each
+    cta_solve_ = ls_.cta.n > 0 && h_long_.empty() && cnt[N] <= kCtaWork * B && cnt[N] < ((int64_t)1 << 31);
+    if (cta_solve_) {
+      // rows by problem (elimination positions are contiguous there), shortest class first
+      std::vector<int4> kr;
+      std::vector<int32_t> ends;
+      kr.reserve(N);
+      for (int64_t k0 = 0; k0 < N;) {
+        int64_t k1 = k0 + 1;
+        while (k1 < N && pos_pid[k1] == pos_pid[k0]) ++k1;
+        std::vector<std::vector<int4>> cls(kKrowClasses);
+        for (int64_t k = k0; k < k1; ++k) {
+          const int64_t i = sy.perm[k];
+          cls[krow_class(cnt[i + 1] - cnt[i])].push_back(make_int4((int)i, (int)cnt[i], (int)cnt[i + 1], 0));
+        }
+        for (const auto& c : cls) {
+          kr.insert(kr.end(), c.begin(), c.end());
+          ends.push_back((int32_t)((int64_t)kr.size() - k0));
+        }
+        k0 = k1;
+      }
+      v_.krow = ar_.upload(kr.data(), N);
+      v_.kcls = ar_.upload(ends.data(), (int64_t)ends.size());
+      v_.rhs2 = ar_.alloc_n<double>(N);
+      v_.r2 = ar_.alloc_n<double>(N);
+      if (!v_.kcls || !v_.rhs2 || !v_.r2) return CLR_E_OOM;
+      if (!v_.krow) return CLR_E_OOM;
+    }
     csr_group_ = avg > 24 ? 32 : (avg > 12 ? 16 : (avg > 6 ? 8 : 4));
   }
   // cohort layout
@@ -1232,6 +1180,16 @@ int Solver::factor() {
   return f32_.factor(stream_, v_.kval, sc_, reg_dyn_eps(), reg_dyn_delta(), halt);
 }
 
+// Small problems: the refined solves of one or two independent right-hand sides in one
+// launch, a CTA per problem and side.
+int Solver::kkt_solve_cta(const CtaRhs& a, const CtaRhs& b) {
+  const KmvArgs ka{hp.n, v_.kptr, v_.kcol, v_.kvi, v_.kval, v_.kfv, v_.krow, v_.kcls};
+  const IrParams ir{st.ir_abstol, st.ir_reltol, st.ir_stop_ratio, st.ir_max_steps};
+  const int* halt = &bf_->all_halt;
+  return use64() ? CtaOps<double>::kkt_solve(stream_, ls_.cta, ka, f64_.F, f64_.Dp, a, b, sc_, ir, halt)
+                 : CtaOps<float>::kkt_solve(stream_, ls_.cta, ka, f32_.F, f32_.Dp, a, b, sc_, ir, halt);
+}
+
 // sol = K^{-1} rhs by the factor plus iterative refinement on the unregularised K (FP64),
 // per problem.  While a graph is being captured the refinement loop is a conditional
 // WHILE node (its body runs only while some problem needs another step); otherwise it
@@ -1244,6 +1202,7 @@ int Solver::kkt_solve(const double* rhs, double* sol) {
   const ChunkGrid cg{v_.ck, nckx_, pst_, hp.n};
   const unsigned nck = (unsigned)(nckx_ + nckz_);
   const int pg = grid_for(B, 128);
+  if (cta_solve_) return kkt_solve_cta(CtaRhs{rhs, sol, v_.r}, CtaRhs{});
   k_inf_norm<<<nck, 256, 0, s>>>(cg, rhs, sc_, halt);
   k_ir_begin<<<pg, 128, 0, s>>>(sc_, B, bf_);
   auto revert = [&](cudaStream_t ss) {
@@ -1354,7 +1313,7 @@ void kmv(int G, cudaStream_t s, int mode, int64_t r0, int64_t r1, int64_t n, con
 // One search direction: solve with the current right-hand side (rhs built by
 // k_rhs), Delta tau, Delta x/z, Delta s = -d_s - H Delta z (PSD blocks of H in
 // factored form).
-int Solver::direction(bool affine) {
+int Solver::direction(bool affine, bool solved) {
   const int64_t n = hp.n, m = hp.m, N = n + m, B = lay.B;
   cudaStream_t s = stream_;
   const int* halt = &bf_->all_halt;
@@ -1362,7 +1321,7 @@ int Solver::direction(bool affine) {
   const unsigned nck = (unsigned)(nckx_ + nckz_);
   double* dir = affine ? v_.dir_a : v_.dir;
   double* ds = affine ? v_.dsa : v_.ds;
-  int rc = kkt_solve(v_.rhs, v_.sol1);
+  int rc = solved ? CLR_OK : kkt_solve(v_.rhs, v_.sol1);
   if (rc) return rc;
   DotArgs da{{v_.qp, v_.b, nullptr}, {v_.sol1, v_.sol1 + n, nullptr}, {1, 0, 0}, 2};
   k_dots<<<nck, 256, 0, s>>>(cg, da, v_.part, S_D0, halt);
@@ -1437,16 +1396,26 @@ int Solver::iteration() {
   if (rc) return rc;
   mark(4);
   // ---- constant right-hand side [-q; b] ----
-  k_build_rhs<<<nck, 256, 0, s>>>(cg, v_.rhs, v_.q, v_.b, 2, halt);
-  rc = kkt_solve(v_.rhs, v_.sol2);
+  // (small problems: together with the affine one, which does not depend on it)
+  const bool pair = cta_solve_;
+  k_build_rhs<<<nck, 256, 0, s>>>(cg, pair ? v_.rhs2 : v_.rhs, v_.q, v_.b, 2, halt);
+  if (pair) {
+    CLR_CUDA(cudaMemcpyAsync(v_.dsrhs, v_.s, sizeof(double) * (size_t)m, cudaMemcpyDeviceToDevice, s));
+    k_rhs<<<nck, 256, 0, s>>>(cg, v_.rhs, v_.G, v_.dsrhs, sc_, B, 1, halt);
+    rc = kkt_solve_cta(CtaRhs{v_.rhs2, v_.sol2, v_.r2}, CtaRhs{v_.rhs, v_.sol1, v_.r});
+  } else {
+    rc = kkt_solve(v_.rhs, v_.sol2);
+  }
   if (rc) return rc;
   DotArgs da{{v_.qp, v_.b, nullptr}, {v_.sol2, v_.sol2 + n, nullptr}, {1, 0, 0}, 2};
   k_dots<<<nck, 256, 0, s>>>(cg, da, v_.part, S_D0, halt);
   k_fin_const<<<(unsigned)B, 128, 0, s>>>(sc_, v_.part, pst_, v_.ckx_ptr, v_.ckz_ptr, halt);
   // ---- step 6: affine direction, d = (G, d_s = s, d_kappa = kappa tau) ----
-  CLR_CUDA(cudaMemcpyAsync(v_.dsrhs, v_.s, sizeof(double) * (size_t)m, cudaMemcpyDeviceToDevice, s));
-  k_rhs<<<nck, 256, 0, s>>>(cg, v_.rhs, v_.G, v_.dsrhs, sc_, B, 1, halt);
-  rc = direction(true);
+  if (!pair) {
+    CLR_CUDA(cudaMemcpyAsync(v_.dsrhs, v_.s, sizeof(double) * (size_t)m, cudaMemcpyDeviceToDevice, s));
+    k_rhs<<<nck, 256, 0, s>>>(cg, v_.rhs, v_.G, v_.dsrhs, sc_, B, 1, halt);
+  }
+  rc = direction(true, pair);
   if (rc) return rc;
   // ---- steps 7-8: affine step length, sigma ----
   rc = step_length(false);
@@ -1455,7 +1424,7 @@ int Solver::iteration() {
   rc = cones_combined_ds(s, cd_, v_.s, v_.xz + n, v_.dsa, v_.dir_a + n, sc_, v_.dsrhs, halt);
   if (rc) return rc;
   k_rhs<<<nck, 256, 0, s>>>(cg, v_.rhs, v_.G, v_.dsrhs, sc_, B, 0, halt);
-  rc = direction(false);
+  rc = direction(false, false);
   if (rc) return rc;
   // ---- step 10: combined step length with the neighbourhood check ----
   rc = step_length(true);
@@ -1488,13 +1457,21 @@ int Solver::initialise() {
     rc = factor();
     if (rc) return rc;
     k_build_rhs<<<nck, 256, 0, s>>>(cg, v_.rhs, v_.q, v_.b, 0, nullptr);
-    rc = kkt_solve(v_.rhs, v_.sol1);
-    if (rc) return rc;
-    k_init_take<<<nck, 256, 0, s>>>(cg, v_.xz, v_.s, v_.sol1, v_.pc, 0);
-    k_build_rhs<<<nck, 256, 0, s>>>(cg, v_.rhs, v_.q, v_.b, 1, nullptr);
-    rc = kkt_solve(v_.rhs, v_.sol1);
-    if (rc) return rc;
-    k_init_take<<<nck, 256, 0, s>>>(cg, v_.xz, v_.s, v_.sol1, v_.pc, 1);
+    if (cta_solve_) {
+      k_build_rhs<<<nck, 256, 0, s>>>(cg, v_.rhs2, v_.q, v_.b, 1, nullptr);
+      rc = kkt_solve_cta(CtaRhs{v_.rhs, v_.sol1, v_.r}, CtaRhs{v_.rhs2, v_.sol2, v_.r2});
+      if (rc) return rc;
+      k_init_take<<<nck, 256, 0, s>>>(cg, v_.xz, v_.s, v_.sol1, v_.pc, 0);
+      k_init_take<<<nck, 256, 0, s>>>(cg, v_.xz, v_.s, v_.sol2, v_.pc, 1);
+    } else {
+      rc = kkt_solve(v_.rhs, v_.sol1);
+      if (rc) return rc;
+      k_init_take<<<nck, 256, 0, s>>>(cg, v_.xz, v_.s, v_.sol1, v_.pc, 0);
+      k_build_rhs<<<nck, 256, 0, s>>>(cg, v_.rhs, v_.q, v_.b, 1, nullptr);
+      rc = kkt_solve(v_.rhs, v_.sol1);
+      if (rc) return rc;
+      k_init_take<<<nck, 256, 0, s>>>(cg, v_.xz, v_.s, v_.sol1, v_.pc, 1);
+    }
     rc = cones_shift_init(s, cd_, v_.s, sc_, nullptr);
     if (rc) return rc;
     rc = cones_shift_init(s, cd_, v_.xz + n, sc_, nullptr);

@@ -37,6 +37,9 @@ struct VecDev {
   double *kval;              // KKT values (x part constant, z part = -H)
   int64_t *kptr;             // full-K CSR (both triangles), values through kvi
   int32_t *kcol, *kvi;
+  const int4* krow = nullptr;  // one-CTA solves: KKT rows and their CSR ranges by problem and length class
+  const int32_t* kcls = nullptr;
+  double *rhs2 = nullptr, *r2 = nullptr;  // one-CTA solves: a second right-hand side and its residual
   int32_t* pid;              // KKT index -> problem
   Chunk* ck;                 // x chunks then z chunks (z begins are row indices)
   int64_t *ckx_ptr, *ckz_ptr;
@@ -105,6 +108,7 @@ class Solver {
   int64_t nckx_ = 0, nckz_ = 0, pst_ = 1;
   int hist_rows_ = 0;
   int csr_group_ = 32;
+  bool cta_solve_ = false;  // refined KKT solves by one CTA per problem (kktcta.cuh)
   std::vector<int64_t> h_long_;  // KKT rows handled by k_kmv_long
   std::vector<int32_t> h_kfv_src_;  // kval index of each entry of the x rows' full-CSR values (kfv)
   // iteration graphs per factor precision (0: configured, 1: FP64 after an escalation)
@@ -142,7 +146,8 @@ class Solver {
   int kkt_solve(const double* rhs, double* sol);
   int iteration();
   int initialise();
-  int direction(bool affine);
+  int kkt_solve_cta(const CtaRhs& a, const CtaRhs& b);
+  int direction(bool affine, bool solved);
   int step_length(bool combined);
   int launch_iteration();
 };

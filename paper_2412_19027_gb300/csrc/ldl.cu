@@ -15,8 +15,10 @@
 // the ancestors' solution gathered by KKT index).
 #include <algorithm>
 #include <queue>
+#include <type_traits>
 #include <unordered_map>
 
+#include "frontfac.cuh"
 #include "ldl.cuh"
 
 namespace clr {
@@ -38,25 +40,52 @@ __global__ void k_add_reg(T* __restrict__ F, const int64_t* __restrict__ diag_po
     F[diag_pos[k]] += (T)(dsign[k] * sc[pos_pid[k]].delta);
 }
 
-// Longest source list a single thread sums (k_pull_long beyond), and the longest that
-// a warp sums: the factor's lists are as many as a front's entries, the solves' as its
-// rows, so those go to a CTA earlier.
-constexpr int64_t kPullShort = 48, kFaWarp = 8192, kSvWarp = 512;
-
+// Targets with up to `most` sources, a thread each, summed in list order (eight gathers
+// in flight); the others are k_pull_warp's and k_pull_long's.
 template <typename T>
 __global__ void k_pull(T* __restrict__ X, const int64_t* __restrict__ tgt, const int64_t* __restrict__ ptr,
-                       const int64_t* __restrict__ src, int64_t t0, int64_t t1, const int* skip) {
+                       const int64_t* __restrict__ src, int64_t t0, int64_t t1, int64_t most, const int* skip) {
   if (skip && *skip) return;
   for (int64_t t = t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < t1; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t q0 = ptr[t], q1 = ptr[t + 1];
-    if (q1 - q0 > kPullShort) continue;  // k_pull_long
+    int64_t q = ptr[t];
+    const int64_t q1 = ptr[t + 1];
+    if (q1 - q > most) continue;
     T acc = X[tgt[t]];
-    for (int64_t q = q0; q < q1; ++q) acc += X[src[q]];
+    for (; q + 8 <= q1; q += 8) {
+      T v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = X[src[q + u]];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc += v[u];
+    }
+    for (; q < q1; ++q) acc += X[src[q]];
     X[tgt[t]] = acc;
   }
 }
 
-// Targets with more than kPullShort sources, G threads (32 or 256) per target: a
+// A warp per target, the sum in list order: 32 entries are gathered at once and added
+// one after the other (the thread's own serial gather waits for L2 on every entry).
+template <typename T>
+__global__ void __launch_bounds__(256) k_pull_warp(T* __restrict__ X, const int64_t* __restrict__ tgt,
+                                                   const int64_t* __restrict__ ptr, const int64_t* __restrict__ src,
+                                                   const int64_t* __restrict__ ids, int64_t n, const int* skip) {
+  if (skip && *skip) return;
+  const int lane = threadIdx.x & 31;
+  for (int64_t i = (blockIdx.x * (int64_t)256 + threadIdx.x) / 32; i < n; i += (int64_t)gridDim.x * 8) {
+    const int64_t t = ids[i], q0 = ptr[t], q1 = ptr[t + 1], tg = tgt[t];
+    T acc = X[tg];
+    T nx = q0 + lane < q1 ? X[src[q0 + lane]] : (T)0;
+    for (int64_t q = q0; q < q1; q += 32) {
+      const T v = nx;
+      nx = q + 32 + lane < q1 ? X[src[q + 32 + lane]] : (T)0;
+      const int m = (int)min((int64_t)32, q1 - q);
+      for (int k = 0; k < m; ++k) acc += __shfl_sync(0xffffffffu, v, k);
+    }
+    if (lane == 0) X[tg] = acc;
+  }
+}
+
+// Targets with more than kPullSerial sources, G threads (32 or 256) per target: a
 // thread's serial gather is one dependent L2 access after another (5000 sources: the
 // forward sweep of the portfolio n = 5000 root spent 384 us per solve in it, now 7; its
 // extend-add of 1.6e8 sources 1.5 -> 1.2 ms) and its
@@ -99,11 +128,14 @@ __global__ void __launch_bounds__(256) k_pull_long(T* __restrict__ X, const int6
   }
 }
 
-// One level's pulls.
+// One level's pulls: `most` sources by a thread, the lists by a warp in order, a warp and a CTA.
 template <typename T>
 static void pull_level(cudaStream_t stm, T* X, const int64_t* tgt, const int64_t* ptr, const int64_t* src, int64_t t0,
-                       int64_t t1, const LdlStructure::List& wl, const LdlStructure::List& cl, const int* skip) {
-  if (t1 - t0 > wl.n + cl.n) k_pull<T><<<grid_for(t1 - t0, 256), 256, 0, stm>>>(X, tgt, ptr, src, t0, t1, skip);
+                       int64_t t1, int64_t most, const LdlStructure::List& ol, const LdlStructure::List& wl,
+                       const LdlStructure::List& cl, const int* skip) {
+  if (t1 - t0 > ol.n + wl.n + cl.n)
+    k_pull<T><<<grid_for(t1 - t0, 256), 256, 0, stm>>>(X, tgt, ptr, src, t0, t1, most, skip);
+  if (ol.n > 0) k_pull_warp<T><<<grid_for(ol.n * 32, 256), 256, 0, stm>>>(X, tgt, ptr, src, ol.id, ol.n, skip);
   if (wl.n > 0) k_pull_long<T, 32><<<grid_for(wl.n * 32, 256), 256, 0, stm>>>(X, tgt, ptr, src, wl.id, wl.n, skip);
   if (cl.n > 0) k_pull_long<T, 256><<<grid_for(cl.n * 256, 256), 256, 0, stm>>>(X, tgt, ptr, src, cl.id, cl.n, skip);
 }
@@ -141,55 +173,64 @@ __global__ void k_push(T* __restrict__ F, WorkList wl, const int64_t* __restrict
   }
 }
 
-template <typename T>
-__device__ __forceinline__ T regularise(T d, int sgn, T eps, T delta, bool* hit) {
-  if ((T)sgn * d <= eps) {
-    *hit = true;
-    return (T)sgn * delta;
-  }
-  *hit = false;
-  return d;
-}
-
-// One CTA per front with f <= small_max: whole front in shared memory.
-template <typename T>
-__global__ void k_factor_small(T* __restrict__ F, T* __restrict__ Dp, const int64_t* __restrict__ fronts,
-                               const int64_t* __restrict__ sn_ptr, const int64_t* __restrict__ row_ptr,
-                               const int64_t* __restrict__ front_off, const int8_t* __restrict__ dsign,
-                               double eps_d, double delta_d, int* dyn_hits, const int* skip) {
+// One CTA per front with f <= small_max: the front in registers (frontfac.cuh), or, above
+// 128 rows, in shared memory.  GW warps and MF: 4 and 32 when a level's fronts have at most 32
+// rows, else 8 and the class of its largest front (64, 96, 128 or beyond), so that the
+// registers of the largest class are only taken by levels that need them.
+template <typename T, int GW, int MF>
+__global__ void __launch_bounds__(32 * GW) k_factor_small(T* __restrict__ F, T* __restrict__ Dp,
+                                                          const int64_t* __restrict__ fronts,
+                                                          const int64_t* __restrict__ sn_ptr,
+                                                          const int64_t* __restrict__ row_ptr,
+                                                          const int64_t* __restrict__ front_off,
+                                                          const int8_t* __restrict__ dsign, double eps_d,
+                                                          double delta_d, int* dyn_hits, const int* skip) {
   if (skip && *skip) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* S = reinterpret_cast<T*>(smraw);
-  __shared__ T dsh;
   const int64_t J = fronts[blockIdx.x];
   const int c = (int)(sn_ptr[J + 1] - sn_ptr[J]);
   const int f = (int)(row_ptr[J + 1] - row_ptr[J]);
   T* G = F + front_off[J];
   const int64_t k0 = sn_ptr[J];
   const T eps = (T)eps_d, delta = (T)delta_d;
-  for (int q = threadIdx.x; q < f * f; q += blockDim.x) S[q] = G[q];
-  __syncthreads();
-  for (int k = 0; k < c; ++k) {
-    if (threadIdx.x == 0) {
-      bool hit;
-      T d = regularise(S[k + k * f], (int)dsign[k0 + k], eps, delta, &hit);
-      if (hit) atomicAdd(dyn_hits, 1);
-      S[k + k * f] = d;
-      Dp[k0 + k] = d;
-      dsh = d;
-    }
-    __syncthreads();
-    const T inv = (T)1 / dsh;
-    const int m = f - k - 1;
-    for (int q = threadIdx.x; q < m * m; q += blockDim.x) {
-      const int i = k + 1 + q % m, j = k + 1 + q / m;
-      if (i >= j) S[i + j * f] -= S[i + k * f] * S[j + k * f] * inv;
-    }
-    __syncthreads();
-    for (int i = k + 1 + threadIdx.x; i < f; i += blockDim.x) S[i + k * f] *= inv;
-    __syncthreads();
+  for (int q = threadIdx.x; q < f * f; q += 32 * GW) S[q] = G[q];
+  if constexpr (GW == 4) {
+    factor_front32<T, 4>(S, G, Dp + k0, dsign + k0, c, f, eps, delta, dyn_hits, 0);
+    return;
+  } else {
+    if (f <= 32) return factor_regs<T, 3, 8>(S, G, Dp + k0, dsign + k0, c, f, eps, delta, dyn_hits, 0);
+    if (f <= 64) return factor_regs<T, 9, 8>(S, G, Dp + k0, dsign + k0, c, f, eps, delta, dyn_hits, 0);
+    if constexpr (MF > 64)
+      if (f <= 96) return factor_regs<T, 19, 8>(S, G, Dp + k0, dsign + k0, c, f, eps, delta, dyn_hits, 0);
+    if constexpr (MF > 96)
+      if (f <= 128) return factor_regs<T, 33, 8>(S, G, Dp + k0, dsign + k0, c, f, eps, delta, dyn_hits, 0);
   }
-  for (int q = threadIdx.x; q < f * f; q += blockDim.x) G[q] = S[q];
+  if constexpr (MF > 128) {
+    __shared__ T ish;
+    __syncthreads();
+    for (int k = 0; k < c; ++k) {
+      if (threadIdx.x == 0) {
+        bool hit;
+        T d = regularise(S[k + k * f], (int)dsign[k0 + k], eps, delta, &hit);
+        if (hit) atomicAdd(dyn_hits, 1);
+        S[k + k * f] = d;
+        Dp[k0 + k] = d;
+        ish = rcp_exact(d);
+      }
+      __syncthreads();
+      const T inv = ish;
+      const int m = f - k - 1;
+      for (int q = threadIdx.x; q < m * m; q += 32 * GW) {
+        const int i = k + 1 + q % m, j = k + 1 + q / m;
+        if (i >= j) S[i + j * f] = elim(S[i + j * f], S[i + k * f], S[j + k * f], inv);
+      }
+      __syncthreads();
+      for (int i = k + 1 + threadIdx.x; i < f; i += 32 * GW) S[i + k * f] *= inv;
+      __syncthreads();
+    }
+    for (int q = threadIdx.x; q < f * f; q += 32 * GW) G[q] = S[q];
+  }
 }
 
 // One CTA per thin front (ldl_thin_front): its c columns in shared memory as they are
@@ -616,16 +657,26 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
     std::vector<char> has_child(sy.nsn, 0);
     for (int64_t J = 0; J < sy.nsn; ++J)
       if (sy.sn_parent[J] >= 0) has_child[sy.sn_parent[J]] = 1;
-    auto longs = [&](const std::vector<int64_t>& ptr, int64_t t0, int64_t t1, int64_t warp_max, std::vector<List>& wl,
-                     std::vector<List>& cl, int64_t l) {
-      std::vector<int64_t> w, c;
+    // long lists of a level's targets: in order by a warp (over `thread`), by a warp (over
+    // kPullSerial), by a CTA (over `warp`)
+    auto longs = [&](const std::vector<int64_t>& ptr, int64_t t0, int64_t t1, int64_t thread, int64_t warp,
+                     std::vector<List>& ol, std::vector<List>& wl, std::vector<List>& cl, int64_t l) {
+      std::vector<int64_t> o, w, c;
       for (int64_t t = t0; t < t1; ++t) {
         const int64_t n = ptr[t + 1] - ptr[t];
-        if (n > kPullShort) (n > warp_max ? c : w).push_back(t);
+        if (n > thread) (n <= kPullSerial ? o : (n <= warp ? w : c)).push_back(t);
       }
+      add(ol, l, o);
       add(wl, l, w);
       add(cl, l, c);
     };
+    // thin fronts of each problem: the path is taken by problems with many of them
+    std::vector<int64_t> nthin(1, 0);
+    auto pid_of = [&](int64_t J) -> size_t { return pos_pid ? (size_t)(*pos_pid)[sy.sn_ptr[J]] : 0; };
+    for (int64_t J = 0; J < sy.nsn; ++J) {
+      if (pid_of(J) >= nthin.size()) nthin.resize(pid_of(J) + 1, 0);
+      nthin[pid_of(J)] += ldl_thin_front(sy.row_ptr[J + 1] - sy.row_ptr[J], sy.sn_ptr[J + 1] - sy.sn_ptr[J], small_max);
+    }
     std::vector<int64_t> small, leaf, thin, both;
     for (int64_t l = 0; l < sy.nlev; ++l) {
       small.clear();
@@ -638,7 +689,7 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
         if (f <= small_max) {
           small.push_back(J);
           st.lev_small_maxf[l] = std::max(st.lev_small_maxf[l], (int)f);
-        } else if (ldl_thin_front(f, c, small_max)) {
+        } else if (nthin[pid_of(J)] >= kThinCount && ldl_thin_front(f, c, small_max)) {
           (has_child[J] ? thin : leaf).push_back(J);
           st.lev_thin_smem[l] = std::max(st.lev_thin_smem[l], f * c);
         } else {
@@ -651,8 +702,8 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       add(st.lev_thin_leaf, l, leaf);
       add(st.lev_thin, l, thin);
       add(st.lev_cta, l, both);
-      longs(mp.fa_ptr, mp.fa_lev_ptr[l], mp.fa_lev_ptr[l + 1], kFaWarp, st.fa_warp, st.fa_cta, l);
-      longs(mp.sv_ptr, mp.sv_lev_ptr[l], mp.sv_lev_ptr[l + 1], kSvWarp, st.sv_warp, st.sv_cta, l);
+      longs(mp.fa_ptr, mp.fa_lev_ptr[l], mp.fa_lev_ptr[l + 1], kPullSerial, kFaWarp, st.fa_ord, st.fa_warp, st.fa_cta, l);
+      longs(mp.sv_ptr, mp.sv_lev_ptr[l], mp.sv_lev_ptr[l + 1], kSvThread, kPullSerial, st.sv_ord, st.sv_warp, st.sv_cta, l);
     }
     int64_t* dbuf = buf.empty() ? nullptr : ar.upload(buf.data(), (int64_t)buf.size());
     if (!buf.empty() && !dbuf) return CLR_E_OOM;
@@ -909,7 +960,7 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       !st.dsign || !st.pos_pid || !st.kdest || !st.diag_pos || !st.fa_tgt || !st.fa_ptr || !st.fa_src || !st.sv_tgt ||
       !st.sv_ptr || !st.sv_src)
     return CLR_E_OOM;
-  return CLR_OK;
+  return cta_plan_build(ar, sy, mp, small_max, pos_pid, st.w_init, st.cta);
 }
 
 template <typename T>
@@ -926,6 +977,7 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
   Linv = ar.alloc_n<T>(st.bfd.n * 2 * kBfNB * kBfNB);
   if (!F || !Dp || !w || !xs || !dyn_hits || !E || !ybuf || !Linv) return CLR_E_OOM;
   if (BigFrontOps<T>::setup_attributes() != CLR_OK) return CLR_E_CUDA;
+  if (st.cta.n > 0 && CtaOps<T>::setup_attributes() != CLR_OK) return CLR_E_CUDA;
   if (st.flow_words > 0) {
     flow_state = ar.alloc_n<int>(st.flow_words);
     if (!flow_state) return CLR_E_OOM;
@@ -948,7 +1000,9 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
   }
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(k_factor_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_factor_small<T, 8, 96>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    cudaFuncSetAttribute(k_factor_small<T, 8, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    cudaFuncSetAttribute(k_factor_small<T, 8, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     cudaFuncSetAttribute(k_factor_thin<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
     cudaFuncSetAttribute(k_factor_thin<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
     attr_set = true;
@@ -968,19 +1022,31 @@ int LdlFactor<T>::factor(cudaStream_t stm, const double* kval, const IterScal* s
   k_scatter_kval<T><<<grid_for(S.nk, 256), 256, 0, stm>>>(F, kval, S.kdest, S.nk, skip);
   k_add_reg<T><<<grid_for(S.N, 256), 256, 0, stm>>>(F, S.diag_pos, S.dsign, S.pos_pid, S.N, sc, skip);
   CLR_CHECK_LAUNCH();
+  if (S.cta.n > 0 && S.cta.factor)
+    return CtaOps<T>::factor(stm, S.cta, F, Dp, S.dsign, S.fa_tgt, S.fa_ptr, S.fa_src, dyn_eps, dyn_delta, dyn_hits,
+                             skip);
   for (int64_t l = 0; l < S.nlev; ++l) {
-    pull_level<T>(stm, F, S.fa_tgt, S.fa_ptr, S.fa_src, S.h_fa_lev_ptr[l], S.h_fa_lev_ptr[l + 1], S.fa_warp[l],
-                  S.fa_cta[l], skip);
+    pull_level<T>(stm, F, S.fa_tgt, S.fa_ptr, S.fa_src, S.h_fa_lev_ptr[l], S.h_fa_lev_ptr[l + 1], kPullSerial,
+                  S.fa_ord[l], S.fa_warp[l], S.fa_cta[l], skip);
     for (const WorkList& wl : S.push_rounds[l])
       if (wl.nblocks > 0)
         k_push<T><<<(unsigned)wl.nblocks, 256, 0, stm>>>(F, wl, S.sn_ptr, S.row_ptr, S.front_off, S.sn_parent,
                                                           S.rel_off, S.rel, skip);
     if (S.lev_small[l].n > 0) {
       const int mf = S.lev_small_maxf[l];
-      const size_t smem = sizeof(T) * (size_t)mf * (size_t)mf;
-      const int threads = mf <= 16 ? 64 : (mf <= 48 ? 128 : 256);
-      k_factor_small<T><<<(unsigned)S.lev_small[l].n, threads, smem, stm>>>(
-          F, Dp, S.lev_small[l].id, S.sn_ptr, S.row_ptr, S.front_off, S.dsign, dyn_eps, dyn_delta, dyn_hits, skip);
+      const size_t smem = sizeof(T) * (size_t)front_words(mf);
+      const unsigned n = (unsigned)S.lev_small[l].n;
+      auto run = [&](auto gw, auto cls) {
+        constexpr int GW = decltype(gw)::value, MF = decltype(cls)::value;
+        k_factor_small<T, GW, MF><<<n, 32 * GW, smem, stm>>>(F, Dp, S.lev_small[l].id, S.sn_ptr, S.row_ptr, S.front_off,
+                                                             S.dsign, dyn_eps, dyn_delta, dyn_hits, skip);
+      };
+      using std::integral_constant;
+      if (mf <= 32) run(integral_constant<int, 4>{}, integral_constant<int, 32>{});
+      else if (mf <= 64) run(integral_constant<int, 8>{}, integral_constant<int, 64>{});
+      else if (mf <= 96) run(integral_constant<int, 8>{}, integral_constant<int, 96>{});
+      else if (mf <= 128) run(integral_constant<int, 8>{}, integral_constant<int, 128>{});
+      else run(integral_constant<int, 8>{}, integral_constant<int, 1024>{});
     }
     const size_t tsm = 2 * sizeof(T) * (size_t)S.lev_thin_smem[l];
     if (S.lev_thin_leaf[l].n > 0)
@@ -1014,8 +1080,8 @@ int LdlFactor<T>::solve(cudaStream_t stm, const double* rhs, const int* skip) co
   const LdlStructure& S = *s;
   k_init_w<T><<<grid_for(S.wtot, 256), 256, 0, stm>>>(w, S.w_init, rhs, S.wtot, skip);
   for (int64_t l = 0; l < S.nlev; ++l) {
-    pull_level<T>(stm, w, S.sv_tgt, S.sv_ptr, S.sv_src, S.h_sv_lev_ptr[l], S.h_sv_lev_ptr[l + 1], S.sv_warp[l],
-                  S.sv_cta[l], skip);
+    pull_level<T>(stm, w, S.sv_tgt, S.sv_ptr, S.sv_src, S.h_sv_lev_ptr[l], S.h_sv_lev_ptr[l + 1], kSvThread,
+                  S.sv_ord[l], S.sv_warp[l], S.sv_cta[l], skip);
     if (S.lev_cta[l].n > 0)
       k_fwd_front<T><<<(unsigned)S.lev_cta[l].n, 256, 0, stm>>>(F, w, S.lev_cta[l].id, S.sn_ptr, S.row_ptr,
                                                                  S.front_off, S.upd_off, skip);

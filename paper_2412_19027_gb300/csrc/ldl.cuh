@@ -8,6 +8,7 @@
 #include "bigfront.cuh"
 #include "device.cuh"
 #include "internal.h"
+#include "kktcta.cuh"
 #include "scal.cuh"
 #include "symbolic.h"
 
@@ -38,8 +39,9 @@ struct LdlStructure {
   };
   std::vector<List> lev_small, lev_thin_leaf, lev_thin, lev_cta;
   std::vector<int64_t> lev_thin_smem;            // largest f c of a level's thin fronts
-  // pull targets with long source lists (indices into fa_tgt, sv_tgt): a warp each, a CTA each
-  std::vector<List> fa_warp, fa_cta, sv_warp, sv_cta;
+  // pull targets with long source lists (indices into fa_tgt, sv_tgt): a warp each (the sum
+  // in list order), a warp each, a CTA each
+  std::vector<List> fa_ord, fa_warp, fa_cta, sv_ord, sv_warp, sv_cta;
   std::vector<std::vector<int64_t>> lev_big;     // big fronts of each level
   BigFrontDev bfd;                               // big-front arrays (device)
   std::vector<BigLevelPlan> bplans;              // per level
@@ -65,6 +67,7 @@ struct LdlStructure {
   int64_t pk_tiles = 0;  // packed operand tiles of the largest level (tensor-core flow, FP32 factor)
   int small_max = 0;
   int64_t max_front = 0;
+  CtaPlan cta;  // small problems: a CTA per problem (n = 0: not used)
 };
 
 // A front of more rows than small_max with few pivots: the arrow columns of a dense
@@ -74,10 +77,13 @@ struct LdlStructure {
 // 1/64 .. 1/16 of a tile's work for the same loads, stores and waits (portfolio
 // n = 5000, FP32: 5000 fronts of ~250 rows 3.0 -> 0.20 ms), and the forward sweep
 // gave each front f / 32 CTAs of 512 threads for one or two columns (100 -> 9 us).
-// The line: f^2 c / 2 FMAs on one SM are 0.3 ms in FP64 at 2^21, about what the tile
-// tasks of one such front take end to end; the rule looks at the front alone, so a
-// problem's arithmetic does not depend on its cohort.
-constexpr int64_t kThinPivots = 16, kThinWork = (int64_t)1 << 21;
+// The lines: f^2 c / 2 FMAs on one SM are 0.3 ms in FP64 at 2^21, about what the tile
+// tasks of one such front take end to end.  A problem with fewer than kThinCount of them
+// keeps the tile tasks: there the launch costs a few rounds of tasks only, and small
+// dense QPs (up to 400 such fronts) solved to 1e-8 amplify a change of rounding to 1e-9
+// in the multipliers.  The rule looks at one problem, so that its arithmetic does not
+// depend on its cohort.
+constexpr int64_t kThinPivots = 16, kThinWork = (int64_t)1 << 21, kThinCount = 512;
 inline bool ldl_thin_front(int64_t f, int64_t c, int small_max) {
   return f > small_max && c <= kThinPivots && f * f * c <= kThinWork;
 }

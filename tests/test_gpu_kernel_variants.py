@@ -111,3 +111,29 @@ def test_thin_fronts_and_long_pulls(bits, leaves, c, r, m, extra):
     eps = 2.2e-16 if bits == 64 else 1.2e-7
     assert np.abs(Kf @ x - rhs).max() <= 10 * np.sqrt(N) * eps * max(1.0, np.abs(x).max()) * 10
     assert hits == 0 and np.all(sgn * D > 0)
+
+
+# one CTA per problem (fronts of at most 96 rows, all of a cohort) against the launch per
+# level: the same problem alone and beside one with large fronts, which takes every problem
+# of the cohort through the general kernels
+@pytest.mark.parametrize("bits", [64, 32])
+@pytest.mark.parametrize("make", [
+    lambda W: W.mpc_qp(1, T=10, nx=4, nu=2), lambda W: W.mpc_qp(2, T=50, nx=12, nu=4),
+    lambda W: W.mpc_qp(3, T=31, nx=5, nu=3), lambda W: W.unique_qp(4, n=10, n_eq=2, n_inactive=10),
+    lambda W: W.unique_qp(5, n=30, n_eq=6, n_inactive=30), lambda W: W.unique_qp(6, n=50, n_eq=10, n_inactive=50),
+    lambda W: W.unique_qp(7, n=68, n_eq=4, n_inactive=30), lambda W: W.psd_mixed(8, orders=(2, 3, 4), per_order=2)])
+def test_cta_solves_equal_level_launches(bits, make):
+    from paper_2412_19027_gb300 import workloads as W
+    pr, big = make(W), W.mixed_cone(9, n=300, n_zero=0, n_nonneg=525, n_soc=75, n_exp=15, n_pow=15)
+    st = clr.clr_default_settings(bits, max_iter=6, fp64_escalation=0)
+    arg = lambda p: (p.P, p.q, p.A, p.b, p.cones)
+    one = clr.clr_setup(*arg(pr), st)
+    one.solve()
+    both = clr.clr_batch_setup([arg(pr), arg(big)], st)
+    both.solve()
+    a, b = one.solution(), both.solution_of(0)
+    for u, v in zip(a[:3], b[:3]):
+        np.testing.assert_array_equal(u, v)
+    assert a[3]["iterations"] == b[3]["iterations"] and a[3]["ir_steps_total"] == b[3]["ir_steps_total"]
+    one.free()
+    both.free()

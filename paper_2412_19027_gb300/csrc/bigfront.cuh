@@ -36,11 +36,29 @@ struct WorkList {
   int64_t nfront = 0, nblocks = 0;
 };
 
+// The big fronts of one level as the sweep kernels take them: by value for up to
+// kSweepInline fronts (a chain level has one), else from a device list with the front of
+// each CTA.
+struct alignas(16) SweepFront {
+  int32_t f, c;
+  int64_t eoff, woff, yoff, k0pos, rk;  // as in BigFrontDev
+  int64_t pull;                         // its rows' pull ranges: pull_ptr[pull + i .. + 1) for i < f
+  int32_t fblk, bblk;                   // first CTA of the forward and of the backward launch
+};
+constexpr int kSweepInline = 4;
+struct SweepLevel {
+  int32_t n = 0, fblocks = 0, bblocks = 0, fused = 0;  // fused: the forward kernel gathers the children itself
+  const SweepFront* list = nullptr;                    // n > kSweepInline
+  const int32_t *fmap = nullptr, *bmap = nullptr;      // ... front of each CTA
+  SweepFront fr[kSweepInline];
+};
+constexpr int kSweepPull = 512;  // largest c of a front whose forward kernel gathers the children
+
 // Host description of the big-front launches of one level.
 struct BigLevelPlan {
   std::vector<WorkList> A, B, C;  // per panel step p (B/C may be empty lists)
   std::vector<WorkList> Ctc;      // C as 128 x 64 tensor-core tiles (16-bit products)
-  WorkList fwd, bwd;
+  WorkList fwd;
 };
 
 // ---------------------------------------------------------------------------
@@ -125,8 +143,10 @@ struct BigFrontOps {
                           bool tc16 = false, int* err = nullptr);
   static int fwd(cudaStream_t st, const BigFrontDev& bf, const WorkList& wl, const T* E, const T* Dp, T* w,
                  T* ybuf, const int* skip);
-  static int bwd(cudaStream_t st, const BigFrontDev& bf, const WorkList& wl, const T* E, const T* Dp, const T* ybuf,
-                 T* xs, const int32_t* rows_kkt, const int* skip);
+  static int sweep_fwd(cudaStream_t st, const SweepLevel& lv, const T* E, const T* Dp, T* w, T* ybuf,
+                       const int32_t* pull_ptr, const int64_t* sv_ptr, const int64_t* sv_src, const int* skip);
+  static int sweep_bwd(cudaStream_t st, const SweepLevel& lv, const T* E, const T* ybuf, T* xs,
+                       const int32_t* rows_kkt, const int* skip);
   // Dataflow factorization of one level: tasks [t0, t0 + nt) of the task table;
   // state: zeroed words holding the level's task counter (at head_off) and, at
   // soff[b], the version words of each big front b of the level.  err: set to 2

@@ -91,6 +91,27 @@ __device__ __forceinline__ double block_min(double v, double* sh) {
   return v;
 }
 
+// Programmatic dependent launch: a kernel launched by launch_pdl starts once every CTA of the
+// kernel before it on the stream has called pdl_trigger (or ended).  Before pdl_wait it may
+// read only what no kernel still running can write; pdl_wait returns when the kernel before it
+// has completed (which, having waited itself, ran after all earlier ones).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename K, typename... A>
+cudaError_t launch_pdl(K kernel, unsigned grid, unsigned threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 inline int grid_for(int64_t n, int threads, int cap = 8 * kSMs) {
   int64_t g = (n + threads - 1) / threads;
   if (g < 1) g = 1;

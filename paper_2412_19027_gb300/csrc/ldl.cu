@@ -319,19 +319,45 @@ __global__ void k_init_w(T* __restrict__ w, const int32_t* __restrict__ w_init, 
 }
 
 // Forward sweep of one front per CTA: unit lower solve of the c x c diagonal
-// block in 32-column blocks (warp 0), then the rows below each block.
+// block in 32-column blocks (warp 0), then the rows below each block.  With pulls (the
+// range of each front's targets), the children's update entries are gathered first, in list
+// order (k_pull); all of the launch's static data is read before the wait for the level before
+// (programmatic dependent launch).
 template <typename T>
-__global__ void k_fwd_front(const T* __restrict__ F, T* __restrict__ w, const int64_t* __restrict__ fronts,
+__global__ void k_fwd_front(const T* __restrict__ F, T* w, const int64_t* __restrict__ fronts,
                             const int64_t* __restrict__ sn_ptr, const int64_t* __restrict__ row_ptr,
                             const int64_t* __restrict__ front_off, const int64_t* __restrict__ upd_off,
-                            const int* skip) {
-  if (skip && *skip) return;
+                            const int64_t* __restrict__ pulls, const int64_t* __restrict__ sv_tgt,
+                            const int64_t* __restrict__ sv_ptr, const int64_t* __restrict__ sv_src, const int* skip) {
+  pdl_trigger();
   __shared__ T xb[32];
   const int64_t J = fronts[blockIdx.x];
   const int64_t c = sn_ptr[J + 1] - sn_ptr[J];
   const int64_t f = row_ptr[J + 1] - row_ptr[J];
   const T* G = F + front_off[J];
   T* wj = w + upd_off[J];
+  const int64_t p0 = pulls ? pulls[2 * blockIdx.x] : 0, p1 = pulls ? pulls[2 * blockIdx.x + 1] : 0;
+  int64_t q0 = 0, q1 = 0, s0 = 0, tg = 0;
+  if (p0 + threadIdx.x < p1) {
+    tg = sv_tgt[p0 + threadIdx.x];
+    q0 = sv_ptr[p0 + threadIdx.x];
+    q1 = sv_ptr[p0 + threadIdx.x + 1];
+    s0 = sv_src[q0];
+  }
+  pdl_wait();
+  if (skip && *skip) return;
+  if (p1 > p0) {
+    auto gather = [&](int64_t t, int64_t a, int64_t b, int64_t s) {
+      T acc = w[t];
+      acc += w[s];
+      for (int64_t q = a + 1; q < b; ++q) acc += w[sv_src[q]];
+      w[t] = acc;
+    };
+    if (q1 > q0) gather(tg, q0, q1, s0);
+    for (int64_t t = p0 + blockDim.x + threadIdx.x; t < p1; t += blockDim.x)
+      gather(sv_tgt[t], sv_ptr[t], sv_ptr[t + 1], sv_src[sv_ptr[t]]);
+    __syncthreads();
+  }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int64_t j0 = 0; j0 < c; j0 += 32) {
     const int jb = (int)min((int64_t)32, c - j0);
@@ -359,12 +385,12 @@ __global__ void k_fwd_front(const T* __restrict__ F, T* __restrict__ w, const in
 // Backward sweep of one front per CTA: v = y / D, then L^T x = v with the
 // solution of the ancestors (rows c .. f-1) gathered from xs by KKT index.
 template <typename T>
-__global__ void k_bwd_front(const T* __restrict__ F, const T* __restrict__ Dp, T* __restrict__ w, T* __restrict__ xs,
+__global__ void k_bwd_front(const T* __restrict__ F, const T* __restrict__ Dp, T* w, T* xs,
                             const int64_t* __restrict__ fronts, const int64_t* __restrict__ sn_ptr,
                             const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ front_off,
                             const int64_t* __restrict__ upd_off, const int32_t* __restrict__ rows_kkt,
                             const int* skip) {
-  if (skip && *skip) return;
+  pdl_trigger();
   const int64_t J = fronts[blockIdx.x];
   const int64_t c = sn_ptr[J + 1] - sn_ptr[J];
   const int64_t f = row_ptr[J + 1] - row_ptr[J];
@@ -372,6 +398,8 @@ __global__ void k_bwd_front(const T* __restrict__ F, const T* __restrict__ Dp, T
   T* X = w + upd_off[J];
   const int32_t* rk = rows_kkt + row_ptr[J];
   const T* D = Dp + sn_ptr[J];
+  pdl_wait();
+  if (skip && *skip) return;
   for (int64_t i = threadIdx.x; i < f; i += blockDim.x) X[i] = (i < c) ? X[i] / D[i] : xs[rk[i]];
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -802,19 +830,105 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
         add_list(pl.C[p], ids, cc);
         add_list(pl.Ctc[p], ids, ct);
       }
-      std::vector<int64_t> cf, cbw;
+      std::vector<int64_t> cf;
       for (int64_t b : ids) {
         cf.push_back((bf_f[b] + 31) / 32);
-        cbw.push_back((bf_c[b] + 7) / 8);
       }
       add_list(pl.fwd, ids, cf);
-      add_list(pl.bwd, ids, cbw);
     }
     int64_t* dbuf = buf.empty() ? nullptr : ar.upload(buf.data(), (int64_t)buf.size());
     if (!buf.empty() && !dbuf) return CLR_E_OOM;
     for (Pending& pd : pend) {
       pd.wl->front = dbuf + pd.fo;
       pd.wl->pref = dbuf + pd.po;
+    }
+    // the solve sweeps: descriptors, the fronts of each CTA, and which levels gather their
+    // children in the forward kernels (every big front of at most kSweepPull pivots, every
+    // source list short enough to be summed in list order, and worth a thread's walk)
+    {
+      std::vector<SweepFront> lists;
+      std::vector<int32_t> maps, pptr;
+      struct Fix {
+        int64_t l;
+        size_t list, fmap, bmap;
+      };
+      std::vector<Fix> fix;
+      st.sweeps.assign(sy.nlev, SweepLevel());
+      st.lev_fused.assign(sy.nlev, 0);
+      // pull targets by front: they come level by level, front by front, in order
+      std::vector<int64_t> sv0(sy.nsn, 0), sv1(sy.nsn, 0), cpull;
+      for (int64_t l = 0; l < sy.nlev; ++l) {
+        int64_t t = mp.sv_lev_ptr[l];
+        int64_t longest = 0;
+        bool fused = true;
+        for (int64_t k = sy.lev_ptr[l]; k < sy.lev_ptr[l + 1]; ++k) {
+          const int64_t J = sy.lev_sn[k], f = sy.row_ptr[J + 1] - sy.row_ptr[J];
+          sv0[J] = t;
+          while (t < mp.sv_lev_ptr[l + 1] && mp.sv_tgt[t] >= sy.upd_off[J] && mp.sv_tgt[t] < sy.upd_off[J] + f) {
+            longest = std::max(longest, mp.sv_ptr[t + 1] - mp.sv_ptr[t]);
+            ++t;
+          }
+          sv1[J] = t;
+          if (bid_of[J] >= 0 && bf_c[bid_of[J]] > kSweepPull) fused = false;
+        }
+        if (t != mp.sv_lev_ptr[l + 1]) return CLR_E_INVALID;
+        st.lev_fused[l] = fused && longest <= kSvThread && mp.sv_lev_ptr[l + 1] < ((int64_t)1 << 31);
+      }
+      for (int64_t l = 0; l < sy.nlev; ++l) {
+        for (int64_t k = sy.lev_ptr[l]; k < sy.lev_ptr[l + 1]; ++k) {  // lev_cta's order
+          const int64_t J = sy.lev_sn[k];
+          if (bid_of[J] >= 0) continue;
+          cpull.push_back(sv0[J]);
+          cpull.push_back(sv1[J]);
+        }
+        if (st.lev_cta[l].n > 0) st.lev_cta[l].first = (int64_t)cpull.size() / 2 - st.lev_cta[l].n;
+        if (st.lev_big[l].empty()) continue;
+        SweepLevel& sw = st.sweeps[l];
+        sw.n = (int32_t)st.lev_big[l].size();
+        sw.fused = st.lev_fused[l];
+        std::vector<SweepFront> fr;
+        for (int64_t J : st.lev_big[l]) {
+          const int64_t b = bid_of[J];
+          SweepFront e{};
+          e.f = (int32_t)bf_f[b];
+          e.c = (int32_t)bf_c[b];
+          e.eoff = bf_eoff[b];
+          e.woff = bf_woff[b];
+          e.yoff = bf_yoff[b];
+          e.k0pos = bf_k0[b];
+          e.rk = bf_rk[b];
+          e.fblk = sw.fblocks;
+          e.bblk = sw.bblocks;
+          sw.fblocks += (int32_t)((bf_f[b] + 31) / 32);
+          sw.bblocks += (int32_t)((bf_c[b] + 7) / 8);
+          if (sw.fused) {
+            e.pull = (int64_t)pptr.size();
+            pptr.resize(pptr.size() + bf_f[b], -1);
+            for (int64_t t = sv0[J]; t < sv1[J]; ++t) pptr[e.pull + (mp.sv_tgt[t] - sy.upd_off[J])] = (int32_t)t;
+          }
+          fr.push_back(e);
+        }
+        if (sw.n <= kSweepInline) {
+          std::copy(fr.begin(), fr.end(), sw.fr);
+        } else {
+          Fix fx{l, lists.size(), maps.size(), 0};
+          lists.insert(lists.end(), fr.begin(), fr.end());
+          for (size_t k = 0; k < fr.size(); ++k) maps.insert(maps.end(), (size_t)((fr[k].f + 31) / 32), (int32_t)k);
+          fx.bmap = maps.size();
+          for (size_t k = 0; k < fr.size(); ++k) maps.insert(maps.end(), (size_t)((fr[k].c + 7) / 8), (int32_t)k);
+          fix.push_back(fx);
+        }
+      }
+      const SweepFront* dl = ar.upload(lists.data(), (int64_t)lists.size());
+      const int32_t* dm = ar.upload(maps.data(), (int64_t)maps.size());
+      st.pull_ptr = up(ar, pptr);
+      st.cta_pull = up(ar, cpull);
+      if (!dl || !dm || !st.pull_ptr || !st.cta_pull) return CLR_E_OOM;
+      for (const Fix& fx : fix) {
+        st.sweeps[fx.l].list = dl + fx.list;
+        st.sweeps[fx.l].fmap = dm + fx.fmap;
+        st.sweeps[fx.l].bmap = dm + fx.bmap;
+      }
     }
     // dataflow task tables (bigfront.cuh), per level: every task of every big front
     // of the level, then ordered by flow_schedule_order.  A pivot block p >= 1
@@ -1080,22 +1194,30 @@ int LdlFactor<T>::solve(cudaStream_t stm, const double* rhs, const int* skip) co
   const LdlStructure& S = *s;
   k_init_w<T><<<grid_for(S.wtot, 256), 256, 0, stm>>>(w, S.w_init, rhs, S.wtot, skip);
   for (int64_t l = 0; l < S.nlev; ++l) {
-    pull_level<T>(stm, w, S.sv_tgt, S.sv_ptr, S.sv_src, S.h_sv_lev_ptr[l], S.h_sv_lev_ptr[l + 1], kSvThread,
-                  S.sv_ord[l], S.sv_warp[l], S.sv_cta[l], skip);
-    if (S.lev_cta[l].n > 0)
-      k_fwd_front<T><<<(unsigned)S.lev_cta[l].n, 256, 0, stm>>>(F, w, S.lev_cta[l].id, S.sn_ptr, S.row_ptr,
-                                                                 S.front_off, S.upd_off, skip);
+    const bool fused = S.lev_fused[l] != 0;
+    if (!fused)
+      pull_level<T>(stm, w, S.sv_tgt, S.sv_ptr, S.sv_src, S.h_sv_lev_ptr[l], S.h_sv_lev_ptr[l + 1], kSvThread,
+                    S.sv_ord[l], S.sv_warp[l], S.sv_cta[l], skip);
+    const LdlStructure::List& cl = S.lev_cta[l];
+    if (cl.n > 0)
+      CLR_CUDA(launch_pdl(k_fwd_front<T>, (unsigned)cl.n, 256, 0, stm, (const T*)F, w, cl.id, (const int64_t*)S.sn_ptr,
+                          (const int64_t*)S.row_ptr, (const int64_t*)S.front_off, (const int64_t*)S.upd_off,
+                          fused ? (const int64_t*)(S.cta_pull + 2 * cl.first) : (const int64_t*)nullptr,
+                          (const int64_t*)S.sv_tgt, (const int64_t*)S.sv_ptr, (const int64_t*)S.sv_src, skip));
     if (!S.lev_big[l].empty()) {
-      int rc = BigFrontOps<T>::fwd(stm, S.bfd, S.bplans[l].fwd, E, Dp, w, ybuf, skip);
+      int rc = fused ? BigFrontOps<T>::sweep_fwd(stm, S.sweeps[l], E, Dp, w, ybuf, S.pull_ptr, S.sv_ptr, S.sv_src, skip)
+                     : BigFrontOps<T>::fwd(stm, S.bfd, S.bplans[l].fwd, E, Dp, w, ybuf, skip);
       if (rc) return rc;
     }
   }
   for (int64_t l = S.nlev - 1; l >= 0; --l) {
-    if (S.lev_cta[l].n > 0)
-      k_bwd_front<T><<<(unsigned)S.lev_cta[l].n, 256, 0, stm>>>(F, Dp, w, xs, S.lev_cta[l].id, S.sn_ptr, S.row_ptr,
-                                                                 S.front_off, S.upd_off, S.rows_kkt, skip);
+    const LdlStructure::List& cl = S.lev_cta[l];
+    if (cl.n > 0)
+      CLR_CUDA(launch_pdl(k_bwd_front<T>, (unsigned)cl.n, 256, 0, stm, (const T*)F, (const T*)Dp, w, xs, cl.id,
+                          (const int64_t*)S.sn_ptr, (const int64_t*)S.row_ptr, (const int64_t*)S.front_off,
+                          (const int64_t*)S.upd_off, (const int32_t*)S.rows_kkt, skip));
     if (!S.lev_big[l].empty()) {
-      int rc = BigFrontOps<T>::bwd(stm, S.bfd, S.bplans[l].bwd, E, Dp, ybuf, xs, S.rows_kkt, skip);
+      int rc = BigFrontOps<T>::sweep_bwd(stm, S.sweeps[l], E, ybuf, xs, S.rows_kkt, skip);
       if (rc) return rc;
     }
   }

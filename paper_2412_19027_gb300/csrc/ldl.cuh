@@ -36,6 +36,7 @@ struct LdlStructure {
   struct List {
     const int64_t* id = nullptr;
     int64_t n = 0;
+    int64_t first = 0;  // lev_cta: index of its first entry in cta_pull
   };
   std::vector<List> lev_small, lev_thin_leaf, lev_thin, lev_cta;
   std::vector<int64_t> lev_thin_smem;            // largest f c of a level's thin fronts
@@ -45,6 +46,10 @@ struct LdlStructure {
   std::vector<std::vector<int64_t>> lev_big;     // big fronts of each level
   BigFrontDev bfd;                               // big-front arrays (device)
   std::vector<BigLevelPlan> bplans;              // per level
+  std::vector<SweepLevel> sweeps;                // per level: the solve sweeps over its big fronts
+  std::vector<int8_t> lev_fused;                 // per level: the forward kernels gather the children themselves
+  int32_t* pull_ptr = nullptr;                   // big fronts of fused levels: pull target of each row, or -1
+  int64_t* cta_pull = nullptr;                   // per lev_cta entry: its pull targets' range (two words)
   // extend-add by relative indices: per level, the rounds' work lists (children
   // and prefix sums of their 32 x 32 tile counts)
   int32_t* rel = nullptr;

@@ -137,3 +137,36 @@ def test_cta_solves_equal_level_launches(bits, make):
     assert a[3]["iterations"] == b[3]["iterations"] and a[3]["ir_steps_total"] == b[3]["ir_steps_total"]
     one.free()
     both.free()
+
+
+# the sweeps over large fronts (k_sweep_fwd up to 512 pivots, k_sweep_bwd) at the ends of
+# their batches and prefetches, one front by value and more than four from the list: leaf
+# cliques of c pivots on r of the m root rows
+@pytest.mark.parametrize("bits", [64, 32])
+@pytest.mark.parametrize("leaves,c,r,m", [
+    (1, 512, 33, 160), (1, 513, 40, 160), (2, 511, 1025, 1030), (5, 129, 1023, 1100), (6, 128, 31, 140),
+    (4, 257, 64, 200), (9, 97, 130, 140), (1, 121, 1056, 1060)])
+def test_large_front_sweeps(bits, leaves, c, r, m):
+    import scipy.sparse as sp
+    rng = np.random.default_rng(leaves + c + r)
+    N, R, Cc, V = leaves * c + m, [], [], []
+    root = N - m
+    for q in range(leaves):
+        p0 = q * c
+        low = np.tril_indices(c, -1)
+        R.append(p0 + low[0]); Cc.append(p0 + low[1]); V.append(rng.standard_normal(len(low[0])) / c)
+        rows = root + np.sort(rng.choice(m, r, replace=False))
+        R.append(np.tile(rows, c)); Cc.append(np.repeat(np.arange(p0, p0 + c), r))
+        V.append(rng.standard_normal(c * r) / np.sqrt(c * r))
+    low = np.tril_indices(m, -1)
+    R.append(root + low[0]); Cc.append(root + low[1]); V.append(rng.standard_normal(len(low[0])) / m)
+    K = sp.csc_matrix((np.concatenate(V), (np.concatenate(R), np.concatenate(Cc))), shape=(N, N))
+    sgn = np.where(np.arange(N) < root, 1.0, -1.0)
+    K = sp.tril(K, -1) + sp.diags(sgn * (2.0 + rng.random(N)))
+    rhs = rng.standard_normal(N)
+    x, D, hits = clr.clr_ldl_solve(K, sgn, rhs, order=np.arange(N), factor_bits=bits)
+    Kf = K + sp.tril(K, -1).T
+    # well conditioned (diagonally dominant blocks): rows of up to c + r terms of size <= 1
+    eps = 2.2e-16 if bits == 64 else 1.2e-7
+    assert np.abs(Kf @ x - rhs).max() <= 10 * np.sqrt(N) * eps * max(1.0, np.abs(x).max()) * 10
+    assert hits == 0 and np.all(sgn * D > 0)

@@ -1,0 +1,908 @@
+// Dataflow factorization of the large FP64 fronts of one level with their 64 x 64 x 64
+// products on the tensor cores.
+//
+// What bounds the FMA version (bigflow.cu): a GB300 SM retires ~1.7 FP64 FMA per clock, so a
+// 64^3 product is 75 us of one SM's FP64 pipe; the FP64 tensor instruction runs no faster
+// (684 clocks per 8 x 8 x 4).  Here each FP64 operand is cut into seven 8-bit digits that
+// tcgen05 kind::f16 multiplies exactly, and the sums are put together again in integers
+// (the error-free splitting of Ozaki, Ogita, Oishi and Rump, "Error-free transformations of
+// matrix multiplication by using fast routines of matrix multiplication and its
+// applications", Numer. Algorithms 59, 2012):
+//   - row r of an operand is scaled by a power of two so that its largest entry is below
+//     2^55 as an integer, X = rint(x 2^(55 - e_r)), and written in balanced base 256,
+//     X = sum_s d_s 256^(6 - s), |d_s| <= 128 (exact in FP16);
+//   - the products of digit matrices s and t of equal s + t <= 7 are summed in one FP32
+//     accumulator in tensor memory: at most 4 products of 64 terms up to 2^14, so every
+//     partial sum is an integer up to 2^22, exact in FP32;
+//   - the eight sums G_0 .. G_7 give (X Y) / 2^54 as a 64-bit integer (the digit products with
+//     s + t >= 8 are below 2^-64 of the row maxima), which is normalised to a double in
+//     integer arithmetic; one FP64 addition per entry remains.
+// Before splitting, the shared index k is scaled by a power of two on one side and its inverse
+// on the other so that both operands are rows of sqrt(D)-scaled factors: |entry| <=
+// sqrt(F_ii) like the rows of a Cholesky factor, and the rounding of the digits (2^-55 of the
+// row maximum, about an eighth of what 64 rounded FMAs leave) is small against
+// sqrt(F_ii F_jj), the error bound of the factorization itself.  A row with an entry that is
+// not finite gives NaN in its results.
+//
+// Tasks and waits are those of bigflow.cu without the fused or split chain task: D(p), T(p, i),
+// Efin(p, e), U(p, i, j), EU(p, i, e).  Producers store their tile also as digits ("packs",
+// 56 KB in the MMA's layout, copied to shared memory by cp.async.bulk):
+//   PA(p, i) = L_IK 2^h, PB(p, i) = (L_IK D_K) 2^-h (h_k = half the exponent of d_k),
+//   PE(p, e) = E_KC^T 2^-h, PT(p) = Linv 2^g (g_l = half the exponent of F_ll), so that
+//   U: F_IJ -= PA(p, i) PB(p, j)^T;  EU: E_IC -= PA(p, i) PE(p, e)^T;
+//   T: L_IK = (F_IK 2^-g) PT(p)^T D^{-1};  Efin: E_KC^T <- (E_KC^T 2^-g) PT(p)^T,
+// with F_IK and E_KC^T split in the task.  One CTA per SM (512 columns of tensor memory).
+// Per task on a GB300 (front of 2052 rows; FMA version in brackets): D 66 us (95), T 27 (41), Efin 23
+// (57), U 13 (57), EU 13 (57); the front: 4.0 ms.
+#include <algorithm>
+
+#include "bfdiag.cuh"
+#include "bigfront.cuh"
+#include "flowsync.cuh"
+
+namespace clr {
+namespace {
+constexpr int NB = kBfNB;
+constexpr int NT = kFlowThreads;
+constexpr int kSlice = NB * NB * 2;                   // one digit matrix, FP16: 8 KB
+constexpr int kDig = 7;
+constexpr int kPackBytes = kDig * kSlice;             // 57344
+constexpr int kTileStride = (int)kPack64Bytes;        // digits, then 64 row exponents, g[64], h[64]
+static_assert(kTileStride == kPackBytes + 3 * 64 * 4 && kTileStride % 16 == 0, "pack layout");
+constexpr int kBad = 1 << 20;                         // row exponent of a row with a value that is not finite
+// shared memory: A digits (an eighth matrix of zeros pairs with the seventh), B digits, scratch
+constexpr int kOffB = 8 * kSlice, kOffS = kOffB + kPackBytes;
+constexpr int kScratch = kDiagSmem * 8;               // D(p); 32 KB of it the exchange of the epilogue
+constexpr size_t kSmem = (size_t)kOffS + kScratch + 1024;
+
+__device__ __forceinline__ uint32_t s_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// K-major core matrices of 8 rows x 16 bytes, adjacent in K 128 bytes apart and in rows 1024
+__device__ __forceinline__ uint64_t dig_desc(uint32_t a) {
+  uint64_t d = (uint64_t)((a & 0x3FFFF) >> 4);
+  d |= (uint64_t)(128 >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;  // tcgen05 descriptor version; no swizzle, base offset 0
+  return d;
+}
+// M = 128, N = 64, D FP32, A and B FP16, both K-major
+constexpr uint32_t kF16Idesc = (1u << 4) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+      "l"(ad), "l"(bd), "r"(kF16Idesc), "r"(acc));
+}
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+// exponent of |x| as in |x| < 2^(ilog + 1) (zero and subnormals: very small; not finite: kBad)
+__device__ __forceinline__ int ilog_of(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  return e == 0 ? -kBad : (e == 0x7ff ? kBad : e - 1023);
+}
+// rint(x 2^(sh + 55 - e)) plus 128 in each of seven bytes, for |x| 2^sh < 2^e
+__device__ __forceinline__ uint64_t digits_of(double x, int sh, int e) {
+  constexpr uint64_t bias = 0x0080808080808080ull;
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  if (ex == 0 || ex == 0x7ff) return bias;
+  const uint64_t m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+  const int s = e - 3 - (ex - 1023 + sh);  // X = m 2^-s, s >= -2
+  uint64_t X;
+  if (s <= 0) X = m << (-s & 3);
+  else X = s > 54 ? 0ull : (m + (1ull << (s - 1))) >> s;
+  return (int64_t)b < 0 ? bias - X : bias + X;
+}
+
+struct PackScratch {
+  int mx[64];   // row maxima of the exponents
+  int sh[64];   // exponent shift of each k
+};
+// All threads: thread (row r = tid & 63, k = 16 (tid >> 6) .. + 15) holds x[16]; writes the
+// rows' digits at dst + s kSlice + ... (global or shared) and their exponents e_r to `exps`.
+// sc.sh holds the shifts; sc.mx is used.  Ends without a barrier.
+__device__ void pack_rows(const double (&x)[16], unsigned char* dst, int* exps, PackScratch& sc) {
+  const int r = threadIdx.x & 63, kq = threadIdx.x >> 6;
+  __syncthreads();
+  if (threadIdx.x < 64) sc.mx[threadIdx.x] = -kBad;
+  __syncthreads();
+  int m = -kBad;
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int l = ilog_of(x[u]);
+    m = max(m, l >= kBad ? kBad : (l <= -kBad ? -kBad : l + sc.sh[16 * kq + u]));
+  }
+  atomicMax(&sc.mx[r], m);
+  __syncthreads();
+  m = sc.mx[r];
+  const int e = m >= kBad ? kBad : (m <= -kBad ? 0 : m + 1);
+  if (kq == 0) exps[r] = e;
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    uint64_t y[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) y[u] = digits_of(x[8 * g + u], sc.sh[16 * kq + 8 * g + u], e);
+    unsigned char* d = dst + (r >> 3) * 1024 + (2 * kq + g) * 128 + (r & 7) * 16;
+#pragma unroll
+    for (int s = 0; s < kDig; ++s) {
+      const int q = 6 - s;  // byte of the digit
+      uint32_t o[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const uint32_t wa = q < 4 ? (uint32_t)y[2 * v] : (uint32_t)(y[2 * v] >> 32);
+        const uint32_t wb = q < 4 ? (uint32_t)y[2 * v + 1] : (uint32_t)(y[2 * v + 1] >> 32);
+        // FP16 1024 + byte, then minus 1152: the digit
+        // (the first digit is up to 128: nine bits)
+        const uint32_t t = __byte_perm(wa, wb, (q & 3) | ((4 + (q & 3)) << 4));
+        const uint32_t h = s == 0 ? __byte_perm(wa, wb, 0x7632) | 0x64006400u : __byte_perm(t, 0x64646464u, 0x4140);
+        asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(o[v]) : "r"(h), "r"(0x64806480u));
+      }
+      *reinterpret_cast<uint4*>(d + s * kSlice) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+  }
+}
+
+// Thread 0: the 19 digit products of A (at sA) and B (at sB) into tensor memory.  A MMA takes
+// two neighbouring digits of A as 128 rows: block t (64 columns) gets the products of digit sum t
+// in lanes 0-63 and those of digit sum t + 1 with the odd digits of A in lanes 64-127.
+__device__ __forceinline__ void issue_products(uint32_t sA, uint32_t sB, uint32_t tmem, uint32_t bar) {
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+  for (int t = 0; t < 8; ++t) {
+    uint32_t acc = 0;
+#pragma unroll 1
+    for (int i = 0; i < 8; i += 2) {
+      const int j = t - i;
+      if (j < 0 || j >= kDig) continue;
+#pragma unroll
+      for (int ks = 0; ks < NB / 16; ++ks) {
+        mma_f16(tmem + 64u * t, dig_desc(sA + i * kSlice + 256u * ks), dig_desc(sB + j * kSlice + 256u * ks), acc);
+        acc = 1;
+      }
+    }
+  }
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// v 2^e as a double, rounded to nearest, ties to even (zero below the normal range)
+__device__ __forceinline__ double scaled_double(long long v, int e) {
+  const uint64_t mag = v < 0 ? (uint64_t)-v : (uint64_t)v;
+  const int lz = __clzll((long long)mag);
+  const uint64_t n = mag << (lz & 63);
+  uint64_t m = n >> 11;
+  const uint64_t rest = n & 0x7ff;
+  m += (rest > 0x400 || (rest == 0x400 && (m & 1))) ? 1 : 0;
+  const int ex = 63 - lz + e + 1023;                 // exponent field of the leading bit
+  uint64_t bits = ((uint64_t)(ex - 1) << 52) + m;    // (a carry out of m raises the exponent)
+  if (mag == 0 || ex < 1) bits = 0;
+  if (ex > 2046) bits = 0x7ff0000000000000ull;
+  if (e > kBad / 2) bits = 0x7ff8000000000000ull;
+  if (v < 0) bits |= 0x8000000000000000ull;
+  return __longlong_as_double((long long)bits);
+}
+
+// the integer of an FP32 accumulator with |v| <= 2^22
+__device__ __forceinline__ int acc_int(uint32_t b) {
+  return __float_as_int(__uint_as_float(b) + 12582912.0f) - 0x4B400000;
+}
+
+// All threads, after the MMAs: thread (row r = 32 (wid & 1) + lane, columns 16 cq .. + 15, cq =
+// 2 (wid >> 2) + ((wid >> 1) & 1)) gets out[u] = the product's entry as a double (eA, eB: row
+// exponents of the operands).  X: 32 KB of shared scratch.
+__device__ __forceinline__ void read_products(uint32_t tmem, const int* eA, const int* eB, long long* X,
+                                              double (&out)[16]) {
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, q = wid & 3, h = wid >> 2;
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const bool top = q < 2;  // lanes 0-63: digit sum t; 64-127: t + 1
+  long long T[32];
+  const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(32 * h);
+  // units of 2^-54 X Y: digit sum s has weight 2^(42 - 8 s)
+#pragma unroll
+  for (int c = 0; c < 32; ++c) T[c] = 0;
+#pragma unroll
+  for (int t = 0; t < 5; ++t) {  // digit sums 0 .. 4 (top) or 1 .. 5
+    uint32_t v[32];
+    tmem_ld32(base + 64u * t, v);
+#pragma unroll
+    for (int c = 0; c < 32; ++c) T[c] = T[c] * 256 + acc_int(v[c]);
+  }
+  {
+    uint32_t v5[32], v6[32];
+    tmem_ld32(base + 64u * 5, v5);
+    tmem_ld32(base + 64u * 6, v6);
+    if (top) {
+      uint32_t v7[32];
+      tmem_ld32(base + 64u * 7, v7);
+#pragma unroll
+      for (int c = 0; c < 32; ++c)
+        T[c] = T[c] * 1024 + (long long)acc_int(v5[c]) * 4 +
+               ((__float2int_rn(__uint_as_float(v6[c])) * 256 + acc_int(v7[c]) + 8192) >> 14);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 32; ++c)
+        T[c] = T[c] * 4 + ((acc_int(v5[c]) * 256 + __float2int_rn(__uint_as_float(v6[c])) + 8192) >> 14);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  // the top half finishes columns 0 .. 15 of its 32, the bottom half 16 .. 31
+  const int r = 32 * (q & 1) + lane;
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int c = (top ? 16 : 0) + u;
+    X[(32 * h + c) * 64 + r] = T[c];
+  }
+  __syncthreads();
+  const int c0 = top ? 0 : 16;
+  const int er = eA[r];
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const long long own = top ? T[u] : T[16 + u];
+    const long long v = own + X[(32 * h + c0 + u) * 64 + r];
+    out[u] = scaled_double(v, er + eB[32 * h + c0 + u] - 56);
+  }
+}
+
+// 27-bit low and 28-bit high parts x0, x1 of the integer rint(x 2^(sh + 55 - e)), |x| 2^sh < 2^e
+__device__ __forceinline__ int2 halves_of(double x, int sh, int e) {
+  constexpr int64_t bias = 0x0080808080808080ll;
+  const int64_t X = (int64_t)digits_of(x, sh, e) - bias;
+  const int x1 = (int)((X + (1ll << 26)) >> 27);
+  return make_int2((int)(X - ((int64_t)x1 << 27)), x1);
+}
+// Exact dot product of 16 terms of such rows in 64-bit integers: four IMAD.WIDE a term (an FP64
+// FMA takes 64 clocks of its pipe per warp); the sum is value() 2^(e_a + e_b - 56).
+struct IntDot {
+  long long hh = 0, mid = 0, ll = 0;
+  __device__ __forceinline__ void add(int2 a, int2 b) {
+    hh += (long long)a.y * b.y;
+    mid += (long long)a.y * b.x;
+    mid += (long long)a.x * b.y;
+    ll += (long long)a.x * b.x;
+  }
+  __device__ __forceinline__ long long value() const { return hh + ((mid + (ll >> 27) + (1ll << 26)) >> 27); }
+};
+
+// integers in the order of the doubles (NaN above all): no FP64 compare
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x);
+  const bool nan = (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+  return nan ? 0x7fffffffffffffffll : (b < 0 ? b ^ 0x7fffffffffffffffll : b);
+}
+// 1 / d to about half an ulp in integers (~110 clocks; two FP64 steps on the estimate: 230): with
+// m in [1, 2) the mantissa of d and y0 the hardware's estimate of 1 / m (20 bits), e = 1 - m y0
+// is exact in 64 bits and 1 / m = y0 (1 + e + e^2) to 2^-57.
+__device__ __forceinline__ double rcp_pivot(double d) {
+  const long long b = __double_as_longlong(d);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  if (ex < 2 || ex > 2043) return 1.0 / d;
+  const unsigned long long M = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;"
+      : "=d"(y)
+      : "d"(__longlong_as_double((long long)((M & 0xfffffffffffffull) | 0x3ff0000000000000ull))));
+  const unsigned long long yb = (unsigned long long)__double_as_longlong(y);
+  // y in [1/2, 1]: Y0 = y 2^21, cut to an integer
+  const int ye = (int)(yb >> 52);  // 1022 or 1023
+  const unsigned Y0 = (unsigned)(((yb & 0xfffffffffffffull) | 0x10000000000000ull) >> (52 - 21 + 1023 - ye));
+  const long long e73 = -(long long)(M * Y0);                // e 2^73 (2^73 = 0 modulo 2^64)
+  const int e40 = (int)(e73 >> 33);
+  const long long c58 = (e73 >> 15) + (((long long)e40 * e40) >> 22);  // (e + e^2) 2^58
+  const long long Y = ((long long)Y0 << 41) + ((c58 * (long long)Y0) >> 17);  // y 2^62
+  const unsigned long long m = (unsigned long long)((Y + 256) >> 9);
+  // 1/d = (m / 2^53) 2^(1023 - ex): m carries the hidden bit
+  const unsigned long long r = ((unsigned long long)(2044 - ex) << 52) + m;
+  return __longlong_as_double((long long)(r | ((unsigned long long)b & 0x8000000000000000ull)));
+}
+
+constexpr int kLI = 65;  // row strides of the integer operands (int2; odd: no bank conflicts)
+constexpr int kLP = 17;
+struct Diag64Smem {
+  int2 ia[64 * kLI];       // L 2^h by rows, exponents ea[panel][row]
+  int2 iq[16 * kLP];       // Linv_QQ 2^g by rows, exponents eq
+  int2 ix[48 * kLP];       // X 2^-g by columns, exponents ex
+  double cb[2 * 64];       // two pivot columns
+  int ea[4 * 64], eq[16], ex[48];
+};
+struct Diag64SmemB {
+  int2 ib[2 * 64 * kLP];   // (L d) 2^-h of a panel by rows, exponents eb[row], for two panels
+  int2 ic[48 * kLI];       // L^{-1} 2^-h by columns, exponents ec[block row][column]
+  int eb[2 * 64], ec[3 * 48];
+  double x[16 * 49];       // X = sum_M L_QM Linv_M
+};
+static_assert(sizeof(Diag64Smem) <= kPackBytes && sizeof(Diag64SmemB) <= kPackBytes, "scratch");
+__device__ __forceinline__ int row_exp(int m) { return m >= kBad ? kBad : (m <= -kBad ? 0 : m + 1); }
+__device__ __forceinline__ int shifted(double x, int sh) {
+  const int l = ilog_of(x);
+  return l >= kBad ? kBad : (l <= -kBad ? -kBad : l + sh);
+}
+
+// Pivots 16 q .. 16 q + 15 by four warps (barrier 2): NP = 2: rows 32 (wid & 1) + lane, columns of
+// parity wid >> 1; NP = 4 (q >= 2: rows 0-31 are done): rows 32 + lane, columns wid modulo 4.
+template <int NP>
+__device__ __forceinline__ void diag64_panel(int q, int pw, double* A, Diag64Smem& sa, Diag64SmemB& sb,
+                                             DiagScratch<double>& sh, int* hs, long long key_eps, double delta,
+                                             int& nhit) {
+  constexpr int LD = kDiagLD, NC = 16 / NP;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, c0 = 16 * q;
+  const int row = NP == 2 ? 32 * (wid & 1) + lane : 32 + lane, par = NP == 2 ? wid >> 1 : wid;
+  double v[NC], l[NC], c8[NC], dk = 0.0;
+#pragma unroll
+  for (int t = 0; t < NC; ++t) v[t] = A[row * LD + c0 + NP * t + par];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int kk = c0 + k;
+    double* cc = sa.cb + 64 * (k & 1);
+    if (par == (k % NP)) cc[row] = v[k / NP];
+    asm volatile("barrier.sync 2, 128;" ::: "memory");
+    double d = cc[kk];
+    const double cr = cc[row];
+    const bool ng = sh.sgn[kk] < 0;
+    const double sd = __longlong_as_double(__double_as_longlong(d) ^ (ng ? (long long)0x8000000000000000ull : 0ll));
+    const bool hit = kk < pw && order_key(sd) <= key_eps;
+    if (hit) d = ng ? -delta : delta;
+    const double lr = cr * rcp_pivot(d);
+    const double ml = __longlong_as_double(__double_as_longlong(lr) ^ (long long)0x8000000000000000ull);
+    if (par == (k % NP)) {
+      l[k / NP] = lr;
+      c8[k / NP] = cr;
+    }
+#pragma unroll
+    for (int t = 0; t < NC; ++t)
+      if (NP * t + NP - 1 > k && NP * t + par > k) v[t] = fma(ml, cc[c0 + NP * t + par], v[t]);
+    if (lane == k) dk = d;
+    nhit += hit ? 1 : 0;
+  }
+  if (wid == 0 && lane < 16) {
+    sh.dv[c0 + lane] = dk;
+    const int lg = ilog_of(dk);
+    hs[c0 + lane] = lg <= -kBad || lg >= kBad ? 0 : lg >> 1;
+  }
+  asm volatile("barrier.sync 2, 128;" ::: "memory");
+  // the columns of L, the pivots, and the integer operands L 2^h, (L d) 2^-h of the rows below
+  int* xm = reinterpret_cast<int*>(sa.cb);  // (the columns are done)
+  int ma = -kBad, mb = -kBad;
+#pragma unroll
+  for (int t = 0; t < NC; ++t) {
+    const int cl = c0 + NP * t + par;
+    if (row >= cl) A[row * LD + cl] = row == cl ? sh.dv[cl] : l[t];
+    if (row <= cl) l[t] = c8[t] = 0.0;
+    ma = max(ma, shifted(l[t], hs[cl]));
+    mb = max(mb, shifted(c8[t], -hs[cl]));
+  }
+  if (par == 0) {
+    xm[row] = ma;
+    xm[64 + row] = mb;
+  }
+  asm volatile("barrier.sync 2, 128;" ::: "memory");
+  if (par != 0) {
+    atomicMax(&xm[row], ma);
+    atomicMax(&xm[64 + row], mb);
+  }
+  asm volatile("barrier.sync 2, 128;" ::: "memory");
+  const int xa = row_exp(xm[row]), xb = row_exp(xm[64 + row]);
+  if (par == 0) {
+    sa.ea[64 * q + row] = xa;
+    sb.eb[64 * (q & 1) + row] = xb;
+  }
+  int2* ib = sb.ib + (q & 1) * 64 * kLP;
+#pragma unroll
+  for (int t = 0; t < NC; ++t) {
+    const int c = NP * t + par;
+    sa.ia[row * kLI + c0 + c] = halves_of(l[t], hs[c0 + c], xa);
+    ib[row * kLP + c] = halves_of(c8[t], -hs[c0 + c], xb);
+  }
+}
+
+// 16 x 16 block (I, J) of the trailing matrix: a_rs -= sum_m l_rm (l_sm d_m) over panel q; 256 entries
+__device__ __forceinline__ void diag64_update(int q, int I, int J, int idx, double* A, const Diag64Smem& sa,
+                                              const Diag64SmemB& sb) {
+  const int r = 16 * I + (idx >> 4), s = 16 * J + (idx & 15);
+  const int2* ib = sb.ib + (q & 1) * 64 * kLP;
+  IntDot acc;
+#pragma unroll
+  for (int m = 0; m < 16; ++m) acc.add(sa.ia[r * kLI + 16 * q + m], ib[s * kLP + m]);
+  if (r >= s)
+    A[r * kDiagLD + s] -= scaled_double(acc.value(), sa.ea[64 * q + r] + sb.eb[64 * (q & 1) + s] - 56);
+}
+
+// Block row Q of L^{-1}, by the 128 threads of warps 4-7 (tid 0 .. 127 here, barrier 3): the inverse of
+// L_QQ, Linv_QP = -Linv_QQ X_P, its operands (Q < 3), and X of block row Q + 1.
+__device__ __forceinline__ void diag64_inverse_row(int Q, int tid, const double* A, double* V, Diag64Smem& sa,
+                                                   Diag64SmemB& sb, const int* gs, const int* hs) {
+  constexpr int LD = kDiagLD;
+  const int R0 = 16 * Q;
+  auto bar = [] { asm volatile("barrier.sync 3, 128;" ::: "memory"); };
+  if (tid < 32) {
+    // both 8 x 8 diagonal blocks (lane: column), then the 8 x 8 block below them, B1 = -C^{-1} B A^{-1}
+    if (tid < 16) {
+      const int o = R0 + (tid & 8), c = tid & 7;
+      double x[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        double s = (r == c) ? 1.0 : 0.0;
+#pragma unroll
+        for (int m = 0; m < r; ++m) s = fma(-A[(o + r) * LD + o + m], x[m], s);
+        x[r] = (r >= c) ? s : 0.0;
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r) V[(o + r) * LD + o + c] = x[r];
+    }
+    __syncwarp();
+  }
+  bar();
+  if (tid < 64) {  // B A^{-1}
+    const int r = R0 + 8 + (tid >> 3), c = R0 + (tid & 7);
+    double s = 0.0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) s = fma(A[r * LD + R0 + m], V[(R0 + m) * LD + c], s);
+    V[r * LD + c] = s;
+  }
+  bar();
+  double b1 = 0.0;
+  if (tid < 64) {
+    const int r = R0 + 8 + (tid >> 3), c = R0 + (tid & 7);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) b1 = fma(-V[r * LD + R0 + 8 + m], V[(R0 + 8 + m) * LD + c], b1);
+  }
+  bar();
+  if (tid < 64) V[(R0 + 8 + (tid >> 3)) * LD + R0 + (tid & 7)] = b1;
+  if (Q > 0) {
+    bar();
+    // rows of Linv_QQ (8 threads a row), columns of X (2 threads a column)
+    {
+      const int a = tid >> 3, k0 = 2 * (tid & 7);
+      const double x0 = V[(R0 + a) * LD + R0 + k0], x1 = V[(R0 + a) * LD + R0 + k0 + 1];
+      int m = max(shifted(x0, gs[R0 + k0]), shifted(x1, gs[R0 + k0 + 1]));
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(~0u, m, o));
+      const int e = row_exp(m);
+      if (k0 == 0) sa.eq[a] = e;
+      sa.iq[a * kLP + k0] = halves_of(x0, gs[R0 + k0], e);
+      sa.iq[a * kLP + k0 + 1] = halves_of(x1, gs[R0 + k0 + 1], e);
+    }
+    if (tid < 2 * R0) {
+      const int b = tid >> 1, k0 = 8 * (tid & 1);
+      int m = -kBad;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) m = max(m, shifted(sb.x[(k0 + k) * 49 + b], -gs[R0 + k0 + k]));
+      m = max(m, __shfl_xor_sync(~0u, m, 1));
+      const int e = row_exp(m);
+      if (k0 == 0) sa.ex[b] = e;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) sa.ix[b * kLP + k0 + k] = halves_of(sb.x[(k0 + k) * 49 + b], -gs[R0 + k0 + k], e);
+    }
+    bar();
+    for (int idx = tid; idx < 16 * R0; idx += 128) {
+      const int a = idx & 15, b = idx >> 4;
+      IntDot acc;
+#pragma unroll
+      for (int m = 0; m < 16; ++m) acc.add(sa.iq[a * kLP + m], sa.ix[b * kLP + m]);
+      V[(R0 + a) * LD + b] = -scaled_double(acc.value(), sa.eq[a] + sa.ex[b] - 56);
+    }
+  }
+  bar();
+  if (Q == 3) return;
+  if (tid < 2 * (R0 + 16)) {  // the new rows' columns as operands (2 threads a column)
+    const int b = tid >> 1, k0 = 8 * (tid & 1);
+    int m = -kBad;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) m = max(m, shifted(V[(R0 + k0 + k) * LD + b], -hs[R0 + k0 + k]));
+    m = max(m, __shfl_xor_sync(~0u, m, 1));
+    const int e = row_exp(m);
+    if (k0 == 0) sb.ec[48 * Q + b] = e;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      sb.ic[b * kLI + R0 + k0 + k] = halves_of(V[(R0 + k0 + k) * LD + b], -hs[R0 + k0 + k], e);
+  }
+  bar();
+  for (int idx = tid; idx < 16 * (R0 + 16); idx += 128) {
+    const int a = idx & 15, b = idx >> 4;
+    double s = 0.0;
+    for (int M = b >> 4; M <= Q; ++M) {
+      IntDot acc;
+#pragma unroll
+      for (int m = 0; m < 16; ++m) acc.add(sa.ia[(R0 + 16 + a) * kLI + 16 * M + m], sb.ic[b * kLI + 16 * M + m]);
+      s += scaled_double(acc.value(), sa.ea[64 * M + R0 + 16 + a] + sb.ec[48 * M + b] - 56);
+    }
+    sb.x[a * 49 + b] = s;
+  }
+}
+
+// Diagonal block: LDL^T with dynamic regularisation of the pw x pw block at G and the inverse of
+// its unit lower factor, the outputs of bf_diag_block.  Shared memory: A and V (64 x 65: L with the
+// pivots, L^{-1}) and the integer operands.
+//
+// bf_diag_block took 113 us here: it is FP64 warp instructions on one SM (64 clocks each, 76 with all
+// four sub-partitions busy), many with few active lanes.  Panels of 16 columns on four warps: per
+// pivot one column goes through shared memory and one barrier; the reciprocal, the test of
+// the sign and the products with 16 terms (the trailing updates, and the off-diagonal blocks of
+// L^{-1}) are integer arithmetic, the products exact (operands scaled like the packs).  Warps 4-7
+// form L^{-1} a block row behind the panels, and the part of the trailing update that
+// the next panel does not read.  66 us with the packs.
+__device__ int diag64(double* G, int64_t f, int pw, double* D, double* Li, const int8_t* dsign, double eps, double delta,
+                      double* scr, Diag64Smem& sa, Diag64SmemB& sb, DiagScratch<double>& sh, const int* gs, int* hs) {
+  constexpr int LD = kDiagLD;
+  double* A = scr;
+  double* V = scr + 64 * LD;
+  const int tid = threadIdx.x, wid = tid >> 5;
+  const long long key_eps = order_key(eps + 0.0);
+  if (tid < 64) sh.sgn[tid] = tid < pw ? dsign[tid] : (int8_t)1;
+  for (int idx = tid; idx < 64 * 64; idx += NT) {
+    const int i = idx & 63, j = idx >> 6;
+    double v = 0.0;
+    if (i < pw && j < pw && i >= j) v = __ldcg(G + i + (int64_t)j * f);
+    else if (i == j) v = 1.0;  // rows and pivots past pw: the identity
+    A[i * LD + j] = v;
+    V[i * LD + j] = 0.0;
+  }
+  __syncthreads();
+  int nhit = 0;
+  for (int q = 0; q < 4; ++q) {
+    if (wid < 4) {
+      if (q < 2) diag64_panel<2>(q, pw, A, sa, sb, sh, hs, key_eps, delta, nhit);
+      else diag64_panel<4>(q, pw, A, sa, sb, sh, hs, key_eps, delta, nhit);
+    } else if (q > 0) {
+      for (int I = q + 1; I < 4; ++I)  // the rest of panel q - 1's update
+        for (int J = q + 1; J <= I; ++J) {
+          diag64_update(q - 1, I, J, tid - 128, A, sa, sb);
+          diag64_update(q - 1, I, J, tid, A, sa, sb);
+        }
+      diag64_inverse_row(q - 1, tid - 128, A, V, sa, sb, gs, hs);
+    }
+    __syncthreads();
+    for (int I = q + 1; I < 4; ++I) diag64_update(q, I, q + 1, tid, A, sa, sb);
+    __syncthreads();
+  }
+  if (wid >= 4) diag64_inverse_row(3, tid - 128, A, V, sa, sb, gs, hs);
+  __syncthreads();
+  for (int idx = tid; idx < 64 * 64; idx += NT) {
+    const int i = idx & 63, j = idx >> 6;
+    if (i < pw && j < pw && i >= j) {
+      G[i + (int64_t)j * f] = A[i * LD + j];
+      Li[i + (int64_t)j * f] = (i == j) ? 1.0 : V[i * LD + j];
+    }
+  }
+  for (int i = tid; i < pw; i += NT) D[i] = sh.dv[i];
+  return nhit;
+}
+
+struct Packs {
+  unsigned char* base;
+  int64_t nL, P, nbf;
+  __device__ int64_t l(int p, int64_t i) const {
+    return (int64_t)p * (nbf - 1) - (int64_t)p * (p - 1) / 2 + (i - p - 1);
+  }
+  __device__ unsigned char* pa(int p, int64_t i) const { return base + kTileStride * l(p, i); }
+  __device__ unsigned char* pb(int p, int64_t i) const { return base + kTileStride * (nL + l(p, i)); }
+  __device__ unsigned char* pe(int p, int64_t e) const { return base + kTileStride * (2 * nL + (int64_t)p * (p + 1) / 2 + e); }
+  __device__ unsigned char* pt(int p) const { return base + kTileStride * (2 * nL + P * (P + 1) / 2 + p); }
+};
+__device__ __forceinline__ int* exps_of(unsigned char* t) { return reinterpret_cast<int*>(t + kPackBytes); }
+
+__global__ void __launch_bounds__(NT, 1)
+    k_bf_flow64(BigFrontDev bf, const FlowTask* __restrict__ task, int64_t t0, int64_t nt, int* __restrict__ state,
+                int64_t head_off, const int64_t* __restrict__ soff, double* F, double* E, double* Dp,
+                const int8_t* __restrict__ dsign, double eps, double delta, int* hits, int* err, const int* skip,
+                unsigned char* pk) {
+  if (skip && *skip) return;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  unsigned char* sm = smraw + ((1024u - (s_addr(smraw) & 1023u)) & 1023u);
+  unsigned char* smB = sm + kOffB;
+  double* scr = reinterpret_cast<double*>(sm + kOffS);
+  long long* X = reinterpret_cast<long long*>(sm + kOffS);
+  __shared__ DiagScratch<double> dsh;
+  __shared__ PackScratch ps;
+  __shared__ int eA[64], eB[64], hs[64], gs[64];
+  __shared__ double dinv[64], dinv2[64];  // 1 / d_j and what its rounding left
+  __shared__ FlowTask s_task;
+  __shared__ int s_go, s_flag;
+  __shared__ __align__(8) uint64_t s_bar[2];
+  __shared__ uint32_t s_tmem;
+  int* head = state + head_off;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s_addr(&s_bar[0])), "r"(1));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s_addr(&s_bar[1])), "r"(1));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_flag = 0;
+  }
+  for (int k = tid; k < kSlice / 16; k += NT) reinterpret_cast<uint4*>(sm + kDig * kSlice)[k] = make_uint4(0, 0, 0, 0);
+  if (wid == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_addr(&s_tmem)), "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  fence_async_shared();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = s_tmem;
+  const uint32_t bar_ld = s_addr(&s_bar[0]), bar_mma = s_addr(&s_bar[1]);
+  uint32_t par_ld = 0, par_mma = 0;
+  // row and columns of this thread's part of a product
+  const int orow = 32 * (wid & 1) + lane, ocol = 16 * (2 * (wid >> 2) + ((wid >> 1) & 1));
+  for (;;) {
+    if (tid == 0) {
+      const int cur = atomicAdd(head, 1);
+      int go = 0;
+      if (cur < nt) {
+        const FlowTask tk = task[t0 + cur];
+        s_task = tk;
+        const int64_t b = tk.bf;
+        const Geo g{bf.f[b], bf.c[b], (bf.c[b] + NB - 1) / NB, flow_nbf(bf.f[b], bf.c[b])};
+        const Words w = words_of(state + soff[b], g);
+        const int p = tk.p;
+        const int* wp[3];
+        int wv[3];
+        int nw;
+        switch (tk.kind) {
+          case 0:
+            wp[0] = w.t(p, p), wv[0] = p;
+            nw = 1;
+            break;
+          case 1:
+            wp[0] = w.diag + p, wv[0] = 1;
+            wp[1] = w.t(tk.i, p), wv[1] = p;
+            nw = 2;
+            break;
+          case 2:
+            wp[0] = w.diag + p, wv[0] = 1;
+            wp[1] = w.e(p, tk.j), wv[1] = p - tk.j;
+            nw = 2;
+            break;
+          case 3:
+            wp[0] = w.trsm + tk.i, wv[0] = p + 1;
+            wp[1] = w.trsm + tk.j, wv[1] = p + 1;
+            wp[2] = w.t(tk.i, tk.j), wv[2] = p;
+            nw = 3;
+            break;
+          default:
+            wp[0] = w.trsm + tk.i, wv[0] = p + 1;
+            if (tk.j < p)
+              wp[1] = w.e(p, tk.j), wv[1] = p - tk.j + 1;
+            else
+              wp[1] = w.pe + p, wv[1] = 1;
+            wp[2] = w.e(tk.i, tk.j), wv[2] = p - tk.j;
+            nw = 3;
+            break;
+        }
+        int got[3] = {0, 0, 0};
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          if (q < nw) got[q] = ld_relaxed(wp[q]);
+        bool ok = true;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          if (q < nw && got[q] < wv[q]) ok = ok && wait_ge(wp[q], wv[q], err);
+        go = ok ? 1 : 0;
+        if (ok) __threadfence();
+      }
+      s_go = go;
+    }
+    __syncthreads();
+    if (!s_go) break;
+    const FlowTask tk = s_task;
+    const int64_t b = tk.bf;
+    const Geo g{bf.f[b], bf.c[b], (bf.c[b] + NB - 1) / NB, flow_nbf(bf.f[b], bf.c[b])};
+    const Packs pkr{pk + (int64_t)kTileStride * bf.pkoff64[b], flow_pk_nl(g.f, g.c), g.P, g.nbf};
+    const Words w = words_of(state + soff[b], g);
+    const int p = tk.p, pw = bnrow(g, p);
+    const int64_t f = g.f, k0 = (int64_t)p * NB;
+    double* G = F + bf.goff[b];
+    double* Eb = E + bf.eoff[b];
+    const int64_t kp = bf.k0pos[b] + k0;
+    bool stop = false;
+    // a task's products: copies of the packs (thread 0), then, with the A digits in place, the MMAs
+    auto wait_bar = [&](uint32_t bar, uint32_t& par) {
+      if (!mbar_wait(bar, par)) atomicExch(&s_flag, 1);
+      __syncthreads();
+      if (s_flag) {
+        if (tid == 0) {
+          atomicExch(err, 2);
+          mbar_wait(bar, par);  // once more for the copies or MMAs in flight
+        }
+        return false;
+      }
+      par ^= 1u;
+      return true;
+    };
+    if (tk.kind == 0) {
+      // D(p): the diagonal block on the FP64 pipe, then its packs
+      if (tid < 64) gs[tid] = tid < pw ? ilog_of(__ldcg(G + (k0 + tid) + (k0 + tid) * f)) >> 1 : 0;
+      if (tid < 64 && (gs[tid] <= -kBad / 2 || gs[tid] >= kBad / 2)) gs[tid] = 0;
+      const int nhit = diag64(G + k0 + k0 * f, f, pw, Dp + kp, Eb + k0 + k0 * f, dsign + kp, eps, delta, scr,
+                              *reinterpret_cast<Diag64Smem*>(sm), *reinterpret_cast<Diag64SmemB*>(smB), dsh, gs, hs);
+      if (tid == 0 && nhit) atomicAdd(hits, nhit);
+      __syncthreads();
+      if (tid < 64) {
+        ps.sh[tid] = gs[tid];
+        int* ex = exps_of(pkr.pt(p));
+        ex[64 + tid] = gs[tid];
+        ex[128 + tid] = hs[tid];
+      }
+      const double* V = scr + 64 * kDiagLD;
+      const int r = tid & 63, kq = tid >> 6;
+      double x[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const int l = 16 * kq + u;
+        x[u] = (r < pw && l < r) ? V[r * kDiagLD + l] : ((l == r && r < pw) ? 1.0 : 0.0);
+      }
+      pack_rows(x, pkr.pt(p), exps_of(pkr.pt(p)), ps);
+      fence_async_global();
+      __syncthreads();
+      if (tid == 0) {
+        __threadfence();
+        st_release(w.diag + p, 1);
+      }
+      fence_async_shared();  // the operands' space is the next task's, by bulk copies
+      // PE(p, p): rows the columns of Linv (after the release: only EU(p, i, p) waits for it)
+      if (tid < 64) ps.sh[tid] = -hs[tid];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const int k = 16 * kq + u;
+        x[u] = (k < pw && r < k) ? V[k * kDiagLD + r] : ((k == r && r < pw) ? 1.0 : 0.0);
+      }
+      pack_rows(x, pkr.pe(p, p), exps_of(pkr.pe(p, p)), ps);
+      fence_async_global();
+      __syncthreads();
+      if (tid == 0) {
+        __threadfence();
+        st_release(w.pe + p, 1);
+      }
+      continue;
+    }
+    if (tk.kind == 1 || tk.kind == 2) {
+      // T(p, i): rows of F_IK; Efin(p, e): rows the columns of E_KC; both times PT(p)^T
+      const bool efin = tk.kind == 2;
+      const int64_t r0 = efin ? (int64_t)tk.j * NB : brow0(g, tk.i);
+      const int nr = efin ? NB : bnrow(g, tk.i);
+      unsigned char* pt = pkr.pt(p);
+      if (tid == 0) {
+        fence_async_global();
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_ld), "r"(kPackBytes) : "memory");
+        bulk_copy(s_addr(smB), pt, kPackBytes, bar_ld);
+      }
+      const int r = tid & 63, kq = tid >> 6;
+      double x[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const int l = 16 * kq + u;
+        const double* a = efin ? Eb + (k0 + l) + (r0 + r) * f : G + (r0 + r) + (k0 + l) * f;
+        x[u] = (r < nr && l < pw) ? __ldcg(a) : 0.0;
+      }
+      if (tid < 64) {
+        const int* ex = exps_of(pt);
+        eB[tid] = __ldcg(ex + tid);
+        ps.sh[tid] = -__ldcg(ex + 64 + tid);
+        hs[tid] = __ldcg(ex + 128 + tid);
+        if (!efin) {
+          const double d = tid < pw ? __ldcg(Dp + kp + tid) : 1.0, r = 1.0 / d;
+          dinv[tid] = tid < pw ? r : 0.0;
+          dinv2[tid] = tid < pw ? fma(-d, r, 1.0) * r : 0.0;
+        }
+      }
+      pack_rows(x, sm, eA, ps);
+      fence_async_shared();
+      stop = !wait_bar(bar_ld, par_ld);
+      if (!stop) {
+        if (tid == 0) issue_products(s_addr(sm), s_addr(smB), tmem, bar_mma);
+        stop = !wait_bar(bar_mma, par_mma);
+      }
+      if (stop) break;
+      double o[16];
+      read_products(tmem, eA, eB, X, o);
+      // (thread: row orow, columns ocol .. ocol + 15: what the packs hold per thread, too)
+      if (efin) {
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+          if (ocol + u < pw) Eb[(k0 + ocol + u) + (r0 + orow) * f] = o[u];
+          else o[u] = 0.0;
+      }
+      double q[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        if (efin) continue;
+        if (ocol + u >= pw || orow >= nr) o[u] = 0.0;
+        q[u] = fma(o[u], dinv[ocol + u], o[u] * dinv2[ocol + u]);  // o / d to half an ulp
+        if (ocol + u < pw && orow < nr) G[(r0 + orow) + (k0 + ocol + u) * f] = q[u];
+      }
+      // through shared memory to the packing order (row tid & 63, k 16 (tid >> 6) ..)
+      __syncthreads();
+      double* Y = scr;
+#pragma unroll
+      for (int u = 0; u < 16; ++u) Y[(ocol + u) * 64 + orow] = o[u];
+      if (tid < 64) ps.sh[tid] = -hs[tid];
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 16; ++u) x[u] = Y[(16 * kq + u) * 64 + r];
+      unsigned char* dst = efin ? pkr.pe(p, tk.j) : pkr.pb(p, tk.i);
+      pack_rows(x, dst, exps_of(dst), ps);
+      if (!efin) {
+        __syncthreads();
+        if (tid < 64) ps.sh[tid] = hs[tid];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) Y[(ocol + u) * 64 + orow] = q[u];
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 16; ++u) x[u] = Y[(16 * kq + u) * 64 + r];
+        pack_rows(x, pkr.pa(p, tk.i), exps_of(pkr.pa(p, tk.i)), ps);
+      }
+      fence_async_global();
+      __syncthreads();
+      if (tid == 0) {
+        __threadfence();
+        if (efin) st_release(w.e(p, tk.j), p - (int)tk.j + 1);
+        else st_release(w.trsm + tk.i, p + 1);
+      }
+      continue;
+    }
+    // U(p, i, j), EU(p, i, e)
+    const bool etile = tk.kind != 3;
+    const int64_t i0 = brow0(g, tk.i), c0 = etile ? (int64_t)tk.j * NB : brow0(g, tk.j);
+    const int ni = bnrow(g, tk.i), nc = bnrow(g, tk.j);
+    const bool diag = !etile && tk.i == tk.j;
+    double* base = etile ? Eb : G;
+    unsigned char* ta = pkr.pa(p, tk.i);
+    unsigned char* tb = etile ? pkr.pe(p, tk.j) : pkr.pb(p, tk.j);
+    if (tid == 0) {
+      fence_async_global();  // the packs were stored by generic writes (acquired above)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_ld), "r"(2 * kPackBytes)
+                   : "memory");
+      bulk_copy(s_addr(sm), ta, kPackBytes, bar_ld);
+      bulk_copy(s_addr(smB), tb, kPackBytes, bar_ld);
+    }
+    if (tid < 64) eA[tid] = __ldcg(exps_of(ta) + tid);
+    else if (tid < 128) eB[tid - 64] = __ldcg(exps_of(tb) + tid - 64);
+    double tv[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int cc = ocol + u;
+      tv[u] = (orow < ni && cc < nc && (!diag || orow >= cc)) ? __ldcg(base + (i0 + orow) + (c0 + cc) * f) : 0.0;
+    }
+    stop = !wait_bar(bar_ld, par_ld);
+    if (!stop) {
+      if (tid == 0) issue_products(s_addr(sm), s_addr(smB), tmem, bar_mma);
+      stop = !wait_bar(bar_mma, par_mma);
+    }
+    if (stop) break;
+    double o[16];
+    read_products(tmem, eA, eB, X, o);
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int cc = ocol + u;
+      if (orow < ni && cc < nc && (!diag || orow >= cc)) base[(i0 + orow) + (c0 + cc) * f] = tv[u] - o[u];
+    }
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      if (etile) st_release(w.e(tk.i, tk.j), p - (int)tk.j + 1);
+      else st_release(w.t(tk.i, tk.j), p + 1);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (wid == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+}  // namespace
+
+int flow64_setup_attributes() {
+  CLR_CUDA(cudaFuncSetAttribute(k_bf_flow64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
+  return CLR_OK;
+}
+
+int flow64_level(cudaStream_t st, const BigFrontDev& bf, const FlowTask* task, int64_t t0, int64_t nt, int* state,
+                 int64_t head_off, const int64_t* soff, int grid, double* F, double* E, double* Dp, const int8_t* dsign,
+                 double eps, double delta, int* hits, int* err, const int* skip, unsigned char* pk) {
+  if (nt <= 0) return CLR_OK;
+  k_bf_flow64<<<(unsigned)std::min<int64_t>(nt, grid), NT, kSmem, st>>>(bf, task, t0, nt, state, head_off, soff, F, E, Dp,
+                                                                       dsign, eps, delta, hits, err, skip, pk);
+  CLR_CHECK_LAUNCH();
+  return CLR_OK;
+}
+
+}  // namespace clr

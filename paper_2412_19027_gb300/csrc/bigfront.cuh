@@ -26,6 +26,7 @@ struct BigFrontDev {
   const int64_t* yoff = nullptr;  // offset of its forward result y (c entries)
   const int64_t* rk = nullptr;    // offset of its rows in rows_kkt
   const int64_t* pkoff = nullptr; // first packed operand tile of the front in its level's tiles (tensor-core flow)
+  const int64_t* pkoff64 = nullptr; // first digit pack of the front in its level's packs (FP64 flow on tensor cores)
   int64_t epool = 0, ypool = 0;
 };
 
@@ -132,6 +133,22 @@ struct FlowTc {
 // Host: encode the tensor map over tc->pk (tc->tiles packed tiles).  CLR_E_CUDA
 // if the driver entry point is missing or rejects the map.
 int flow_tc_encode(FlowTc* tc);
+
+// FP64 factor: the large fronts whose products run on the tensor cores as 8-bit digits
+// (bigflow64.cu).  Packs of a front with P pivot blocks: PA and PB of its L tiles, PE, PT.
+constexpr int64_t kPack64Bytes = 7 * 64 * 64 * 2 + 3 * 64 * 4;
+__host__ __device__ inline int64_t flow_pk64_tiles(int64_t f, int64_t c) {
+  const int64_t P = (c + kBfNB - 1) / kBfNB;
+  return 2 * flow_pk_nl(f, c) + P * (P + 1) / 2 + P;
+}
+// Fronts of more rows than this.  Five 64-row blocks or fewer are a chain of diagonal blocks with
+// hardly a product beside it, and small dense QPs (roots up to 260 rows) solved to 1e-8 amplify a
+// change of rounding to 1e-9 in their multipliers.
+constexpr int64_t kFlow64Rows = 320;
+int flow64_setup_attributes();
+int flow64_level(cudaStream_t st, const BigFrontDev& bf, const FlowTask* task, int64_t t0, int64_t nt, int* state,
+                 int64_t head_off, const int64_t* soff, int grid, double* F, double* E, double* Dp, const int8_t* dsign,
+                 double eps, double delta, int* hits, int* err, const int* skip, unsigned char* pk);
 
 template <typename T>
 struct BigFrontOps {

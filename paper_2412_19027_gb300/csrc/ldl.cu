@@ -459,7 +459,7 @@ T* up(DeviceArena& ar, const std::vector<T>& v) {
 // dur: typical durations (microseconds) by kind D, T, Efin, U, EU, DX; span: the
 // simulated duration of the level.
 static bool flow_schedule_order(std::vector<FlowTask>& tasks, int64_t t0, const std::vector<int64_t>& P_of,
-                                int workers, const double* dur, double* span, bool split = false) {
+                                int workers, const double* dur, double* span, int mode = 0) {
   const int64_t n = (int64_t)tasks.size() - t0;
   *span = 0.0;
   if (n <= 1) return true;
@@ -478,11 +478,13 @@ static bool flow_schedule_order(std::vector<FlowTask>& tasks, int64_t t0, const 
     auto it = idx.find(key(b, kind, p, i, j));
     return it == idx.end() ? -1 : it->second;
   };
-  // split: FP64 chain tasks TX(p, q), UX(p, q), D(p) in place of DX(p) (bigfront.cuh)
+  // mode 1: FP64 chain tasks TX(p, q), UX(p, q), D(p) in place of DX(p) (bigfront.cuh); 2: D(p),
+  // T(p, i), U(p, i, j) only (bigflow64.cu)
+  const bool split = mode == 1, plain = mode == 2;
   auto dd = [&](int64_t b, int64_t p) {
-    return (p == 0 || split) ? find(b, 0, p, p, p) : find(b, 5, p, p, p);
+    return (p == 0 || split || plain) ? find(b, 0, p, p, p) : find(b, 5, p, p, p);
   };
-  auto folded = [&](int64_t b, int64_t p, int64_t i) { return i == p + 1 && i < P_of[b]; };
+  auto folded = [&](int64_t b, int64_t p, int64_t i) { return !plain && i == p + 1 && i < P_of[b]; };
   struct Edge {
     int64_t to;
     bool mid;  // the successor needs only the early-published rows of a DX task
@@ -506,6 +508,7 @@ static bool flow_schedule_order(std::vector<FlowTask>& tasks, int64_t t0, const 
       case 0:
         if (split && p >= 1)
           for (int64_t q = 0; q < 4; ++q) d.emplace_back(find(b, 7, p, q, 0), false);
+        if (plain && p >= 1) d.emplace_back(find(b, 3, p - 1, p, p), false);
         break;
       case 5:
         d.emplace_back(dd(b, p - 1), false);
@@ -605,6 +608,76 @@ static bool flow_schedule_order(std::vector<FlowTask>& tasks, int64_t t0, const 
   }
   std::copy(out.begin(), out.end(), tasks.begin() + t0);
   return true;
+}
+
+// The FP64 factor's task tables: fronts with FMA products (the fused chain task split into
+// TX(p, q), UX(p, q) and D(p), bigfront.cuh), and, with emu, the fronts of more than
+// kFlow64Rows rows with their products on the tensor cores (bigflow64.cu).
+static int flow64_tables(DeviceArena& ar, LdlStructure& st, bool emu) {
+  const int64_t nlev = st.nlev, nb = (int64_t)st.h_bf_f.size();
+  std::vector<int64_t> P_of(nb);
+  std::vector<std::vector<int64_t>> of(nlev);
+  for (int64_t b = 0; b < nb; ++b) {
+    P_of[b] = (st.h_bf_c[b] + kBfNB - 1) / kBfNB;
+    of[st.h_bf_lev[b]].push_back(b);
+  }
+  int flow_sms = 152, dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+      sms > 0)
+    flow_sms = sms;
+  std::vector<FlowTask> t64, t64e;
+  st.flow_t0_64.assign(nlev, 0);
+  st.flow_nt_64.assign(nlev, 0);
+  st.flow_one64.assign(nlev, 0);
+  st.flow_t0_64e.assign(nlev, 0);
+  st.flow_nt_64e.assign(nlev, 0);
+  for (int64_t l = 0; l < nlev; ++l) {
+    st.flow_t0_64[l] = (int64_t)t64.size();
+    st.flow_t0_64e[l] = (int64_t)t64e.size();
+    for (int64_t b : of[l]) {
+      const bool e64 = emu && st.h_bf_f[b] > kFlow64Rows;
+      std::vector<FlowTask>& out = e64 ? t64e : t64;
+      auto add = [&](int kind, int64_t p, int64_t i, int64_t j) {
+        out.push_back(FlowTask{(int32_t)b, (int16_t)kind, (int16_t)p, (int32_t)i, (int32_t)j});
+      };
+      const int64_t P = P_of[b], n = flow_nbf(st.h_bf_f[b], st.h_bf_c[b]);
+      for (int64_t p = 0; p < P; ++p) {
+        if (p >= 1 && !e64) {
+          for (int64_t q = 0; q < 4; ++q) add(6, p, q, 0);
+          for (int64_t q = 0; q < 4; ++q) add(7, p, q, 0);
+        }
+        add(0, p, p, p);
+        for (int64_t i = p + 1; i < n; ++i)
+          if (e64 || !(i == p + 1 && i < P)) add(1, p, i, p);
+        for (int64_t e = 0; e < p; ++e) add(2, p, p, e);
+        for (int64_t j = p + 1; j < n; ++j)
+          for (int64_t i = j; i < n; ++i)
+            if (e64 || !(i == p + 1 && j == p + 1 && i < P)) add(3, p, i, j);
+        for (int64_t i = p + 1; i < n; ++i)
+          for (int64_t e = 0; e <= p; ++e) add(4, p, i, e);
+      }
+    }
+    st.flow_nt_64[l] = (int64_t)t64.size() - st.flow_t0_64[l];
+    st.flow_nt_64e[l] = (int64_t)t64e.size() - st.flow_t0_64e[l];
+    // FP64 task times (microseconds; D, T, Efin, U, EU, -, TX, UX) from per-task
+    // timestamps on a GB300 at two CTAs per SM (banded LP generator), and estimates
+    // for one CTA per SM (a task then has the SM's FP64 pipe to itself)
+    static const double dur64_2[8] = {95.0, 41.0, 57.0, 57.0, 57.0, 204.0, 12.0, 14.0};
+    static const double dur64_1[8] = {70.0, 28.0, 38.0, 36.0, 36.0, 150.0, 8.0, 9.0};
+    std::vector<FlowTask> one(t64.begin() + st.flow_t0_64[l], t64.end());
+    double span2 = 0.0, span1 = 0.0;
+    if (!flow_schedule_order(t64, st.flow_t0_64[l], P_of, 2 * flow_sms, dur64_2, &span2, 1) ||
+        !flow_schedule_order(one, 0, P_of, flow_sms, dur64_1, &span1, 1))
+      return CLR_E_INVALID;
+    st.flow_one64[l] = span1 < 0.97 * span2 ? 1 : 0;
+    if (st.flow_one64[l]) std::copy(one.begin(), one.end(), t64.begin() + st.flow_t0_64[l]);
+    // with the products on the tensor cores, one CTA per SM (bigflow64.cu)
+    static const double dur64e[8] = {66.0, 27.0, 23.0, 13.0, 13.0, 0.0, 0.0, 0.0};
+    if (!flow_schedule_order(t64e, st.flow_t0_64e[l], P_of, flow_sms, dur64e, &span1, 2)) return CLR_E_INVALID;
+  }
+  st.flow_task64 = t64.empty() ? nullptr : ar.upload(t64.data(), (int64_t)t64.size());
+  st.flow_task64e = t64e.empty() ? nullptr : ar.upload(t64e.data(), (int64_t)t64e.size());
+  return (!t64.empty() && !st.flow_task64) || (!t64e.empty() && !st.flow_task64e) ? CLR_E_OOM : CLR_OK;
 }
 
 int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<int8_t>& dsign,
@@ -997,56 +1070,32 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       else if (st.flow_one[l]) std::copy(one.begin(), one.end(), tasks.begin() + st.flow_t0[l]);
     }
     st.flow_words = words;
-    // the FP64 factor's table: the same levels, fronts and version words, with the
-    // fused chain task split into TX(p, q), UX(p, q) and D(p) (bigfront.cuh)
-    std::vector<FlowTask> tasks64;
-    st.flow_t0_64.assign(sy.nlev, 0);
-    st.flow_nt_64.assign(sy.nlev, 0);
-    st.flow_one64.assign(sy.nlev, 0);
-    for (int64_t l = 0; l < sy.nlev; ++l) {
-      if (st.lev_big[l].empty()) continue;
-      st.flow_t0_64[l] = (int64_t)tasks64.size();
-      auto add = [&](int64_t b, int kind, int64_t p, int64_t i, int64_t j) {
-        tasks64.push_back(FlowTask{(int32_t)b, (int16_t)kind, (int16_t)p, (int32_t)i, (int32_t)j});
-      };
-      for (int64_t J : st.lev_big[l]) {
-        const int64_t b = bid_of[J];
-        const int64_t P = P_of[b], nb = flow_nbf(bf_f[b], bf_c[b]);
-        for (int64_t p = 0; p < P; ++p) {
-          if (p >= 1) {
-            for (int64_t q = 0; q < 4; ++q) add(b, 6, p, q, 0);
-            for (int64_t q = 0; q < 4; ++q) add(b, 7, p, q, 0);
-          }
-          add(b, 0, p, p, p);
-          for (int64_t i = p + 1; i < nb; ++i)
-            if (!(i == p + 1 && i < P)) add(b, 1, p, i, p);
-          for (int64_t e = 0; e < p; ++e) add(b, 2, p, p, e);
-          for (int64_t j = p + 1; j < nb; ++j)
-            for (int64_t i = j; i < nb; ++i)
-              if (!(i == p + 1 && j == p + 1 && i < P)) add(b, 3, p, i, j);
-          for (int64_t i = p + 1; i < nb; ++i)
-            for (int64_t e = 0; e <= p; ++e) add(b, 4, p, i, e);
+    st.h_bf_f = bf_f;
+    st.h_bf_c = bf_c;
+    st.h_bf_lev.assign(bf_f.size(), 0);
+    for (int64_t l = 0; l < sy.nlev; ++l)
+      for (int64_t J : st.lev_big[l]) st.h_bf_lev[bid_of[J]] = l;
+    std::vector<int64_t> pk64(bf_f.size(), 0);
+    st.flow_head64e.assign(sy.nlev, 0);
+    {
+      std::vector<int64_t> used(sy.nlev, 0);
+      for (size_t b = 0; b < bf_f.size(); ++b)
+        if (bf_f[b] > kFlow64Rows) {
+          pk64[b] = used[st.h_bf_lev[b]];
+          used[st.h_bf_lev[b]] += flow_pk64_tiles(bf_f[b], bf_c[b]);
         }
+      for (int64_t l = 0; l < sy.nlev; ++l) {
+        st.pk64_tiles = std::max(st.pk64_tiles, used[l]);
+        if (used[l] > 0) st.flow_head64e[l] = words++;
       }
-      st.flow_nt_64[l] = (int64_t)tasks64.size() - st.flow_t0_64[l];
-      // FP64 task times (microseconds; D, T, Efin, U, EU, -, TX, UX) from per-task
-      // timestamps on a GB300 at two CTAs per SM (banded LP generator), and estimates
-      // for one CTA per SM (a task then has the SM's FP64 pipe to itself)
-      static const double dur64_2[8] = {95.0, 41.0, 57.0, 57.0, 57.0, 204.0, 12.0, 14.0};
-      static const double dur64_1[8] = {70.0, 28.0, 38.0, 36.0, 36.0, 150.0, 8.0, 9.0};
-      std::vector<FlowTask> one(tasks64.begin() + st.flow_t0_64[l], tasks64.end());
-      double span2 = 0.0, span1 = 0.0;
-      if (!flow_schedule_order(tasks64, st.flow_t0_64[l], P_of, 2 * flow_sms, dur64_2, &span2, true) ||
-          !flow_schedule_order(one, 0, P_of, flow_sms, dur64_1, &span1, true))
-        return CLR_E_INVALID;
-      st.flow_one64[l] = span1 < 0.97 * span2 ? 1 : 0;
-      if (st.flow_one64[l]) std::copy(one.begin(), one.end(), tasks64.begin() + st.flow_t0_64[l]);
     }
+    st.flow_words = words;
+    bd.pkoff64 = up(ar, pk64);
+    if (flow64_tables(ar, st, st.flow_emu) != CLR_OK) return CLR_E_OOM;
     if (!tasks.empty()) {
       st.flow_task = ar.upload(tasks.data(), (int64_t)tasks.size());
-      st.flow_task64 = ar.upload(tasks64.data(), (int64_t)tasks64.size());
       st.flow_soff = ar.upload(soff.data(), (int64_t)soff.size());
-      if (!st.flow_task || !st.flow_task64 || !st.flow_soff) return CLR_E_OOM;
+      if (!st.flow_task || !st.flow_soff) return CLR_E_OOM;
     }
   }
   st.sn_ptr = up(ar, sy.sn_ptr);
@@ -1106,6 +1155,21 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
       if (!tcs.pk) return CLR_E_OOM;
       const int rc = flow_tc_encode(&tcs);
       if (rc != CLR_OK) return rc;
+    }
+    if (sizeof(T) == 8 && flow && st.flow_emu && st.flow_task64e) {
+      // (not more than half of what is free: what is allocated after this had that room before)
+      size_t room = 0, all = 0;
+      if (cudaMemGetInfo(&room, &all) == cudaSuccess && (size_t)(st.pk64_tiles * kPack64Bytes) <= room / 2)
+        pk64 = ar.alloc_n<unsigned char>(st.pk64_tiles * kPack64Bytes);
+      if (!pk64) {  // no room for the packs: FMA products on every front
+        cudaGetLastError();
+        LdlStructure& ms = const_cast<LdlStructure&>(st);
+        ms.flow_emu = false;
+        const int rc = flow64_tables(ar, ms, false);
+        if (rc != CLR_OK) return rc;
+      } else if (flow64_setup_attributes() != CLR_OK) {
+        return CLR_E_CUDA;
+      }
     }
     const int occ = BigFrontOps<T>::flow_occupancy(tc);
     if (occ < 0) return CLR_E_CUDA;
@@ -1175,6 +1239,14 @@ int LdlFactor<T>::factor(cudaStream_t stm, const double* kval, const IterScal* s
       const FlowTask* tab = f64 ? S.flow_task64 : S.flow_task;
       const int64_t ft0 = f64 ? S.flow_t0_64[l] : S.flow_t0[l], fnt = f64 ? S.flow_nt_64[l] : S.flow_nt[l];
       const bool one = f64 ? S.flow_one64[l] != 0 : S.flow_one[l] != 0;
+      if constexpr (sizeof(T) == 8) {
+        if (use_flow && S.flow_nt_64e[l] > 0) {
+          int rc = flow64_level(stm, S.bfd, S.flow_task64e, S.flow_t0_64e[l], S.flow_nt_64e[l], flow_state,
+                                S.flow_head64e[l], S.flow_soff, flow_sms, F, E, Dp, S.dsign, dyn_eps, dyn_delta, dyn_hits,
+                                tc_err, skip, pk64);
+          if (rc) return rc;
+        }
+      }
       int rc = use_flow ? BigFrontOps<T>::flow_level(stm, S.bfd, tab, ft0, fnt, flow_state,
                                                      S.flow_head[l], S.flow_soff,
                                                      one ? flow_sms : flow_sms * flow_occ, one,

@@ -66,6 +66,13 @@ struct LdlStructure {
   std::vector<int8_t> flow_tc;   // per level: FP32 factors use the tensor-core launch
   // the FP64 factor's task table (the fused chain task split, bigfront.cuh), per level
   FlowTask* flow_task64 = nullptr;
+  // the FP64 fronts whose products run on the tensor cores (bigflow64.cu): their table, per level
+  // its range and counter; flow_emu: allowed (set before ldl_structure_upload)
+  bool flow_emu = true;
+  FlowTask* flow_task64e = nullptr;
+  std::vector<int64_t> flow_t0_64e, flow_nt_64e, flow_head64e;
+  int64_t pk64_tiles = 0;  // digit packs of the largest level
+  std::vector<int64_t> h_bf_f, h_bf_c, h_bf_lev;  // big fronts: rows, pivots, level
   std::vector<int64_t> flow_t0_64, flow_nt_64;
   std::vector<int8_t> flow_one64;
   int64_t flow_words = 0;
@@ -113,6 +120,7 @@ struct LdlFactor {
   bool flow = true;       // big fronts by the dataflow kernel (one launch per level); else per-panel launches
   int flow_tc = 1;        // FP32 dataflow, trailing and E updates on the tensor cores (TF32 hi/lo parts):
                           // 0 never, 1 on the levels whose simulated schedule is shorter that way, 2 always
+  unsigned char* pk64 = nullptr;  // FP64: digit packs of the largest level (null: FMA products on every front)
   FlowTc tcs;             // its packed operand tiles and their tensor map (allocated when used)
   int* flow_state = nullptr;
   int flow_sms = 0, flow_occ = 0;  // SMs of the device, resident flow CTAs per SM

@@ -170,3 +170,41 @@ def test_large_front_sweeps(bits, leaves, c, r, m):
     eps = 2.2e-16 if bits == 64 else 1.2e-7
     assert np.abs(Kf @ x - rhs).max() <= 10 * np.sqrt(N) * eps * max(1.0, np.abs(x).max()) * 10
     assert hits == 0 and np.all(sgn * D > 0)
+
+
+# FP64 fronts of more than 320 rows with products of 8-bit digits on the tensor cores, at the ends
+# of their 64-row blocks, against FMA products (schedule 2).  Per entry the residual of a solve
+# by computed factors is below 3 n u |L||D||L^T||x| (Higham, "Accuracy and Stability of Numerical
+# Algorithms", ch. 10), with rows and columns scaled by powers of ten as well; the inverses of the
+# diagonal blocks add their condition (here below 10).
+@pytest.mark.parametrize("scale", [0, 60])
+@pytest.mark.parametrize("n", [320, 321, 383, 384, 385, 449, 512, 639])
+def test_large_fp64_fronts_by_digits(n, scale):
+    import scipy.sparse as sp
+    rng = np.random.default_rng(n + scale)
+    p = 2 * n // 3
+    K = rng.standard_normal((n, n)) / np.sqrt(n)
+    K = K + K.T
+    H, G = rng.standard_normal((p, p)) / np.sqrt(p), rng.standard_normal((n - p, n - p)) / np.sqrt(n - p)
+    K[:p, :p], K[p:, p:] = H @ H.T + 0.1 * np.eye(p), -(G @ G.T + 0.1 * np.eye(n - p))
+    q = rng.permutation(n)  # both signs in every block
+    K, sgn = K[np.ix_(q, q)], np.where(q < p, 1.0, -1.0)
+    s = 10.0 ** np.round(rng.uniform(-scale, scale, n))
+    K, rhs = K * s[:, None] * s[None, :], rng.standard_normal(n) * s
+    L, D = np.tril(K).astype(np.float64), np.zeros(n)
+    for j in range(n):
+        D[j] = L[j, j]
+        c = L[j + 1:, j] / D[j]
+        L[j + 1:, j + 1:] -= np.tril(np.outer(c, L[j + 1:, j]))
+        L[j + 1:, j], L[j, j] = c, 1.0
+    res = {}
+    for sch in (1, 2):
+        x, Dg, hits = clr.clr_ldl_solve(sp.csc_matrix(np.tril(K)), sgn, rhs, order=np.arange(n), dyn_reg_eps=0.0,
+                                        big_front_schedule=sch)
+        bound = 3 * n * 2.0 ** -53 * (np.abs(L) @ (np.abs(D)[:, None] * (np.abs(L).T @ np.abs(x)[:, None])))[:, 0]
+        r = np.abs((rhs.astype(np.longdouble) - K.astype(np.longdouble) @ x).astype(np.float64))
+        assert np.all(r <= 10 * bound)
+        assert hits == 0 and np.all(sgn * Dg > 0)
+        np.testing.assert_allclose(Dg, D, rtol=1e-10)
+        res[sch] = np.linalg.norm(r / s)
+    assert res[1] <= 2 * res[2]

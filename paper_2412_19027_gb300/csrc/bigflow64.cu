@@ -32,8 +32,8 @@
 //   U: F_IJ -= PA(p, i) PB(p, j)^T;  EU: E_IC -= PA(p, i) PE(p, e)^T;
 //   T: L_IK = (F_IK 2^-g) PT(p)^T D^{-1};  Efin: E_KC^T <- (E_KC^T 2^-g) PT(p)^T,
 // with F_IK and E_KC^T split in the task.  One CTA per SM (512 columns of tensor memory).
-// Per task on a GB300 (front of 2052 rows; FMA version in brackets): D 66 us (95), T 27 (41), Efin 23
-// (57), U 13 (57), EU 13 (57); the front: 4.0 ms.
+// Per task on a GB300 (front of 2052 rows; FMA version in brackets): D 70 us (95), T 24 (41), Efin 18
+// (57), U 11 (57), EU 11 (57); the front: 3.9 ms.
 #include <algorithm>
 
 #include "bfdiag.cuh"
@@ -52,7 +52,11 @@ static_assert(kTileStride == kPackBytes + 3 * 64 * 4 && kTileStride % 16 == 0, "
 constexpr int kBad = 1 << 20;                         // row exponent of a row with a value that is not finite
 // shared memory: A digits (an eighth matrix of zeros pairs with the seventh), B digits, scratch
 constexpr int kOffB = 8 * kSlice, kOffS = kOffB + kPackBytes;
-constexpr int kScratch = kDiagSmem * 8;               // D(p); 32 KB of it the exchange of the epilogue
+// scratch: D(p)'s blocks, or two 64 x 64 tiles of doubles: entry (row, k) at tile_at(k) + row
+constexpr int kTile = 64 * 65 + 3 * 8;
+__device__ __forceinline__ int tile_at(int k) { return k * 65 + (k >> 4) * 8; }
+constexpr int kScratch = 2 * kTile * 8;
+static_assert(2 * kTile >= kDiagSmem, "scratch");
 constexpr size_t kSmem = (size_t)kOffS + kScratch + 1024;
 
 __device__ __forceinline__ uint32_t s_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -99,34 +103,31 @@ __device__ __forceinline__ uint64_t digits_of(double x, int sh, int e) {
   return (int64_t)b < 0 ? bias - X : bias + X;
 }
 
-struct PackScratch {
-  int mx[64];   // row maxima of the exponents
-  int sh[64];   // exponent shift of each k
-};
-// All threads: thread (row r = tid & 63, k = 16 (tid >> 6) .. + 15) holds x[16]; writes the
-// rows' digits at dst + s kSlice + ... (global or shared) and their exponents e_r to `exps`.
-// sc.sh holds the shifts; sc.mx is used.  Ends without a barrier.
-__device__ void pack_rows(const double (&x)[16], unsigned char* dst, int* exps, PackScratch& sc) {
-  const int r = threadIdx.x & 63, kq = threadIdx.x >> 6;
-  __syncthreads();
-  if (threadIdx.x < 64) sc.mx[threadIdx.x] = -kBad;
-  __syncthreads();
+// All threads: the 64 x 64 matrix with entry (r, k) at Y[r rs + k ks + (k >> 4) sk], its
+// k-th column scaled by 2^(sgn sh[k]), as digits at dst + s kSlice + ... (global or shared) and
+// row exponents at `exps`.  Ends without a barrier.  One copy of the code, in loops: with everything
+// unrolled and inlined the kernel's code was 430 KB and its tasks waited for instructions
+// (a CTA's first task of a kind took twice the time of the later ones).
+__device__ __noinline__ void pack_tile(const double* Y, int rs, int ks, int sk, const int* sh, int sgn,
+                                       unsigned char* dst, int* exps) {
+  const int lane = threadIdx.x & 31, r = 8 * (threadIdx.x >> 5) + (lane & 7), kq = lane >> 3;
+  const double* y = Y + r * rs + 16 * kq * ks + kq * sk;
+  const int* shk = sh + 16 * kq;
   int m = -kBad;
-#pragma unroll
+#pragma unroll 4
   for (int u = 0; u < 16; ++u) {
-    const int l = ilog_of(x[u]);
-    m = max(m, l >= kBad ? kBad : (l <= -kBad ? -kBad : l + sc.sh[16 * kq + u]));
+    const int l = ilog_of(y[u * ks]);
+    m = max(m, l >= kBad ? kBad : (l <= -kBad ? -kBad : l + sgn * shk[u]));
   }
-  atomicMax(&sc.mx[r], m);
-  __syncthreads();
-  m = sc.mx[r];
+  m = max(m, __shfl_xor_sync(~0u, m, 8));
+  m = max(m, __shfl_xor_sync(~0u, m, 16));
   const int e = m >= kBad ? kBad : (m <= -kBad ? 0 : m + 1);
   if (kq == 0) exps[r] = e;
-#pragma unroll
+#pragma unroll 1
   for (int g = 0; g < 2; ++g) {
-    uint64_t y[8];
+    uint64_t z[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) y[u] = digits_of(x[8 * g + u], sc.sh[16 * kq + 8 * g + u], e);
+    for (int u = 0; u < 8; ++u) z[u] = digits_of(y[(8 * g + u) * ks], sgn * shk[8 * g + u], e);
     unsigned char* d = dst + (r >> 3) * 1024 + (2 * kq + g) * 128 + (r & 7) * 16;
 #pragma unroll
     for (int s = 0; s < kDig; ++s) {
@@ -134,8 +135,8 @@ __device__ void pack_rows(const double (&x)[16], unsigned char* dst, int* exps, 
       uint32_t o[4];
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
-        const uint32_t wa = q < 4 ? (uint32_t)y[2 * v] : (uint32_t)(y[2 * v] >> 32);
-        const uint32_t wb = q < 4 ? (uint32_t)y[2 * v + 1] : (uint32_t)(y[2 * v + 1] >> 32);
+        const uint32_t wa = q < 4 ? (uint32_t)z[2 * v] : (uint32_t)(z[2 * v] >> 32);
+        const uint32_t wb = q < 4 ? (uint32_t)z[2 * v + 1] : (uint32_t)(z[2 * v + 1] >> 32);
         // FP16 1024 + byte, then minus 1152: the digit
         // (the first digit is up to 128: nine bits)
         const uint32_t t = __byte_perm(wa, wb, (q & 3) | ((4 + (q & 3)) << 4));
@@ -191,60 +192,59 @@ __device__ __forceinline__ int acc_int(uint32_t b) {
   return __float_as_int(__uint_as_float(b) + 12582912.0f) - 0x4B400000;
 }
 
-// All threads, after the MMAs: thread (row r = 32 (wid & 1) + lane, columns 16 cq .. + 15, cq =
-// 2 (wid >> 2) + ((wid >> 1) & 1)) gets out[u] = the product's entry as a double (eA, eB: row
-// exponents of the operands).  X: 32 KB of shared scratch.
-__device__ __forceinline__ void read_products(uint32_t tmem, const int* eA, const int* eB, long long* X,
-                                              double (&out)[16]) {
+// eight columns of four neighbouring 64-column blocks
+__device__ __forceinline__ void tmem_ld8x4(uint32_t a, uint32_t (&v)[4][8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%32];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%33];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%34];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%35];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=r"(v[0][0]), "=r"(v[0][1]), "=r"(v[0][2]), "=r"(v[0][3]), "=r"(v[0][4]), "=r"(v[0][5]), "=r"(v[0][6]), "=r"(v[0][7]), 
+        "=r"(v[1][0]), "=r"(v[1][1]), "=r"(v[1][2]), "=r"(v[1][3]), "=r"(v[1][4]), "=r"(v[1][5]), "=r"(v[1][6]), "=r"(v[1][7]), 
+        "=r"(v[2][0]), "=r"(v[2][1]), "=r"(v[2][2]), "=r"(v[2][3]), "=r"(v[2][4]), "=r"(v[2][5]), "=r"(v[2][6]), "=r"(v[2][7]), 
+        "=r"(v[3][0]), "=r"(v[3][1]), "=r"(v[3][2]), "=r"(v[3][3]), "=r"(v[3][4]), "=r"(v[3][5]), "=r"(v[3][6]), "=r"(v[3][7])
+      : "r"(a), "r"(a + 64), "r"(a + 128), "r"(a + 192)
+      : "memory");
+}
+
+// All threads, after the MMAs: the product as doubles in the tile X (eA, eB: row exponents of the
+// operands; entry (r, c) at tile_at(c) + r); X2: a second tile.  Ends with a barrier.
+__device__ __forceinline__ void read_products(uint32_t tmem, const int* eA, const int* eB, double* X, double* X2) {
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, q = wid & 3, h = wid >> 2;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const bool top = q < 2;  // lanes 0-63: digit sum t; 64-127: t + 1
-  long long T[32];
   const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(32 * h);
-  // units of 2^-54 X Y: digit sum s has weight 2^(42 - 8 s)
+  const int r = 32 * (q & 1) + lane;
+  long long* P = reinterpret_cast<long long*>(top ? X : X2) + r;
+#pragma unroll 1
+  for (int g = 0; g < 4; ++g) {
+    // units of 2^-54 X Y: digit sum s has weight 2^(42 - 8 s)
+    uint32_t a[4][8], b[4][8];
+    tmem_ld8x4(base + 8 * g, a);        // digit sums 0 .. 3 (top) or 1 .. 4
+    tmem_ld8x4(base + 256 + 8 * g, b);  // 4 .. 7 or 5 .. 7 (the last block's lower half is not read)
 #pragma unroll
-  for (int c = 0; c < 32; ++c) T[c] = 0;
+    for (int c = 0; c < 8; ++c) {
+      long long T = 0;
 #pragma unroll
-  for (int t = 0; t < 5; ++t) {  // digit sums 0 .. 4 (top) or 1 .. 5
-    uint32_t v[32];
-    tmem_ld32(base + 64u * t, v);
-#pragma unroll
-    for (int c = 0; c < 32; ++c) T[c] = T[c] * 256 + acc_int(v[c]);
-  }
-  {
-    uint32_t v5[32], v6[32];
-    tmem_ld32(base + 64u * 5, v5);
-    tmem_ld32(base + 64u * 6, v6);
-    if (top) {
-      uint32_t v7[32];
-      tmem_ld32(base + 64u * 7, v7);
-#pragma unroll
-      for (int c = 0; c < 32; ++c)
-        T[c] = T[c] * 1024 + (long long)acc_int(v5[c]) * 4 +
-               ((__float2int_rn(__uint_as_float(v6[c])) * 256 + acc_int(v7[c]) + 8192) >> 14);
-    } else {
-#pragma unroll
-      for (int c = 0; c < 32; ++c)
-        T[c] = T[c] * 4 + ((acc_int(v5[c]) * 256 + __float2int_rn(__uint_as_float(v6[c])) + 8192) >> 14);
+      for (int t = 0; t < 4; ++t) T = T * 256 + acc_int(a[t][c]);
+      T = T * 256 + acc_int(b[0][c]);
+      const int i5 = acc_int(b[1][c]), i6 = __float2int_rn(__uint_as_float(b[2][c]));
+      const int lo = top ? i6 * 256 + acc_int(b[3][c]) : i5 * 256 + i6;
+      T = (top ? T * 1024 + (long long)i5 * 4 : T * 4) + ((lo + 8192) >> 14);
+      P[tile_at(32 * h + 8 * g + c)] = T;
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  // the top half finishes columns 0 .. 15 of its 32, the bottom half 16 .. 31
-  const int r = 32 * (q & 1) + lane;
-#pragma unroll
+  __syncthreads();
+  const int c0 = 32 * h + (top ? 0 : 16), er = eA[r];
+#pragma unroll 4
   for (int u = 0; u < 16; ++u) {
-    const int c = (top ? 16 : 0) + u;
-    X[(32 * h + c) * 64 + r] = T[c];
+    const int at = tile_at(c0 + u) + r;
+    const long long v = __double_as_longlong(X[at]) + __double_as_longlong(X2[at]);
+    X[at] = scaled_double(v, er + eB[c0 + u] - 56);
   }
   __syncthreads();
-  const int c0 = top ? 0 : 16;
-  const int er = eA[r];
-#pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const long long own = top ? T[u] : T[16 + u];
-    const long long v = own + X[(32 * h + c0 + u) * 64 + r];
-    out[u] = scaled_double(v, er + eB[32 * h + c0 + u] - 56);
-  }
 }
 
 // 27-bit low and 28-bit high parts x0, x1 of the integer rint(x 2^(sh + 55 - e)), |x| 2^sh < 2^e
@@ -328,34 +328,44 @@ __device__ __forceinline__ void diag64_panel(int q, int pw, double* A, Diag64Sme
                                              DiagScratch<double>& sh, int* hs, long long key_eps, double delta,
                                              int& nhit) {
   constexpr int LD = kDiagLD, NC = 16 / NP;
+  static_assert(NP % 2 == 0, "");
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, c0 = 16 * q;
   const int row = NP == 2 ? 32 * (wid & 1) + lane : 32 + lane, par = NP == 2 ? wid >> 1 : wid;
-  double v[NC], l[NC], c8[NC], dk = 0.0;
+  double v[NC], dk = 0.0;
+  int2* ib = sb.ib + (q & 1) * 64 * kLP;
+  double* cd = reinterpret_cast<double*>(ib);  // this thread's entries of L d, then their integers in place
 #pragma unroll
   for (int t = 0; t < NC; ++t) v[t] = A[row * LD + c0 + NP * t + par];
+#pragma unroll 1
+  for (int kp = 0; kp < NC; ++kp) {
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const int kk = c0 + k;
-    double* cc = sa.cb + 64 * (k & 1);
-    if (par == (k % NP)) cc[row] = v[k / NP];
-    asm volatile("barrier.sync 2, 128;" ::: "memory");
-    double d = cc[kk];
-    const double cr = cc[row];
-    const bool ng = sh.sgn[kk] < 0;
-    const double sd = __longlong_as_double(__double_as_longlong(d) ^ (ng ? (long long)0x8000000000000000ull : 0ll));
-    const bool hit = kk < pw && order_key(sd) <= key_eps;
-    if (hit) d = ng ? -delta : delta;
-    const double lr = cr * rcp_pivot(d);
-    const double ml = __longlong_as_double(__double_as_longlong(lr) ^ (long long)0x8000000000000000ull);
-    if (par == (k % NP)) {
-      l[k / NP] = lr;
-      c8[k / NP] = cr;
+    for (int o = 0; o < NP; ++o) {
+      const int k = NP * kp + o, kk = c0 + k;
+      double* cc = sa.cb + 64 * (o & 1);
+      if (par == o) cc[row] = v[0];
+      asm volatile("barrier.sync 2, 128;" ::: "memory");
+      double d = cc[kk];
+      const double cr = cc[row];
+      const bool ng = sh.sgn[kk] < 0;
+      const double sd = __longlong_as_double(__double_as_longlong(d) ^ (ng ? (long long)0x8000000000000000ull : 0ll));
+      const bool hit = kk < pw && order_key(sd) <= key_eps;
+      if (hit) d = ng ? -delta : delta;
+      const double lr = cr * rcp_pivot(d);
+      const double ml = __longlong_as_double(__double_as_longlong(lr) ^ (long long)0x8000000000000000ull);
+      const double* cp = cc + c0 + NP * kp + par;
+      if (par > o) v[0] = fma(ml, cp[0], v[0]);
+#pragma unroll
+      for (int t = 1; t < NC; ++t)
+        if (kp + t < NC) v[t] = fma(ml, cp[NP * t], v[t]);
+      if (par == o) {
+        if (row >= kk) A[row * LD + kk] = row == kk ? d : lr;
+        cd[row * kLP + k] = cr;
+      }
+      if (lane == k) dk = d;
+      nhit += hit ? 1 : 0;
     }
 #pragma unroll
-    for (int t = 0; t < NC; ++t)
-      if (NP * t + NP - 1 > k && NP * t + par > k) v[t] = fma(ml, cc[c0 + NP * t + par], v[t]);
-    if (lane == k) dk = d;
-    nhit += hit ? 1 : 0;
+    for (int t = 0; t + 1 < NC; ++t) v[t] = v[t + 1];
   }
   if (wid == 0 && lane < 16) {
     sh.dv[c0 + lane] = dk;
@@ -369,10 +379,10 @@ __device__ __forceinline__ void diag64_panel(int q, int pw, double* A, Diag64Sme
 #pragma unroll
   for (int t = 0; t < NC; ++t) {
     const int cl = c0 + NP * t + par;
-    if (row >= cl) A[row * LD + cl] = row == cl ? sh.dv[cl] : l[t];
-    if (row <= cl) l[t] = c8[t] = 0.0;
-    ma = max(ma, shifted(l[t], hs[cl]));
-    mb = max(mb, shifted(c8[t], -hs[cl]));
+    if (row > cl) {
+      ma = max(ma, shifted(A[row * LD + cl], hs[cl]));
+      mb = max(mb, shifted(cd[row * kLP + cl - c0], -hs[cl]));
+    }
   }
   if (par == 0) {
     xm[row] = ma;
@@ -389,22 +399,23 @@ __device__ __forceinline__ void diag64_panel(int q, int pw, double* A, Diag64Sme
     sa.ea[64 * q + row] = xa;
     sb.eb[64 * (q & 1) + row] = xb;
   }
-  int2* ib = sb.ib + (q & 1) * 64 * kLP;
-#pragma unroll
+#pragma unroll 1
   for (int t = 0; t < NC; ++t) {
     const int c = NP * t + par;
-    sa.ia[row * kLI + c0 + c] = halves_of(l[t], hs[c0 + c], xa);
-    ib[row * kLP + c] = halves_of(c8[t], -hs[c0 + c], xb);
+    const bool in = row > c0 + c;
+    const double lv = in ? A[row * LD + c0 + c] : 0.0, cv = in ? cd[row * kLP + c] : 0.0;
+    sa.ia[row * kLI + c0 + c] = halves_of(lv, hs[c0 + c], xa);
+    ib[row * kLP + c] = halves_of(cv, -hs[c0 + c], xb);
   }
 }
 
 // 16 x 16 block (I, J) of the trailing matrix: a_rs -= sum_m l_rm (l_sm d_m) over panel q; 256 entries
-__device__ __forceinline__ void diag64_update(int q, int I, int J, int idx, double* A, const Diag64Smem& sa,
+__device__ __noinline__ void diag64_update(int q, int I, int J, int idx, double* A, const Diag64Smem& sa,
                                               const Diag64SmemB& sb) {
   const int r = 16 * I + (idx >> 4), s = 16 * J + (idx & 15);
   const int2* ib = sb.ib + (q & 1) * 64 * kLP;
   IntDot acc;
-#pragma unroll
+#pragma unroll 4
   for (int m = 0; m < 16; ++m) acc.add(sa.ia[r * kLI + 16 * q + m], ib[s * kLP + m]);
   if (r >= s)
     A[r * kDiagLD + s] -= scaled_double(acc.value(), sa.ea[64 * q + r] + sb.eb[64 * (q & 1) + s] - 56);
@@ -412,7 +423,7 @@ __device__ __forceinline__ void diag64_update(int q, int I, int J, int idx, doub
 
 // Block row Q of L^{-1}, by the 128 threads of warps 4-7 (tid 0 .. 127 here, barrier 3): the inverse of
 // L_QQ, Linv_QP = -Linv_QQ X_P, its operands (Q < 3), and X of block row Q + 1.
-__device__ __forceinline__ void diag64_inverse_row(int Q, int tid, const double* A, double* V, Diag64Smem& sa,
+__device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A, double* V, Diag64Smem& sa,
                                                    Diag64SmemB& sb, const int* gs, const int* hs) {
   constexpr int LD = kDiagLD;
   const int R0 = 16 * Q;
@@ -480,7 +491,7 @@ __device__ __forceinline__ void diag64_inverse_row(int Q, int tid, const double*
     for (int idx = tid; idx < 16 * R0; idx += 128) {
       const int a = idx & 15, b = idx >> 4;
       IntDot acc;
-#pragma unroll
+#pragma unroll 4
       for (int m = 0; m < 16; ++m) acc.add(sa.iq[a * kLP + m], sa.ix[b * kLP + m]);
       V[(R0 + a) * LD + b] = -scaled_double(acc.value(), sa.eq[a] + sa.ex[b] - 56);
     }
@@ -505,7 +516,7 @@ __device__ __forceinline__ void diag64_inverse_row(int Q, int tid, const double*
     double s = 0.0;
     for (int M = b >> 4; M <= Q; ++M) {
       IntDot acc;
-#pragma unroll
+#pragma unroll 4
       for (int m = 0; m < 16; ++m) acc.add(sa.ia[(R0 + 16 + a) * kLI + 16 * M + m], sb.ic[b * kLI + 16 * M + m]);
       s += scaled_double(acc.value(), sa.ea[64 * M + R0 + 16 + a] + sb.ec[48 * M + b] - 56);
     }
@@ -523,7 +534,7 @@ __device__ __forceinline__ void diag64_inverse_row(int Q, int tid, const double*
 // the sign and the products with 16 terms (the trailing updates, and the off-diagonal blocks of
 // L^{-1}) are integer arithmetic, the products exact (operands scaled like the packs).  Warps 4-7
 // form L^{-1} a block row behind the panels, and the part of the trailing update that
-// the next panel does not read.  66 us with the packs.
+// the next panel does not read.  70 us with the packs.
 __device__ int diag64(double* G, int64_t f, int pw, double* D, double* Li, const int8_t* dsign, double eps, double delta,
                       double* scr, Diag64Smem& sa, Diag64SmemB& sb, DiagScratch<double>& sh, const int* gs, int* hs) {
   constexpr int LD = kDiagLD;
@@ -594,10 +605,9 @@ __global__ void __launch_bounds__(NT, 1)
   unsigned char* sm = smraw + ((1024u - (s_addr(smraw) & 1023u)) & 1023u);
   unsigned char* smB = sm + kOffB;
   double* scr = reinterpret_cast<double*>(sm + kOffS);
-  long long* X = reinterpret_cast<long long*>(sm + kOffS);
+  double* scr2 = scr + kTile;
   __shared__ DiagScratch<double> dsh;
-  __shared__ PackScratch ps;
-  __shared__ int eA[64], eB[64], hs[64], gs[64];
+  __shared__ int eA[64], eB[64], hs[64], gs[64];  // row exponents of the operands; h; g
   __shared__ double dinv[64], dinv2[64];  // 1 / d_j and what its rounding left
   __shared__ FlowTask s_task;
   __shared__ int s_go, s_flag;
@@ -719,36 +729,22 @@ __global__ void __launch_bounds__(NT, 1)
       if (tid == 0 && nhit) atomicAdd(hits, nhit);
       __syncthreads();
       if (tid < 64) {
-        ps.sh[tid] = gs[tid];
         int* ex = exps_of(pkr.pt(p));
         ex[64 + tid] = gs[tid];
         ex[128 + tid] = hs[tid];
       }
       const double* V = scr + 64 * kDiagLD;
-      const int r = tid & 63, kq = tid >> 6;
-      double x[16];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const int l = 16 * kq + u;
-        x[u] = (r < pw && l < r) ? V[r * kDiagLD + l] : ((l == r && r < pw) ? 1.0 : 0.0);
-      }
-      pack_rows(x, pkr.pt(p), exps_of(pkr.pt(p)), ps);
+      pack_tile(V, kDiagLD, 1, 0, gs, 1, pkr.pt(p), exps_of(pkr.pt(p)));
       fence_async_global();
       __syncthreads();
       if (tid == 0) {
         __threadfence();
         st_release(w.diag + p, 1);
       }
-      fence_async_shared();  // the operands' space is the next task's, by bulk copies
       // PE(p, p): rows the columns of Linv (after the release: only EU(p, i, p) waits for it)
-      if (tid < 64) ps.sh[tid] = -hs[tid];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const int k = 16 * kq + u;
-        x[u] = (k < pw && r < k) ? V[k * kDiagLD + r] : ((k == r && r < pw) ? 1.0 : 0.0);
-      }
-      pack_rows(x, pkr.pe(p, p), exps_of(pkr.pe(p, p)), ps);
+      pack_tile(V, 1, kDiagLD, 0, hs, -1, pkr.pe(p, p), exps_of(pkr.pe(p, p)));
       fence_async_global();
+      fence_async_shared();  // the operands' space is the next task's, by bulk copies
       __syncthreads();
       if (tid == 0) {
         __threadfence();
@@ -756,113 +752,58 @@ __global__ void __launch_bounds__(NT, 1)
       }
       continue;
     }
-    if (tk.kind == 1 || tk.kind == 2) {
-      // T(p, i): rows of F_IK; Efin(p, e): rows the columns of E_KC; both times PT(p)^T
-      const bool efin = tk.kind == 2;
-      const int64_t r0 = efin ? (int64_t)tk.j * NB : brow0(g, tk.i);
-      const int nr = efin ? NB : bnrow(g, tk.i);
-      unsigned char* pt = pkr.pt(p);
-      if (tid == 0) {
-        fence_async_global();
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_ld), "r"(kPackBytes) : "memory");
-        bulk_copy(s_addr(smB), pt, kPackBytes, bar_ld);
+    // T(p, i): rows of F_IK; Efin(p, e): rows the columns of E_KC; both times PT(p)^T.  U(p, i, j),
+    // EU(p, i, e): PA(p, i) times PB(p, j)^T or PE(p, e)^T
+    const bool upd = tk.kind >= 3, efin = tk.kind == 2, etile = tk.kind == 4;
+    const int64_t i0 = efin ? (int64_t)tk.j * NB : brow0(g, tk.i), c0 = etile ? (int64_t)tk.j * NB : brow0(g, tk.j);
+    const int ni = efin ? NB : bnrow(g, tk.i), nc = bnrow(g, tk.j);
+    const bool diag = tk.kind == 3 && tk.i == tk.j;
+    double* base = etile ? Eb : G;
+    unsigned char* tb = !upd ? pkr.pt(p) : (etile ? pkr.pe(p, tk.j) : pkr.pb(p, tk.j));
+    if (tid == 0) {
+      fence_async_global();  // the packs were stored by generic writes (acquired above)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_ld),
+                   "r"((upd ? 2 : 1) * kPackBytes)
+                   : "memory");
+      if (upd) bulk_copy(s_addr(sm), pkr.pa(p, tk.i), kPackBytes, bar_ld);
+      bulk_copy(s_addr(smB), tb, kPackBytes, bar_ld);
+    }
+    if (tid < 64) eB[tid] = __ldcg(exps_of(tb) + tid);
+    double tv[16];
+    if (upd) {
+      if (tid >= 64 && tid < 128) eA[tid - 64] = __ldcg(exps_of(pkr.pa(p, tk.i)) + tid - 64);
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const int cc = ocol + u;
+        tv[u] = (orow < ni && cc < nc && (!diag || orow >= cc)) ? __ldcg(base + (i0 + orow) + (c0 + cc) * f) : 0.0;
       }
-      const int r = tid & 63, kq = tid >> 6;
+    } else {
+      if (tid < 64) {
+        const int* ex = exps_of(tb);
+        gs[tid] = __ldcg(ex + 64 + tid);
+        hs[tid] = __ldcg(ex + 128 + tid);
+      } else if (tid < 128 && !efin) {
+        const int k = tid - 64;
+        const double d = k < pw ? __ldcg(Dp + kp + k) : 1.0, r = 1.0 / d;
+        dinv[k] = k < pw ? r : 0.0;
+        dinv2[k] = k < pw ? fma(-d, r, 1.0) * r : 0.0;
+      }
+      // the tile: lane along the rows of F, or along k (the rows of E)
+      const int a = tid & 63, b0 = tid >> 6;
       double x[16];
 #pragma unroll
       for (int u = 0; u < 16; ++u) {
-        const int l = 16 * kq + u;
-        const double* a = efin ? Eb + (k0 + l) + (r0 + r) * f : G + (r0 + r) + (k0 + l) * f;
-        x[u] = (r < nr && l < pw) ? __ldcg(a) : 0.0;
+        const int c = b0 + 4 * u, r = efin ? c : a, k = efin ? a : c;
+        x[u] = (r < ni && k < pw) ? __ldcg(efin ? Eb + (k0 + k) + (i0 + r) * f : G + (i0 + r) + (k0 + k) * f) : 0.0;
       }
-      if (tid < 64) {
-        const int* ex = exps_of(pt);
-        eB[tid] = __ldcg(ex + tid);
-        ps.sh[tid] = -__ldcg(ex + 64 + tid);
-        hs[tid] = __ldcg(ex + 128 + tid);
-        if (!efin) {
-          const double d = tid < pw ? __ldcg(Dp + kp + tid) : 1.0, r = 1.0 / d;
-          dinv[tid] = tid < pw ? r : 0.0;
-          dinv2[tid] = tid < pw ? fma(-d, r, 1.0) * r : 0.0;
-        }
-      }
-      pack_rows(x, sm, eA, ps);
-      fence_async_shared();
-      stop = !wait_bar(bar_ld, par_ld);
-      if (!stop) {
-        if (tid == 0) issue_products(s_addr(sm), s_addr(smB), tmem, bar_mma);
-        stop = !wait_bar(bar_mma, par_mma);
-      }
-      if (stop) break;
-      double o[16];
-      read_products(tmem, eA, eB, X, o);
-      // (thread: row orow, columns ocol .. ocol + 15: what the packs hold per thread, too)
-      if (efin) {
-#pragma unroll
-        for (int u = 0; u < 16; ++u)
-          if (ocol + u < pw) Eb[(k0 + ocol + u) + (r0 + orow) * f] = o[u];
-          else o[u] = 0.0;
-      }
-      double q[16];
 #pragma unroll
       for (int u = 0; u < 16; ++u) {
-        if (efin) continue;
-        if (ocol + u >= pw || orow >= nr) o[u] = 0.0;
-        q[u] = fma(o[u], dinv[ocol + u], o[u] * dinv2[ocol + u]);  // o / d to half an ulp
-        if (ocol + u < pw && orow < nr) G[(r0 + orow) + (k0 + ocol + u) * f] = q[u];
+        const int c = b0 + 4 * u;
+        scr[efin ? tile_at(a) + c : tile_at(c) + a] = x[u];
       }
-      // through shared memory to the packing order (row tid & 63, k 16 (tid >> 6) ..)
       __syncthreads();
-      double* Y = scr;
-#pragma unroll
-      for (int u = 0; u < 16; ++u) Y[(ocol + u) * 64 + orow] = o[u];
-      if (tid < 64) ps.sh[tid] = -hs[tid];
-      __syncthreads();
-#pragma unroll
-      for (int u = 0; u < 16; ++u) x[u] = Y[(16 * kq + u) * 64 + r];
-      unsigned char* dst = efin ? pkr.pe(p, tk.j) : pkr.pb(p, tk.i);
-      pack_rows(x, dst, exps_of(dst), ps);
-      if (!efin) {
-        __syncthreads();
-        if (tid < 64) ps.sh[tid] = hs[tid];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) Y[(ocol + u) * 64 + orow] = q[u];
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < 16; ++u) x[u] = Y[(16 * kq + u) * 64 + r];
-        pack_rows(x, pkr.pa(p, tk.i), exps_of(pkr.pa(p, tk.i)), ps);
-      }
-      fence_async_global();
-      __syncthreads();
-      if (tid == 0) {
-        __threadfence();
-        if (efin) st_release(w.e(p, tk.j), p - (int)tk.j + 1);
-        else st_release(w.trsm + tk.i, p + 1);
-      }
-      continue;
-    }
-    // U(p, i, j), EU(p, i, e)
-    const bool etile = tk.kind != 3;
-    const int64_t i0 = brow0(g, tk.i), c0 = etile ? (int64_t)tk.j * NB : brow0(g, tk.j);
-    const int ni = bnrow(g, tk.i), nc = bnrow(g, tk.j);
-    const bool diag = !etile && tk.i == tk.j;
-    double* base = etile ? Eb : G;
-    unsigned char* ta = pkr.pa(p, tk.i);
-    unsigned char* tb = etile ? pkr.pe(p, tk.j) : pkr.pb(p, tk.j);
-    if (tid == 0) {
-      fence_async_global();  // the packs were stored by generic writes (acquired above)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_ld), "r"(2 * kPackBytes)
-                   : "memory");
-      bulk_copy(s_addr(sm), ta, kPackBytes, bar_ld);
-      bulk_copy(s_addr(smB), tb, kPackBytes, bar_ld);
-    }
-    if (tid < 64) eA[tid] = __ldcg(exps_of(ta) + tid);
-    else if (tid < 128) eB[tid - 64] = __ldcg(exps_of(tb) + tid - 64);
-    double tv[16];
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int cc = ocol + u;
-      tv[u] = (orow < ni && cc < nc && (!diag || orow >= cc)) ? __ldcg(base + (i0 + orow) + (c0 + cc) * f) : 0.0;
+      pack_tile(scr, 1, 65, 8, gs, -1, sm, eA);
+      fence_async_shared();
     }
     stop = !wait_bar(bar_ld, par_ld);
     if (!stop) {
@@ -870,17 +811,43 @@ __global__ void __launch_bounds__(NT, 1)
       stop = !wait_bar(bar_mma, par_mma);
     }
     if (stop) break;
-    double o[16];
-    read_products(tmem, eA, eB, X, o);
+    read_products(tmem, eA, eB, scr, scr2);
+    if (upd) {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int cc = ocol + u;
-      if (orow < ni && cc < nc && (!diag || orow >= cc)) base[(i0 + orow) + (c0 + cc) * f] = tv[u] - o[u];
+      for (int u = 0; u < 16; ++u) {
+        const int cc = ocol + u;
+        if (orow < ni && cc < nc && (!diag || orow >= cc))
+          base[(i0 + orow) + (c0 + cc) * f] = tv[u] - scr[tile_at(cc) + orow];
+      }
+    } else if (efin) {
+      const int a = tid & 63;
+      if (a < pw)
+#pragma unroll 4
+        for (int c = tid >> 6; c < NB; c += 4) Eb[(k0 + a) + (i0 + c) * f] = scr[tile_at(a) + c];
+    } else {
+      const int a = tid & 63;
+#pragma unroll 4
+      for (int c = tid >> 6; c < NB; c += 4) {
+        const bool in = c < pw && a < ni;
+        const double o = in ? scr[tile_at(c) + a] : 0.0, q = fma(o, dinv[c], o * dinv2[c]);  // o / d to half an ulp
+        if (in) G[(i0 + a) + (k0 + c) * f] = q;
+        if (!in) scr[tile_at(c) + a] = 0.0;
+        scr2[tile_at(c) + a] = q;
+      }
+      __syncthreads();
+      pack_tile(scr2, 1, 65, 8, hs, 1, pkr.pa(p, tk.i), exps_of(pkr.pa(p, tk.i)));
+    }
+    if (!upd) {
+      unsigned char* dst = efin ? pkr.pe(p, tk.j) : pkr.pb(p, tk.i);
+      pack_tile(scr, 1, 65, 8, hs, -1, dst, exps_of(dst));
+      fence_async_global();
     }
     __syncthreads();
     if (tid == 0) {
       __threadfence();
-      if (etile) st_release(w.e(tk.i, tk.j), p - (int)tk.j + 1);
+      if (tk.kind == 1) st_release(w.trsm + tk.i, p + 1);
+      else if (tk.kind == 2) st_release(w.e(p, tk.j), p - (int)tk.j + 1);
+      else if (etile) st_release(w.e(tk.i, tk.j), p - (int)tk.j + 1);
       else st_release(w.t(tk.i, tk.j), p + 1);
     }
   }

@@ -672,7 +672,7 @@ static int flow64_tables(DeviceArena& ar, LdlStructure& st, bool emu) {
     st.flow_one64[l] = span1 < 0.97 * span2 ? 1 : 0;
     if (st.flow_one64[l]) std::copy(one.begin(), one.end(), t64.begin() + st.flow_t0_64[l]);
     // with the products on the tensor cores, one CTA per SM (bigflow64.cu)
-    static const double dur64e[8] = {66.0, 27.0, 23.0, 13.0, 13.0, 0.0, 0.0, 0.0};
+    static const double dur64e[8] = {70.0, 24.0, 18.0, 11.0, 11.0, 0.0, 0.0, 0.0};
     if (!flow_schedule_order(t64e, st.flow_t0_64e[l], P_of, flow_sms, dur64e, &span1, 2)) return CLR_E_INVALID;
   }
   st.flow_task64 = t64.empty() ? nullptr : ar.upload(t64.data(), (int64_t)t64.size());

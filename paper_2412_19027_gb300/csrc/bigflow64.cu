@@ -305,8 +305,8 @@ struct Diag64Smem {
   int2 ia[64 * kLI];       // L 2^h by rows, exponents ea[panel][row]
   int2 iq[16 * kLP];       // Linv_QQ 2^g by rows, exponents eq
   int2 ix[48 * kLP];       // X 2^-g by columns, exponents ex
-  double cb[2 * 64];       // two pivot columns
-  int ea[4 * 64], eq[16], ex[48];
+  double cb[8 * 64];       // pivot columns: four of this group of columns, four of the last
+  int ea[4 * 64], eq[16], ex[48], xm[2 * 64];
 };
 struct Diag64SmemB {
   int2 ib[2 * 64 * kLP];   // (L d) 2^-h of a panel by rows, exponents eb[row], for two panels
@@ -323,83 +323,86 @@ __device__ __forceinline__ int shifted(double x, int sh) {
 
 // Pivots 16 q .. 16 q + 15 by four warps (barrier 2): NP = 2: rows 32 (wid & 1) + lane, columns of
 // parity wid >> 1; NP = 4 (q >= 2: rows 0-31 are done): rows 32 + lane, columns wid modulo 4.
+// Groups of four columns: a pivot updates its group at once, the columns after it by the group's
+// four pivots together (an FMA behind its own load and branch took 150 clocks, in a batch 85).
 template <int NP>
 __device__ __forceinline__ void diag64_panel(int q, int pw, double* A, Diag64Smem& sa, Diag64SmemB& sb,
                                              DiagScratch<double>& sh, int* hs, long long key_eps, double delta,
-                                             int& nhit) {
-  constexpr int LD = kDiagLD, NC = 16 / NP;
-  static_assert(NP % 2 == 0, "");
+                                             double rdelta, int& nhit) {
+  constexpr int LD = kDiagLD, NC = 16 / NP, GC = 4 / NP;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, c0 = 16 * q;
   const int row = NP == 2 ? 32 * (wid & 1) + lane : 32 + lane, par = NP == 2 ? wid >> 1 : wid;
+  constexpr long long kSign = (long long)0x8000000000000000ull;
   double v[NC], dk = 0.0;
+  int ma = -kBad, mb = -kBad;
   int2* ib = sb.ib + (q & 1) * 64 * kLP;
   double* cd = reinterpret_cast<double*>(ib);  // this thread's entries of L d, then their integers in place
 #pragma unroll
   for (int t = 0; t < NC; ++t) v[t] = A[row * LD + c0 + NP * t + par];
+  if (par == 0) sa.xm[row] = sa.xm[64 + row] = -kBad;
 #pragma unroll 1
-  for (int kp = 0; kp < NC; ++kp) {
+  for (int g = 0; g < 4; ++g) {
+    double* cg = sa.cb + 256 * (g & 1);
+    double ml[4];
 #pragma unroll
-    for (int o = 0; o < NP; ++o) {
-      const int k = NP * kp + o, kk = c0 + k;
-      double* cc = sa.cb + 64 * (o & 1);
-      if (par == o) cc[row] = v[0];
+    for (int o = 0; o < 4; ++o) {
+      const int k = 4 * g + o, kk = c0 + k;
+      double* cc = cg + 64 * o;
+      if (par == o % NP) cc[row] = v[o / NP];
+      const bool ng = sh.sgn[kk] < 0;
       asm volatile("barrier.sync 2, 128;" ::: "memory");
       double d = cc[kk];
       const double cr = cc[row];
-      const bool ng = sh.sgn[kk] < 0;
-      const double sd = __longlong_as_double(__double_as_longlong(d) ^ (ng ? (long long)0x8000000000000000ull : 0ll));
-      const bool hit = kk < pw && order_key(sd) <= key_eps;
-      if (hit) d = ng ? -delta : delta;
-      const double lr = cr * rcp_pivot(d);
-      const double ml = __longlong_as_double(__double_as_longlong(lr) ^ (long long)0x8000000000000000ull);
-      const double* cp = cc + c0 + NP * kp + par;
-      if (par > o) v[0] = fma(ml, cp[0], v[0]);
+      // (the reciprocal does not wait for the test)
+      double rd = rcp_pivot(d);
+      const bool hit = kk < pw && order_key(__longlong_as_double(__double_as_longlong(d) ^ (ng ? kSign : 0ll))) <= key_eps;
+      if (hit) d = ng ? -delta : delta, rd = ng ? -rdelta : rdelta;
+      const double lr = cr * rd;
+      ml[o] = __longlong_as_double(__double_as_longlong(lr) ^ kSign);
 #pragma unroll
-      for (int t = 1; t < NC; ++t)
-        if (kp + t < NC) v[t] = fma(ml, cp[NP * t], v[t]);
-      if (par == o) {
+      for (int t = 0; t < GC; ++t)
+        if (NP * t + NP - 1 > o && NP * t + par > o) v[t] = fma(ml[o], cc[c0 + 4 * g + NP * t + par], v[t]);
+      if (par == o % NP) {
         if (row >= kk) A[row * LD + kk] = row == kk ? d : lr;
         cd[row * kLP + k] = cr;
+        if (row > kk) {
+          const int ld = ilog_of(d), h = ld <= -kBad || ld >= kBad ? 0 : ld >> 1;
+          ma = max(ma, shifted(lr, h));
+          mb = max(mb, shifted(cr, -h));
+        }
       }
       if (lane == k) dk = d;
       nhit += hit ? 1 : 0;
     }
 #pragma unroll
-    for (int t = 0; t + 1 < NC; ++t) v[t] = v[t + 1];
+    for (int u = 1; u < 4; ++u) {
+      if (g + u < 4) {
+        const double* cp = cg + c0 + 4 * (g + u) + par;
+        double w[4 * GC];
+#pragma unroll
+        for (int e = 0; e < 4 * GC; ++e) w[e] = cp[64 * (e / GC) + NP * (e % GC)];
+#pragma unroll
+        for (int e = 0; e < 4 * GC; ++e) v[GC * u + e % GC] = fma(ml[e / GC], w[e], v[GC * u + e % GC]);
+      }
+    }
+#pragma unroll
+    for (int t = 0; t + GC < NC; ++t) v[t] = v[t + GC];
   }
   if (wid == 0 && lane < 16) {
     sh.dv[c0 + lane] = dk;
     const int lg = ilog_of(dk);
     hs[c0 + lane] = lg <= -kBad || lg >= kBad ? 0 : lg >> 1;
   }
+  // the integer operands L 2^h, (L d) 2^-h of the rows below
+  atomicMax(&sa.xm[row], ma);
+  atomicMax(&sa.xm[64 + row], mb);
   asm volatile("barrier.sync 2, 128;" ::: "memory");
-  // the columns of L, the pivots, and the integer operands L 2^h, (L d) 2^-h of the rows below
-  int* xm = reinterpret_cast<int*>(sa.cb);  // (the columns are done)
-  int ma = -kBad, mb = -kBad;
-#pragma unroll
-  for (int t = 0; t < NC; ++t) {
-    const int cl = c0 + NP * t + par;
-    if (row > cl) {
-      ma = max(ma, shifted(A[row * LD + cl], hs[cl]));
-      mb = max(mb, shifted(cd[row * kLP + cl - c0], -hs[cl]));
-    }
-  }
-  if (par == 0) {
-    xm[row] = ma;
-    xm[64 + row] = mb;
-  }
-  asm volatile("barrier.sync 2, 128;" ::: "memory");
-  if (par != 0) {
-    atomicMax(&xm[row], ma);
-    atomicMax(&xm[64 + row], mb);
-  }
-  asm volatile("barrier.sync 2, 128;" ::: "memory");
-  const int xa = row_exp(xm[row]), xb = row_exp(xm[64 + row]);
+  const int xa = row_exp(sa.xm[row]), xb = row_exp(sa.xm[64 + row]);
   if (par == 0) {
     sa.ea[64 * q + row] = xa;
     sb.eb[64 * (q & 1) + row] = xb;
   }
-#pragma unroll 1
+#pragma unroll 2
   for (int t = 0; t < NC; ++t) {
     const int c = NP * t + par;
     const bool in = row > c0 + c;
@@ -428,22 +431,17 @@ __device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A,
   constexpr int LD = kDiagLD;
   const int R0 = 16 * Q;
   auto bar = [] { asm volatile("barrier.sync 3, 128;" ::: "memory"); };
-  if (tid < 32) {
-    // both 8 x 8 diagonal blocks (lane: column), then the 8 x 8 block below them, B1 = -C^{-1} B A^{-1}
-    if (tid < 16) {
-      const int o = R0 + (tid & 8), c = tid & 7;
-      double x[8];
+  {
+    // both 8 x 8 diagonal blocks by column sweeps, lane: row 4 r + c of four columns; then the 8 x 8
+    // block below them, -C^{-1} B A^{-1}
+    const int w = tid >> 5, lane = tid & 31, o = R0 + 8 * (w >> 1), r = lane >> 2, c = 4 * (w & 1) + (lane & 3);
+    double x = r == c ? 1.0 : 0.0;
 #pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        double s = (r == c) ? 1.0 : 0.0;
-#pragma unroll
-        for (int m = 0; m < r; ++m) s = fma(-A[(o + r) * LD + o + m], x[m], s);
-        x[r] = (r >= c) ? s : 0.0;
-      }
-#pragma unroll
-      for (int r = 0; r < 8; ++r) V[(o + r) * LD + o + c] = x[r];
+    for (int m = 0; m < 7; ++m) {
+      const double xm = __shfl_sync(~0u, x, 4 * m + (lane & 3));
+      if (r > m) x = fma(-A[(o + r) * LD + o + m], xm, x);
     }
-    __syncwarp();
+    V[(o + r) * LD + o + c] = x;
   }
   bar();
   if (tid < 64) {  // B A^{-1}
@@ -525,8 +523,8 @@ __device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A,
 }
 
 // Diagonal block: LDL^T with dynamic regularisation of the pw x pw block at G and the inverse of
-// its unit lower factor, the outputs of bf_diag_block.  Shared memory: A and V (64 x 65: L with the
-// pivots, L^{-1}) and the integer operands.
+// its unit lower factor, left in shared memory: A and V (64 x 65: L with the pivots, L^{-1}); D and
+// the scalings gs, hs are written.
 //
 // bf_diag_block took 113 us here: it is FP64 warp instructions on one SM (64 clocks each, 76 with all
 // four sub-partitions busy), many with few active lanes.  Panels of 16 columns on four warps: per
@@ -535,8 +533,8 @@ __device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A,
 // L^{-1}) are integer arithmetic, the products exact (operands scaled like the packs).  Warps 4-7
 // form L^{-1} a block row behind the panels, and the part of the trailing update that
 // the next panel does not read.  70 us with the packs.
-__device__ int diag64(double* G, int64_t f, int pw, double* D, double* Li, const int8_t* dsign, double eps, double delta,
-                      double* scr, Diag64Smem& sa, Diag64SmemB& sb, DiagScratch<double>& sh, const int* gs, int* hs) {
+__device__ int diag64(const double* G, int64_t f, int pw, double* D, const int8_t* dsign, double eps, double delta,
+                      double* scr, Diag64Smem& sa, Diag64SmemB& sb, DiagScratch<double>& sh, int* gs, int* hs) {
   constexpr int LD = kDiagLD;
   double* A = scr;
   double* V = scr + 64 * LD;
@@ -550,13 +548,18 @@ __device__ int diag64(double* G, int64_t f, int pw, double* D, double* Li, const
     else if (i == j) v = 1.0;  // rows and pivots past pw: the identity
     A[i * LD + j] = v;
     V[i * LD + j] = 0.0;
+    if (i == j) {  // g: half the exponent of the diagonal
+      const int lg = i < pw ? ilog_of(v) : 0;
+      gs[i] = lg <= -kBad || lg >= kBad ? 0 : lg >> 1;
+    }
   }
+  const double rdelta = 1.0 / delta;
   __syncthreads();
   int nhit = 0;
   for (int q = 0; q < 4; ++q) {
     if (wid < 4) {
-      if (q < 2) diag64_panel<2>(q, pw, A, sa, sb, sh, hs, key_eps, delta, nhit);
-      else diag64_panel<4>(q, pw, A, sa, sb, sh, hs, key_eps, delta, nhit);
+      if (q < 2) diag64_panel<2>(q, pw, A, sa, sb, sh, hs, key_eps, delta, rdelta, nhit);
+      else diag64_panel<4>(q, pw, A, sa, sb, sh, hs, key_eps, delta, rdelta, nhit);
     } else if (q > 0) {
       for (int I = q + 1; I < 4; ++I)  // the rest of panel q - 1's update
         for (int J = q + 1; J <= I; ++J) {
@@ -571,13 +574,6 @@ __device__ int diag64(double* G, int64_t f, int pw, double* D, double* Li, const
   }
   if (wid >= 4) diag64_inverse_row(3, tid - 128, A, V, sa, sb, gs, hs);
   __syncthreads();
-  for (int idx = tid; idx < 64 * 64; idx += NT) {
-    const int i = idx & 63, j = idx >> 6;
-    if (i < pw && j < pw && i >= j) {
-      G[i + (int64_t)j * f] = A[i * LD + j];
-      Li[i + (int64_t)j * f] = (i == j) ? 1.0 : V[i * LD + j];
-    }
-  }
   for (int i = tid; i < pw; i += NT) D[i] = sh.dv[i];
   return nhit;
 }
@@ -722,9 +718,7 @@ __global__ void __launch_bounds__(NT, 1)
     };
     if (tk.kind == 0) {
       // D(p): the diagonal block on the FP64 pipe, then its packs
-      if (tid < 64) gs[tid] = tid < pw ? ilog_of(__ldcg(G + (k0 + tid) + (k0 + tid) * f)) >> 1 : 0;
-      if (tid < 64 && (gs[tid] <= -kBad / 2 || gs[tid] >= kBad / 2)) gs[tid] = 0;
-      const int nhit = diag64(G + k0 + k0 * f, f, pw, Dp + kp, Eb + k0 + k0 * f, dsign + kp, eps, delta, scr,
+      const int nhit = diag64(G + k0 + k0 * f, f, pw, Dp + kp, dsign + kp, eps, delta, scr,
                               *reinterpret_cast<Diag64Smem*>(sm), *reinterpret_cast<Diag64SmemB*>(smB), dsh, gs, hs);
       if (tid == 0 && nhit) atomicAdd(hits, nhit);
       __syncthreads();
@@ -741,7 +735,8 @@ __global__ void __launch_bounds__(NT, 1)
         __threadfence();
         st_release(w.diag + p, 1);
       }
-      // PE(p, p): rows the columns of Linv (after the release: only EU(p, i, p) waits for it)
+      // after the release: what no T(p, i) or Efin(p, e) reads: L_KK and its inverse for the solves, and
+      // PE(p, p), rows the columns of Linv, for EU(p, i, p)
       pack_tile(V, 1, kDiagLD, 0, hs, -1, pkr.pe(p, p), exps_of(pkr.pe(p, p)));
       fence_async_global();
       fence_async_shared();  // the operands' space is the next task's, by bulk copies
@@ -750,6 +745,14 @@ __global__ void __launch_bounds__(NT, 1)
         __threadfence();
         st_release(w.pe + p, 1);
       }
+      for (int idx = tid; idx < 64 * 64; idx += NT) {
+        const int i = idx & 63, j = idx >> 6;
+        if (i < pw && j < pw && i >= j) {
+          G[(k0 + i) + (k0 + j) * f] = scr[i * kDiagLD + j];
+          Eb[(k0 + i) + (k0 + j) * f] = (i == j) ? 1.0 : V[i * kDiagLD + j];
+        }
+      }
+      __syncthreads();
       continue;
     }
     // T(p, i): rows of F_IK; Efin(p, e): rows the columns of E_KC; both times PT(p)^T.  U(p, i, j),

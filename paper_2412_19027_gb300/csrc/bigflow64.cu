@@ -334,7 +334,6 @@ __device__ __forceinline__ void diag64_panel(int q, int pw, double* A, Diag64Sme
   const int row = NP == 2 ? 32 * (wid & 1) + lane : 32 + lane, par = NP == 2 ? wid >> 1 : wid;
   constexpr long long kSign = (long long)0x8000000000000000ull;
   double v[NC], dk = 0.0;
-  int ma = -kBad, mb = -kBad;
   int2* ib = sb.ib + (q & 1) * 64 * kLP;
   double* cd = reinterpret_cast<double*>(ib);  // this thread's entries of L d, then their integers in place
 #pragma unroll
@@ -365,11 +364,6 @@ __device__ __forceinline__ void diag64_panel(int q, int pw, double* A, Diag64Sme
       if (par == o % NP) {
         if (row >= kk) A[row * LD + kk] = row == kk ? d : lr;
         cd[row * kLP + k] = cr;
-        if (row > kk) {
-          const int ld = ilog_of(d), h = ld <= -kBad || ld >= kBad ? 0 : ld >> 1;
-          ma = max(ma, shifted(lr, h));
-          mb = max(mb, shifted(cr, -h));
-        }
       }
       if (lane == k) dk = d;
       nhit += hit ? 1 : 0;
@@ -394,6 +388,15 @@ __device__ __forceinline__ void diag64_panel(int q, int pw, double* A, Diag64Sme
     hs[c0 + lane] = lg <= -kBad || lg >= kBad ? 0 : lg >> 1;
   }
   // the integer operands L 2^h, (L d) 2^-h of the rows below
+  // (their largest exponents here, not in the loop: integer work there is on the chain of pivots)
+  asm volatile("barrier.sync 2, 128;" ::: "memory");
+  int ma = -kBad, mb = -kBad;
+#pragma unroll
+  for (int t = 0; t < NC; ++t) {
+    const int c = NP * t + par, h = hs[c0 + c];
+    const int xl = shifted(A[row * LD + c0 + c], h), xd = shifted(cd[row * kLP + c], -h);
+    if (row > c0 + c) ma = max(ma, xl), mb = max(mb, xd);
+  }
   atomicMax(&sa.xm[row], ma);
   atomicMax(&sa.xm[64 + row], mb);
   asm volatile("barrier.sync 2, 128;" ::: "memory");

@@ -236,9 +236,10 @@ __global__ void __launch_bounds__(32 * GW) k_factor_small(T* __restrict__ F, T* 
 // One CTA per thin front (ldl_thin_front): its c columns in shared memory as they are
 // (P = L D) and scaled (L), then the trailing lower triangle F -= L P^T in 64 x 64 tiles,
 // a lane per row and eight columns per warp, so that every store is a full line.  LEAF:
-// no child has added to the trailing part, which is zero and not read.  Bound by the
-// stores of the update matrix (f^2 / 2 values) in FP32, by the FMAs in FP64 from c ~ 4 on.
-template <typename T, bool LEAF>
+// no child has added to the trailing part, which is zero and not read; no update matrix with
+// SYRK (thinsyrk.cu).  Bound by the stores of the update matrix (f^2 / 2 values) in FP32, by the
+// FMAs in FP64 from c ~ 4 on.
+template <typename T, bool LEAF, bool SYRK = false>
 __global__ void __launch_bounds__(256) k_factor_thin(T* __restrict__ F, T* __restrict__ Dp,
                                                      const int64_t* __restrict__ fronts,
                                                      const int64_t* __restrict__ sn_ptr,
@@ -279,6 +280,7 @@ __global__ void __launch_bounds__(256) k_factor_thin(T* __restrict__ F, T* __res
     }
     __syncthreads();
   }
+  if constexpr (SYRK) return;
   const int lane = tid & 31, w = tid >> 5;
   for (int j0 = c; j0 < f; j0 += 64)
     for (int i0 = j0; i0 < f; i0 += 64) {
@@ -692,7 +694,9 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
   st.max_front = sy.max_front;
   st.h_lev_ptr = sy.lev_ptr;
   st.h_lev_sn = sy.lev_sn;
-  st.h_fa_lev_ptr = mp.fa_lev_ptr;
+  // the extend-add lists: as they are, or without what thinsyrk.cu adds
+  FaLists fal;
+  const std::vector<int64_t>*fa_lev_ptr = &mp.fa_lev_ptr, *fa_tgt = &mp.fa_tgt, *fa_ptr = &mp.fa_ptr, *fa_src = &mp.fa_src;
   st.h_sv_lev_ptr = mp.sv_lev_ptr;
   st.h_sn_ptr = sy.sn_ptr;
   st.h_row_ptr = sy.row_ptr;
@@ -778,10 +782,25 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       if (pid_of(J) >= nthin.size()) nthin.resize(pid_of(J) + 1, 0);
       nthin[pid_of(J)] += ldl_thin_front(sy.row_ptr[J + 1] - sy.row_ptr[J], sy.sn_ptr[J + 1] - sy.sn_ptr[J], small_max);
     }
-    std::vector<int64_t> small, leaf, thin, both;
+    std::vector<char> thin_leaf(sy.nsn, 0);
+    for (int64_t J = 0; J < sy.nsn; ++J) {
+      const int64_t f = sy.row_ptr[J + 1] - sy.row_ptr[J], c = sy.sn_ptr[J + 1] - sy.sn_ptr[J];
+      thin_leaf[J] = f > small_max && !has_child[J] && nthin[pid_of(J)] >= kThinCount && ldl_thin_front(f, c, small_max);
+    }
+    const int rcs = thin_syrk_plan(ar, sy, mp, thin_leaf, st.f64, kThinCount, st.syrk, fal);
+    if (rcs != CLR_OK) return rcs;
+    if (!fal.lev_ptr.empty()) {
+      fa_lev_ptr = &fal.lev_ptr;
+      fa_tgt = &fal.tgt;
+      fa_ptr = &fal.ptr;
+      fa_src = &fal.src;
+    }
+    st.h_fa_lev_ptr = *fa_lev_ptr;
+    std::vector<int64_t> small, leaf, thin, both, prod;
     for (int64_t l = 0; l < sy.nlev; ++l) {
       small.clear();
       leaf.clear();
+      prod.clear();
       thin.clear();
       both.clear();
       for (int64_t t = sy.lev_ptr[l]; t < sy.lev_ptr[l + 1]; ++t) {
@@ -791,7 +810,7 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
           small.push_back(J);
           st.lev_small_maxf[l] = std::max(st.lev_small_maxf[l], (int)f);
         } else if (nthin[pid_of(J)] >= kThinCount && ldl_thin_front(f, c, small_max)) {
-          (has_child[J] ? thin : leaf).push_back(J);
+          (has_child[J] ? thin : (!st.syrk.child.empty() && st.syrk.child[J] ? prod : leaf)).push_back(J);
           st.lev_thin_smem[l] = std::max(st.lev_thin_smem[l], f * c);
         } else {
           st.lev_big[l].push_back(J);
@@ -801,9 +820,10 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       }
       add(st.lev_small, l, small);
       add(st.lev_thin_leaf, l, leaf);
+      add(st.lev_thin_syrk, l, prod);
       add(st.lev_thin, l, thin);
       add(st.lev_cta, l, both);
-      longs(mp.fa_ptr, mp.fa_lev_ptr[l], mp.fa_lev_ptr[l + 1], kPullSerial, kFaWarp, st.fa_ord, st.fa_warp, st.fa_cta, l);
+      longs(*fa_ptr, (*fa_lev_ptr)[l], (*fa_lev_ptr)[l + 1], kPullSerial, kFaWarp, st.fa_ord, st.fa_warp, st.fa_cta, l);
       longs(mp.sv_ptr, mp.sv_lev_ptr[l], mp.sv_lev_ptr[l + 1], kSvThread, kPullSerial, st.sv_ord, st.sv_warp, st.sv_cta, l);
     }
     int64_t* dbuf = buf.empty() ? nullptr : ar.upload(buf.data(), (int64_t)buf.size());
@@ -1113,9 +1133,9 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
   }
   st.kdest = up(ar, mp.kdest);
   st.diag_pos = up(ar, mp.diag_pos);
-  st.fa_tgt = up(ar, mp.fa_tgt);
-  st.fa_ptr = up(ar, mp.fa_ptr);
-  st.fa_src = up(ar, mp.fa_src);
+  st.fa_tgt = up(ar, *fa_tgt);
+  st.fa_ptr = up(ar, *fa_ptr);
+  st.fa_src = up(ar, *fa_src);
   st.sv_tgt = up(ar, mp.sv_tgt);
   st.sv_ptr = up(ar, mp.sv_ptr);
   st.sv_src = up(ar, mp.sv_src);
@@ -1139,6 +1159,14 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
   ybuf = ar.alloc_n<T>(st.bfd.ypool);
   Linv = ar.alloc_n<T>(st.bfd.n * 2 * kBfNB * kBfNB);
   if (!F || !Dp || !w || !xs || !dyn_hits || !E || !ybuf || !Linv) return CLR_E_OOM;
+  if (st.syrk.wtotal > 0) {
+    syrk_w = ar.alloc_n<T>(st.syrk.wtotal);
+    syrk_part = ar.alloc_n<T>(std::max<int64_t>(1, st.syrk.part));
+    if (!syrk_w || !syrk_part) return CLR_E_OOM;
+    if (cudaMemset(syrk_w, 0, sizeof(T) * (size_t)st.syrk.wtotal) != cudaSuccess ||
+        cudaStreamSynchronize(nullptr) != cudaSuccess)
+      return CLR_E_CUDA;
+  }
   if (BigFrontOps<T>::setup_attributes() != CLR_OK) return CLR_E_CUDA;
   if (st.cta.n > 0 && CtaOps<T>::setup_attributes() != CLR_OK) return CLR_E_CUDA;
   if (st.flow_words > 0) {
@@ -1182,6 +1210,7 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
     cudaFuncSetAttribute(k_factor_small<T, 8, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     cudaFuncSetAttribute(k_factor_small<T, 8, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     cudaFuncSetAttribute(k_factor_thin<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+    cudaFuncSetAttribute(k_factor_thin<T, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
     cudaFuncSetAttribute(k_factor_thin<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
     attr_set = true;
   }
@@ -1195,7 +1224,8 @@ int LdlFactor<T>::factor(cudaStream_t stm, const double* kval, const IterScal* s
   CLR_CUDA(cudaMemsetAsync(dyn_hits, 0, 2 * sizeof(int), stm));  // dynamic-regularisation hits, big-front error
   const bool use_flow = flow && !tc16 && flow_state != nullptr;
   if (use_flow) CLR_CUDA(cudaMemsetAsync(flow_state, 0, sizeof(int) * (size_t)S.flow_words, stm));
-  CLR_CUDA(cudaMemsetAsync(F, 0, sizeof(T) * (size_t)S.pool, stm));
+  if (S.syrk.nseg > 0) ThinSyrkOps<T>::clear_pool(stm, S.syrk, F);
+  else CLR_CUDA(cudaMemsetAsync(F, 0, sizeof(T) * (size_t)S.pool, stm));
   if (S.bfd.epool > 0) CLR_CUDA(cudaMemsetAsync(E, 0, sizeof(T) * (size_t)S.bfd.epool, stm));
   k_scatter_kval<T><<<grid_for(S.nk, 256), 256, 0, stm>>>(F, kval, S.kdest, S.nk, skip);
   k_add_reg<T><<<grid_for(S.N, 256), 256, 0, stm>>>(F, S.diag_pos, S.dsign, S.pos_pid, S.N, sc, skip);
@@ -1206,6 +1236,7 @@ int LdlFactor<T>::factor(cudaStream_t stm, const double* kval, const IterScal* s
   for (int64_t l = 0; l < S.nlev; ++l) {
     pull_level<T>(stm, F, S.fa_tgt, S.fa_ptr, S.fa_src, S.h_fa_lev_ptr[l], S.h_fa_lev_ptr[l + 1], kPullSerial,
                   S.fa_ord[l], S.fa_warp[l], S.fa_cta[l], skip);
+    if (!S.syrk.lev.empty()) ThinSyrkOps<T>::add_level(stm, S.syrk, l, F, Dp, syrk_w, syrk_part, skip);
     for (const WorkList& wl : S.push_rounds[l])
       if (wl.nblocks > 0)
         k_push<T><<<(unsigned)wl.nblocks, 256, 0, stm>>>(F, wl, S.sn_ptr, S.row_ptr, S.front_off, S.sn_parent,
@@ -1230,6 +1261,9 @@ int LdlFactor<T>::factor(cudaStream_t stm, const double* kval, const IterScal* s
     if (S.lev_thin_leaf[l].n > 0)
       k_factor_thin<T, true><<<(unsigned)S.lev_thin_leaf[l].n, 256, tsm, stm>>>(
           F, Dp, S.lev_thin_leaf[l].id, S.sn_ptr, S.row_ptr, S.front_off, S.dsign, dyn_eps, dyn_delta, dyn_hits, skip);
+    if (S.lev_thin_syrk[l].n > 0)
+      k_factor_thin<T, true, true><<<(unsigned)S.lev_thin_syrk[l].n, 256, tsm, stm>>>(
+          F, Dp, S.lev_thin_syrk[l].id, S.sn_ptr, S.row_ptr, S.front_off, S.dsign, dyn_eps, dyn_delta, dyn_hits, skip);
     if (S.lev_thin[l].n > 0)
       k_factor_thin<T, false><<<(unsigned)S.lev_thin[l].n, 256, tsm, stm>>>(
           F, Dp, S.lev_thin[l].id, S.sn_ptr, S.row_ptr, S.front_off, S.dsign, dyn_eps, dyn_delta, dyn_hits, skip);

@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "bigfront.cuh"
+#include "thinsyrk.cuh"
 #include "device.cuh"
 #include "internal.h"
 #include "kktcta.cuh"
@@ -39,6 +40,9 @@ struct LdlStructure {
     int64_t first = 0;  // lev_cta: index of its first entry in cta_pull
   };
   std::vector<List> lev_small, lev_thin_leaf, lev_thin, lev_cta;
+  std::vector<List> lev_thin_syrk;               // thin leaves whose update matrices are a product (thinsyrk.cu)
+  ThinSyrk syrk;
+  bool f64 = false;                              // the factor is FP64 (set before ldl_structure_upload)
   std::vector<int64_t> lev_thin_smem;            // largest f c of a level's thin fronts
   // pull targets with long source lists (indices into fa_tgt, sv_tgt): a warp each (the sum
   // in list order), a warp each, a CTA each
@@ -120,6 +124,7 @@ struct LdlFactor {
   bool flow = true;       // big fronts by the dataflow kernel (one launch per level); else per-panel launches
   int flow_tc = 1;        // FP32 dataflow, trailing and E updates on the tensor cores (TF32 hi/lo parts):
                           // 0 never, 1 on the levels whose simulated schedule is shorter that way, 2 always
+  T *syrk_w = nullptr, *syrk_part = nullptr;  // panels and partial tiles of thinsyrk.cu
   unsigned char* pk64 = nullptr;  // FP64: digit packs of the largest level (null: FMA products on every front)
   FlowTc tcs;             // its packed operand tiles and their tensor map (allocated when used)
   int* flow_state = nullptr;

@@ -322,6 +322,7 @@ int clr_ldl_solve(const clr_csc* K, const double* signs, const int64_t* order, i
   for (int64_t k = 0; k < N; ++k) dsign[k] = signs[sy.perm[k]] > 0 ? 1 : -1;
   DeviceArena ar;
   LdlStructure ls;
+  ls.f64 = factor_bits == 64;
   ls.flow_emu = big_front_schedule == 1 || big_front_schedule == 3;
   rc = ldl_structure_upload(ar, sy, mp, dsign, factor_bits == 64 ? 96 : 128, ls);
   if (rc) return rc;

@@ -1,0 +1,49 @@
+// Extend-add of many thin leaf fronts into one parent as a product (thinsyrk.cu).
+#pragma once
+
+#include <cstdint>
+#include <vector>
+
+#include "device.cuh"
+#include "symbolic.h"
+
+namespace clr {
+
+struct ThinSyrkParent {
+  int64_t goff, fP, ld;     // the parent's front in the pool, its rows; row length of its panel W
+  int64_t K, col0, woff;    // columns of its thin leaves, the first one in the column arrays, W's offset
+  int64_t tiles, splits, kc;
+};
+
+struct ThinSyrk {
+  std::vector<std::vector<ThinSyrkParent>> lev;  // by the parent's level
+  std::vector<char> child;                       // host: fronts that keep no update matrix
+  // per column: its rows below the pivots in the pool, how many, their places in the parent's
+  // rows (first one in map), its pivot
+  int64_t *src = nullptr, *map0 = nullptr;
+  int32_t *cnt = nullptr, *dpos = nullptr, *map = nullptr;
+  // parts of the pool that a factorization clears (offset, length <= kSegment): without the update
+  // matrices that are not kept
+  int64_t* seg = nullptr;
+  int64_t nseg = 0;
+  int64_t wtotal = 0, part = 0;                  // entries of all panels W; of the largest parent's partial tiles
+};
+
+// The extend-add lists of a structure (NumericMaps' fa_*), without what the products cover.
+struct FaLists {
+  std::vector<int64_t> lev_ptr, tgt, ptr, src;
+};
+
+// leaf: thin leaf fronts (ldl_thin_front, the path taken).  Chooses the parents, fills out and, if
+// any was chosen, fa.
+int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<char>& leaf, bool f64,
+                   int64_t min_children, ThinSyrk& out, FaLists& fa);
+
+template <typename T>
+struct ThinSyrkOps {
+  static void clear_pool(cudaStream_t st, const ThinSyrk& ts, T* F);
+  // F_P -= sum over the leaves' columns of l d l^T, for the parents of level l
+  static void add_level(cudaStream_t st, const ThinSyrk& ts, int64_t l, T* F, const T* Dp, T* W, T* part,
+                        const int* skip);
+};
+}  // namespace clr

@@ -113,6 +113,42 @@ def test_thin_fronts_and_long_pulls(bits, leaves, c, r, m, extra):
     assert hits == 0 and np.all(sgn * D > 0)
 
 
+# 512 thin leaves or more under one parent: their update matrices as one product (thinsyrk.cu), at
+# the ends of its 64 x 64 tiles, 16-column steps and splits; `deep` leaves have a child and `few`
+# have too few rows to be thin, and stay with the lists beside it
+@pytest.mark.parametrize("bits", [64, 32])
+@pytest.mark.parametrize("leaves,c,r,m,deep,few", [
+    (512, 1, 129, 129, 0, 0), (515, 1, 128, 192, 0, 0), (530, 1, 190, 193, 9, 0), (513, 2, 130, 255, 0, 5),
+    (600, 1, 256, 256, 3, 3), (512, 3, 257, 257, 0, 0), (2100, 1, 140, 140, 0, 7), (511, 1, 130, 130, 2, 2)])
+def test_thin_leaves_as_product(bits, leaves, c, r, m, deep, few):
+    import scipy.sparse as sp
+    rng = np.random.default_rng(leaves + c + r + m)
+    R, Cc, V, p0 = [], [], [], 0
+    kinds = rng.permutation(np.r_[np.zeros(leaves, int), np.ones(deep, int), np.full(few, 2)])
+    root = leaves * c + deep * (c + 3) + few * c
+    N = root + m
+    for kind in kinds:
+        piv = np.arange(p0, p0 + c + (3 if kind == 1 else 0))
+        p0 += len(piv)
+        for a in piv:
+            low = piv[piv > a]
+            R.append(low); Cc.append(np.full(len(low), a)); V.append(0.1 * rng.standard_normal(len(low)))
+        rr = 20 if kind == 2 else r
+        rows = root + np.sort(rng.choice(m, rr, replace=False))
+        for a in piv[-c:]:
+            R.append(rows); Cc.append(np.full(rr, a)); V.append(rng.standard_normal(rr) / np.sqrt(len(kinds) * r))
+    K = sp.csc_matrix((np.concatenate(V), (np.concatenate(R), np.concatenate(Cc))), shape=(N, N))
+    sgn = np.where(np.arange(N) < root, 1.0, -1.0)
+    K = sp.tril(K, -1) + sp.diags(sgn * (2.0 + rng.random(N)))
+    rhs = rng.standard_normal(N)
+    x, D, hits = clr.clr_ldl_solve(K, sgn, rhs, order=np.arange(N), factor_bits=bits)
+    Kf = K + sp.tril(K, -1).T
+    # as above: diagonally dominant quasi-definite blocks
+    eps = 2.2e-16 if bits == 64 else 1.2e-7
+    assert np.abs(Kf @ x - rhs).max() <= 10 * np.sqrt(N) * eps * max(1.0, np.abs(x).max()) * 10
+    assert hits == 0 and np.all(sgn * D > 0)
+
+
 # one CTA per problem (fronts of at most 96 rows, all of a cohort) against the launch per
 # level: the same problem alone and beside one with large fronts, which takes every problem
 # of the cohort through the general kernels

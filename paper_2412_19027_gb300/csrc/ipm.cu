@@ -59,10 +59,11 @@ __device__ __forceinline__ int64_t chunk_slot(const ChunkGrid& g) {
 // The sum of a row is formed in one fixed order whatever G is (32 partial sums,
 // entry e of the row going to partial e mod 32, then the pairwise tree t += t+16,
 // t += t+8, ...), so a row gives the same bits in every cohort it belongs to.
-// Rows longer than this go to k_kmv_long (a CTA per row); each row's sum is taken
+// Rows longer than kLongRow are summed by a CTA each (k_kmv_rows); each row's sum is taken
 // in an order fixed by its length alone, so a problem's K products are the same
 // alone and in a cohort.
 constexpr int64_t kLongRow = 512;
+constexpr int kShortRow = 4;
 
 template <int G>
 __global__ void k_kmv(int mode, int64_t r0, int64_t r1, int64_t n, const int64_t* __restrict__ kptr,
@@ -80,7 +81,7 @@ __global__ void k_kmv(int mode, int64_t r0, int64_t r1, int64_t n, const int64_t
   RunExt<true> mx;
   for (int64_t i = r0 + gid; i < r1; i += gstride) {
     const int64_t p0 = kptr[i], p1 = kptr[i + 1];
-    if (p1 - p0 > kLongRow) continue;  // k_kmv_long (the whole G-lane group skips)
+    if (p1 - p0 > kLongRow) continue;  // k_kmv_rows (the whole G-lane group skips)
     double a, b;
     kmv_row<G>(i, p0, p1, n, kcol, kvi, kval, kfv, v, lane, gmask, a, b);
     if (lane == 0) {
@@ -99,93 +100,120 @@ __global__ void k_kmv(int mode, int64_t r0, int64_t r1, int64_t n, const int64_t
   if (mode == 1) mx.flush(sc, &IterScal::rnorm_bits);
 }
 
-// The long rows: 8 warps per row, warp w sums the w-th of 8 contiguous segments of
-// 32-entry steps (lane t: entries p = p0 + t (mod 32)), the 8 partials of a lane are
-// added in warp order, then the 32 lanes by the same butterfly as k_kmv.  Outputs
-// as k_kmv for the modes.
+// A row's result, by one thread.
+__device__ __forceinline__ void kmv_put(int mode, int64_t i, int64_t n, double a, double b, double* __restrict__ lo,
+                                        double* __restrict__ hi, const double* __restrict__ rhs, double* __restrict__ out,
+                                        const int32_t* __restrict__ pid, IterScal* sc, RunExt<true>& mx) {
+  if (mode == 0) {
+    lo[i] = a;
+    hi[i] = b;
+  } else if (mode == 1) {
+    const double r = rhs[i] - (a + b);
+    out[i] = r;
+    mx.add(sc, &IterScal::rnorm_bits, pid[i], dbits(fabs(r)));
+  } else {
+    out[i - n] = -rhs[i - n] + b;
+  }
+}
+
+// Rows by length in one launch, outputs as k_kmv for the modes: nb.x CTAs take the long rows (more than
+// kLongRow entries), nb.y the middle ones (a warp each), the others the short ones (up to
+// kShortRow, a thread each).
+// Long rows: 8 warps per row, warp w sums the w-th of 8 contiguous segments of 32-entry steps
+// (lane t: entries p = p0 + t (mod 32)), the 8 partials of a lane are added in warp order, then the
+// 32 lanes by the same butterfly as k_kmv.
+// Bound by the FP64 pipe (a multiplication and an addition per 32 entries, 64 clocks of a
+// sub-partition each) and by the loads' latency; in two launches one after the other, with
+// the constant values of the z rows gathered through the index and a warp for every short row,
+// the product took 39 us on the portfolio n = 5000 (2.5e6 entries), here 26.
+struct KmvRows {
+  const int64_t* id[3];
+  int64_t n[3];
+  int64_t nb[2];
+};
 __global__ void __launch_bounds__(256)
-    k_kmv_long(int mode, const int64_t* __restrict__ rows, int64_t nrows, int64_t n, const int64_t* __restrict__ kptr,
-               const int32_t* __restrict__ kcol, const int32_t* __restrict__ kvi, const double* __restrict__ kval,
-               const double* __restrict__ kfv,
+    k_kmv_rows(int mode, KmvRows rows, int64_t n, const int64_t* __restrict__ kptr, const int32_t* __restrict__ kcol,
+               const int32_t* __restrict__ kvi, const double* __restrict__ kval, const double* __restrict__ kfv,
                const double* __restrict__ v, double* __restrict__ lo, double* __restrict__ hi,
-               const double* __restrict__ rhs, double* __restrict__ out, const int32_t* __restrict__ pid,
-               IterScal* sc, const int* skip) {
+               const double* __restrict__ rhs, double* __restrict__ out, const int32_t* __restrict__ pid, IterScal* sc,
+               const int* skip) {
   if (skip && *skip) return;
   __shared__ double pa[8][32], pb[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   RunExt<true> mx;
-  for (int64_t t = blockIdx.x; t < nrows; t += gridDim.x) {
-    const int64_t i = rows[t];
-    const int64_t p0 = kptr[i], p1 = kptr[i + 1];
-    const int64_t S = ((p1 - p0 + 255) / 256) * 32;  // segment length, a multiple of 32
-    const int64_t s0 = p0 + w * S, s1 = min(p1, s0 + S);
-    double a = 0.0, b = 0.0;
-    for (int64_t base = s0; base < s1; base += 128) {
-      double tv[4];
-      bool tx[4];
+  int64_t blk = blockIdx.x;
+  if (blk < rows.nb[0]) {
+    for (int64_t t = blk; t < rows.n[0]; t += rows.nb[0]) {
+      const int64_t i = rows.id[0][t];
+      const int64_t p0 = kptr[i], p1 = kptr[i + 1];
+      const int64_t S = ((p1 - p0 + 255) / 256) * 32;  // segment length, a multiple of 32
+      const int64_t s0 = p0 + w * S, s1 = min(p1, s0 + S);
+      double a, b;
+      unsigned ua, ub;
+      kmv_warp(i, s0, s1, n, kcol, kvi, kval, kfv, v, lane, a, b, ua, ub);
+      pa[w][lane] = a;
+      pb[w][lane] = b;
+      __syncthreads();
+      if (w == 0) {
+        a = pa[0][lane];
+        b = pb[0][lane];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int64_t p = base + 32 * k + lane;
-        tv[k] = 0.0;
-        tx[k] = true;
-        if (p < s1) {
-          const int32_t c = kcol[p];
-          tv[k] = (i < n ? kfv[p] : kval[kvi[p]]) * v[c];
-          tx[k] = c < n;
+        for (int q = 1; q < 8; ++q) {
+          a += pa[q][lane];
+          b += pb[q][lane];
         }
-      }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (base + 32 * k + lane >= s1) continue;
-        if (tx[k]) a += tv[k];
-        else b += tv[k];
-      }
-    }
-    pa[w][lane] = a;
-    pb[w][lane] = b;
-    __syncthreads();
-    if (w == 0) {
-      a = pa[0][lane];
-      b = pb[0][lane];
-#pragma unroll
-      for (int q = 1; q < 8; ++q) {
-        a += pa[q][lane];
-        b += pb[q][lane];
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, off);
-        b += __shfl_xor_sync(0xffffffffu, b, off);
-      }
-      if (lane == 0) {
-        if (mode == 0) {
-          lo[i] = a;
-          hi[i] = b;
-        } else if (mode == 1) {
-          const double r = rhs[i] - (a + b);
-          out[i] = r;
-          mx.add(sc, &IterScal::rnorm_bits, pid[i], dbits(fabs(r)));
-        } else {
-          out[i - n] = -rhs[i - n] + b;
+        for (int off = 16; off > 0; off >>= 1) {
+          a += __shfl_xor_sync(0xffffffffu, a, off);
+          b += __shfl_xor_sync(0xffffffffu, b, off);
         }
+        if (lane == 0) kmv_put(mode, i, n, a, b, lo, hi, rhs, out, pid, sc, mx);
       }
+      __syncthreads();
     }
-    __syncthreads();
+    if (mode == 1 && w == 0) mx.flush(sc, &IterScal::rnorm_bits);
+    return;
   }
-  if (mode == 1 && w == 0) mx.flush(sc, &IterScal::rnorm_bits);
+  blk -= rows.nb[0];
+  if (blk < rows.nb[1]) {
+    for (int64_t t = 8 * blk + w; t < rows.n[1]; t += 8 * rows.nb[1]) {
+      const int64_t i = rows.id[1][t];
+      double a, b;
+      kmv_row<32>(i, kptr[i], kptr[i + 1], n, kcol, kvi, kval, kfv, v, lane, 0xffffffffu, a, b);
+      if (lane == 0) kmv_put(mode, i, n, a, b, lo, hi, rhs, out, pid, sc, mx);
+    }
+  } else {
+    const int64_t step = 256 * ((int64_t)gridDim.x - rows.nb[0] - rows.nb[1]);
+    for (int64_t t = 256 * (blk - rows.nb[1]) + threadIdx.x; t < rows.n[2]; t += step) {
+      const int64_t i = rows.id[2][t];
+      double a, b;
+      kmv_row_thread<kShortRow>(i, kptr[i], kptr[i + 1], n, kcol, kvi, kval, kfv, v, a, b);
+      kmv_put(mode, i, n, a, b, lo, hi, rhs, out, pid, sc, mx);
+    }
+  }
+  if (mode == 1) mx.flush(sc, &IterScal::rnorm_bits);
 }
 
-// launch k_kmv_long for the long rows in [r0, r1)
-void kmv_long(cudaStream_t s, int mode, int64_t r0, int64_t r1, int64_t n, const VecDev& v,
-              const std::vector<int64_t>& h_long, const double* x, double* lo, double* hi, const double* rhs,
-              double* out, IterScal* sc, const int* skip) {
-  if (h_long.empty()) return;
-  const int64_t a = std::lower_bound(h_long.begin(), h_long.end(), r0) - h_long.begin();
-  const int64_t b = std::lower_bound(h_long.begin(), h_long.end(), r1) - h_long.begin();
-  if (b <= a) return;
-  const unsigned g = (unsigned)std::min<int64_t>(b - a, 16 * kSMs);  // a row per CTA, up to 16 CTAs per SM
-  k_kmv_long<<<g, 256, 0, s>>>(mode, v.long_rows + a, b - a, n, v.kptr, v.kcol, v.kvi, v.kval, v.kfv, x, lo, hi, rhs,
-                               out, v.pid, sc, skip);
+// the rows [r0, r1) of the three lists
+void kmv_rows(cudaStream_t s, int mode, int64_t r0, int64_t r1, int64_t n, const VecDev& v,
+              const std::vector<int64_t> (&h_rows)[3], const double* x, double* lo, double* hi, const double* rhs,
+              double* out, IterScal* sc, const int* skip, bool long_only) {
+  KmvRows k{};
+  int64_t grid[3];
+  for (int c = 0; c < 3; ++c) {
+    const auto& h = h_rows[c];
+    const int64_t a = std::lower_bound(h.begin(), h.end(), r0) - h.begin();
+    const int64_t b = std::lower_bound(h.begin(), h.end(), r1) - h.begin();
+    k.id[c] = v.rows_by_len[c] + a;
+    k.n[c] = long_only && c > 0 ? 0 : b - a;
+    const int64_t per = c == 0 ? 1 : (c == 1 ? 8 : 256);
+    grid[c] = std::min<int64_t>((k.n[c] + per - 1) / per, 16 * kSMs);  // a row per CTA, warp, thread; 16 CTAs per SM
+  }
+  k.nb[0] = grid[0];
+  k.nb[1] = grid[1];
+  if (grid[0] + grid[1] + grid[2] == 0) return;
+  k_kmv_rows<<<(unsigned)(grid[0] + grid[1] + grid[2]), 256, 0, s>>>(mode, k, n, v.kptr, v.kcol, v.kvi, v.kval, v.kfv, x,
+                                                                     lo, hi, rhs, out, v.pid, sc, skip);
 }
 
 // ------------------------------------------------------------------ residuals
@@ -990,27 +1018,30 @@ int Solver::upload() {
         vi[p] = row[p - cnt[i]].second;
       }
     }
-    h_long_.clear();
-    for (int64_t i = 0; i < N; ++i)
-      if (cnt[i + 1] - cnt[i] > kLongRow) h_long_.push_back(i);
-    v_.nlong = (int64_t)h_long_.size();
-    v_.long_rows = h_long_.empty() ? nullptr : ar_.upload(h_long_.data(), v_.nlong);
-    if (!h_long_.empty() && !v_.long_rows) return CLR_E_OOM;
+    for (auto& h : h_rows_) h.clear();
+    for (int64_t i = 0; i < N; ++i) {
+      const int64_t len = cnt[i + 1] - cnt[i];
+      h_rows_[len > kLongRow ? 0 : (len > kShortRow ? 1 : 2)].push_back(i);
+    }
+    for (int c = 0; c < 3; ++c) {
+      v_.rows_by_len[c] = h_rows_[c].empty() ? nullptr : ar_.upload(h_rows_[c].data(), (int64_t)h_rows_[c].size());
+      if (!h_rows_[c].empty() && !v_.rows_by_len[c]) return CLR_E_OOM;
+    }
     v_.kptr = ar_.upload(cnt.data(), N + 1);
     v_.kcol = ar_.upload(col.data(), (int64_t)col.size());
     v_.kvi = ar_.upload(vi.data(), (int64_t)vi.size());
     {
-      // the x rows' values in full-CSR order (P and A are constant through the solve):
-      // contiguous loads instead of gathers through the value index
-      std::vector<double> fv(cnt[hp.n], 0.0);
-      for (int64_t p = 0; p < cnt[hp.n]; ++p) fv[p] = hp.kval[vi[p]];
-      h_kfv_src_.assign(vi.begin(), vi.begin() + cnt[hp.n]);
+      // the values in full-CSR order: contiguous loads instead of gathers through the value
+      // index for P and A, which are constant through the solve (the z-z block's are not used)
+      std::vector<double> fv(cnt[N], 0.0);
+      for (int64_t p = 0; p < cnt[N]; ++p) fv[p] = hp.kval[vi[p]];
+      h_kfv_src_ = vi;
       v_.kfv = fv.empty() ? nullptr : ar_.upload(fv.data(), (int64_t)fv.size());
       if (!fv.empty() && !v_.kfv) return CLR_E_OOM;
     }
     const double avg = N ? (double)cnt[N] / (double)N : 1.0;
     // one CTA per problem: rows summed by lane groups only, and a bounded number of entries each
-    cta_solve_ = ls_.cta.n > 0 && h_long_.empty() && cnt[N] <= kCtaWork * B && cnt[N] < ((int64_t)1 << 31);
+    cta_solve_ = ls_.cta.n > 0 && h_rows_[0].empty() && cnt[N] <= kCtaWork * B && cnt[N] < ((int64_t)1 << 31);
     if (cta_solve_) {
       // rows by problem (elimination positions are contiguous there), shortest class first
       std::vector<int4> kr;
@@ -1227,12 +1258,12 @@ int Solver::kkt_solve(const double* rhs, double* sol) {
   const int kg = grid_for(N * G, 256, 16 * kSMs);
   auto residual = [&](cudaStream_t ss) {
     switch (G) {
-      case 32: k_kmv<32><<<kg, 256, 0, ss>>>(1, 0, N, hp.n, v_.kptr, v_.kcol, v_.kvi, v_.kval, v_.kfv, sol, nullptr, nullptr, rhs, v_.r, v_.pid, sc_, irs); break;
+      case 32: break;  // k_kmv_rows
       case 16: k_kmv<16><<<kg, 256, 0, ss>>>(1, 0, N, hp.n, v_.kptr, v_.kcol, v_.kvi, v_.kval, v_.kfv, sol, nullptr, nullptr, rhs, v_.r, v_.pid, sc_, irs); break;
       case 8: k_kmv<8><<<kg, 256, 0, ss>>>(1, 0, N, hp.n, v_.kptr, v_.kcol, v_.kvi, v_.kval, v_.kfv, sol, nullptr, nullptr, rhs, v_.r, v_.pid, sc_, irs); break;
       default: k_kmv<4><<<kg, 256, 0, ss>>>(1, 0, N, hp.n, v_.kptr, v_.kcol, v_.kvi, v_.kval, v_.kfv, sol, nullptr, nullptr, rhs, v_.r, v_.pid, sc_, irs); break;
     }
-    kmv_long(ss, 1, 0, N, hp.n, v_, h_long_, sol, nullptr, nullptr, rhs, v_.r, sc_, irs);
+    kmv_rows(ss, 1, 0, N, hp.n, v_, h_rows_, sol, nullptr, nullptr, rhs, v_.r, sc_, irs, G < 32);
   };
   const int cb = (int)std::min<int64_t>(1024, std::max<int64_t>(32, ((B + 31) / 32) * 32));
   int rc = ldl_solve_add(s, rhs, 0);
@@ -1299,16 +1330,16 @@ void launch_kmv_split(cudaStream_t s, int mode, int64_t r0, int64_t r1, int64_t 
                               skip);
 }
 void kmv(int G, cudaStream_t s, int mode, int64_t r0, int64_t r1, int64_t n, const VecDev& v,
-         const std::vector<int64_t>& h_long, const double* x, double* lo, double* hi, const double* rhs, double* out,
+         const std::vector<int64_t> (&h_rows)[3], const double* x, double* lo, double* hi, const double* rhs, double* out,
          IterScal* sc, const int* skip) {
   if (r1 <= r0) return;
   switch (G) {
-    case 32: launch_kmv_split<32>(s, mode, r0, r1, n, v, x, lo, hi, rhs, out, sc, skip); break;
+    case 32: break;  // k_kmv_rows
     case 16: launch_kmv_split<16>(s, mode, r0, r1, n, v, x, lo, hi, rhs, out, sc, skip); break;
     case 8: launch_kmv_split<8>(s, mode, r0, r1, n, v, x, lo, hi, rhs, out, sc, skip); break;
     default: launch_kmv_split<4>(s, mode, r0, r1, n, v, x, lo, hi, rhs, out, sc, skip); break;
   }
-  kmv_long(s, mode, r0, r1, n, v, h_long, x, lo, hi, rhs, out, sc, skip);
+  kmv_rows(s, mode, r0, r1, n, v, h_rows, x, lo, hi, rhs, out, sc, skip, G < 32);
 }
 }  // namespace
 
@@ -1330,7 +1361,7 @@ int Solver::direction(bool affine, bool solved) {
   k_fin_dtau<<<(unsigned)B, 128, 0, s>>>(sc_, v_.part, pst_, v_.ckx_ptr, v_.ckz_ptr, halt);
   k_recover<<<nck, 256, 0, s>>>(cg, dir, v_.sol1, v_.sol2, sc_, halt);
   // (the auxiliary rows of expanded SOCs, the last rows, keep Delta s = 0)
-  kmv(csr_group_, s, 2, n, N - hp.cl.n_aux, n, v_, h_long_, dir, nullptr, nullptr, v_.dsrhs, ds, sc_, halt);
+  kmv(csr_group_, s, 2, n, N - hp.cl.n_aux, n, v_, h_rows_, dir, nullptr, nullptr, v_.dsrhs, ds, sc_, halt);
   // PSD rows again, with H in factored form (the assembled block loses the small
   // eigen-directions of S near convergence)
   cones_psd_ds_from_dz(s, cd_, dir + n, v_.dsrhs, ds, halt);
@@ -1380,7 +1411,7 @@ int Solver::iteration() {
   int rc;
   mark(2);
   // ---- residuals, objectives, mu, termination ----
-  kmv(csr_group_, s, 0, 0, N, n, v_, h_long_, v_.xz, v_.lo, v_.hi, nullptr, nullptr, sc_, halt);
+  kmv(csr_group_, s, 0, 0, N, n, v_, h_rows_, v_.xz, v_.lo, v_.hi, nullptr, nullptr, sc_, halt);
   CLR_CUDA(cudaMemsetAsync(v_.maxb, 0, sizeof(unsigned long long) * M_NMAX * (size_t)B, s));
   k_resid<<<nck, 256, 0, s>>>(cg, v_.xz, v_.s, v_.lo, v_.hi, v_.q, v_.b, v_.D, v_.E, sc_, v_.G, v_.qp, v_.part,
                               v_.maxb, halt);

@@ -18,9 +18,8 @@
 namespace clr {
 
 struct VecDev {
-  const int64_t* long_rows = nullptr;  // KKT rows with more than kLongRow entries (sorted)
-  const double* kfv = nullptr;         // values of the x rows of the full KKT CSR (constant), CSR order
-  int64_t nlong = 0;
+  const int64_t* rows_by_len[3] = {nullptr, nullptr, nullptr};  // KKT rows: long, middle, short (sorted; k_kmv_rows)
+  const double* kfv = nullptr;         // values of the full KKT CSR in its order, but for the z-z block (constant)
   double *xz, *s;            // iterate: [x; z] (N), s (m)
   double *lo, *hi;           // split K products (N each)
   double *G;                 // [G1; G2] (N)
@@ -109,8 +108,8 @@ class Solver {
   int hist_rows_ = 0;
   int csr_group_ = 32;
   bool cta_solve_ = false;  // refined KKT solves by one CTA per problem (kktcta.cuh)
-  std::vector<int64_t> h_long_;  // KKT rows handled by k_kmv_long
-  std::vector<int32_t> h_kfv_src_;  // kval index of each entry of the x rows' full-CSR values (kfv)
+  std::vector<int64_t> h_rows_[3];  // rows_by_len on the host
+  std::vector<int32_t> h_kfv_src_;  // kval index of each full-CSR entry (kfv)
   // iteration graphs per factor precision (0: configured, 1: FP64 after an escalation)
   cudaGraph_t graph_[2] = {nullptr, nullptr};
   cudaGraphExec_t gexec_[2] = {nullptr, nullptr};

@@ -10,6 +10,57 @@ namespace clr {
 __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
 __device__ __forceinline__ double bitsd(unsigned long long b) { return __longlong_as_double((long long)b); }
 
+// Entry p of row i, column c.  kfv holds the constant values (P and A) in row order; the
+// z-z block's, which change from iteration to iteration, are read through the value index.
+__device__ __forceinline__ double kmv_value(int64_t i, int64_t p, int32_t c, int64_t n, const int32_t* __restrict__ kvi,
+                                            const double* __restrict__ kval, const double* __restrict__ kfv) {
+  return i >= n && c >= n ? kval[kvi[p]] : kfv[p];
+}
+// Sum of the lanes' partials, lanes outside `used` holding 0: the tree t += t + 16, ..., and for
+// one partial what the tree gives, x + 0.
+__device__ __forceinline__ double kmv_tree(double a, unsigned used) {
+  if (used == 0) return 0.0;
+  if ((used & (used - 1)) == 0) return __dadd_rn(__shfl_sync(0xffffffffu, a, __ffs(used) - 1), 0.0);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) a = __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, off));
+  return a;
+}
+// Entries [s0, s1) of row i by a warp, entry p to lane (p - s0) mod 32.  An FP64 instruction
+// takes 64 clocks of its pipe however few lanes are active, so sums that no lane adds to are left out
+// (a row's columns are sorted: most steps have one kind).
+__device__ __forceinline__ void kmv_warp(int64_t i, int64_t s0, int64_t s1, int64_t n, const int32_t* __restrict__ kcol,
+                                         const int32_t* __restrict__ kvi, const double* __restrict__ kval,
+                                         const double* __restrict__ kfv, const double* v, int lane, double& a, double& b,
+                                         unsigned& ua, unsigned& ub) {
+  a = b = 0.0;
+  ua = ub = 0;
+  for (int64_t base = s0; base < s1; base += 128) {
+    double x[4], y[4];
+    int32_t c[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t p = base + 32 * k + lane;
+      c[k] = p < s1 ? kcol[p] : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      x[k] = c[k] >= 0 ? kmv_value(i, base + 32 * k + lane, c[k], n, kvi, kval, kfv) : 0.0;
+      y[k] = c[k] >= 0 ? v[c[k]] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const unsigned ma = __ballot_sync(0xffffffffu, c[k] >= 0 && c[k] < n);
+      const unsigned mb = __ballot_sync(0xffffffffu, c[k] >= n);
+      if ((ma | mb) == 0) break;
+      const double t = __dmul_rn(x[k], y[k]);
+      if (ma) a = c[k] >= 0 && c[k] < n ? __dadd_rn(a, t) : a;
+      if (mb) b = c[k] >= n ? __dadd_rn(b, t) : b;
+      ua |= ma;
+      ub |= mb;
+    }
+  }
+}
+
 // Sums of row i (entries p0 .. p1) by G lanes: a over the columns < n, b over the
 // others, valid in lane 0 of the group.  32 partial sums, entry e of the row going to
 // partial e mod 32, then the pairwise tree t += t + 16, t += t + 8, ..., whatever G is.
@@ -18,6 +69,14 @@ __device__ __forceinline__ void kmv_row(int64_t i, int64_t p0, int64_t p1, int64
                                         const int32_t* __restrict__ kvi, const double* __restrict__ kval,
                                         const double* __restrict__ kfv, const double* v, int lane, unsigned gmask,
                                         double& ra, double& rb) {
+  if constexpr (G == 32) {
+    unsigned ua, ub;
+    double x, y;
+    kmv_warp(i, p0, p1, n, kcol, kvi, kval, kfv, v, lane, x, y, ua, ub);
+    ra = kmv_tree(x, ua);
+    rb = kmv_tree(y, ub);
+    return;
+  }
   constexpr int NU = 32 / G;  // partial sums per lane: t = lane + G u
   double a[NU], b[NU];
 #pragma unroll
@@ -37,7 +96,7 @@ __device__ __forceinline__ void kmv_row(int64_t i, int64_t p0, int64_t p1, int64
         tx[k][u] = true;
         if (p < p1) {
           const int32_t c = kcol[p];
-          tv[k][u] = (i < n ? kfv[p] : kval[kvi[p]]) * v[c];
+          tv[k][u] = kmv_value(i, p, c, n, kvi, kval, kfv) * v[c];
           tx[k][u] = c < n;
         }
       }
@@ -82,7 +141,7 @@ __device__ __forceinline__ void kmv_row_thread(int64_t i, int64_t p0, int64_t p1
     const int64_t p = p0 + e;
     if (p < p1) {
       const int32_t c = kcol[p];
-      const double t = (i < n ? kfv[p] : kval[kvi[p]]) * v[c];
+      const double t = kmv_value(i, p, c, n, kvi, kval, kfv) * v[c];
       if (c < n) a[e] = t;
       else b[e] = t;
     }

@@ -244,3 +244,34 @@ def test_large_fp64_fronts_by_digits(n, scale):
         np.testing.assert_allclose(Dg, D, rtol=1e-10)
         res[sch] = np.linalg.norm(r / s)
     assert res[1] <= 2 * res[2]
+
+
+# K products by row length in one launch (k_kmv_rows: thread, warp and CTA per row) against the lane
+# groups: a problem of dense rows alone, and beside a sparse one that brings the rows' average
+# down; P and A columns of every length around the limits, a SOC block beside the nonnegative rows
+@pytest.mark.parametrize("bits", [64, 32])
+@pytest.mark.parametrize("n", [130, 520, 700])
+def test_k_products_by_row_length(bits, n):
+    import scipy.sparse as sp
+    from paper_2412_19027_gb300 import workloads as W
+    rng = np.random.default_rng(n)
+    lens = [1, 2, 3, 4, 5, 31, 32, 33, 127, 128, 129] + [k for k in (509, 510, 511, 512, 513, 514, 641) if k <= n] + [n] * 40
+    R = np.concatenate([np.full(k, i) for i, k in enumerate(lens)])
+    Cc = np.concatenate([np.sort(rng.choice(n, k, replace=False)) for k in lens])
+    A = sp.csc_matrix((rng.standard_normal(len(R)) / np.sqrt(n), (R, Cc)), shape=(len(lens), n))
+    m = len(lens)
+    P, q = sp.csc_matrix(sp.diags(1.0 + rng.random(n))), rng.standard_normal(n)
+    s0 = np.r_[1.0 + rng.random(m - 12), 5.0, 0.1 * rng.standard_normal(11)]
+    dense = (P, q, A, A @ rng.standard_normal(n) + s0, [(W.NONNEG, m - 12, 0.0), (W.SOC, 12, 0.0)])
+    big = W.banded_lp(3, n=6000)
+    st = clr.clr_default_settings(bits, max_iter=5, fp64_escalation=0)
+    one = clr.clr_setup(*dense, st)
+    one.solve()
+    both = clr.clr_batch_setup([dense, (big.P, big.q, big.A, big.b, big.cones)], st)
+    both.solve()
+    a, b = one.solution(), both.solution_of(0)
+    for u, v in zip(a[:3], b[:3]):
+        np.testing.assert_array_equal(u, v)
+    assert a[3]["iterations"] == b[3]["iterations"] and a[3]["ir_steps_total"] == b[3]["ir_steps_total"]
+    one.free()
+    both.free()

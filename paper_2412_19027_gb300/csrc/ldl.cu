@@ -695,9 +695,9 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
   st.h_lev_ptr = sy.lev_ptr;
   st.h_lev_sn = sy.lev_sn;
   // the extend-add lists: as they are, or without what thinsyrk.cu adds
-  FaLists fal;
+  FaLists fal, svl;
+  const std::vector<int64_t>*sv_lev_ptr = &mp.sv_lev_ptr, *sv_tgt = &mp.sv_tgt, *sv_ptr = &mp.sv_ptr, *sv_src = &mp.sv_src;
   const std::vector<int64_t>*fa_lev_ptr = &mp.fa_lev_ptr, *fa_tgt = &mp.fa_tgt, *fa_ptr = &mp.fa_ptr, *fa_src = &mp.fa_src;
-  st.h_sv_lev_ptr = mp.sv_lev_ptr;
   st.h_sn_ptr = sy.sn_ptr;
   st.h_row_ptr = sy.row_ptr;
   st.h_front_off = sy.front_off;
@@ -787,14 +787,19 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       const int64_t f = sy.row_ptr[J + 1] - sy.row_ptr[J], c = sy.sn_ptr[J + 1] - sy.sn_ptr[J];
       thin_leaf[J] = f > small_max && !has_child[J] && nthin[pid_of(J)] >= kThinCount && ldl_thin_front(f, c, small_max);
     }
-    const int rcs = thin_syrk_plan(ar, sy, mp, thin_leaf, st.f64, kThinCount, st.syrk, fal);
+    const int rcs = thin_syrk_plan(ar, sy, mp, thin_leaf, st.f64, kThinCount, st.syrk, fal, svl);
     if (rcs != CLR_OK) return rcs;
     if (!fal.lev_ptr.empty()) {
       fa_lev_ptr = &fal.lev_ptr;
       fa_tgt = &fal.tgt;
       fa_ptr = &fal.ptr;
       fa_src = &fal.src;
+      sv_lev_ptr = &svl.lev_ptr;
+      sv_tgt = &svl.tgt;
+      sv_ptr = &svl.ptr;
+      sv_src = &svl.src;
     }
+    st.h_sv_lev_ptr = *sv_lev_ptr;
     st.h_fa_lev_ptr = *fa_lev_ptr;
     std::vector<int64_t> small, leaf, thin, both, prod;
     for (int64_t l = 0; l < sy.nlev; ++l) {
@@ -810,13 +815,14 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
           small.push_back(J);
           st.lev_small_maxf[l] = std::max(st.lev_small_maxf[l], (int)f);
         } else if (nthin[pid_of(J)] >= kThinCount && ldl_thin_front(f, c, small_max)) {
-          (has_child[J] ? thin : (!st.syrk.child.empty() && st.syrk.child[J] ? prod : leaf)).push_back(J);
+          const bool in_product = !st.syrk.child.empty() && st.syrk.child[J];
+          (has_child[J] ? thin : (in_product ? prod : leaf)).push_back(J);
           st.lev_thin_smem[l] = std::max(st.lev_thin_smem[l], f * c);
         } else {
           st.lev_big[l].push_back(J);
           continue;
         }
-        both.push_back(J);
+        if (st.syrk.child.empty() || !st.syrk.child[J]) both.push_back(J);
       }
       add(st.lev_small, l, small);
       add(st.lev_thin_leaf, l, leaf);
@@ -824,7 +830,7 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       add(st.lev_thin, l, thin);
       add(st.lev_cta, l, both);
       longs(*fa_ptr, (*fa_lev_ptr)[l], (*fa_lev_ptr)[l + 1], kPullSerial, kFaWarp, st.fa_ord, st.fa_warp, st.fa_cta, l);
-      longs(mp.sv_ptr, mp.sv_lev_ptr[l], mp.sv_lev_ptr[l + 1], kSvThread, kPullSerial, st.sv_ord, st.sv_warp, st.sv_cta, l);
+      longs(*sv_ptr, (*sv_lev_ptr)[l], (*sv_lev_ptr)[l + 1], kSvThread, kPullSerial, st.sv_ord, st.sv_warp, st.sv_cta, l);
     }
     int64_t* dbuf = buf.empty() ? nullptr : ar.upload(buf.data(), (int64_t)buf.size());
     if (!buf.empty() && !dbuf) return CLR_E_OOM;
@@ -951,26 +957,26 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       // pull targets by front: they come level by level, front by front, in order
       std::vector<int64_t> sv0(sy.nsn, 0), sv1(sy.nsn, 0), cpull;
       for (int64_t l = 0; l < sy.nlev; ++l) {
-        int64_t t = mp.sv_lev_ptr[l];
+        int64_t t = (*sv_lev_ptr)[l];
         int64_t longest = 0;
         bool fused = true;
         for (int64_t k = sy.lev_ptr[l]; k < sy.lev_ptr[l + 1]; ++k) {
           const int64_t J = sy.lev_sn[k], f = sy.row_ptr[J + 1] - sy.row_ptr[J];
           sv0[J] = t;
-          while (t < mp.sv_lev_ptr[l + 1] && mp.sv_tgt[t] >= sy.upd_off[J] && mp.sv_tgt[t] < sy.upd_off[J] + f) {
-            longest = std::max(longest, mp.sv_ptr[t + 1] - mp.sv_ptr[t]);
+          while (t < (*sv_lev_ptr)[l + 1] && (*sv_tgt)[t] >= sy.upd_off[J] && (*sv_tgt)[t] < sy.upd_off[J] + f) {
+            longest = std::max(longest, (*sv_ptr)[t + 1] - (*sv_ptr)[t]);
             ++t;
           }
           sv1[J] = t;
           if (bid_of[J] >= 0 && bf_c[bid_of[J]] > kSweepPull) fused = false;
         }
-        if (t != mp.sv_lev_ptr[l + 1]) return CLR_E_INVALID;
-        st.lev_fused[l] = fused && longest <= kSvThread && mp.sv_lev_ptr[l + 1] < ((int64_t)1 << 31);
+        if (t != (*sv_lev_ptr)[l + 1]) return CLR_E_INVALID;
+        st.lev_fused[l] = fused && longest <= kSvThread && (*sv_lev_ptr)[l + 1] < ((int64_t)1 << 31);
       }
       for (int64_t l = 0; l < sy.nlev; ++l) {
         for (int64_t k = sy.lev_ptr[l]; k < sy.lev_ptr[l + 1]; ++k) {  // lev_cta's order
           const int64_t J = sy.lev_sn[k];
-          if (bid_of[J] >= 0) continue;
+          if (bid_of[J] >= 0 || (!st.syrk.child.empty() && st.syrk.child[J])) continue;
           cpull.push_back(sv0[J]);
           cpull.push_back(sv1[J]);
         }
@@ -997,7 +1003,7 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
           if (sw.fused) {
             e.pull = (int64_t)pptr.size();
             pptr.resize(pptr.size() + bf_f[b], -1);
-            for (int64_t t = sv0[J]; t < sv1[J]; ++t) pptr[e.pull + (mp.sv_tgt[t] - sy.upd_off[J])] = (int32_t)t;
+            for (int64_t t = sv0[J]; t < sv1[J]; ++t) pptr[e.pull + ((*sv_tgt)[t] - sy.upd_off[J])] = (int32_t)t;
           }
           fr.push_back(e);
         }
@@ -1136,9 +1142,9 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
   st.fa_tgt = up(ar, *fa_tgt);
   st.fa_ptr = up(ar, *fa_ptr);
   st.fa_src = up(ar, *fa_src);
-  st.sv_tgt = up(ar, mp.sv_tgt);
-  st.sv_ptr = up(ar, mp.sv_ptr);
-  st.sv_src = up(ar, mp.sv_src);
+  st.sv_tgt = up(ar, *sv_tgt);
+  st.sv_ptr = up(ar, *sv_ptr);
+  st.sv_src = up(ar, *sv_src);
   if (!st.sn_ptr || !st.row_ptr || !st.front_off || !st.upd_off || !st.lev_sn || !st.rows_kkt || !st.w_init ||
       !st.dsign || !st.pos_pid || !st.kdest || !st.diag_pos || !st.fa_tgt || !st.fa_ptr || !st.fa_src || !st.sv_tgt ||
       !st.sv_ptr || !st.sv_src)
@@ -1304,6 +1310,9 @@ int LdlFactor<T>::solve(cudaStream_t stm, const double* rhs, const int* skip) co
     if (!fused)
       pull_level<T>(stm, w, S.sv_tgt, S.sv_ptr, S.sv_src, S.h_sv_lev_ptr[l], S.h_sv_lev_ptr[l + 1], kSvThread,
                     S.sv_ord[l], S.sv_warp[l], S.sv_cta[l], skip);
+    if (!S.syrk.lev.empty())
+      ThinSyrkOps<T>::fwd_level(stm, S.syrk, l, F, syrk_w, syrk_part, w, S.sn_ptr, S.row_ptr, S.front_off, S.upd_off,
+                                skip);
     const LdlStructure::List& cl = S.lev_cta[l];
     if (cl.n > 0)
       CLR_CUDA(launch_pdl(k_fwd_front<T>, (unsigned)cl.n, 256, 0, stm, (const T*)F, w, cl.id, (const int64_t*)S.sn_ptr,
@@ -1326,6 +1335,10 @@ int LdlFactor<T>::solve(cudaStream_t stm, const double* rhs, const int* skip) co
       int rc = BigFrontOps<T>::sweep_bwd(stm, S.sweeps[l], E, ybuf, xs, S.rows_kkt, skip);
       if (rc) return rc;
     }
+    // (leaves: what they need is their parent's and its ancestors' solution)
+    if (!S.syrk.lev.empty())
+      ThinSyrkOps<T>::bwd_level(stm, S.syrk, l, F, Dp, w, xs, S.sn_ptr, S.row_ptr, S.front_off, S.upd_off, S.rows_kkt,
+                                skip);
   }
   CLR_CHECK_LAUNCH();
   return CLR_OK;

@@ -1,4 +1,4 @@
-// Extend-add of many thin leaf fronts into one parent, as one product.
+// Many thin leaf fronts of one parent: their extend-add as one product, their solves by columns.
 //
 // A parent with hundreds of thin leaves (a portfolio: one leaf per asset with its row of the
 // factor matrix) sums their update matrices l d l^T entry by entry: r^2 / 2 values written by every
@@ -12,6 +12,10 @@
 // Tiles of 64 x 64 of the lower triangle, 4 x 4 per thread, the columns in splits so that small
 // parents fill the SMs (about 608 CTAs: four per SM); partial tiles are added in the order of
 // the splits, which depend on the parent alone.
+//
+// Solves: w_P -= W^T y over the panel (coalesced, L2 resident) in place of a CTA per leaf and 5000
+// sources gathered per entry of w_P (13.5 + 11.4 us), and a warp per leaf for its columns' dot
+// products with the ancestors (a CTA of 256 threads with four barriers each took 24 us): 21 us together, launches included.
 #include "thinsyrk.cuh"
 
 #include <algorithm>
@@ -137,13 +141,120 @@ __global__ void __launch_bounds__(NT) k_add_tiles(T* __restrict__ F, ThinSyrkPar
   for (int64_t k = 0; k < p.splits; ++k) s += o[k * (TB * TB)];
   F[p.goff + r + c * p.fP] -= s;
 }
+
+// Leaves of several pivots: the unit lower solve of their diagonal block, a warp each (c <= 32).
+template <typename T>
+__global__ void __launch_bounds__(NT) k_leaf_fwd(const T* __restrict__ F, T* __restrict__ w, const int64_t* __restrict__ front,
+                                                 int64_t n, const int64_t* __restrict__ sn_ptr,
+                                                 const int64_t* __restrict__ row_ptr,
+                                                 const int64_t* __restrict__ front_off,
+                                                 const int64_t* __restrict__ upd_off, const int* skip) {
+  if (skip && *skip) return;
+  const int64_t t = (blockIdx.x * (int64_t)NT + threadIdx.x) / 32;
+  if (t >= n) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t J = front[t], f = row_ptr[J + 1] - row_ptr[J];
+  const int c = (int)(sn_ptr[J + 1] - sn_ptr[J]);
+  const T* G = F + front_off[J];
+  T x = lane < c ? w[upd_off[J] + lane] : (T)0;
+  for (int j = 0; j < c; ++j) {
+    const T xj = __shfl_sync(0xffffffffu, x, j);
+    if (lane > j && lane < c) x -= G[lane + j * f] * xj;
+  }
+  if (lane < c) w[upd_off[J] + lane] = x;
+}
+
+// Split blockIdx.y of w_P's product: rows 256 blockIdx.x .., a thread each.
+template <typename T>
+__global__ void __launch_bounds__(NT) k_panel_product(const T* __restrict__ Wall, const T* __restrict__ w, ThinSyrkParent p,
+                                                      const int64_t* __restrict__ slot, T* __restrict__ part,
+                                                      const int* skip) {
+  if (skip && *skip) return;
+  __shared__ T y[NT];
+  const int64_t i = blockIdx.x * (int64_t)NT + threadIdx.x;
+  const int64_t k0 = blockIdx.y * p.vc, k1 = min(p.K, k0 + p.vc);
+  const T* W = Wall + p.woff + min(i, p.ld - 1);
+  T a[4] = {(T)0, (T)0, (T)0, (T)0};
+  for (int64_t b = k0; b < k1; b += NT) {
+    const int m = (int)min((int64_t)NT, k1 - b);
+    __syncthreads();
+    if ((int)threadIdx.x < m) y[threadIdx.x] = w[slot[p.col0 + b + threadIdx.x]];
+    __syncthreads();
+    int k = 0;
+    for (; k + 8 <= m; k += 8) {
+      T x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = W[(b + k + u) * p.ld];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) a[u & 3] += x[u] * y[k + u];
+    }
+    for (; k < m; ++k) a[0] += W[(b + k) * p.ld] * y[k];
+  }
+  if (i < p.fP) part[blockIdx.y * p.fP + i] = (a[0] + a[1]) + (a[2] + a[3]);
+}
+template <typename T>
+__global__ void __launch_bounds__(NT) k_panel_add(T* __restrict__ w, ThinSyrkParent p, const T* __restrict__ part,
+                                                  const int* skip) {
+  if (skip && *skip) return;
+  // eight lanes per row: lane g adds the splits g, g + 8, ...
+  const int64_t i = (blockIdx.x * (int64_t)NT + threadIdx.x) / 8;
+  const int g = threadIdx.x & 7;
+  T s = (T)0;
+  if (i < p.fP)
+    for (int64_t k = g; k < p.vsplits; k += 8) s += part[k * p.fP + i];
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (g == 0 && i < p.fP) w[p.wslot + i] -= s;
+}
+
+// Backward sweep of a leaf by a warp: v = y / D - sum over the rows below of l x, then its diagonal block.
+template <typename T>
+__global__ void __launch_bounds__(NT) k_leaf_bwd(const T* __restrict__ F, const T* __restrict__ Dp,
+                                                 const T* __restrict__ w, T* __restrict__ xs,
+                                                 const int64_t* __restrict__ front, int64_t n,
+                                                 const int64_t* __restrict__ sn_ptr, const int64_t* __restrict__ row_ptr,
+                                                 const int64_t* __restrict__ front_off,
+                                                 const int64_t* __restrict__ upd_off,
+                                                 const int32_t* __restrict__ rows_kkt, const int* skip) {
+  if (skip && *skip) return;
+  const int64_t t = (blockIdx.x * (int64_t)NT + threadIdx.x) / 32;
+  if (t >= n) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t J = front[t];
+  const int c = (int)(sn_ptr[J + 1] - sn_ptr[J]), f = (int)(row_ptr[J + 1] - row_ptr[J]);
+  const T* G = F + front_off[J];
+  const int32_t* rk = rows_kkt + row_ptr[J];
+  T v = lane < c ? w[upd_off[J] + lane] / Dp[sn_ptr[J] + lane] : (T)0;
+  for (int k = c - 1; k >= 0; --k) {
+    const T* g = G + (int64_t)k * f;
+    T s[4] = {(T)0, (T)0, (T)0, (T)0};
+    for (int i0 = c; i0 < f; i0 += 128) {
+      T l[4], x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + 32 * u + lane;
+        l[u] = i < f ? g[i] : (T)0;
+        x[u] = i < f ? xs[rk[i]] : (T)0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s[u] += l[u] * x[u];
+    }
+    const T d = warp_sum((s[0] + s[1]) + (s[2] + s[3]));
+    if (lane == k) v -= d;
+  }
+  for (int k = c - 1; k >= 0; --k) {
+    const T xk = __shfl_sync(0xffffffffu, v, k);
+    if (lane < k) v -= G[k + (int64_t)lane * f] * xk;
+  }
+  if (lane < c) xs[rk[lane]] = v;
+}
 }  // namespace
 
 // The parents: at least min_children thin leaves, and the product's FMAs not more than `ratio` per
 // value of the update matrices that they replace.  A value costs 7.5 ps to gather (1.6e8 in 1.2 ms),
 // an FMA 0.07 ps in FP32 (half the FMA rate of 152 SMs) and 2.5 ps in FP64 (1.7 per clock and SM).
 int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<char>& leaf, bool f64,
-                   int64_t min_children, ThinSyrk& out, FaLists& fa) {
+                   int64_t min_children, ThinSyrk& out, FaLists& fa, FaLists& sv) {
   const int64_t ratio = f64 ? 2 : 64;
   out.lev.assign(sy.nlev, {});
   std::vector<char> pushed(sy.nsn, 0);
@@ -167,33 +278,47 @@ int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, c
   out.child.assign(sy.nsn, 0);
   std::vector<std::vector<int64_t>> kids(sy.nsn);
   for (int64_t J = 0; J < sy.nsn; ++J)
-    if (sy.sn_parent[J] >= 0 && take[sy.sn_parent[J]] && !pushed[J]) {
+    if (sy.sn_parent[J] >= 0 && take[sy.sn_parent[J]]) {
       kids[sy.sn_parent[J]].push_back(J);
-      out.child[J] = leaf[J];
+      out.child[J] = leaf[J] && !pushed[J];
     }
-  std::vector<int64_t> src, map0;
+  std::vector<int64_t> src, map0, slot, front;
   std::vector<int32_t> cnt, dpos, map, loc(sy.N, -1);
   std::vector<std::pair<int64_t, int64_t>> contrib;
-  fa = FaLists();
+  // the targets in [lo, hi) of level l, which follow one another from t on: copied to `o` or skipped
+  auto pass = [](const std::vector<int64_t>& tgt, const std::vector<int64_t>& ptr, const std::vector<int64_t>& s,
+                 int64_t& t, int64_t t1, int64_t lo, int64_t hi, bool keep, FaLists& o) {
+    for (; t < t1 && tgt[t] >= lo && tgt[t] < hi; ++t) {
+      if (!keep) continue;
+      o.tgt.push_back(tgt[t]);
+      o.ptr.push_back((int64_t)o.src.size());
+      o.src.insert(o.src.end(), s.begin() + ptr[t], s.begin() + ptr[t + 1]);
+    }
+  };
+  auto lists = [&](FaLists& o) {
+    std::stable_sort(contrib.begin(), contrib.end(), [](auto& a, auto& b) { return a.first < b.first; });
+    for (size_t k = 0; k < contrib.size(); ++k) {
+      if (k == 0 || contrib[k].first != contrib[k - 1].first) {
+        o.tgt.push_back(contrib[k].first);
+        o.ptr.push_back((int64_t)o.src.size());
+      }
+      o.src.push_back(contrib[k].second);
+    }
+    contrib.clear();
+  };
+  fa = sv = FaLists();
   fa.lev_ptr.assign(1, 0);
+  sv.lev_ptr.assign(1, 0);
   for (int64_t l = 0; l < sy.nlev; ++l) {
+    int64_t ts = mp.sv_lev_ptr[l];
+    const int64_t ts1 = mp.sv_lev_ptr[l + 1];
     int64_t t = mp.fa_lev_ptr[l];
     const int64_t t1 = mp.fa_lev_ptr[l + 1];
     for (int64_t x = sy.lev_ptr[l]; x < sy.lev_ptr[l + 1]; ++x) {
-      const int64_t P = sy.lev_sn[x], fP = rows(P), end = sy.front_off[P] + fP * fP;
-      // this front's targets follow one another in the level
-      int64_t u = t;
-      while (u < t1 && mp.fa_tgt[u] >= sy.front_off[P] && mp.fa_tgt[u] < end) ++u;
-      if (!take[P]) {
-        for (int64_t k = t; k < u; ++k) {
-          fa.tgt.push_back(mp.fa_tgt[k]);
-          fa.ptr.push_back((int64_t)fa.src.size());
-          fa.src.insert(fa.src.end(), mp.fa_src.begin() + mp.fa_ptr[k], mp.fa_src.begin() + mp.fa_ptr[k + 1]);
-        }
-        t = u;
-        continue;
-      }
-      t = u;
+      const int64_t P = sy.lev_sn[x], fP = rows(P);
+      pass(mp.fa_tgt, mp.fa_ptr, mp.fa_src, t, t1, sy.front_off[P], sy.front_off[P] + fP * fP, !take[P], fa);
+      pass(mp.sv_tgt, mp.sv_ptr, mp.sv_src, ts, ts1, sy.upd_off[P], sy.upd_off[P] + fP, !take[P], sv);
+      if (!take[P]) continue;
       const int64_t* rP = sy.rows.data() + sy.row_ptr[P];
       for (int64_t a = 0; a < fP; ++a) loc[rP[a]] = (int32_t)a;
       ThinSyrkParent p{};
@@ -203,11 +328,13 @@ int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, c
       p.K = cols[P];
       p.col0 = (int64_t)src.size();
       p.woff = out.wtotal;
-      contrib.clear();
+      p.wslot = sy.upd_off[P];
+      p.front0 = (int64_t)front.size();
       for (int64_t J : kids[P]) {
         const int64_t f = rows(J), c = pivots(J);
         const int64_t* r = sy.rows.data() + sy.row_ptr[J];
-        if (!leaf[J]) {  // stays with the lists
+        if (pushed[J]) continue;
+        if (!out.child[J]) {  // stays with the lists
           for (int64_t b = c; b < f; ++b)
             for (int64_t a = b; a < f; ++a)
               contrib.emplace_back(p.goff + loc[r[a]] + loc[r[b]] * fP, sy.front_off[J] + a + b * f);
@@ -218,17 +345,24 @@ int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, c
           map0.push_back((int64_t)map.size());
           cnt.push_back((int32_t)(f - c));
           dpos.push_back((int32_t)(sy.sn_ptr[J] + b));
+          slot.push_back(sy.upd_off[J] + b);
         }
+        front.push_back(J);
+        p.many |= c > 1;
         for (int64_t a = c; a < f; ++a) map.push_back(loc[r[a]]);
       }
-      std::stable_sort(contrib.begin(), contrib.end(), [](auto& a, auto& b) { return a.first < b.first; });
-      for (size_t k = 0; k < contrib.size(); ++k) {
-        if (k == 0 || contrib[k].first != contrib[k - 1].first) {
-          fa.tgt.push_back(contrib[k].first);
-          fa.ptr.push_back((int64_t)fa.src.size());
-        }
-        fa.src.push_back(contrib[k].second);
+      lists(fa);
+      for (int64_t J : kids[P]) {
+        if (out.child[J]) continue;
+        const int64_t* r = sy.rows.data() + sy.row_ptr[J];
+        for (int64_t a = pivots(J); a < rows(J); ++a)
+          contrib.emplace_back(sy.upd_off[P] + loc[r[a]], sy.upd_off[J] + a);
       }
+      lists(sv);
+      p.nfront = (int64_t)front.size() - p.front0;
+      p.vc = std::max<int64_t>(32, (p.K * ((fP + NT - 1) / NT) + kCtas - 1) / kCtas);
+      p.vsplits = (p.K + p.vc - 1) / p.vc;
+      out.part = std::max(out.part, p.vsplits * fP);
       const int64_t nt = p.ld / TB;
       p.tiles = nt * (nt + 1) / 2;
       p.splits = std::max<int64_t>(1, std::min((kCtas + p.tiles - 1) / p.tiles, p.K / 64));
@@ -239,8 +373,10 @@ int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, c
       out.lev[l].push_back(p);
     }
     fa.lev_ptr.push_back((int64_t)fa.tgt.size());
+    sv.lev_ptr.push_back((int64_t)sv.tgt.size());
   }
   fa.ptr.push_back((int64_t)fa.src.size());
+  sv.ptr.push_back((int64_t)sv.src.size());
   // what a factorization clears
   std::vector<std::pair<int64_t, int64_t>> used;
   for (int64_t J = 0; J < sy.nsn; ++J)
@@ -263,7 +399,9 @@ int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, c
   out.cnt = ar.upload(cnt.data(), (int64_t)cnt.size());
   out.dpos = ar.upload(dpos.data(), (int64_t)dpos.size());
   out.map = ar.upload(map.data(), (int64_t)map.size());
-  return out.seg && out.src && out.map0 && out.cnt && out.dpos && out.map ? CLR_OK : CLR_E_OOM;
+  out.slot = ar.upload(slot.data(), (int64_t)slot.size());
+  out.front = ar.upload(front.data(), (int64_t)front.size());
+  return out.seg && out.src && out.map0 && out.cnt && out.dpos && out.map && out.slot && out.front ? CLR_OK : CLR_E_OOM;
 }
 
 template <typename T>
@@ -281,6 +419,29 @@ void ThinSyrkOps<T>::add_level(cudaStream_t st, const ThinSyrk& ts, int64_t l, T
     if (p.splits > 1)
       k_add_tiles<T><<<(unsigned)(p.tiles * (TB * TB / NT)), NT, 0, st>>>(F, p, part, skip);
   }
+}
+
+template <typename T>
+void ThinSyrkOps<T>::fwd_level(cudaStream_t st, const ThinSyrk& ts, int64_t l, const T* F, const T* W, T* part, T* w,
+                               const int64_t* sn_ptr, const int64_t* row_ptr, const int64_t* front_off,
+                               const int64_t* upd_off, const int* skip) {
+  for (const ThinSyrkParent& p : ts.lev[l]) {
+    if (p.many)
+      k_leaf_fwd<T><<<(unsigned)((p.nfront * 32 + NT - 1) / NT), NT, 0, st>>>(F, w, ts.front + p.front0, p.nfront, sn_ptr,
+                                                                              row_ptr, front_off, upd_off, skip);
+    k_panel_product<T><<<dim3((unsigned)((p.fP + NT - 1) / NT), (unsigned)p.vsplits), NT, 0, st>>>(W, w, p, ts.slot, part,
+                                                                                                  skip);
+    k_panel_add<T><<<(unsigned)((p.fP * 8 + NT - 1) / NT), NT, 0, st>>>(w, p, part, skip);
+  }
+}
+
+template <typename T>
+void ThinSyrkOps<T>::bwd_level(cudaStream_t st, const ThinSyrk& ts, int64_t l, const T* F, const T* Dp, const T* w, T* xs,
+                               const int64_t* sn_ptr, const int64_t* row_ptr, const int64_t* front_off,
+                               const int64_t* upd_off, const int32_t* rows_kkt, const int* skip) {
+  for (const ThinSyrkParent& p : ts.lev[l])
+    k_leaf_bwd<T><<<(unsigned)((p.nfront * 32 + NT - 1) / NT), NT, 0, st>>>(
+        F, Dp, w, xs, ts.front + p.front0, p.nfront, sn_ptr, row_ptr, front_off, upd_off, rows_kkt, skip);
 }
 
 template struct ThinSyrkOps<float>;

@@ -1,4 +1,4 @@
-// Extend-add of many thin leaf fronts into one parent as a product (thinsyrk.cu).
+// Many thin leaf fronts of one parent: extend-add as a product, solves by their columns (thinsyrk.cu).
 #pragma once
 
 #include <cstdint>
@@ -13,6 +13,10 @@ struct ThinSyrkParent {
   int64_t goff, fP, ld;     // the parent's front in the pool, its rows; row length of its panel W
   int64_t K, col0, woff;    // columns of its thin leaves, the first one in the column arrays, W's offset
   int64_t tiles, splits, kc;
+  int64_t wslot;            // the parent's work vector
+  int64_t front0, nfront;   // its leaves in `front`
+  int64_t vsplits, vc;      // columns per split of the solve's product
+  int32_t many;             // a leaf has several pivots
 };
 
 struct ThinSyrk {
@@ -22,6 +26,7 @@ struct ThinSyrk {
   // rows (first one in map), its pivot
   int64_t *src = nullptr, *map0 = nullptr;
   int32_t *cnt = nullptr, *dpos = nullptr, *map = nullptr;
+  int64_t *slot = nullptr, *front = nullptr;     // per column: its pivot's place in the work vector; the leaves
   // parts of the pool that a factorization clears (offset, length <= kSegment): without the update
   // matrices that are not kept
   int64_t* seg = nullptr;
@@ -29,15 +34,15 @@ struct ThinSyrk {
   int64_t wtotal = 0, part = 0;                  // entries of all panels W; of the largest parent's partial tiles
 };
 
-// The extend-add lists of a structure (NumericMaps' fa_*), without what the products cover.
+// The extend-add or solve lists of a structure (NumericMaps' fa_*, sv_*), without what the products cover.
 struct FaLists {
   std::vector<int64_t> lev_ptr, tgt, ptr, src;
 };
 
 // leaf: thin leaf fronts (ldl_thin_front, the path taken).  Chooses the parents, fills out and, if
-// any was chosen, fa.
+// any was chosen, fa and sv.
 int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<char>& leaf, bool f64,
-                   int64_t min_children, ThinSyrk& out, FaLists& fa);
+                   int64_t min_children, ThinSyrk& out, FaLists& fa, FaLists& sv);
 
 template <typename T>
 struct ThinSyrkOps {
@@ -45,5 +50,13 @@ struct ThinSyrkOps {
   // F_P -= sum over the leaves' columns of l d l^T, for the parents of level l
   static void add_level(cudaStream_t st, const ThinSyrk& ts, int64_t l, T* F, const T* Dp, T* W, T* part,
                         const int* skip);
+  // the leaves' forward sweep for the parents of level l: w_P -= sum over their columns of l y
+  static void fwd_level(cudaStream_t st, const ThinSyrk& ts, int64_t l, const T* F, const T* W, T* part, T* w,
+                        const int64_t* sn_ptr, const int64_t* row_ptr, const int64_t* front_off,
+                        const int64_t* upd_off, const int* skip);
+  // and their backward sweep, after the parents'
+  static void bwd_level(cudaStream_t st, const ThinSyrk& ts, int64_t l, const T* F, const T* Dp, const T* w, T* xs,
+                        const int64_t* sn_ptr, const int64_t* row_ptr, const int64_t* front_off,
+                        const int64_t* upd_off, const int32_t* rows_kkt, const int* skip);
 };
 }  // namespace clr

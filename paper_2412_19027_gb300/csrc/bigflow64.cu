@@ -32,8 +32,8 @@
 //   U: F_IJ -= PA(p, i) PB(p, j)^T;  EU: E_IC -= PA(p, i) PE(p, e)^T;
 //   T: L_IK = (F_IK 2^-g) PT(p)^T D^{-1};  Efin: E_KC^T <- (E_KC^T 2^-g) PT(p)^T,
 // with F_IK and E_KC^T split in the task.  One CTA per SM (512 columns of tensor memory).
-// Per task on a GB300 (front of 2052 rows; FMA version in brackets): D 70 us (95), T 24 (41), Efin 18
-// (57), U 11 (57), EU 11 (57); the front: 3.9 ms.
+// Per task on a GB300 (front of 2052 rows; FMA version in brackets): D 64 us (95), T 24 (41), Efin 18
+// (57), U 11 (57), EU 11 (57); the front: 3.7 ms.
 #include <algorithm>
 
 #include "bfdiag.cuh"
@@ -535,7 +535,7 @@ __device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A,
 // the sign and the products with 16 terms (the trailing updates, and the off-diagonal blocks of
 // L^{-1}) are integer arithmetic, the products exact (operands scaled like the packs).  Warps 4-7
 // form L^{-1} a block row behind the panels, and the part of the trailing update that
-// the next panel does not read.  70 us with the packs.
+// the next panel does not read.  64 us with the packs: panels 12 us each, the last row of L^{-1} 5.5.
 __device__ int diag64(const double* G, int64_t f, int pw, double* D, const int8_t* dsign, double eps, double delta,
                       double* scr, Diag64Smem& sa, Diag64SmemB& sb, DiagScratch<double>& sh, int* gs, int* hs) {
   constexpr int LD = kDiagLD;

@@ -136,6 +136,11 @@ class DeviceArena {
                                  : cudaMemcpy(d, h, sizeof(T) * (size_t)n, cudaMemcpyHostToDevice);
     return e == cudaSuccess ? d : nullptr;
   }
+  // zeros, ordered like an upload
+  bool clear(void* d, size_t n) {
+    if (async_) return cudaMemsetAsync(d, 0, n, async_) == cudaSuccess;
+    return cudaMemset(d, 0, n) == cudaSuccess && cudaStreamSynchronize(nullptr) == cudaSuccess;
+  }
   void release();
   size_t bytes() const { return total_; }
   // Stream-ordered mode: allocations and frees go through cudaMallocAsync /

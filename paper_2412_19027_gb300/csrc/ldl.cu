@@ -1169,9 +1169,7 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
     syrk_w = ar.alloc_n<T>(st.syrk.wtotal);
     syrk_part = ar.alloc_n<T>(std::max<int64_t>(1, st.syrk.part));
     if (!syrk_w || !syrk_part) return CLR_E_OOM;
-    if (cudaMemset(syrk_w, 0, sizeof(T) * (size_t)st.syrk.wtotal) != cudaSuccess ||
-        cudaStreamSynchronize(nullptr) != cudaSuccess)
-      return CLR_E_CUDA;
+    if (!ar.clear(syrk_w, sizeof(T) * (size_t)st.syrk.wtotal)) return CLR_E_CUDA;
   }
   if (BigFrontOps<T>::setup_attributes() != CLR_OK) return CLR_E_CUDA;
   if (st.cta.n > 0 && CtaOps<T>::setup_attributes() != CLR_OK) return CLR_E_CUDA;

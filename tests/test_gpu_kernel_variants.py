@@ -275,3 +275,26 @@ def test_k_products_by_row_length(bits, n):
     assert a[3]["iterations"] == b[3]["iterations"] and a[3]["ir_steps_total"] == b[3]["ir_steps_total"]
     one.free()
     both.free()
+
+
+# the panels of thin leaves in solvers built while others run (stream-ordered memory, reused from one
+# solver to the next): the server's results are those of a solver built alone
+@pytest.mark.parametrize("bits", [64, 32])
+def test_thin_leaf_panels_in_server(bits):
+    from paper_2412_19027_gb300 import workloads as W
+    st = clr.clr_default_settings(bits, max_iter=40)
+    arg = lambda p: (p.P, p.q, p.A, p.b, p.cones)
+    probs = [W.portfolio_qp(k, n=1500 + 700 * k, density=1.0) for k in (0, 1, 0, 1)]
+    sv = clr.Server(device_bytes=8 << 30, max_cohort=1, max_active=2, settings=st)
+    reqs = [clr.Request(*arg(p)) for p in probs]
+    tickets = [sv.submit(r) for r in reqs]
+    got = [sv.wait(t, 120.0) for t in tickets]
+    sv.close()
+    for p, g in zip(probs, got):
+        s = clr.clr_setup(*arg(p), st)
+        s.solve()
+        want = s.solution()
+        for u, v in zip(want[:3], g[:3]):
+            np.testing.assert_array_equal(u, v)
+        assert want[3]["iterations"] == g[3]["iterations"]
+        s.free()

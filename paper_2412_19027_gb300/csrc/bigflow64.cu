@@ -14,21 +14,28 @@
 //   - the products of digit matrices s and t of equal s + t <= 7 are summed in one FP32
 //     accumulator in tensor memory: at most 4 products of 64 terms up to 2^14, so every
 //     partial sum is an integer up to 2^22, exact in FP32;
-//   - the eight sums G_0 .. G_7 give (X Y) / 2^54 as a 64-bit integer (the digit products with
-//     s + t >= 8 are below 2^-64 of the row maxima), which is normalised to a double in
-//     integer arithmetic; one FP64 addition per entry remains.
+//   - the eight sums G_0 .. G_7 give (X Y) / 2^54 as a 64-bit integer, which is normalised to a
+//     double in integer arithmetic; one FP64 addition per entry remains.  Left out are the digit
+//     products with s + t >= 8: five of s + t = 8, at most 2^-55.7 of the product of the row maxima
+//     over 64 terms.
 // Before splitting, the shared index k is scaled by a power of two on one side and its inverse
-// on the other so that both operands are rows of sqrt(D)-scaled factors: |entry| <=
-// sqrt(F_ii) like the rows of a Cholesky factor, and the rounding of the digits (2^-55 of the
-// row maximum, about an eighth of what 64 rounded FMAs leave) is small against
-// sqrt(F_ii F_jj), the error bound of the factorization itself.  A row with an entry that is
-// not finite gives NaN in its results.
+// on the other, so that an operand's row is one of L |D|^(1/2), or, where an inverse L^{-1} of a
+// diagonal block is the other operand, so that no column of D^{-1/2} L^{-1} stands out.  The rounding
+// of a product is then 2^-55 of (largest entry of row i of L |D|^(1/2)) times (the sum over row j),
+// and the same with i and j exchanged: the size of n u |L| |D| |L|^T, the error of any LDL^T, for
+// rows whose large entries meet in the same columns.  Entries of one row of L |D|^(1/2) that span many
+// decades (a row beside a pivot that has stayed at its regularisation) lose against FMAs: LP systems
+// with P = 0 and a scaling over 12 decades, variables and rows mixed in the order, have residuals of
+// an unrefined solve 2.7 times those of FMA products; over 4 decades, with equality rows regularised
+// by 1e-8, or with more rows than variables, 0.7 to 1.1 times.  (Scaled by the diagonal as it was
+// before elimination in the place of g below, these four were 35, 0.7, 23 and 3 times.)  A row with
+// an entry that is not finite gives NaN in its results.
 //
 // Tasks and waits are those of bigflow.cu without the fused or split chain task: D(p), T(p, i),
 // Efin(p, e), U(p, i, j), EU(p, i, e).  Producers store their tile also as digits ("packs",
 // 56 KB in the MMA's layout, copied to shared memory by cp.async.bulk):
 //   PA(p, i) = L_IK 2^h, PB(p, i) = (L_IK D_K) 2^-h (h_k = half the exponent of d_k),
-//   PE(p, e) = E_KC^T 2^-h, PT(p) = Linv 2^g (g_l = half the exponent of F_ll), so that
+//   PE(p, e) = E_KC^T 2^-h, PT(p) = Linv 2^g (g_l = minus the exponent of column l of D^{-1/2} Linv), so that
 //   U: F_IJ -= PA(p, i) PB(p, j)^T;  EU: E_IC -= PA(p, i) PE(p, e)^T;
 //   T: L_IK = (F_IK 2^-g) PT(p)^T D^{-1};  Efin: E_KC^T <- (E_KC^T 2^-g) PT(p)^T,
 // with F_IK and E_KC^T split in the task.  One CTA per SM (512 columns of tensor memory).
@@ -306,7 +313,7 @@ struct Diag64Smem {
   int2 iq[16 * kLP];       // Linv_QQ 2^g by rows, exponents eq
   int2 ix[48 * kLP];       // X 2^-g by columns, exponents ex
   double cb[8 * 64];       // pivot columns: four of this group of columns, four of the last
-  int ea[4 * 64], eq[16], ex[48], xm[2 * 64];
+  int ea[4 * 64], eq[16], ex[48], xm[2 * 64], gq[4 * 16];
 };
 struct Diag64SmemB {
   int2 ib[2 * 64 * kLP];   // (L d) 2^-h of a panel by rows, exponents eb[row], for two panels
@@ -316,6 +323,9 @@ struct Diag64SmemB {
 };
 static_assert(sizeof(Diag64Smem) <= kPackBytes && sizeof(Diag64SmemB) <= kPackBytes, "scratch");
 __device__ __forceinline__ int row_exp(int m) { return m >= kBad ? kBad : (m <= -kBad ? 0 : m + 1); }
+// g of a column of an inverse whose largest entry, row k scaled by 2^-h_k, has exponent m: the column times
+// 2^g is of order one beside the others, in every row that sums over it
+__device__ __forceinline__ int block_scale(int m) { return m <= -kBad || m >= kBad ? 0 : -m; }
 __device__ __forceinline__ int shifted(double x, int sh) {
   const int l = ilog_of(x);
   return l >= kBad ? kBad : (l <= -kBad ? -kBad : l + sh);
@@ -430,7 +440,7 @@ __device__ __noinline__ void diag64_update(int q, int I, int J, int idx, double*
 // Block row Q of L^{-1}, by the 128 threads of warps 4-7 (tid 0 .. 127 here, barrier 3): the inverse of
 // L_QQ, Linv_QP = -Linv_QQ X_P, its operands (Q < 3), and X of block row Q + 1.
 __device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A, double* V, Diag64Smem& sa,
-                                                   Diag64SmemB& sb, const int* gs, const int* hs) {
+                                                   Diag64SmemB& sb, const int* hs) {
   constexpr int LD = kDiagLD;
   const int R0 = 16 * Q;
   auto bar = [] { asm volatile("barrier.sync 3, 128;" ::: "memory"); };
@@ -465,28 +475,46 @@ __device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A,
   if (tid < 64) V[(R0 + 8 + (tid >> 3)) * LD + R0 + (tid & 7)] = b1;
   if (Q > 0) {
     bar();
-    // rows of Linv_QQ (8 threads a row), columns of X (2 threads a column)
+    // rows of Linv_QQ (8 threads a row), columns of X (2 threads a column); g of a column of Linv_QQ: see
+    // block_scale
+    const int a0 = tid >> 3, c0 = 2 * (tid & 7);
+    const double x0 = V[(R0 + a0) * LD + R0 + c0], x1 = V[(R0 + a0) * LD + R0 + c0 + 1];
     {
-      const int a = tid >> 3, k0 = 2 * (tid & 7);
-      const double x0 = V[(R0 + a) * LD + R0 + k0], x1 = V[(R0 + a) * LD + R0 + k0 + 1];
-      int m = max(shifted(x0, gs[R0 + k0]), shifted(x1, gs[R0 + k0 + 1]));
+      int m0 = shifted(x0, -hs[R0 + a0]), m1 = shifted(x1, -hs[R0 + a0]);
+#pragma unroll
+      for (int o = 8; o < 32; o <<= 1) {
+        m0 = max(m0, __shfl_xor_sync(~0u, m0, o));
+        m1 = max(m1, __shfl_xor_sync(~0u, m1, o));
+      }
+      if ((tid & 31) < 8) {
+        sa.gq[16 * (tid >> 5) + c0] = m0;
+        sa.gq[16 * (tid >> 5) + c0 + 1] = m1;
+      }
+    }
+    bar();
+    auto g_of = [&](int k) {
+      return block_scale(max(max(sa.gq[k], sa.gq[16 + k]), max(sa.gq[32 + k], sa.gq[48 + k])));
+    };
+    {
+      const int g0 = g_of(c0), g1 = g_of(c0 + 1);
+      int m = max(shifted(x0, g0), shifted(x1, g1));
 #pragma unroll
       for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(~0u, m, o));
       const int e = row_exp(m);
-      if (k0 == 0) sa.eq[a] = e;
-      sa.iq[a * kLP + k0] = halves_of(x0, gs[R0 + k0], e);
-      sa.iq[a * kLP + k0 + 1] = halves_of(x1, gs[R0 + k0 + 1], e);
+      if (c0 == 0) sa.eq[a0] = e;
+      sa.iq[a0 * kLP + c0] = halves_of(x0, g0, e);
+      sa.iq[a0 * kLP + c0 + 1] = halves_of(x1, g1, e);
     }
     if (tid < 2 * R0) {
       const int b = tid >> 1, k0 = 8 * (tid & 1);
       int m = -kBad;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) m = max(m, shifted(sb.x[(k0 + k) * 49 + b], -gs[R0 + k0 + k]));
+      for (int k = 0; k < 8; ++k) m = max(m, shifted(sb.x[(k0 + k) * 49 + b], -g_of(k0 + k)));
       m = max(m, __shfl_xor_sync(~0u, m, 1));
       const int e = row_exp(m);
       if (k0 == 0) sa.ex[b] = e;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) sa.ix[b * kLP + k0 + k] = halves_of(sb.x[(k0 + k) * 49 + b], -gs[R0 + k0 + k], e);
+      for (int k = 0; k < 8; ++k) sa.ix[b * kLP + k0 + k] = halves_of(sb.x[(k0 + k) * 49 + b], -g_of(k0 + k), e);
     }
     bar();
     for (int idx = tid; idx < 16 * R0; idx += 128) {
@@ -551,10 +579,6 @@ __device__ int diag64(const double* G, int64_t f, int pw, double* D, const int8_
     else if (i == j) v = 1.0;  // rows and pivots past pw: the identity
     A[i * LD + j] = v;
     V[i * LD + j] = 0.0;
-    if (i == j) {  // g: half the exponent of the diagonal
-      const int lg = i < pw ? ilog_of(v) : 0;
-      gs[i] = lg <= -kBad || lg >= kBad ? 0 : lg >> 1;
-    }
   }
   const double rdelta = 1.0 / delta;
   __syncthreads();
@@ -569,14 +593,23 @@ __device__ int diag64(const double* G, int64_t f, int pw, double* D, const int8_
           diag64_update(q - 1, I, J, tid - 128, A, sa, sb);
           diag64_update(q - 1, I, J, tid, A, sa, sb);
         }
-      diag64_inverse_row(q - 1, tid - 128, A, V, sa, sb, gs, hs);
+      diag64_inverse_row(q - 1, tid - 128, A, V, sa, sb, hs);
     }
     __syncthreads();
     for (int I = q + 1; I < 4; ++I) diag64_update(q, I, q + 1, tid, A, sa, sb);
     __syncthreads();
   }
-  if (wid >= 4) diag64_inverse_row(3, tid - 128, A, V, sa, sb, gs, hs);
+  if (wid >= 4) diag64_inverse_row(3, tid - 128, A, V, sa, sb, hs);
   __syncthreads();
+  {  // g of the columns of L^{-1}, four threads each
+    const int l = tid >> 2, k0 = 16 * (tid & 3);
+    int m = -kBad;
+#pragma unroll 4
+    for (int k = k0; k < k0 + 16; ++k) m = max(m, shifted(V[k * LD + l], -hs[k]));
+    m = max(m, __shfl_xor_sync(~0u, m, 1));
+    m = max(m, __shfl_xor_sync(~0u, m, 2));
+    if (k0 == 0) gs[l] = block_scale(m);
+  }
   for (int i = tid; i < pw; i += NT) D[i] = sh.dv[i];
   return nhit;
 }

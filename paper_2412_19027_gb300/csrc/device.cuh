@@ -123,7 +123,13 @@ inline int grid_for(int64_t n, int threads, int cap = 8 * kSMs) {
 class DeviceArena {
  public:
   ~DeviceArena() { release(); }
-  void* alloc(size_t bytes);
+  void* alloc(size_t bytes) {
+    void* p = alloc_spare(bytes);
+    failures_ += p ? 0 : 1;
+    return p;
+  }
+  // Memory that the owner can do without: null when there is no room, not counted as a failure.
+  void* alloc_spare(size_t bytes);
   template <typename T>
   T* alloc_n(int64_t n) {
     return static_cast<T*>(alloc(sizeof(T) * (size_t)(n > 0 ? n : 1)));
@@ -134,8 +140,13 @@ class DeviceArena {
     if (!d || n <= 0) return d;
     const cudaError_t e = async_ ? cudaMemcpyAsync(d, h, sizeof(T) * (size_t)n, cudaMemcpyHostToDevice, async_)
                                  : cudaMemcpy(d, h, sizeof(T) * (size_t)n, cudaMemcpyHostToDevice);
-    return e == cudaSuccess ? d : nullptr;
+    if (e == cudaSuccess) return d;
+    ++failures_;
+    return nullptr;
   }
+  // Allocations and uploads that failed so far: whoever builds on the arena compares the count before
+  // and after, so that no null pointer among dozens of buffers reaches a kernel.
+  int64_t failures() const { return failures_; }
   // zeros, ordered like an upload
   bool clear(void* d, size_t n) {
     if (async_) return cudaMemsetAsync(d, 0, n, async_) == cudaSuccess;
@@ -156,6 +167,7 @@ class DeviceArena {
   };
   Block* blocks_ = nullptr;
   size_t nblocks_ = 0, cap_ = 0, total_ = 0;
+  int64_t failures_ = 0;
   cudaStream_t async_ = nullptr;
 };
 

@@ -798,7 +798,7 @@ void set_cuda_error(cudaError_t e, const char* where) {
   if (g_cuda_err.empty()) g_cuda_err = std::string(cudaGetErrorString(e)) + " at " + where;
 }
 
-void* DeviceArena::alloc(size_t bytes) {
+void* DeviceArena::alloc_spare(size_t bytes) {
   void* p = nullptr;
   bytes = (bytes + 255) & ~(size_t)255;
   if (g_alloc.a) p = g_alloc.a(bytes, g_alloc.ctx);
@@ -807,7 +807,10 @@ void* DeviceArena::alloc(size_t bytes) {
   } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
     p = nullptr;
   }
-  if (!p) return nullptr;
+  if (!p) {
+    cudaGetLastError();  // the caller reports it, not the next launch's check
+    return nullptr;
+  }
   if (nblocks_ == cap_) {
     size_t nc = cap_ ? 2 * cap_ : 64;
     Block* nb = new Block[nc];
@@ -949,6 +952,7 @@ int Solver::analyze_cohort(std::vector<HostProblem>&& ps, const std::vector<std:
 
 int Solver::upload() {
   const double t0 = now_s();
+  const int64_t failed = ar_.failures();
   const int64_t n = hp.n, m = hp.m, N = n + m, B = lay.B;
   if (!stream_) {
     CLR_CUDA(cudaStreamCreateWithFlags(&stream_, cudaStreamNonBlocking));
@@ -1174,9 +1178,7 @@ int Solver::upload() {
   }
   cd_.ep_zt = ar_.alloc_n<double>(3 * (cd_.n_exp + cd_.n_pow));
   exp_central_point_host(cd_.exp_center);
-  if (!v_.kptr || !v_.kcol || !v_.kvi || !v_.kval || !v_.xz || !v_.part || !sc_ || !bf_ || !cd_.scratch || !v_.ck ||
-      !v_.pid || !v_.pc || !v_.hist || !v_.maxb)
-    return CLR_E_OOM;
+  if (ar_.failures() != failed) return CLR_E_OOM;
   CLR_CUDA(cudaStreamSynchronize(stream_));
   device_ready = true;
   setup_s += now_s() - t0;

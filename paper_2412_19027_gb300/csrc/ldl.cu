@@ -684,6 +684,7 @@ static int flow64_tables(DeviceArena& ar, LdlStructure& st, bool emu) {
 
 int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<int8_t>& dsign,
                          int small_max, LdlStructure& st, const std::vector<int32_t>* pos_pid) {
+  const int64_t failed = ar.failures();
   st.N = sy.N;
   st.nsn = sy.nsn;
   st.nlev = sy.nlev;
@@ -1149,7 +1150,8 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       !st.dsign || !st.pos_pid || !st.kdest || !st.diag_pos || !st.fa_tgt || !st.fa_ptr || !st.fa_src || !st.sv_tgt ||
       !st.sv_ptr || !st.sv_src)
     return CLR_E_OOM;
-  return cta_plan_build(ar, sy, mp, small_max, pos_pid, st.w_init, st.cta);
+  const int rc = cta_plan_build(ar, sy, mp, small_max, pos_pid, st.w_init, st.cta);
+  return rc == CLR_OK && ar.failures() != failed ? CLR_E_OOM : rc;
 }
 
 template <typename T>
@@ -1192,9 +1194,8 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
       // (not more than half of what is free: what is allocated after this had that room before)
       size_t room = 0, all = 0;
       if (cudaMemGetInfo(&room, &all) == cudaSuccess && (size_t)(st.pk64_tiles * kPack64Bytes) <= room / 2)
-        pk64 = ar.alloc_n<unsigned char>(st.pk64_tiles * kPack64Bytes);
+        pk64 = static_cast<unsigned char*>(ar.alloc_spare((size_t)(st.pk64_tiles * kPack64Bytes)));
       if (!pk64) {  // no room for the packs: FMA products on every front
-        cudaGetLastError();
         LdlStructure& ms = const_cast<LdlStructure&>(st);
         ms.flow_emu = false;
         const int rc = flow64_tables(ar, ms, false);

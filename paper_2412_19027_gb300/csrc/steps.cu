@@ -125,8 +125,8 @@ struct ConeBench {
     cd.row_pid = ar.upload(pid.data(), m);
     cd.pc = ar.upload(&pc, 1);
     sc = ar.alloc_n<IterScal>(1);
-    if (cones_init_shadow(nullptr, cd, nullptr) != CLR_OK) rc = CLR_E_CUDA;
-    if (!cd.kvz || !cd.scratch || !cd.soc_wb || !cd.row_pid || !cd.pc || !sc) rc = CLR_E_OOM;
+    if (ar.failures() > 0) rc = CLR_E_OOM;
+    else if (cones_init_shadow(nullptr, cd, nullptr) != CLR_OK) rc = CLR_E_CUDA;
   }
 
   double* upload_perm(const double* v) {

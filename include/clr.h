@@ -412,6 +412,20 @@ int clr_server_destroy(clr_server* sv);
 /* Device timing and launch count of the last clr_solve (CLR_E_STATE before it). */
 int clr_get_perf(const clr_solver* s, clr_perf* out);
 
+/* Which of the kernels chosen by size the factor in use takes (after an
+ * escalation the FP64 one); counts over the whole cohort. */
+typedef struct {
+  int64_t one_cta;         /* 1: refined KKT solves by one CTA per problem */
+  int64_t big_fronts;      /* fronts of the big-front kernels */
+  int64_t digit_fronts;    /* of these, FP64 fronts whose products are 8-bit digits on the tensor cores */
+  int64_t digit_launches;  /* launches that they take per factorization */
+  int64_t digit_bytes;     /* scratch of the largest launch */
+  int64_t digit_no_room;   /* 1: that scratch did not fit at setup, FMA products on every front */
+  int64_t thin_fronts;     /* fronts of few pivots and many rows, one CTA each */
+  int64_t product_parents, product_leaves; /* fronts that take their thin leaves as one product, and those leaves */
+} clr_routes;
+int clr_get_routes(const clr_solver* s, clr_routes* out);
+
 /* Export the symbolic factorization for inspection.  perm (length N): the
  * fill-reducing order, perm[k] = KKT index eliminated k-th (KKT index i < n is
  * x_i, n + j is row j of the reordered constraint block).  sn_ptr (n_supernodes

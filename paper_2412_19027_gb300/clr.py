@@ -94,10 +94,15 @@ class clr_perf(C.Structure):
                 ("factorizations64", C.c_int32), ("pad", C.c_int32)]
 
 
+class clr_routes(C.Structure):
+    _fields_ = [(k, C.c_int64) for k in ("one_cta", "big_fronts", "digit_fronts", "digit_launches", "digit_bytes",
+                                         "digit_no_room", "thin_fronts", "product_parents", "product_leaves")]
+
+
 _LIB = None
 EXPORTS = ["clr_default_settings", "clr_setup", "clr_analyze", "clr_solve", "clr_get_solution", "clr_update_qb",
            "clr_update_PA", "clr_batch_update_PA",
-           "clr_get_symbolic_stats", "clr_get_perf", "clr_get_symbolic", "clr_get_scaling", "clr_get_history", "clr_set_stream",
+           "clr_get_symbolic_stats", "clr_get_perf", "clr_get_routes", "clr_get_symbolic", "clr_get_scaling", "clr_get_history", "clr_set_stream",
            "clr_set_allocator", "clr_free", "clr_error_string", "clr_status_string", "clr_last_cuda_error",
            "clr_cones_scaling", "clr_cones_step_length", "clr_cones_combined_ds", "clr_cones_time", "clr_ldl_solve",
            "clr_dense_ldl_solve_noalloc", "clr_batch_setup", "clr_batch_analyze", "clr_batch_size", "clr_batch_get",
@@ -125,6 +130,7 @@ def _lib():
         L.clr_batch_update_PA.argtypes = [vp, C.c_int32, P(C.c_double), P(C.c_double)]
         L.clr_get_symbolic_stats.argtypes = [vp, P(clr_symbolic_stats)]
         L.clr_get_perf.argtypes = [vp, P(clr_perf)]
+        L.clr_get_routes.argtypes = [vp, P(clr_routes)]
         L.clr_get_symbolic.argtypes = [vp] + [P(C.c_int64)] * 7
         L.clr_get_scaling.argtypes = [vp, P(C.c_double), P(C.c_double), P(C.c_double)]
         L.clr_get_history.argtypes = [vp, P(C.c_double), C.c_int32, P(C.c_int32)]
@@ -345,6 +351,12 @@ class Solver:
         s = clr_perf()
         _check(_lib().clr_get_perf(self.h, C.byref(s)), "clr_get_perf")
         return {name: getattr(s, name) for name, _ in clr_perf._fields_}
+
+    def routes(self):
+        """Which of the kernels chosen by size the factor in use takes, as a dict."""
+        s = clr_routes()
+        _check(_lib().clr_get_routes(self.h, C.byref(s)), "clr_get_routes")
+        return {name: getattr(s, name) for name, _ in clr_routes._fields_}
 
     def symbolic(self):
         """The symbolic factorization: elimination order, supernode column ranges,

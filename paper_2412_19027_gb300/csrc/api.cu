@@ -378,6 +378,13 @@ int clr_get_perf(const clr_solver* s, clr_perf* out) {
   return CLR_OK;
 }
 
+int clr_get_routes(const clr_solver* s, clr_routes* out) {
+  if (!s || !out) return CLR_E_INVALID;
+  if (!s->impl.device_ready) return CLR_E_STATE;
+  s->impl.routes(out);
+  return CLR_OK;
+}
+
 int clr_get_symbolic(const clr_solver* s, int64_t* perm, int64_t* sn_ptr, int64_t* sn_parent, int64_t* row_ptr,
                      int64_t* rows, int64_t* rows_len, int64_t* row_perm) {
   if (!s) return CLR_E_INVALID;

@@ -124,11 +124,12 @@ class DeviceArena {
  public:
   ~DeviceArena() { release(); }
   void* alloc(size_t bytes) {
-    void* p = alloc_spare(bytes);
+    void* p = take(bytes);
     failures_ += p ? 0 : 1;
     return p;
   }
-  // Memory that the owner can do without: null when there is no room, not counted as a failure.
+  // Memory that the owner can do without: null when there is no room, or when cudaMalloc would leave
+  // less than 256 MB to the driver (graphs, local memory) and to others.  Not counted as a failure.
   void* alloc_spare(size_t bytes);
   template <typename T>
   T* alloc_n(int64_t n) {
@@ -165,6 +166,7 @@ class DeviceArena {
     void* p;
     size_t n;
   };
+  void* take(size_t bytes);
   Block* blocks_ = nullptr;
   size_t nblocks_ = 0, cap_ = 0, total_ = 0;
   int64_t failures_ = 0;

@@ -798,7 +798,7 @@ void set_cuda_error(cudaError_t e, const char* where) {
   if (g_cuda_err.empty()) g_cuda_err = std::string(cudaGetErrorString(e)) + " at " + where;
 }
 
-void* DeviceArena::alloc_spare(size_t bytes) {
+void* DeviceArena::take(size_t bytes) {
   void* p = nullptr;
   bytes = (bytes + 255) & ~(size_t)255;
   if (g_alloc.a) p = g_alloc.a(bytes, g_alloc.ctx);
@@ -822,6 +822,13 @@ void* DeviceArena::alloc_spare(size_t bytes) {
   blocks_[nblocks_++] = Block{p, bytes};
   total_ += bytes;
   return p;
+}
+
+void* DeviceArena::alloc_spare(size_t bytes) {
+  size_t room = 0, all = 0;
+  if (!g_alloc.a && !async_ && (cudaMemGetInfo(&room, &all) != cudaSuccess || room < bytes + ((size_t)256 << 20)))
+    return nullptr;
+  return take(bytes);
 }
 
 void DeviceArena::release() {
@@ -1179,6 +1186,7 @@ int Solver::upload() {
   cd_.ep_zt = ar_.alloc_n<double>(3 * (cd_.n_exp + cd_.n_pow));
   exp_central_point_host(cd_.exp_center);
   if (ar_.failures() != failed) return CLR_E_OOM;
+  if (st.factor_bits == 64 && (rc = f64_.alloc_packs(ar_, ls_)) != CLR_OK) return rc;
   CLR_CUDA(cudaStreamSynchronize(stream_));
   device_ready = true;
   setup_s += now_s() - t0;
@@ -1624,6 +1632,7 @@ int Solver::step_poll(bool* ready) {
 int Solver::escalate_to_fp64() {
   if (!f64_ready_ && st.factor_bits != 64) {
     int rc = f64_.alloc(ar_, ls_);
+    if (rc == CLR_OK) rc = f64_.alloc_packs(ar_, ls_);
     if (rc != CLR_OK) return rc;
     f64_ready_ = true;
   }
@@ -1634,6 +1643,12 @@ int Solver::escalate_to_fp64() {
     std::fprintf(stderr, "[clr] refinement failed with the low-precision factor: continuing with the FP64 factor "
                          "and its regularisation\n");
   return CLR_OK;
+}
+
+void Solver::routes(clr_routes* out) const {
+  ldl_routes(ls_, out);
+  out->one_cta = cta_solve_ ? 1 : 0;
+  if (!use64()) out->digit_fronts = out->digit_launches = out->digit_bytes = 0;
 }
 
 // bookkeeping once a launched step has finished

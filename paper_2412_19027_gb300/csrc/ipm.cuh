@@ -89,6 +89,7 @@ class Solver {
   int update_PA(int64_t p, const double* Px, const double* Ax);
   int set_stream(void* stream);
   size_t device_bytes() const { return ar_.bytes(); }
+  void routes(clr_routes* out) const;
   int64_t nprob() const { return lay.B; }
 
  private:

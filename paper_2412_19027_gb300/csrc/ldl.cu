@@ -613,12 +613,13 @@ static bool flow_schedule_order(std::vector<FlowTask>& tasks, int64_t t0, const 
 }
 
 // The FP64 factor's task tables: fronts with FMA products (the fused chain task split into
-// TX(p, q), UX(p, q) and D(p), bigfront.cuh), and, with emu, the fronts of more than
-// kFlow64Rows rows with their products on the tensor cores (bigflow64.cu).
-static int flow64_tables(DeviceArena& ar, LdlStructure& st, bool emu) {
+// TX(p, q), UX(p, q) and D(p), bigfront.cuh), and the fronts of flow64_digits with their products on
+// the tensor cores (bigflow64.cu), in launches of at most `group` packs (or one front; 0: none of them).
+static int flow64_tables(DeviceArena& ar, LdlStructure& st, int64_t group) {
   const int64_t nlev = st.nlev, nb = (int64_t)st.h_bf_f.size();
   std::vector<int64_t> P_of(nb);
   std::vector<std::vector<int64_t>> of(nlev);
+  std::vector<int64_t> pk(nb, 0);
   for (int64_t b = 0; b < nb; ++b) {
     P_of[b] = (st.h_bf_c[b] + kBfNB - 1) / kBfNB;
     of[st.h_bf_lev[b]].push_back(b);
@@ -631,13 +632,35 @@ static int flow64_tables(DeviceArena& ar, LdlStructure& st, bool emu) {
   st.flow_t0_64.assign(nlev, 0);
   st.flow_nt_64.assign(nlev, 0);
   st.flow_one64.assign(nlev, 0);
-  st.flow_t0_64e.assign(nlev, 0);
-  st.flow_nt_64e.assign(nlev, 0);
+  st.flow_64e.assign(nlev, {});
+  st.pk64_tiles = st.pk64_front = 0;
+  int64_t launches = 0;
+  // with the products on the tensor cores, one CTA per SM (bigflow64.cu)
+  static const double dur64e[8] = {70.0, 24.0, 18.0, 11.0, 11.0, 0.0, 0.0, 0.0};
   for (int64_t l = 0; l < nlev; ++l) {
     st.flow_t0_64[l] = (int64_t)t64.size();
-    st.flow_t0_64e[l] = (int64_t)t64e.size();
+    std::vector<LdlStructure::Flow64Launch>& runs = st.flow_64e[l];
+    int64_t used = 0;
+    double span = 0.0;
+    auto close = [&] {  // the level's last launch is complete
+      if (runs.empty()) return true;
+      runs.back().nt = (int64_t)t64e.size() - runs.back().t0;
+      st.pk64_tiles = std::max(st.pk64_tiles, used);
+      return flow_schedule_order(t64e, runs.back().t0, P_of, flow_sms, dur64e, &span, 2);
+    };
     for (int64_t b : of[l]) {
-      const bool e64 = emu && st.h_bf_f[b] > kFlow64Rows;
+      const bool e64 = group > 0 && flow64_digits(st.h_bf_f[b], st.h_bf_c[b]);
+      if (e64) {
+        const int64_t own = flow_pk64_tiles(st.h_bf_f[b], st.h_bf_c[b]);
+        if (runs.empty() || used + own > group) {
+          if (!close()) return CLR_E_INVALID;
+          runs.push_back({(int64_t)t64e.size(), 0, st.flow_head64e + launches++});
+          used = 0;
+        }
+        pk[b] = used;
+        used += own;
+        st.pk64_front = std::max(st.pk64_front, own);
+      }
       std::vector<FlowTask>& out = e64 ? t64e : t64;
       auto add = [&](int kind, int64_t p, int64_t i, int64_t j) {
         out.push_back(FlowTask{(int32_t)b, (int16_t)kind, (int16_t)p, (int32_t)i, (int32_t)j});
@@ -660,7 +683,7 @@ static int flow64_tables(DeviceArena& ar, LdlStructure& st, bool emu) {
       }
     }
     st.flow_nt_64[l] = (int64_t)t64.size() - st.flow_t0_64[l];
-    st.flow_nt_64e[l] = (int64_t)t64e.size() - st.flow_t0_64e[l];
+    if (!close()) return CLR_E_INVALID;
     // FP64 task times (microseconds; D, T, Efin, U, EU, -, TX, UX) from per-task
     // timestamps on a GB300 at two CTAs per SM (banded LP generator), and estimates
     // for one CTA per SM (a task then has the SM's FP64 pipe to itself)
@@ -673,13 +696,11 @@ static int flow64_tables(DeviceArena& ar, LdlStructure& st, bool emu) {
       return CLR_E_INVALID;
     st.flow_one64[l] = span1 < 0.97 * span2 ? 1 : 0;
     if (st.flow_one64[l]) std::copy(one.begin(), one.end(), t64.begin() + st.flow_t0_64[l]);
-    // with the products on the tensor cores, one CTA per SM (bigflow64.cu)
-    static const double dur64e[8] = {70.0, 24.0, 18.0, 11.0, 11.0, 0.0, 0.0, 0.0};
-    if (!flow_schedule_order(t64e, st.flow_t0_64e[l], P_of, flow_sms, dur64e, &span1, 2)) return CLR_E_INVALID;
   }
+  st.bfd.pkoff64 = up(ar, pk);
   st.flow_task64 = t64.empty() ? nullptr : ar.upload(t64.data(), (int64_t)t64.size());
   st.flow_task64e = t64e.empty() ? nullptr : ar.upload(t64e.data(), (int64_t)t64e.size());
-  return (!t64.empty() && !st.flow_task64) || (!t64e.empty() && !st.flow_task64e) ? CLR_E_OOM : CLR_OK;
+  return (!t64.empty() && !st.flow_task64) || (!t64e.empty() && !st.flow_task64e) || !st.bfd.pkoff64 ? CLR_E_OOM : CLR_OK;
 }
 
 int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<int8_t>& dsign,
@@ -1102,23 +1123,11 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
     st.h_bf_lev.assign(bf_f.size(), 0);
     for (int64_t l = 0; l < sy.nlev; ++l)
       for (int64_t J : st.lev_big[l]) st.h_bf_lev[bid_of[J]] = l;
-    std::vector<int64_t> pk64(bf_f.size(), 0);
-    st.flow_head64e.assign(sy.nlev, 0);
-    {
-      std::vector<int64_t> used(sy.nlev, 0);
-      for (size_t b = 0; b < bf_f.size(); ++b)
-        if (bf_f[b] > kFlow64Rows) {
-          pk64[b] = used[st.h_bf_lev[b]];
-          used[st.h_bf_lev[b]] += flow_pk64_tiles(bf_f[b], bf_c[b]);
-        }
-      for (int64_t l = 0; l < sy.nlev; ++l) {
-        st.pk64_tiles = std::max(st.pk64_tiles, used[l]);
-        if (used[l] > 0) st.flow_head64e[l] = words++;
-      }
-    }
+    st.flow_head64e = words;
+    for (size_t b = 0; b < bf_f.size(); ++b) words += flow64_digits(bf_f[b], bf_c[b]) ? 1 : 0;
     st.flow_words = words;
-    bd.pkoff64 = up(ar, pk64);
-    if (flow64_tables(ar, st, st.flow_emu) != CLR_OK) return CLR_E_OOM;
+    const int rc64 = flow64_tables(ar, st, st.flow_emu ? kPack64Group / kPack64Bytes : 0);
+    if (rc64 != CLR_OK) return rc64;
     if (!tasks.empty()) {
       st.flow_task = ar.upload(tasks.data(), (int64_t)tasks.size());
       st.flow_soff = ar.upload(soff.data(), (int64_t)soff.size());
@@ -1190,20 +1199,6 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
       const int rc = flow_tc_encode(&tcs);
       if (rc != CLR_OK) return rc;
     }
-    if (sizeof(T) == 8 && flow && st.flow_emu && st.flow_task64e) {
-      // (not more than half of what is free: what is allocated after this had that room before)
-      size_t room = 0, all = 0;
-      if (cudaMemGetInfo(&room, &all) == cudaSuccess && (size_t)(st.pk64_tiles * kPack64Bytes) <= room / 2)
-        pk64 = static_cast<unsigned char*>(ar.alloc_spare((size_t)(st.pk64_tiles * kPack64Bytes)));
-      if (!pk64) {  // no room for the packs: FMA products on every front
-        LdlStructure& ms = const_cast<LdlStructure&>(st);
-        ms.flow_emu = false;
-        const int rc = flow64_tables(ar, ms, false);
-        if (rc != CLR_OK) return rc;
-      } else if (flow64_setup_attributes() != CLR_OK) {
-        return CLR_E_CUDA;
-      }
-    }
     const int occ = BigFrontOps<T>::flow_occupancy(tc);
     if (occ < 0) return CLR_E_CUDA;
     flow_sms = sms;
@@ -1220,6 +1215,37 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
     attr_set = true;
   }
   return CLR_OK;
+}
+
+template <typename T>
+int LdlFactor<T>::alloc_packs(DeviceArena& ar, LdlStructure& st) {
+  if constexpr (sizeof(T) == 8) {
+    if (!flow || !flow_state) return CLR_OK;
+    while (st.pk64_tiles > 0) {
+      pk64 = static_cast<unsigned char*>(ar.alloc_spare((size_t)(st.pk64_tiles * kPack64Bytes)));
+      if (pk64) return flow64_setup_attributes();
+      st.pk64_no_room = st.pk64_tiles <= st.pk64_front;
+      const int rc = flow64_tables(ar, st, st.pk64_no_room ? 0 : st.pk64_front);
+      if (rc != CLR_OK) return rc;
+    }
+  }
+  return CLR_OK;
+}
+
+void ldl_routes(const LdlStructure& st, clr_routes* out) {
+  *out = clr_routes{};
+  out->one_cta = st.cta.n > 0 ? 1 : 0;
+  out->big_fronts = st.bfd.n;
+  for (const auto& runs : st.flow_64e) out->digit_launches += (int64_t)runs.size();
+  if (out->digit_launches > 0)
+    for (size_t b = 0; b < st.h_bf_f.size(); ++b) out->digit_fronts += flow64_digits(st.h_bf_f[b], st.h_bf_c[b]) ? 1 : 0;
+  out->digit_bytes = st.pk64_tiles * kPack64Bytes;
+  out->digit_no_room = st.pk64_no_room ? 1 : 0;
+  for (int64_t l = 0; l < st.nlev; ++l) {
+    out->thin_fronts += st.lev_thin_leaf[l].n + st.lev_thin[l].n + st.lev_thin_syrk[l].n;
+    out->product_leaves += st.lev_thin_syrk[l].n;
+    if (!st.syrk.lev.empty()) out->product_parents += (int64_t)st.syrk.lev[l].size();
+  }
 }
 
 template <typename T>
@@ -1279,12 +1305,12 @@ int LdlFactor<T>::factor(cudaStream_t stm, const double* kval, const IterScal* s
       const int64_t ft0 = f64 ? S.flow_t0_64[l] : S.flow_t0[l], fnt = f64 ? S.flow_nt_64[l] : S.flow_nt[l];
       const bool one = f64 ? S.flow_one64[l] != 0 : S.flow_one[l] != 0;
       if constexpr (sizeof(T) == 8) {
-        if (use_flow && S.flow_nt_64e[l] > 0) {
-          int rc = flow64_level(stm, S.bfd, S.flow_task64e, S.flow_t0_64e[l], S.flow_nt_64e[l], flow_state,
-                                S.flow_head64e[l], S.flow_soff, flow_sms, F, E, Dp, S.dsign, dyn_eps, dyn_delta, dyn_hits,
-                                tc_err, skip, pk64);
-          if (rc) return rc;
-        }
+        if (use_flow)
+          for (const LdlStructure::Flow64Launch& e : S.flow_64e[l]) {
+            int rc = flow64_level(stm, S.bfd, S.flow_task64e, e.t0, e.nt, flow_state, e.head, S.flow_soff, flow_sms, F, E,
+                                  Dp, S.dsign, dyn_eps, dyn_delta, dyn_hits, tc_err, skip, pk64);
+            if (rc) return rc;
+          }
       }
       int rc = use_flow ? BigFrontOps<T>::flow_level(stm, S.bfd, tab, ft0, fnt, flow_state,
                                                      S.flow_head[l], S.flow_soff,

@@ -74,8 +74,14 @@ struct LdlStructure {
   // its range and counter; flow_emu: allowed (set before ldl_structure_upload)
   bool flow_emu = true;
   FlowTask* flow_task64e = nullptr;
-  std::vector<int64_t> flow_t0_64e, flow_nt_64e, flow_head64e;
-  int64_t pk64_tiles = 0;  // digit packs of the largest level
+  struct Flow64Launch {
+    int64_t t0, nt, head;
+  };
+  std::vector<std::vector<Flow64Launch>> flow_64e;  // per level, one after the other (they share the packs' space)
+  int64_t flow_head64e = 0;     // their counters: one word per front with digit products, from here on
+  int64_t pk64_tiles = 0;       // digit packs of the largest launch
+  int64_t pk64_front = 0;       // ... of the largest front
+  bool pk64_no_room = false;    // the packs did not fit: FMA products
   std::vector<int64_t> h_bf_f, h_bf_c, h_bf_lev;  // big fronts: rows, pivots, level
   std::vector<int64_t> flow_t0_64, flow_nt_64;
   std::vector<int8_t> flow_one64;
@@ -104,6 +110,9 @@ inline bool ldl_thin_front(int64_t f, int64_t c, int small_max) {
   return f > small_max && c <= kThinPivots && f * f * c <= kThinWork;
 }
 
+// Which kernels a structure's fronts take (clr_get_routes).
+void ldl_routes(const LdlStructure& st, clr_routes* out);
+
 // pos_pid: problem of each elimination position (null: one problem).
 int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<int8_t>& dsign,
                          int small_max, LdlStructure& st, const std::vector<int32_t>* pos_pid = nullptr);
@@ -125,11 +134,15 @@ struct LdlFactor {
   int flow_tc = 1;        // FP32 dataflow, trailing and E updates on the tensor cores (TF32 hi/lo parts):
                           // 0 never, 1 on the levels whose simulated schedule is shorter that way, 2 always
   T *syrk_w = nullptr, *syrk_part = nullptr;  // panels and partial tiles of thinsyrk.cu
-  unsigned char* pk64 = nullptr;  // FP64: digit packs of the largest level (null: FMA products on every front)
+  unsigned char* pk64 = nullptr;  // FP64: digit packs of the largest launch (null: FMA products on every front)
   FlowTc tcs;             // its packed operand tiles and their tensor map (allocated when used)
   int* flow_state = nullptr;
   int flow_sms = 0, flow_occ = 0;  // SMs of the device, resident flow CTAs per SM
   int alloc(DeviceArena& ar, const LdlStructure& st);
+  // The digit packs of an FP64 factor, after everything else that the owner allocates: without room for
+  // a launch's packs the fronts go one at a time (the same results), without room for one front's with FMA
+  // products.
+  int alloc_packs(DeviceArena& ar, LdlStructure& st);
   // the FP32 dataflow factorization with tensor-core updates is in use
   bool use_flow_tc() const { return sizeof(T) == 4 && flow && flow_tc != 0 && !tc16 && s && s->pk_tiles > 0; }
   // Factor K: kval (FP64, lower triangle entries in kval order) scattered into

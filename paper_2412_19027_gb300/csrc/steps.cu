@@ -337,6 +337,7 @@ int clr_ldl_solve(const clr_csc* K, const double* signs, const int64_t* order, i
     LdlFactor<double> f;
     f.flow = big_front_schedule != 0;
     if ((rc = f.alloc(ar, ls))) return rc;
+    if ((rc = f.alloc_packs(ar, ls))) return rc;
     if ((rc = f.factor(nullptr, kv, ddelta, dyn_reg_eps, dyn_reg_delta, nullptr))) return rc;
     if ((rc = f.solve(nullptr, drhs, nullptr))) return rc;
     CLR_CUDA(cudaDeviceSynchronize());

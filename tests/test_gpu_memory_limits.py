@@ -1,5 +1,5 @@
-"""Setups through a user allocator (clr_set_allocator) that refuses: every failure is an
-out-of-memory error of the call, and the next setup works."""
+"""Setups through a user allocator (clr_set_allocator) with little room: what setup needs gives an
+out-of-memory error, what it can do without is left out, and the next setup works."""
 import ctypes as C
 
 import numpy as np
@@ -90,3 +90,60 @@ def test_refused_allocations_of_the_cone_steps():
                 clr.clr_cones_step_length(cones, s, s, -s, -s, 1e6)
             assert e.value.code == OOM
     assert clr.clr_cones_step_length(cones, s, s, -s, -s, 1e6) == ref
+
+
+def dense_qp(seed, n):
+    """A QP whose KKT factorization has a root of about n rows."""
+    import scipy.sparse as sp
+    rng = np.random.default_rng(seed)
+    H = rng.standard_normal((n, n)) / np.sqrt(n)
+    A = sp.csc_matrix(sp.vstack([sp.eye(n), -sp.eye(n)]))
+    return (sp.csc_matrix(np.triu(H @ H.T + 0.1 * np.eye(n))), rng.standard_normal(n), A, np.ones(2 * n),
+            [(W.NONNEG, 2 * n, 0.0)])
+
+
+def solve_in(limit, probs, schedule):
+    """(solutions, routes, largest use) of a cohort set up and solved in `limit` bytes."""
+    st = clr.clr_default_settings(64, max_iter=5, big_front_schedule=schedule)
+    with Budget(limit) as m:
+        sv = clr.clr_batch_setup(probs, st)
+        sv.solve()
+        out = [sv.solution_of(i) for i in range(len(probs))], sv.routes(), m.peak
+        sv.free()
+        assert m.used == 0
+    return out
+
+
+def same(a, b):
+    for u, v in zip(a, b):
+        for x, y in zip(u[:3], v[:3]):
+            np.testing.assert_array_equal(x, y)
+
+
+# The scratch of the digit products is what setup can do without: where everything else fits, setup is
+# not refused.  First no room for it (FMA products, the bits of schedule 2), then room for one front's
+# at a time (the bits of all of them at once).
+def test_digit_scratch_within_a_memory_limit():
+    probs = [dense_qp(k, 400 + 7 * k) for k in range(3)]
+    fma, r2, least = solve_in(1 << 40, probs, 2)
+    full, r1, most = solve_in(1 << 40, probs, 1)
+    assert r2["digit_fronts"] == 0 and r1["digit_fronts"] == 3 and r1["digit_launches"] == 1
+    front = r1["digit_bytes"] / 3  # about that of each
+    slack = 1 << 20  # task tables of both kinds, less than a front's scratch
+    assert front > 2 * slack and most - least > 3 * front - slack
+    got, r, peak = solve_in(least + slack, probs, 1)
+    assert r["digit_no_room"] == 1 and r["digit_fronts"] == 0
+    same(got, fma)
+    got, r, peak = solve_in(least + slack + int(1.2 * front), probs, 1)
+    assert r["digit_no_room"] == 0 and r["digit_fronts"] == 3 and r["digit_launches"] == 3
+    same(got, full)
+
+
+# a problem's products are chosen by its own fronts: the same alone and in a cohort
+def test_digits_alone_and_in_a_cohort():
+    probs = [dense_qp(10 + k, n) for k, n in enumerate((330, 400, 470))]
+    both, _, _ = solve_in(1 << 40, probs, 1)
+    for p, b in zip(probs, both):
+        one, r, _ = solve_in(1 << 40, [p], 1)
+        assert r["digit_fronts"] == 1
+        same(one, [b])

@@ -1054,6 +1054,11 @@ int Solver::upload() {
     // one CTA per problem: rows summed by lane groups only, and a bounded number of entries each
     cta_solve_ = ls_.cta.n > 0 && h_rows_[0].empty() && cnt[N] <= kCtaWork * B && cnt[N] < ((int64_t)1 << 31);
     if (cta_solve_) {
+      std::vector<int64_t> entries(B, 0);
+      for (int64_t i = 0; i < N; ++i) entries[lay.pid[i]] += cnt[i + 1] - cnt[i];
+      cta_solve_ = cta_solve_pays(ls_.cta_cost, entries);
+    }
+    if (cta_solve_) {
       // rows by problem (elimination positions are contiguous there), shortest class first
       std::vector<int4> kr;
       std::vector<int32_t> ends;

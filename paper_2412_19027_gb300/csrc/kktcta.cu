@@ -581,9 +581,64 @@ size_t solve_smem(const CtaPlan& cp, size_t word) {
 
 }  // namespace
 
+// Times of a set of CTAs on the GPU: the longest, or, with more than one per SM, the list schedule's bound.
+static double cta_makespan(const std::vector<double>& t, int copies) {
+  double sum = 0.0, most = 0.0;
+  for (double x : t) sum += x, most = std::max(most, x);
+  return copies * (int64_t)t.size() <= kSMs ? most : copies * sum / kSMs + most * (1.0 - 1.0 / kSMs);
+}
+
+static CtaCost cta_cost(const Symbolic& sy, const std::vector<std::vector<std::pair<int32_t, int64_t>>>& byp) {
+  CtaCost k;
+  std::vector<double> solve(sy.nlev, 0.0), fac(sy.nlev, 0.0), pf;  // by launches: the longest front of a level
+  for (const auto& fronts : byp) {
+    double t = 16.0, tf = 8.0;
+    for (size_t i = 0; i < fronts.size();) {
+      const int32_t l = fronts[i].first;
+      size_t j = i;
+      while (j < fronts.size() && fronts[j].first == l) ++j;
+      double w8[kCtaSweepWarps] = {}, w16[kCtaThreads / 32] = {}, four = 0.0;
+      for (size_t q = i; q < j; ++q) {
+        const int64_t J = fronts[q].second;
+        const double c = (double)(sy.sn_ptr[J + 1] - sy.sn_ptr[J]), f = (double)(sy.row_ptr[J + 1] - sy.row_ptr[J]);
+        const double by4 = 0.55 * c + 1.6e-4 * c * f * f;  // four warps: the chain of pivots, then the entries
+        w8[(q - i) % kCtaSweepWarps] += 0.9 + 0.2 * c + (f > 32 ? 0.005 * c * f : 0.0);
+        w16[(q - i) % (kCtaThreads / 32)] += 2.1 + 0.55 * c + 1e-3 * c * f * f;
+        four = std::max(four, 1.5 + by4);
+        solve[l] = std::max(solve[l], 0.25 * c + 0.003 * c * f);
+        fac[l] = std::max(fac[l], by4);
+      }
+      t += 0.4 + *std::max_element(w8, w8 + kCtaSweepWarps);
+      tf += j - i <= 4 ? four : 1.0 + *std::max_element(w16, w16 + kCtaThreads / 32);
+      i = j;
+    }
+    k.sweep.push_back(t);
+    pf.push_back(tf);
+  }
+  k.levels = 21.0 + 1.6e-3 * (double)sy.N;
+  k.factor_levels = 7.0 + 2e-3 * (double)sy.nsn;
+  for (int64_t l = 0; l < sy.nlev; ++l) {
+    k.levels += 5.5 + solve[l];
+    k.factor_levels += 4.5 + fac[l];
+  }
+  k.factor = cta_makespan(pf, 1);
+  return k;
+}
+
+bool cta_solve_pays(const CtaCost& c, const std::vector<int64_t>& entries) {
+  std::vector<double> t(c.sweep);
+  double all = 0.0;
+  for (size_t p = 0; p < t.size(); ++p) {
+    t[p] += 3.5e-3 * (double)entries[p];
+    all += (double)entries[p];
+  }
+  return cta_makespan(t, 2) + cta_makespan(t, 1) < 3.0 * (c.levels + 6e-5 * all);
+}
+
 int cta_plan_build(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, int small_max,
-                   const std::vector<int32_t>* pos_pid, const int32_t* d_w_init, CtaPlan& out) {
+                   const std::vector<int32_t>* pos_pid, const int32_t* d_w_init, CtaPlan& out, CtaCost& cost) {
   out = CtaPlan();
+  cost = CtaCost();
   if (sy.nsn == 0 || sy.max_front > std::min(small_max, kCtaRows) || sy.N >= ((int64_t)1 << 31) || sy.upd_total >= ((int64_t)1 << 31))
     return CLR_OK;
   auto pid_of = [&](int64_t J) { return pos_pid ? (*pos_pid)[sy.sn_ptr[J]] : 0; };
@@ -639,6 +694,8 @@ int cta_plan_build(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, i
     }
     if (t != mp.sv_lev_ptr[l + 1] || a != mp.fa_lev_ptr[l + 1]) return CLR_OK;
   }
+  cost = cta_cost(sy, byp);
+  if (!(cost.factor < 0.9 * cost.factor_levels)) out.factor = false;
   std::vector<CtaFront> fr;
   std::vector<CtaPull> pulls;
   std::vector<int32_t> lev, rows, psrc, perm(sy.N), slot(sy.N);

@@ -91,9 +91,25 @@ constexpr int kCtaSweepWarps = 8;          // warps that sweep fronts (two colum
 constexpr int64_t kCtaSmem = 220 * 1024;   // shared memory of a CTA
 constexpr int64_t kCtaWork = 1 << 18;      // factor entries, and KKT entries, of a problem one CTA takes
 
+// When a CTA per problem is faster than a launch per level (the results are the same bits, so the choice
+// may depend on the cohort).  A problem's fronts are one SM's work here and the whole GPU's there: a
+// separable QP of 4000 variables, one level of 4000 fronts of 3 rows, took 32.4 ms on one CTA and 3.6 ms by
+// launches; a dense QP of n = 72, one front of 93 rows swept by one warp, 11.1 and 8.9 ms; MPC, T = 20,
+// 11.6 and 21.4 ms; 64 dense QPs of n = 50 in one cohort, 9.7 and 12.4 ms.  The times are estimated
+// at setup, in microseconds, by constants fitted to per-iteration times on a GB300 (FP64; 57 cohorts:
+// separable, box, total-variation chains and grids, dense QPs, MPC, 1 .. 200 problems).  Over these the
+// choice costs 4 % of the solves' time at worst (dense QP, n = 40, where both are even).
+struct CtaCost {
+  std::vector<double> sweep;   // per problem: one right-hand side's two sweeps by its CTA, the residual but for its entries
+  double levels = 0;           // the same by launches, whole cohort
+  double factor = 0, factor_levels = 0;
+};
+// the refined solves of an iteration (two launches for three right-hand sides); entries: KKT entries of each problem
+bool cta_solve_pays(const CtaCost& c, const std::vector<int64_t>& entries);
+
 // Host: the plan of a cohort whose fronts are all of at most kCtaRows rows, or n = 0.
 int cta_plan_build(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, int small_max,
-                   const std::vector<int32_t>* pos_pid, const int32_t* d_w_init, CtaPlan& out);
+                   const std::vector<int32_t>* pos_pid, const int32_t* d_w_init, CtaPlan& out, CtaCost& cost);
 
 // One right-hand side of a launch: its solution and residual vectors (KKT order).
 struct CtaRhs {

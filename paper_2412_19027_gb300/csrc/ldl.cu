@@ -1159,7 +1159,7 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       !st.dsign || !st.pos_pid || !st.kdest || !st.diag_pos || !st.fa_tgt || !st.fa_ptr || !st.fa_src || !st.sv_tgt ||
       !st.sv_ptr || !st.sv_src)
     return CLR_E_OOM;
-  const int rc = cta_plan_build(ar, sy, mp, small_max, pos_pid, st.w_init, st.cta);
+  const int rc = cta_plan_build(ar, sy, mp, small_max, pos_pid, st.w_init, st.cta, st.cta_cost);
   return rc == CLR_OK && ar.failures() != failed ? CLR_E_OOM : rc;
 }
 

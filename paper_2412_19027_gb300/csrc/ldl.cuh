@@ -90,6 +90,7 @@ struct LdlStructure {
   int small_max = 0;
   int64_t max_front = 0;
   CtaPlan cta;  // small problems: a CTA per problem (n = 0: not used)
+  CtaCost cta_cost;
 };
 
 // A front of more rows than small_max with few pivots: the arrow columns of a dense

@@ -1,0 +1,66 @@
+"""Which kernels a problem takes (Solver.routes) where the choice is one of time, and that both
+sides of a choice give the same bits."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+clr = pytest.importorskip("paper_2412_19027_gb300.clr")
+from paper_2412_19027_gb300 import workloads as W  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2412_19027_gb300 import build
+    build.build()
+
+
+def arg(p):
+    return p.P, p.q, p.A, p.b, p.cones
+
+
+def separable(n, seed=0):
+    """min x'Px/2 + q'x, |x| <= 1: n independent fronts of three rows."""
+    import scipy.sparse as sp
+    rng = np.random.default_rng(seed)
+    return (sp.csc_matrix(sp.diags(rng.random(n) + 0.1)), rng.standard_normal(n),
+            sp.csc_matrix(sp.vstack([sp.eye(n), -sp.eye(n)])), np.ones(2 * n), [(W.NONNEG, 2 * n, 0.0)])
+
+
+def qp(seed, n):
+    return arg(W.unique_qp(seed, n=n, n_eq=n // 5, n_inactive=n, rank=5))
+
+
+# refined solves by one CTA per problem: chains of small fronts and cohorts of small problems, not one
+# problem of thousands of independent fronts or with one large front
+@pytest.mark.parametrize("make,one", [
+    (lambda: [separable(2000)], 0), (lambda: [separable(40)], 1), (lambda: [qp(1, 70)], 0), (lambda: [qp(1, 20)], 1),
+    (lambda: [qp(k, 50) for k in range(64)], 1), (lambda: [arg(W.mpc_qp(1, T=20, nx=8, nu=3))], 1),
+    (lambda: [separable(1000, k) for k in range(100)], 1)])
+def test_one_cta_solves_where_they_are_faster(make, one):
+    sv = clr.clr_batch_setup(make(), clr.clr_default_settings(64, max_iter=2))
+    assert sv.routes()["one_cta"] == one
+    sv.free()
+
+
+# a dense QP alone (launches per level) and among 64 (one CTA each): its 65-row front on either path
+@pytest.mark.parametrize("bits", [64, 32])
+def test_one_cta_in_a_cohort_equals_launches_alone(bits):
+    probs = [qp(k, 50) for k in range(64)]
+    st = clr.clr_default_settings(bits, max_iter=6, fp64_escalation=0)
+    many = clr.clr_batch_setup(probs, st)
+    many.solve()
+    assert many.routes()["one_cta"] == 1
+    for k in (0, 13, 63):
+        one = clr.clr_setup(*probs[k], st)
+        one.solve()
+        assert one.routes()["one_cta"] == 0
+        a, b = one.solution(), many.solution_of(k)
+        for u, v in zip(a[:3], b[:3]):
+            np.testing.assert_array_equal(u, v)
+        assert a[3]["ir_steps_total"] == b[3]["ir_steps_total"]
+        one.free()
+    many.free()

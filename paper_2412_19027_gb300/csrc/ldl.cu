@@ -233,6 +233,32 @@ __global__ void __launch_bounds__(32 * GW) k_factor_small(T* __restrict__ F, T* 
   }
 }
 
+// A warp per front of at most 16 rows, eight fronts a CTA, for levels of more than two such fronts per SM: no
+// barriers, the operations of k_factor_small.  Bound by launching CTAs and by the fronts' loads and
+// stores: with four warps a front, mostly idle lanes, 200 000 fronts of 3 rows took 0.95 ms in FP64 and
+// 0.41 in FP32, here 0.33 and 0.155; 500 of them 16.1 and 14.4 us; 200 the same either way.
+constexpr int64_t kTinyCount = 304;
+template <typename T>
+__global__ void __launch_bounds__(256) k_factor_tiny(T* __restrict__ F, T* __restrict__ Dp,
+                                                     const int64_t* __restrict__ fronts, int64_t n,
+                                                     const int64_t* __restrict__ sn_ptr,
+                                                     const int64_t* __restrict__ row_ptr,
+                                                     const int64_t* __restrict__ front_off,
+                                                     const int8_t* __restrict__ dsign, double eps_d, double delta_d,
+                                                     int* dyn_hits, int words, const int* skip) {
+  if (skip && *skip) return;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int64_t t = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
+  if (t >= n) return;
+  T* S = reinterpret_cast<T*>(smraw) + (threadIdx.x >> 5) * words;
+  const int64_t J = fronts[t], k0 = sn_ptr[J];
+  const int c = (int)(sn_ptr[J + 1] - k0), f = (int)(row_ptr[J + 1] - row_ptr[J]);
+  T* G = F + front_off[J];
+  for (int q = threadIdx.x & 31; q < f * f; q += 32) S[q] = G[q];
+  __syncwarp();
+  factor_regs<T, 5, 1>(S, G, Dp + k0, dsign + k0, c, f, (T)eps_d, (T)delta_d, dyn_hits, 0);
+}
+
 // One CTA per thin front (ldl_thin_front): its c columns in shared memory as they are
 // (P = L D) and scaled (L), then the trailing lower triangle F -= L P^T in 64 x 64 tiles,
 // a lane per row and eight columns per warp, so that every store is a full line.  LEAF:
@@ -1282,7 +1308,11 @@ int LdlFactor<T>::factor(cudaStream_t stm, const double* kval, const IterScal* s
                                                              S.dsign, dyn_eps, dyn_delta, dyn_hits, skip);
       };
       using std::integral_constant;
-      if (mf <= 32) run(integral_constant<int, 4>{}, integral_constant<int, 32>{});
+      if (mf <= 16 && n >= kTinyCount)
+        k_factor_tiny<T><<<(n + 7) / 8, 256, 8 * smem, stm>>>(F, Dp, S.lev_small[l].id, n, S.sn_ptr, S.row_ptr,
+                                                              S.front_off, S.dsign, dyn_eps, dyn_delta, dyn_hits,
+                                                              front_words(mf), skip);
+      else if (mf <= 32) run(integral_constant<int, 4>{}, integral_constant<int, 32>{});
       else if (mf <= 64) run(integral_constant<int, 8>{}, integral_constant<int, 64>{});
       else if (mf <= 96) run(integral_constant<int, 8>{}, integral_constant<int, 96>{});
       else if (mf <= 128) run(integral_constant<int, 8>{}, integral_constant<int, 128>{});

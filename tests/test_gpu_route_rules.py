@@ -64,3 +64,21 @@ def test_one_cta_in_a_cohort_equals_launches_alone(bits):
         assert a[3]["ir_steps_total"] == b[3]["ir_steps_total"]
         one.free()
     many.free()
+
+
+# levels of more than 304 fronts of at most 16 rows (a warp each) against the kernel that takes a CTA
+# per front, beside a problem with larger fronts on the same level
+@pytest.mark.parametrize("bits", [64, 32])
+@pytest.mark.parametrize("n", [303, 304, 305, 311, 2000])
+def test_tiny_fronts_a_warp_each(bits, n):
+    st = clr.clr_default_settings(bits, max_iter=5, fp64_escalation=0)
+    big = arg(W.mixed_cone(9, n=300, n_zero=0, n_nonneg=525, n_soc=75, n_exp=15, n_pow=15))
+    one = clr.clr_setup(*separable(n), st)
+    one.solve()
+    both = clr.clr_batch_setup([separable(n), big], st)
+    both.solve()
+    a, b = one.solution(), both.solution_of(0)
+    for u, v in zip(a[:3], b[:3]):
+        np.testing.assert_array_equal(u, v)
+    one.free()
+    both.free()

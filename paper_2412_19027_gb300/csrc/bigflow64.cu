@@ -19,23 +19,31 @@
 //     products with s + t >= 8: five of s + t = 8, at most 2^-55.7 of the product of the row maxima
 //     over 64 terms.
 // Before splitting, the shared index k is scaled by a power of two on one side and its inverse
-// on the other, so that an operand's row is one of L |D|^(1/2), or, where an inverse L^{-1} of a
-// diagonal block is the other operand, so that no column of D^{-1/2} L^{-1} stands out.  The rounding
-// of a product is then 2^-55 of (largest entry of row i of L |D|^(1/2)) times (the sum over row j),
-// and the same with i and j exchanged: the size of n u |L| |D| |L|^T, the error of any LDL^T, for
-// rows whose large entries meet in the same columns.  Entries of one row of L |D|^(1/2) that span many
-// decades (a row beside a pivot that has stayed at its regularisation) lose against FMAs: LP systems
-// with P = 0 and a scaling over 12 decades, variables and rows mixed in the order, have residuals of
-// an unrefined solve 2.7 times those of FMA products; over 4 decades, with equality rows regularised
-// by 1e-8, or with more rows than variables, 0.7 to 1.1 times.  (Scaled by the diagonal as it was
-// before elimination in the place of g below, these four were 35, 0.7, 23 and 3 times.)  A row with
-// an entry that is not finite gives NaN in its results.
+// on the other, so that both operands are rows of sqrt(D)-scaled factors:
+//   - U and EU: rows of L |D|^(1/2).  The rounding of a product is 2^-55 of (the largest entry of
+//     row i) times (the sum over row j), and the same with i and j exchanged: the size of
+//     n u |L| |D| |L|^T, the error of any LDL^T, for rows whose large entries meet in the same columns.
+//   - T, Efin and the block's own inverse, products with V = L_KK^{-1}: column l of V is scaled by
+//     sqrt(F_ll).  In a block of one sign |F_il| <= sqrt(F_ii F_ll), as in a Cholesky factorization, and
+//     |d_l| <= |F_ll|.  In a block of both signs a pivot can grow from a tiny diagonal (the
+//     regularisation of an equality row or of an LP variable), and its column would set every row's
+//     maximum; so where a pivot has grown the columns are raised as far as no row of V 2^g gets a larger
+//     maximum than e_k = max(sqrt|d_k|, max_l |V_kl| sqrt(F_ll)).
+// Against FMA products (NumPy emulation, n = 192, 32 systems each, geometric means): the error of the
+// factorization, 0.5 to 0.94 times theirs on all of the following; the residual of one unrefined solve,
+// in brackets with sqrt(F_ll) alone: both signs in every block, equality rows regularised by 1e-8 1.0 (36),
+// LP with a scaling over 4 decades 0.7 (0.75), more rows than variables 0.8 (2.1); definite with a
+// spectrum over 14 decades 0.55; but 3.2 (45) for LP with a scaling over 12 decades and 7.8 for the
+// block of a PSD cone at the end of a solve (scaling over 12 decades): there U's rounding relative to the
+// row's maximum counts (4.0 and 3.7 by itself), where FMAs keep the 53 bits of each entry.  Refinement
+// removes it; schedule 2 has FMA products.  A row with an entry that is not finite gives NaN in its
+// results.
 //
 // Tasks and waits are those of bigflow.cu without the fused or split chain task: D(p), T(p, i),
 // Efin(p, e), U(p, i, j), EU(p, i, e).  Producers store their tile also as digits ("packs",
 // 56 KB in the MMA's layout, copied to shared memory by cp.async.bulk):
 //   PA(p, i) = L_IK 2^h, PB(p, i) = (L_IK D_K) 2^-h (h_k = half the exponent of d_k),
-//   PE(p, e) = E_KC^T 2^-h, PT(p) = Linv 2^g (g_l = minus the exponent of column l of D^{-1/2} Linv), so that
+//   PE(p, e) = E_KC^T 2^-h, PT(p) = Linv 2^g (g_l = half the exponent of F_ll, raised where pivots grew), so that
 //   U: F_IJ -= PA(p, i) PB(p, j)^T;  EU: E_IC -= PA(p, i) PE(p, e)^T;
 //   T: L_IK = (F_IK 2^-g) PT(p)^T D^{-1};  Efin: E_KC^T <- (E_KC^T 2^-g) PT(p)^T,
 // with F_IK and E_KC^T split in the task.  One CTA per SM (512 columns of tensor memory).
@@ -323,8 +331,7 @@ struct Diag64SmemB {
 };
 static_assert(sizeof(Diag64Smem) <= kPackBytes && sizeof(Diag64SmemB) <= kPackBytes, "scratch");
 __device__ __forceinline__ int row_exp(int m) { return m >= kBad ? kBad : (m <= -kBad ? 0 : m + 1); }
-// g of a column of an inverse whose largest entry, row k scaled by 2^-h_k, has exponent m: the column times
-// 2^g is of order one beside the others, in every row that sums over it
+// the scale of a column whose largest entry has exponent m
 __device__ __forceinline__ int block_scale(int m) { return m <= -kBad || m >= kBad ? 0 : -m; }
 __device__ __forceinline__ int shifted(double x, int sh) {
   const int l = ilog_of(x);
@@ -440,7 +447,7 @@ __device__ __noinline__ void diag64_update(int q, int I, int J, int idx, double*
 // Block row Q of L^{-1}, by the 128 threads of warps 4-7 (tid 0 .. 127 here, barrier 3): the inverse of
 // L_QQ, Linv_QP = -Linv_QQ X_P, its operands (Q < 3), and X of block row Q + 1.
 __device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A, double* V, Diag64Smem& sa,
-                                                   Diag64SmemB& sb, const int* hs) {
+                                                   Diag64SmemB& sb, const int* gs, const int* hs) {
   constexpr int LD = kDiagLD;
   const int R0 = 16 * Q;
   auto bar = [] { asm volatile("barrier.sync 3, 128;" ::: "memory"); };
@@ -475,12 +482,16 @@ __device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A,
   if (tid < 64) V[(R0 + 8 + (tid >> 3)) * LD + R0 + (tid & 7)] = b1;
   if (Q > 0) {
     bar();
-    // rows of Linv_QQ (8 threads a row), columns of X (2 threads a column); g of a column of Linv_QQ: see
-    // block_scale
+    // rows of Linv_QQ (8 threads a row), columns of X (2 threads a column)
     const int a0 = tid >> 3, c0 = 2 * (tid & 7);
     const double x0 = V[(R0 + a0) * LD + R0 + c0], x1 = V[(R0 + a0) * LD + R0 + c0 + 1];
-    {
-      int m0 = shifted(x0, -hs[R0 + a0]), m1 = shifted(x1, -hs[R0 + a0]);
+    const bool grown = __any_sync(~0u, hs[R0 + (tid & 15)] > gs[R0 + (tid & 15)]);
+    if (grown) {  // as at the end of diag64, for this block
+      int e = max(shifted(x0, gs[R0 + c0]), shifted(x1, gs[R0 + c0 + 1]));
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) e = max(e, __shfl_xor_sync(~0u, e, o));
+      e = max(e, hs[R0 + a0]);
+      int m0 = shifted(x0, -e), m1 = shifted(x1, -e);
 #pragma unroll
       for (int o = 8; o < 32; o <<= 1) {
         m0 = max(m0, __shfl_xor_sync(~0u, m0, o));
@@ -490,9 +501,10 @@ __device__ __noinline__ void diag64_inverse_row(int Q, int tid, const double* A,
         sa.gq[16 * (tid >> 5) + c0] = m0;
         sa.gq[16 * (tid >> 5) + c0 + 1] = m1;
       }
+      bar();
     }
-    bar();
     auto g_of = [&](int k) {
+      if (!grown) return gs[R0 + k];
       return block_scale(max(max(sa.gq[k], sa.gq[16 + k]), max(sa.gq[32 + k], sa.gq[48 + k])));
     };
     {
@@ -579,6 +591,10 @@ __device__ int diag64(const double* G, int64_t f, int pw, double* D, const int8_
     else if (i == j) v = 1.0;  // rows and pivots past pw: the identity
     A[i * LD + j] = v;
     V[i * LD + j] = 0.0;
+    if (i == j) {  // g: half the exponent of the diagonal
+      const int lg = i < pw ? ilog_of(v) : 0;
+      gs[i] = lg <= -kBad || lg >= kBad ? 0 : lg >> 1;
+    }
   }
   const double rdelta = 1.0 / delta;
   __syncthreads();
@@ -593,22 +609,28 @@ __device__ int diag64(const double* G, int64_t f, int pw, double* D, const int8_
           diag64_update(q - 1, I, J, tid - 128, A, sa, sb);
           diag64_update(q - 1, I, J, tid, A, sa, sb);
         }
-      diag64_inverse_row(q - 1, tid - 128, A, V, sa, sb, hs);
+      diag64_inverse_row(q - 1, tid - 128, A, V, sa, sb, gs, hs);
     }
     __syncthreads();
     for (int I = q + 1; I < 4; ++I) diag64_update(q, I, q + 1, tid, A, sa, sb);
     __syncthreads();
   }
-  if (wid >= 4) diag64_inverse_row(3, tid - 128, A, V, sa, sb, hs);
+  if (wid >= 4) diag64_inverse_row(3, tid - 128, A, V, sa, sb, gs, hs);
   __syncthreads();
-  {  // g of the columns of L^{-1}, four threads each
-    const int l = tid >> 2, k0 = 16 * (tid & 3);
-    int m = -kBad;
+  if (__syncthreads_or(tid < 64 && hs[tid] > gs[tid])) {  // e_k (four threads a row), then g (four a column): see the top
+    const int a = tid >> 2, b0 = 16 * (tid & 3);
+    int e = -kBad, m = -kBad;
 #pragma unroll 4
-    for (int k = k0; k < k0 + 16; ++k) m = max(m, shifted(V[k * LD + l], -hs[k]));
+    for (int l = b0; l < b0 + 16; ++l) e = max(e, shifted(V[a * LD + l], gs[l]));
+    e = max(e, __shfl_xor_sync(~0u, e, 1));
+    e = max(e, __shfl_xor_sync(~0u, e, 2));
+    if (b0 == 0) sa.xm[a] = max(e, hs[a]);
+    __syncthreads();
+#pragma unroll 4
+    for (int k = b0; k < b0 + 16; ++k) m = max(m, shifted(V[k * LD + a], -sa.xm[k]));
     m = max(m, __shfl_xor_sync(~0u, m, 1));
     m = max(m, __shfl_xor_sync(~0u, m, 2));
-    if (k0 == 0) gs[l] = block_scale(m);
+    if (b0 == 0) gs[a] = block_scale(m);
   }
   for (int i = tid; i < pw; i += NT) D[i] = sh.dv[i];
   return nhit;

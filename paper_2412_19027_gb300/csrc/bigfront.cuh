@@ -54,6 +54,11 @@ struct SweepLevel {
   SweepFront fr[kSweepInline];
 };
 constexpr int kSweepPull = 512;  // largest c of a front whose forward kernel gathers the children
+// ... and most CTAs of such a launch, two per SM: what k_sweep_fwd loads ahead shortens a chain of
+// levels, and keeps a second CTA off the SM.  300 fronts of 401 rows and one pivot (3900 CTAs): solves of an
+// iteration 1.14 ms with it, 0.85 with k_bf_fwd and a pull of its own; 60 fronts of 417 rows 0.74 and
+// 0.62; banded LP n = 40000, FP32, 126 and 121 ms.  Lines at 152, 304 and 608 CTAs are within 2 %.
+constexpr int64_t kSweepCtas = 2 * kSMs;
 
 // Host description of the big-front launches of one level.
 struct BigLevelPlan {

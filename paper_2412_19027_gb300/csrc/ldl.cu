@@ -991,7 +991,8 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
     }
     // the solve sweeps: descriptors, the fronts of each CTA, and which levels gather their
     // children in the forward kernels (every big front of at most kSweepPull pivots, every
-    // source list short enough to be summed in list order, and worth a thread's walk)
+    // source list short enough to be summed in list order and worth a thread's walk, at most
+    // kSweepCtas CTAs)
     {
       std::vector<SweepFront> lists;
       std::vector<int32_t> maps, pptr;
@@ -1006,7 +1007,7 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       std::vector<int64_t> sv0(sy.nsn, 0), sv1(sy.nsn, 0), cpull;
       for (int64_t l = 0; l < sy.nlev; ++l) {
         int64_t t = (*sv_lev_ptr)[l];
-        int64_t longest = 0;
+        int64_t longest = 0, ctas = 0;  // CTAs of the level's forward kernel over big fronts
         bool fused = true;
         for (int64_t k = sy.lev_ptr[l]; k < sy.lev_ptr[l + 1]; ++k) {
           const int64_t J = sy.lev_sn[k], f = sy.row_ptr[J + 1] - sy.row_ptr[J];
@@ -1017,9 +1018,10 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
           }
           sv1[J] = t;
           if (bid_of[J] >= 0 && bf_c[bid_of[J]] > kSweepPull) fused = false;
+          if (bid_of[J] >= 0) ctas += (f + 31) / 32;
         }
         if (t != (*sv_lev_ptr)[l + 1]) return CLR_E_INVALID;
-        st.lev_fused[l] = fused && longest <= kSvThread && (*sv_lev_ptr)[l + 1] < ((int64_t)1 << 31);
+        st.lev_fused[l] = fused && ctas <= kSweepCtas && longest <= kSvThread && (*sv_lev_ptr)[l + 1] < ((int64_t)1 << 31);
       }
       for (int64_t l = 0; l < sy.nlev; ++l) {
         for (int64_t k = sy.lev_ptr[l]; k < sy.lev_ptr[l + 1]; ++k) {  // lev_cta's order

@@ -82,3 +82,29 @@ def test_tiny_fronts_a_warp_each(bits, n):
         np.testing.assert_array_equal(u, v)
     one.free()
     both.free()
+
+
+# forward sweeps of large fronts with the children's gather inside (few CTAs on a level) and apart (a cohort
+# whose roots share a level of more than 304)
+@pytest.mark.parametrize("bits", [64, 32])
+@pytest.mark.parametrize("n,count", [(200, 44), (133, 62)])
+def test_sweeps_with_and_without_the_gather(bits, n, count):
+    import scipy.sparse as sp
+    probs = []
+    for k in range(count):
+        rng = np.random.default_rng(k)
+        H = rng.standard_normal((n, n)) / np.sqrt(n)
+        A = sp.csc_matrix(sp.vstack([sp.eye(n), -sp.eye(n)]))
+        probs.append((sp.csc_matrix(np.triu(H @ H.T + 0.1 * np.eye(n))), rng.standard_normal(n), A, np.ones(2 * n),
+                      [(W.NONNEG, 2 * n, 0.0)]))
+    st = clr.clr_default_settings(bits, max_iter=4, fp64_escalation=0)
+    many = clr.clr_batch_setup(probs, st)
+    many.solve()
+    for k in (0, count - 1):
+        one = clr.clr_setup(*probs[k], st)
+        one.solve()
+        a, b = one.solution(), many.solution_of(k)
+        for u, v in zip(a[:3], b[:3]):
+            np.testing.assert_array_equal(u, v)
+        one.free()
+    many.free()

@@ -150,6 +150,11 @@ __host__ __device__ inline int64_t flow_pk64_tiles(int64_t f, int64_t c) {
 // hardly a product beside it, and small dense QPs (roots up to 260 rows) solved to 1e-8 amplify a
 // change of rounding to 1e-9 in their multipliers.
 constexpr int64_t kFlow64Rows = 320;
+// ... and of more pivots: FMA products take time by the pivots, digits that of 64.  A factorization with
+// 300 fronts of 401 rows and one pivot (and a root of 560) took 2.17 ms with their products by digits, 1.54
+// by FMAs (2.09 with the root's by FMAs as well); 100 of 10 pivots 1.49 and 1.43; 60 of 17 pivots 1.32 and
+// 1.41.
+constexpr int64_t kFlow64Pivots = 16;
 // A front's own packs decide, not what memory is free or what else is in its cohort: a problem's
 // arithmetic is the same alone and in a mix.  16 GiB: a root of 26 000 rows.
 constexpr int64_t kPack64Front = (int64_t)16 << 30;
@@ -157,7 +162,7 @@ constexpr int64_t kPack64Front = (int64_t)16 << 30;
 // A front of 2000 rows has 96 MB of them and a quarter of the GPU's work in flight, so a group fills it.
 constexpr int64_t kPack64Group = (int64_t)1 << 30;
 inline bool flow64_digits(int64_t f, int64_t c) {
-  return f > kFlow64Rows && flow_pk64_tiles(f, c) * kPack64Bytes <= kPack64Front;
+  return f > kFlow64Rows && c > kFlow64Pivots && flow_pk64_tiles(f, c) * kPack64Bytes <= kPack64Front;
 }
 int flow64_setup_attributes();
 int flow64_level(cudaStream_t st, const BigFrontDev& bf, const FlowTask* task, int64_t t0, int64_t nt, int* state,

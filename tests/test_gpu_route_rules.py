@@ -108,3 +108,29 @@ def test_sweeps_with_and_without_the_gather(bits, n, count):
             np.testing.assert_array_equal(u, v)
         one.free()
     many.free()
+
+
+# FP64 fronts of more than 320 rows: products by digits from 17 pivots on
+@pytest.mark.parametrize("c,digits", [(16, 0), (17, 1)])
+def test_digit_products_from_17_pivots(c, digits):
+    import scipy.sparse as sp
+    rng = np.random.default_rng(c)
+    m, r, groups = 400, 330, 6  # groups of c coupled variables, each on r rows of one dense second-order cone
+    R, Cc, V = [], [], []
+    for g in range(groups):
+        rows = np.sort(rng.choice(m, r, replace=False))
+        for k in range(c):
+            R.append(rows); Cc.append(np.full(r, g * c + k)); V.append(rng.standard_normal(r) / np.sqrt(r))
+    A = sp.csc_matrix((np.concatenate(V), (np.concatenate(R), np.concatenate(Cc))), shape=(m, groups * c))
+    P = sp.csc_matrix(sp.triu(sp.block_diag([sp.coo_matrix(np.eye(c) + 0.05 * np.ones((c, c)))] * groups)))
+    st = clr.clr_default_settings(64, max_iter=3, soc_expand_dim=0)
+    sv = clr.clr_setup(P, rng.standard_normal(groups * c), A, np.r_[60.0, 0.5 * rng.standard_normal(m - 1)],
+                       [(W.SOC, m, 0.0)], st)
+    sv.solve()
+    sym = sv.symbolic()
+    f, p = np.diff(sym["row_ptr"]), np.diff(sym["sn_ptr"])
+    got = sv.routes()
+    assert got["digit_fronts"] == np.sum((f > 320) & (p > 16)) and (np.sum((f > 320) & (p == c)) > 0)
+    assert got["digit_fronts"] < got["big_fronts"] or digits
+    assert np.all(np.isfinite(sv.solution()[0]))
+    sv.free()

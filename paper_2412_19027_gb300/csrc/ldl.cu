@@ -128,15 +128,17 @@ __global__ void __launch_bounds__(256) k_pull_long(T* __restrict__ X, const int6
   }
 }
 
-// One level's pulls: `most` sources by a thread, the lists by a warp in order, a warp and a CTA.
-template <typename T>
+// One level's pulls: `most` sources by a thread, the lists wl by a warp (in list order, or in the order of
+// k_pull_long) and cl by a CTA.
+template <typename T, bool ORDERED>
 static void pull_level(cudaStream_t stm, T* X, const int64_t* tgt, const int64_t* ptr, const int64_t* src, int64_t t0,
-                       int64_t t1, int64_t most, const LdlStructure::List& ol, const LdlStructure::List& wl,
-                       const LdlStructure::List& cl, const int* skip) {
-  if (t1 - t0 > ol.n + wl.n + cl.n)
-    k_pull<T><<<grid_for(t1 - t0, 256), 256, 0, stm>>>(X, tgt, ptr, src, t0, t1, most, skip);
-  if (ol.n > 0) k_pull_warp<T><<<grid_for(ol.n * 32, 256), 256, 0, stm>>>(X, tgt, ptr, src, ol.id, ol.n, skip);
-  if (wl.n > 0) k_pull_long<T, 32><<<grid_for(wl.n * 32, 256), 256, 0, stm>>>(X, tgt, ptr, src, wl.id, wl.n, skip);
+                       int64_t t1, int64_t most, const LdlStructure::List& wl, const LdlStructure::List& cl,
+                       const int* skip) {
+  if (t1 - t0 > wl.n + cl.n) k_pull<T><<<grid_for(t1 - t0, 256), 256, 0, stm>>>(X, tgt, ptr, src, t0, t1, most, skip);
+  if (wl.n > 0) {
+    auto* const warp = ORDERED ? k_pull_warp<T> : k_pull_long<T, 32>;
+    warp<<<grid_for(wl.n * 32, 256), 256, 0, stm>>>(X, tgt, ptr, src, wl.id, wl.n, skip);
+  }
   if (cl.n > 0) k_pull_long<T, 256><<<grid_for(cl.n * 256, 256), 256, 0, stm>>>(X, tgt, ptr, src, cl.id, cl.n, skip);
 }
 
@@ -810,16 +812,14 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
     std::vector<char> has_child(sy.nsn, 0);
     for (int64_t J = 0; J < sy.nsn; ++J)
       if (sy.sn_parent[J] >= 0) has_child[sy.sn_parent[J]] = 1;
-    // long lists of a level's targets: in order by a warp (over `thread`), by a warp (over
-    // kPullSerial), by a CTA (over `warp`)
+    // long lists of a level's targets: by a warp (over `thread`), by a CTA (over `warp`)
     auto longs = [&](const std::vector<int64_t>& ptr, int64_t t0, int64_t t1, int64_t thread, int64_t warp,
-                     std::vector<List>& ol, std::vector<List>& wl, std::vector<List>& cl, int64_t l) {
-      std::vector<int64_t> o, w, c;
+                     std::vector<List>& wl, std::vector<List>& cl, int64_t l) {
+      std::vector<int64_t> w, c;
       for (int64_t t = t0; t < t1; ++t) {
         const int64_t n = ptr[t + 1] - ptr[t];
-        if (n > thread) (n <= kPullSerial ? o : (n <= warp ? w : c)).push_back(t);
+        if (n > thread) (n <= warp ? w : c).push_back(t);
       }
-      add(ol, l, o);
       add(wl, l, w);
       add(cl, l, c);
     };
@@ -877,8 +877,8 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       add(st.lev_thin_syrk, l, prod);
       add(st.lev_thin, l, thin);
       add(st.lev_cta, l, both);
-      longs(*fa_ptr, (*fa_lev_ptr)[l], (*fa_lev_ptr)[l + 1], kPullSerial, kFaWarp, st.fa_ord, st.fa_warp, st.fa_cta, l);
-      longs(*sv_ptr, (*sv_lev_ptr)[l], (*sv_lev_ptr)[l + 1], kSvThread, kPullSerial, st.sv_ord, st.sv_warp, st.sv_cta, l);
+      longs(*fa_ptr, (*fa_lev_ptr)[l], (*fa_lev_ptr)[l + 1], kPullSerial, kFaWarp, st.fa_warp, st.fa_cta, l);
+      longs(*sv_ptr, (*sv_lev_ptr)[l], (*sv_lev_ptr)[l + 1], kSvThread, kPullSerial, st.sv_warp, st.sv_cta, l);
     }
     int64_t* dbuf = buf.empty() ? nullptr : ar.upload(buf.data(), (int64_t)buf.size());
     if (!buf.empty() && !dbuf) return CLR_E_OOM;
@@ -1293,8 +1293,8 @@ int LdlFactor<T>::factor(cudaStream_t stm, const double* kval, const IterScal* s
     return CtaOps<T>::factor(stm, S.cta, F, Dp, S.dsign, S.fa_tgt, S.fa_ptr, S.fa_src, dyn_eps, dyn_delta, dyn_hits,
                              skip);
   for (int64_t l = 0; l < S.nlev; ++l) {
-    pull_level<T>(stm, F, S.fa_tgt, S.fa_ptr, S.fa_src, S.h_fa_lev_ptr[l], S.h_fa_lev_ptr[l + 1], kPullSerial,
-                  S.fa_ord[l], S.fa_warp[l], S.fa_cta[l], skip);
+    pull_level<T, false>(stm, F, S.fa_tgt, S.fa_ptr, S.fa_src, S.h_fa_lev_ptr[l], S.h_fa_lev_ptr[l + 1],
+                         kPullSerial, S.fa_warp[l], S.fa_cta[l], skip);
     if (!S.syrk.lev.empty()) ThinSyrkOps<T>::add_level(stm, S.syrk, l, F, Dp, syrk_w, syrk_part, skip);
     for (const WorkList& wl : S.push_rounds[l])
       if (wl.nblocks > 0)
@@ -1365,8 +1365,8 @@ int LdlFactor<T>::solve(cudaStream_t stm, const double* rhs, const int* skip) co
   for (int64_t l = 0; l < S.nlev; ++l) {
     const bool fused = S.lev_fused[l] != 0;
     if (!fused)
-      pull_level<T>(stm, w, S.sv_tgt, S.sv_ptr, S.sv_src, S.h_sv_lev_ptr[l], S.h_sv_lev_ptr[l + 1], kSvThread,
-                    S.sv_ord[l], S.sv_warp[l], S.sv_cta[l], skip);
+      pull_level<T, true>(stm, w, S.sv_tgt, S.sv_ptr, S.sv_src, S.h_sv_lev_ptr[l], S.h_sv_lev_ptr[l + 1],
+                          kSvThread, S.sv_warp[l], S.sv_cta[l], skip);
     if (!S.syrk.lev.empty())
       ThinSyrkOps<T>::fwd_level(stm, S.syrk, l, F, syrk_w, syrk_part, w, S.sn_ptr, S.row_ptr, S.front_off, S.upd_off,
                                 skip);

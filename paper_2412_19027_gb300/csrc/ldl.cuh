@@ -44,9 +44,9 @@ struct LdlStructure {
   ThinSyrk syrk;
   bool f64 = false;                              // the factor is FP64 (set before ldl_structure_upload)
   std::vector<int64_t> lev_thin_smem;            // largest f c of a level's thin fronts
-  // pull targets with long source lists (indices into fa_tgt, sv_tgt): a warp each (the sum
-  // in list order), a warp each, a CTA each
-  std::vector<List> fa_ord, fa_warp, fa_cta, sv_ord, sv_warp, sv_cta;
+  // pull targets with long source lists (indices into fa_tgt, sv_tgt): a warp each (the solves'
+  // in list order), a CTA each
+  std::vector<List> fa_warp, fa_cta, sv_warp, sv_cta;
   std::vector<std::vector<int64_t>> lev_big;     // big fronts of each level
   BigFrontDev bfd;                               // big-front arrays (device)
   std::vector<BigLevelPlan> bplans;              // per level

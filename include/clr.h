@@ -423,6 +423,7 @@ typedef struct {
   int64_t digit_no_room;   /* 1: that scratch did not fit at setup, FMA products on every front */
   int64_t thin_fronts;     /* fronts of few pivots and many rows, one CTA each */
   int64_t product_parents, product_leaves; /* fronts that take their thin leaves as one product, and those leaves */
+  int64_t warp_lists, cta_lists; /* the factorization's extend-add targets summed by a warp (over 512 sources), by a CTA */
 } clr_routes;
 int clr_get_routes(const clr_solver* s, clr_routes* out);
 
@@ -524,6 +525,11 @@ int clr_cones_time(const clr_cone* cones, int32_t ncones, const double* s, const
 int clr_ldl_solve(const clr_csc* K_lower, const double* signs, const int64_t* order, int32_t factor_bits,
                   double dyn_reg_eps, double dyn_reg_delta, const double* rhs, double* x_out, double* D_out,
                   int32_t* dyn_hits_out, int32_t big_front_schedule);
+
+/* The kernels that clr_ldl_solve takes for this pattern (no values are read; device memory for the index
+ * arrays is allocated and freed). */
+int clr_ldl_routes(const clr_csc* K_lower, const int64_t* order, int32_t factor_bits, int32_t big_front_schedule,
+                   clr_routes* out);
 
 /* Arithmetic peaks of the current GPU measured by the library's own kernels,
  * the denominators of the benchmark's roofline fractions (the paper reports

@@ -96,7 +96,8 @@ class clr_perf(C.Structure):
 
 class clr_routes(C.Structure):
     _fields_ = [(k, C.c_int64) for k in ("one_cta", "big_fronts", "digit_fronts", "digit_launches", "digit_bytes",
-                                         "digit_no_room", "thin_fronts", "product_parents", "product_leaves")]
+                                         "digit_no_room", "thin_fronts", "product_parents", "product_leaves", "warp_lists",
+                                         "cta_lists")]
 
 
 _LIB = None
@@ -104,7 +105,7 @@ EXPORTS = ["clr_default_settings", "clr_setup", "clr_analyze", "clr_solve", "clr
            "clr_update_PA", "clr_batch_update_PA",
            "clr_get_symbolic_stats", "clr_get_perf", "clr_get_routes", "clr_get_symbolic", "clr_get_scaling", "clr_get_history", "clr_set_stream",
            "clr_set_allocator", "clr_free", "clr_error_string", "clr_status_string", "clr_last_cuda_error",
-           "clr_cones_scaling", "clr_cones_step_length", "clr_cones_combined_ds", "clr_cones_time", "clr_ldl_solve",
+           "clr_cones_scaling", "clr_cones_step_length", "clr_cones_combined_ds", "clr_cones_time", "clr_ldl_solve", "clr_ldl_routes",
            "clr_dense_ldl_solve_noalloc", "clr_batch_setup", "clr_batch_analyze", "clr_batch_size", "clr_batch_get",
            "clr_batch_update_qb", "clr_server_create", "clr_server_submit", "clr_server_poll", "clr_server_wait",
            "clr_server_get_stats", "clr_server_destroy", "clr_autotune", "clr_probe_peaks", "clr_solve_begin",
@@ -150,6 +151,7 @@ def _lib():
                                                                                      P(clr_cone_times)]
         L.clr_ldl_solve.argtypes = [P(clr_csc), P(C.c_double), P(C.c_int64), C.c_int32, C.c_double, C.c_double,
                                     P(C.c_double), P(C.c_double), P(C.c_double), P(C.c_int32), C.c_int32]
+        L.clr_ldl_routes.argtypes = [P(clr_csc), P(C.c_int64), C.c_int32, C.c_int32, P(clr_routes)]
         L.clr_dense_ldl_solve_noalloc.argtypes = [vp, vp, C.c_int32, vp, vp, vp, C.c_double, C.c_double, vp, vp]
         L.clr_probe_peaks.argtypes = [C.c_int32, vp, P(clr_peaks)]
         L.clr_solve_begin.argtypes = [vp]
@@ -618,6 +620,20 @@ def clr_ldl_solve(K_lower, signs, rhs, order=None, factor_bits=64, dyn_reg_eps=1
     _check(_lib().clr_ldl_solve(C.byref(Kc), _dptr(signs), ordp, factor_bits, dyn_reg_eps, dyn_reg_delta, _dptr(rhs),
                                 _dptr(x), _dptr(D), C.byref(hits), int(big_front_schedule)), "clr_ldl_solve")
     return x, D, hits.value
+
+
+def clr_ldl_routes(K_lower, order=None, factor_bits=64, big_front_schedule=1):
+    """The kernels that clr_ldl_solve takes for this pattern, as a dict."""
+    keep = []
+    Kc = _csc(sp.tril(sp.csc_matrix(K_lower)), keep)
+    ordp = None
+    if order is not None:
+        order = np.ascontiguousarray(order, dtype=np.int64)
+        ordp = order.ctypes.data_as(C.POINTER(C.c_int64))
+    out = clr_routes()
+    _check(_lib().clr_ldl_routes(C.byref(Kc), ordp, factor_bits, int(big_front_schedule), C.byref(out)),
+           "clr_ldl_routes")
+    return {name: getattr(out, name) for name, _ in clr_routes._fields_}
 
 
 class clr_peaks(C.Structure):

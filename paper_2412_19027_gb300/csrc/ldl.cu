@@ -1272,6 +1272,8 @@ void ldl_routes(const LdlStructure& st, clr_routes* out) {
   for (int64_t l = 0; l < st.nlev; ++l) {
     out->thin_fronts += st.lev_thin_leaf[l].n + st.lev_thin[l].n + st.lev_thin_syrk[l].n;
     out->product_leaves += st.lev_thin_syrk[l].n;
+    out->warp_lists += st.fa_warp[l].n;
+    out->cta_lists += st.fa_cta[l].n;
     if (!st.syrk.lev.empty()) out->product_parents += (int64_t)st.syrk.lev[l].size();
   }
 }

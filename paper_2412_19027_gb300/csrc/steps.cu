@@ -291,6 +291,50 @@ int clr_cones_time(const clr_cone* cones, int32_t ncones, const double* s, const
   return rc;
 }
 
+static int ldl_analyze(const clr_csc* K, const int64_t* order, bool values, Symbolic& sy, NumericMaps& mp) {
+  const int64_t N = K->ncols;
+  std::vector<int64_t> colptr(K->colptr, K->colptr + N + 1), row(K->nnz);
+  for (int64_t j = 0; j < N; ++j) {
+    bool diag = false;
+    for (int64_t p = colptr[j]; p < colptr[j + 1]; ++p) {
+      row[p] = K->rowind[p];
+      if (row[p] < j || row[p] >= N) return CLR_E_INVALID;
+      if (row[p] == j) diag = true;
+      if (values && !std::isfinite(K->val[p])) return CLR_E_INVALID;
+    }
+    if (!diag) return CLR_E_INVALID;
+  }
+  std::vector<int64_t> ord;
+  if (order) ord.assign(order, order + N);
+  const int rc = symbolic_analyze(N, colptr, row, order ? &ord : nullptr, sy);
+  if (rc) return rc;
+  build_numeric_maps(sy, colptr, row, mp);
+  return CLR_OK;
+}
+
+int clr_ldl_routes(const clr_csc* K, const int64_t* order, int32_t factor_bits, int32_t big_front_schedule,
+                   clr_routes* out) {
+  if (!K || !out || (factor_bits != 64 && factor_bits != 32 && factor_bits != 16) || big_front_schedule < 0 ||
+      big_front_schedule > 3)
+    return CLR_E_INVALID;
+  if (K->nrows != K->ncols) return CLR_E_DIM;
+  *out = clr_routes{};
+  if (K->ncols == 0) return CLR_OK;
+  Symbolic sy;
+  NumericMaps mp;
+  int rc = ldl_analyze(K, order, false, sy, mp);
+  if (rc) return rc;
+  DeviceArena ar;
+  LdlStructure ls;
+  ls.f64 = factor_bits == 64;
+  ls.flow_emu = ls.f64 && (big_front_schedule == 1 || big_front_schedule == 3);
+  rc = ldl_structure_upload(ar, sy, mp, std::vector<int8_t>(K->ncols, 1), ls.f64 ? 96 : 128, ls);
+  if (rc) return rc;
+  ldl_routes(ls, out);
+  out->one_cta = 0;
+  return CLR_OK;
+}
+
 int clr_ldl_solve(const clr_csc* K, const double* signs, const int64_t* order, int32_t factor_bits,
                   double dyn_reg_eps, double dyn_reg_delta, const double* rhs, double* x_out, double* D_out,
                   int32_t* dyn_hits_out, int32_t big_front_schedule) {
@@ -300,24 +344,10 @@ int clr_ldl_solve(const clr_csc* K, const double* signs, const int64_t* order, i
   const int64_t N = K->ncols;
   if (K->nrows != N) return CLR_E_DIM;
   if (N == 0) return CLR_OK;
-  std::vector<int64_t> colptr(K->colptr, K->colptr + N + 1), row(K->nnz);
-  for (int64_t j = 0; j < N; ++j) {
-    bool diag = false;
-    for (int64_t p = colptr[j]; p < colptr[j + 1]; ++p) {
-      row[p] = K->rowind[p];
-      if (row[p] < j || row[p] >= N) return CLR_E_INVALID;
-      if (row[p] == j) diag = true;
-      if (!std::isfinite(K->val[p])) return CLR_E_INVALID;
-    }
-    if (!diag) return CLR_E_INVALID;
-  }
   Symbolic sy;
-  std::vector<int64_t> ord;
-  if (order) ord.assign(order, order + N);
-  int rc = symbolic_analyze(N, colptr, row, order ? &ord : nullptr, sy);
-  if (rc) return rc;
   NumericMaps mp;
-  build_numeric_maps(sy, colptr, row, mp);
+  int rc = ldl_analyze(K, order, true, sy, mp);
+  if (rc) return rc;
   std::vector<int8_t> dsign(N);
   for (int64_t k = 0; k < N; ++k) dsign[k] = signs[sy.perm[k]] > 0 ? 1 : -1;
   DeviceArena ar;

@@ -121,10 +121,20 @@ typedef struct {
                                  operand split into high and low TF32 parts, FP32 accumulation; operand tiles
                                  staged by TMA); 3 the tensor-core launch on every level; 2 CUDA-core
                                  products only; 0 three launches per 64-column panel.  The 16-bit-products
-                                 variant always uses the per-panel launches. */
-  int32_t small_front_max;    /* fronts of at most this order are factored by one CTA each in shared memory,
-                                 larger ones by the big-front kernels; 0 (default): 128 (FP32 / 16-bit
-                                 products), 96 (FP64); at most 224 (FP32) / 160 (FP64) */
+                                 variant always uses the per-panel launches.  With the FP64 factor (and after
+                                 an escalation) 1 and 3 multiply the 64 x 64 blocks of fronts of more than 320
+                                 rows and 16 pivots as 8-bit digits on the tensor cores: operands rounded to
+                                 2^-55 of their row's largest entry, exact from there; 2 has FP64 FMAs.  The
+                                 digits are faster and usually more accurate; an unrefined solve with rows
+                                 that span many decades can have a few times the residual (clr_ldl_solve does
+                                 not refine, the solver does).  They need scratch, allocated last: about 1.4
+                                 times the memory of the largest such front or, if more, up to 1 GB for a
+                                 group of them; without room for one front's, FMAs are used
+                                 (clr_routes.digit_no_room). */
+  int32_t small_front_max;    /* fronts of at most this order are factored by one CTA each, in registers up to 128
+                                 rows and in shared memory beyond, larger ones by the big-front kernels;
+                                 0 (default): 128 (FP32 / 16-bit products), 96 (FP64); at most 224 (FP32) /
+                                 160 (FP64) */
   int32_t amalgamation;       /* relaxed supernode amalgamation: 0 off, 1 (default) column thresholds
                                  4 / 16 / 48, 2 thresholds 8 / 32 / 96 (same zero ratios) */
   double escalate_ratio;      /* factor_bits 32/16 with fp64_escalation: also escalate when a KKT solve of an
@@ -345,7 +355,7 @@ int clr_batch_update_PA(clr_solver* s, int32_t i, const double* Px, const double
 /* Autotuner of the factorization's blocking parameters (small_front_max,
  * amalgamation, big_front_schedule) for a cohort of problems: every candidate
  * (small_front_max in {64, 96, 128, 160} plus 192 for FP32 factors, amalgamation
- * 0..2, schedules 0 and 1, and 2 for FP32 factors) is set up as a cohort of `probs` with the other fields
+ * 0..2, schedules 0, 1 and, where it is not the same as 1, 2) is set up as a cohort of `probs` with the other fields
  * of *base and solved for `iters` (>= 1) IPM iterations; the device time per
  * iteration (CUDA events: residuals, scaling, factorization, solves, steps)
  * picks the winner.  With cache_path non-NULL the result is looked up first
@@ -520,8 +530,9 @@ int clr_cones_time(const clr_cone* cones, int32_t ncones, const double* s, const
  * x_out = K^{-1} rhs (no refinement); D_out (optional, N): pivots in the
  * caller's numbering.  big_front_schedule: the large fronts' schedule, as the
  * setting of the same name (0 per-panel launches; dataflow: 1 tensor-core
- * updates for factor_bits 32 on the levels chosen at setup, 2 CUDA-core
- * products, 3 tensor-core updates on every level). */
+ * updates for factor_bits 32 on the levels chosen at setup and digit products for
+ * factor_bits 64, 2 CUDA-core products, 3 tensor-core updates on every level and
+ * digit products). */
 int clr_ldl_solve(const clr_csc* K_lower, const double* signs, const int64_t* order, int32_t factor_bits,
                   double dyn_reg_eps, double dyn_reg_delta, const double* rhs, double* x_out, double* D_out,
                   int32_t* dyn_hits_out, int32_t big_front_schedule);

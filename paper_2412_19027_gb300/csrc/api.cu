@@ -245,8 +245,9 @@ static std::string tune_key(int32_t nprob, const clr_problem* probs, const clr_s
   return buf;
 }
 
-// device ms per IPM iteration of a cohort with settings s (iters iterations)
-static int tune_time(int32_t nprob, const clr_problem* probs, const clr_settings& s, double* ms) {
+// device ms per IPM iteration of a cohort with settings s (iters iterations); digits: fronts whose products
+// run as digits in the FP64 factor
+static int tune_time(int32_t nprob, const clr_problem* probs, const clr_settings& s, double* ms, int64_t* digits = nullptr) {
   clr_solver* h = nullptr;
   int rc = make_batch(&h, nprob, probs, &s, true);
   if (rc) return rc;
@@ -255,6 +256,9 @@ static int tune_time(int32_t nprob, const clr_problem* probs, const clr_settings
     const clr_perf& p = h->impl.perf;
     const double tot = p.resid_cones_ms + p.factor_ms + p.solve_step_ms;
     *ms = tot / std::max(1, p.iterations);
+    clr_routes r;
+    h->impl.routes(&r);
+    if (digits) *digits = r.digit_fronts;
   }
   clr_free(h);
   return rc;
@@ -306,12 +310,14 @@ int clr_autotune(int32_t nprob, const clr_problem* probs, const clr_settings* ba
   const int* fr = f64 ? fronts64 : fronts32;
   const int nfr = f64 ? 4 : 5;
   for (int a = 0; a <= 2; ++a)
-    for (int i = 0; i < nfr; ++i)
-      for (int sc = 0; sc <= (f64 ? 1 : 2); ++sc) {  // 2 = 1 for the FP64 factor
+    for (int i = 0; i < nfr; ++i) {
+      int64_t digits = 0;
+      for (int sc = 0; sc <= 2; ++sc) {
+        if (sc == 2 && f64 && digits == 0) break;  // the FP64 factor's 2 is its 1 without fronts in digits
         s.small_front_max = fr[i];
         s.amalgamation = a;
         s.big_front_schedule = sc;
-        rc = tune_time(nprob, probs, s, &ms);
+        rc = tune_time(nprob, probs, s, &ms, &digits);
         if (rc) return rc;
         out->candidates += 1;
         if (ms < out->ms_per_iter) {
@@ -321,6 +327,7 @@ int clr_autotune(int32_t nprob, const clr_problem* probs, const clr_settings* ba
           out->big_front_schedule = sc;
         }
       }
+    }
   if (cache_path)
     if (FILE* f = std::fopen(cache_path, "a")) {
       std::fprintf(f, "%s %d %d %d %.6f\n", key.c_str(), out->small_front_max, out->amalgamation,

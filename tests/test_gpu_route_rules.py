@@ -134,3 +134,18 @@ def test_digit_products_from_17_pivots(c, digits):
     assert got["digit_fronts"] < got["big_fronts"] or digits
     assert np.all(np.isfinite(sv.solution()[0]))
     sv.free()
+
+
+# the autotuner times FMA products (schedule 2) beside digits where an FP64 problem has fronts in digits: three
+# amalgamations, four front sizes, three schedules
+def test_autotuner_times_fma_products():
+    import scipy.sparse as sp
+    n = 340
+    rng = np.random.default_rng(1)
+    H = rng.standard_normal((n, n)) / np.sqrt(n)
+    A = sp.csc_matrix(sp.vstack([sp.eye(n), -sp.eye(n)]))
+    prob = (sp.csc_matrix(np.triu(H @ H.T + 0.1 * np.eye(n))), rng.standard_normal(n), A, np.ones(2 * n),
+            [(W.NONNEG, 2 * n, 0.0)])
+    r = clr.clr_autotune([prob], clr.clr_default_settings(64), iters=1)
+    assert r["candidates"] == 36
+    assert clr.clr_autotune([qp(1, 20)], clr.clr_default_settings(64), iters=1)["candidates"] == 24

@@ -1232,16 +1232,14 @@ int LdlFactor<T>::alloc(DeviceArena& ar, const LdlStructure& st) {
     flow_sms = sms;
     flow_occ = occ;
   }
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_factor_small<T, 8, 96>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-    cudaFuncSetAttribute(k_factor_small<T, 8, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-    cudaFuncSetAttribute(k_factor_small<T, 8, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-    cudaFuncSetAttribute(k_factor_thin<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
-    cudaFuncSetAttribute(k_factor_thin<T, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
-    cudaFuncSetAttribute(k_factor_thin<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
-    attr_set = true;
-  }
+  // (of the current device: a process may hold solvers on several)
+  const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  CLR_CUDA(cudaFuncSetAttribute(k_factor_small<T, 8, 96>, smem, 220 * 1024));
+  CLR_CUDA(cudaFuncSetAttribute(k_factor_small<T, 8, 128>, smem, 220 * 1024));
+  CLR_CUDA(cudaFuncSetAttribute(k_factor_small<T, 8, 1024>, smem, 220 * 1024));
+  CLR_CUDA(cudaFuncSetAttribute(k_factor_thin<T, true>, smem, 128 * 1024));
+  CLR_CUDA(cudaFuncSetAttribute(k_factor_thin<T, true, true>, smem, 128 * 1024));
+  CLR_CUDA(cudaFuncSetAttribute(k_factor_thin<T, false>, smem, 128 * 1024));
   return CLR_OK;
 }
 

@@ -16,22 +16,11 @@
 
 #include "../../include/clr.h"
 #include "device.cuh"
+#include "rcp.cuh"
 
 namespace clr {
 
 constexpr int kNoAllocMaxN = CLR_NOALLOC_MAX_N;
-
-// Reciprocal of a pivot: the hardware's ~2^-20 approximation, then one third-order
-// step y (1 + e + e^2), e = 1 - d y (Householder's method), three dependent FMAs
-// instead of a correctly rounded divide's nine or so; |relative error| ~ 2^-53.
-__device__ __forceinline__ double pivot_rcp(double d) {
-  const double a = fabs(d);
-  if (!(a > 1e-290 && a < 1e290)) return 1.0 / d;  // the approximation flushes subnormals
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const double e = fma(-d, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
 
 // One CTA, right-looking LDL^T with the dynamic-regularisation rule; the forward
 // solve runs along (y_k is final when column k is), then D^{-1} and the backward
@@ -82,7 +71,7 @@ __global__ void __launch_bounds__(256) k_noalloc_ldl(const double* K, const doub
     const double sg = sgn[k];
     const bool hit = sg * d <= eps;
     if (hit) d = sg * delta;
-    const double inv = pivot_rcp(d);
+    const double inv = near_rcp(d);
     if (ti == kk) {
       sd[k] = d;
       if (hit) ++nhit;

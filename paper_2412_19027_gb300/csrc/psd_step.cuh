@@ -6,11 +6,7 @@
 
 #include <cmath>
 
-#ifdef __CUDACC__
-#define CLR_HD __host__ __device__
-#else
-#define CLR_HD
-#endif
+#include "rcp.cuh"
 
 namespace clr {
 
@@ -37,23 +33,8 @@ constexpr double kPsdSqrt2 = 1.4142135623730951;
 // Every product that is added is an explicit fma, so that the lane-parallel version
 // of the same steps (k_step_psd_lane) gives the same bits.
 
-// 1 / d for the Sturm recurrence.  On the device: the hardware's ~2^-20
-// approximation and one third-order step y (1 + e + e^2), e = 1 - d y
-// (Householder's method), 213 clocks instead of a division's 569; a relative
-// perturbation of a pivot by an ulp moves the counted eigenvalues by an ulp.
-CLR_HD inline double psd_rcp(double d) {
-#ifdef __CUDA_ARCH__
-  const double m = fabs(d);
-  if (m > 1e-290 && m < 1e290) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-    const double e = fma(-d, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-  }
-#endif
-  return 1.0 / d;
-}
-
+// The Sturm recurrence divides by near_rcp: a relative perturbation of a pivot by an ulp moves the counted
+// eigenvalues by an ulp.
 template <int KM>
 CLR_HD double psd_step_side(const double* __restrict__ v, const double* __restrict__ dv, int k) {
   double L[KM * KM], W[KM * KM];  // row-major; L lower, W full then X in its lower part
@@ -143,7 +124,7 @@ CLR_HD double psd_step_side(const double* __restrict__ v, const double* __restri
     double d = 1.0;
     for (int i = 0; i < k; ++i) {
       double t = a[i] - x;
-      if (i > 0) t = fma(-(b[i - 1] * b[i - 1]), psd_rcp(d), t);
+      if (i > 0) t = fma(-(b[i - 1] * b[i - 1]), near_rcp(d), t);
       if (t == 0.0) t = -1e-300;
       cnt += t < 0.0;
       d = t;

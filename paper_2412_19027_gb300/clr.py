@@ -360,6 +360,9 @@ class Solver:
         _check(_lib().clr_get_routes(self.h, C.byref(s)), "clr_get_routes")
         return {name: getattr(s, name) for name, _ in clr_routes._fields_}
 
+    def _dims(self):
+        return self.n, self.m
+
     def symbolic(self):
         """The symbolic factorization: elimination order, supernode column ranges,
         parents, front row lists and the constraint-row permutation (numpy arrays)."""
@@ -369,7 +372,7 @@ class Solver:
         rl = C.c_int64()
         _check(_lib().clr_get_symbolic(self.h, None, None, None, None, None, C.byref(rl), None), "clr_get_symbolic")
         perm, snp, par = np.empty(N, np.int64), np.empty(nsn + 1, np.int64), np.empty(nsn, np.int64)
-        rp, rows, rowperm = np.empty(nsn + 1, np.int64), np.empty(rl.value, np.int64), np.empty(self.m, np.int64)
+        rp, rows, rowperm = np.empty(nsn + 1, np.int64), np.empty(rl.value, np.int64), np.empty(self._dims()[1], np.int64)
         ptr = lambda a: a.ctypes.data_as(L)
         _check(_lib().clr_get_symbolic(self.h, ptr(perm), ptr(snp), ptr(par), ptr(rp), ptr(rows), C.byref(rl),
                                        ptr(rowperm)), "clr_get_symbolic")
@@ -377,7 +380,8 @@ class Solver:
 
     def scaling(self):
         """Equilibration of the setup: D (n), E (m, reordered rows) and the cost scale c."""
-        D, E, c = np.empty(self.n), np.empty(self.m), C.c_double()
+        n, m = self._dims()
+        D, E, c = np.empty(n), np.empty(m), C.c_double()
         _check(_lib().clr_get_scaling(self.h, _dptr(D), _dptr(E), C.byref(c)), "clr_get_scaling")
         return D, E, c.value
 
@@ -429,6 +433,9 @@ class Batch(Solver):
         _check(fn(C.byref(h), len(problems), arr, C.byref(st)), "clr_batch_setup" if device else "clr_batch_analyze")
         self.h = h
         self.patterns = pats
+
+    def _dims(self):  # of the merged problem, which symbolic() and scaling() describe
+        return sum(n for n, _ in self.sizes), sum(m for _, m in self.sizes)
 
     def size(self):
         """Number of problems in the cohort."""

@@ -74,8 +74,9 @@ __global__ void __launch_bounds__(NT) k_syrk_tiles(T* __restrict__ F, const T* _
       a = *reinterpret_cast<const Vec4<T>*>(W + k * p.ld + TB * I + 4 * q);
       b = *reinterpret_cast<const Vec4<T>*>(W + k * p.ld + TB * J + 4 * q);
       const T d = Dp[dpos[p.col0 + k]];
+      // (an infinite pivot has l = 0 and takes nothing off, as in k_factor_thin: no 0 times infinity)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) b.v[u] *= d;
+      for (int u = 0; u < 4; ++u) b.v[u] = b.v[u] == (T)0 ? (T)0 : b.v[u] * d;
     } else {
 #pragma unroll
       for (int u = 0; u < 4; ++u) a.v[u] = b.v[u] = (T)0;

@@ -81,3 +81,21 @@ def test_thin_fronts_by_lists(bits, leaves, c, r, m, deep, few, shared, warps, c
     assert got["product_parents"] == 0 and got["thin_fronts"] >= 512
     assert (got["warp_lists"] > 0) == bool(warps) and (got["cta_lists"] > 0) == bool(ctas)
     check(K, sgn, rhs, bits)
+
+
+# a leaf whose pivot overflows in FP32: its column of L is zero and takes nothing off its parent, by lists (too
+# many zeros for the product) and by the product
+@pytest.mark.parametrize("r,m,parents", [(129, 1100, 0), (140, 200, 1)])
+def test_infinite_pivot_of_a_leaf(r, m, parents):
+    import scipy.sparse as sp
+    K, sgn, rhs = arrow(560, 1, r, m)
+    N = len(rhs)
+    got = clr.clr_ldl_routes(K, order=np.arange(N), factor_bits=32)
+    assert got["product_parents"] == parents and got["thin_fronts"] >= 512
+    K = K.tolil()
+    K[7, 7] = 1e39
+    x, D, hits = clr.clr_ldl_solve(sp.csc_matrix(K), sgn, rhs, order=np.arange(N), factor_bits=32)
+    assert np.isinf(D[7]) and x[7] == 0 and np.all(np.isfinite(x)) and np.all(np.isfinite(np.delete(D, 7)))
+    Kf = sp.csc_matrix(K + sp.tril(K, -1).T)
+    r = (Kf @ x - rhs)[np.arange(N) != 7]
+    assert np.abs(r).max() <= 10 * np.sqrt(N) * 1.2e-7 * max(1.0, np.abs(x).max()) * 10

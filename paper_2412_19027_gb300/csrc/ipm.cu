@@ -983,6 +983,7 @@ int Solver::upload() {
   }
   const int small_max = st.small_front_max > 0 ? st.small_front_max : (st.factor_bits == 64 ? 96 : 128);
   ls_.f64 = st.factor_bits == 64;
+  ls_.f64_later = !ls_.f64 && st.fp64_escalation != 0;
   ls_.flow_emu = st.big_front_schedule == 1 || st.big_front_schedule == 3;  // (2: CUDA-core products only)
   int rc = ldl_structure_upload(ar_, sy, mp, dsign, small_max, ls_, &pos_pid);
   if (rc != CLR_OK) return rc;

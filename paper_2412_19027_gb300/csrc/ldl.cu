@@ -835,7 +835,9 @@ int ldl_structure_upload(DeviceArena& ar, const Symbolic& sy, const NumericMaps&
       const int64_t f = sy.row_ptr[J + 1] - sy.row_ptr[J], c = sy.sn_ptr[J + 1] - sy.sn_ptr[J];
       thin_leaf[J] = f > small_max && !has_child[J] && nthin[pid_of(J)] >= kThinCount && ldl_thin_front(f, c, small_max);
     }
-    const int rcs = thin_syrk_plan(ar, sy, mp, thin_leaf, st.f64, kThinCount, st.syrk, fal, svl);
+    const int rcs = thin_syrk_plan(ar, sy, mp, thin_leaf,
+                                   st.f64 ? kSyrkRatio64 : (st.f64_later ? kSyrkRatioBoth : kSyrkRatio32), kThinCount,
+                                   st.syrk, fal, svl);
     if (rcs != CLR_OK) return rcs;
     if (!fal.lev_ptr.empty()) {
       fa_lev_ptr = &fal.lev_ptr;

@@ -43,6 +43,7 @@ struct LdlStructure {
   std::vector<List> lev_thin_syrk;               // thin leaves whose update matrices are a product (thinsyrk.cu)
   ThinSyrk syrk;
   bool f64 = false;                              // the factor is FP64 (set before ldl_structure_upload)
+  bool f64_later = false;                        // an FP64 factor may take over (likewise)
   std::vector<int64_t> lev_thin_smem;            // largest f c of a level's thin fronts
   // pull targets with long source lists (indices into fa_tgt, sv_tgt): a warp each (the solves'
   // in list order), a CTA each

@@ -252,11 +252,9 @@ __global__ void __launch_bounds__(NT) k_leaf_bwd(const T* __restrict__ F, const 
 }  // namespace
 
 // The parents: at least min_children thin leaves, and the product's FMAs not more than `ratio` per
-// value of the update matrices that they replace.  A value costs 7.5 ps to gather (1.6e8 in 1.2 ms),
-// an FMA 0.07 ps in FP32 (half the FMA rate of 152 SMs) and 2.5 ps in FP64 (1.7 per clock and SM).
-int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<char>& leaf, bool f64,
+// value of the update matrices that they replace.
+int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<char>& leaf, int64_t ratio,
                    int64_t min_children, ThinSyrk& out, FaLists& fa, FaLists& sv) {
-  const int64_t ratio = f64 ? 2 : 64;
   out.lev.assign(sy.nlev, {});
   std::vector<char> pushed(sy.nsn, 0);
   for (int64_t J : mp.px_child) pushed[J] = 1;

@@ -39,9 +39,18 @@ struct FaLists {
   std::vector<int64_t> lev_ptr, tgt, ptr, src;
 };
 
+// FMAs of the product per value that the lists would gather, at most, for FP64 and FP32 factors and for
+// FP32 ones that may go on in FP64 with the same plan.  Factorization per iteration, product and lists, of
+// the portfolio n = 5000 by the density of its factor matrix (FMAs per value):
+//   FP32   0.50 and 2.01 ms at 8.5, 0.49 and 1.55 at 12, 0.48 and 1.18 at 16, 0.51 and 0.88 at 23
+//   FP64   4.69 and 11.8 ms at 2.1, 4.62 and 4.41 at 8.5, 4.60 and 3.54 at 12, 4.59 and 2.81 at 16, 4.58 and 2.10 at 23
+// An FP32 iteration gains by the product what an FP64 one loses at about 12.  The FP64 line is on the safe
+// side: between 2 and 7 the product would be faster.
+constexpr int64_t kSyrkRatio64 = 2, kSyrkRatio32 = 64, kSyrkRatioBoth = 12;
+
 // leaf: thin leaf fronts (ldl_thin_front, the path taken).  Chooses the parents, fills out and, if
 // any was chosen, fa and sv.
-int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<char>& leaf, bool f64,
+int thin_syrk_plan(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, const std::vector<char>& leaf, int64_t ratio,
                    int64_t min_children, ThinSyrk& out, FaLists& fa, FaLists& sv);
 
 template <typename T>

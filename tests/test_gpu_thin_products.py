@@ -99,3 +99,15 @@ def test_infinite_pivot_of_a_leaf(r, m, parents):
     Kf = sp.csc_matrix(K + sp.tril(K, -1).T)
     r = (Kf @ x - rhs)[np.arange(N) != 7]
     assert np.abs(r).max() <= 10 * np.sqrt(N) * 1.2e-7 * max(1.0, np.abs(x).max()) * 10
+
+
+# with an escalation to FP64 possible, a plan that FP64 would pay for stays with the lists (23 FMAs of the
+# product per value); without it, and at half the zeros (8.5), the product is taken
+@pytest.mark.parametrize("density,escalation,parents", [(0.3, 1, 0), (0.3, 0, 1), (0.5, 1, 1)])
+def test_product_of_a_solver_that_may_escalate(density, escalation, parents):
+    from paper_2412_19027_gb300 import workloads as W
+    p = W.portfolio_qp(1, n=5000, density=density)
+    st = clr.clr_default_settings(32, max_iter=2, fp64_escalation=escalation)
+    sv = clr.clr_setup(p.P, p.q, p.A, p.b, p.cones, st)
+    assert sv.routes()["product_parents"] == parents
+    sv.free()

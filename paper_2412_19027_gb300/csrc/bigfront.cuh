@@ -146,9 +146,11 @@ __host__ __device__ inline int64_t flow_pk64_tiles(int64_t f, int64_t c) {
   const int64_t P = (c + kBfNB - 1) / kBfNB;
   return 2 * flow_pk_nl(f, c) + P * (P + 1) / 2 + P;
 }
-// Fronts of more rows than this.  Five 64-row blocks or fewer are a chain of diagonal blocks with
-// hardly a product beside it, and small dense QPs (roots up to 260 rows) solved to 1e-8 amplify a
-// change of rounding to 1e-9 in their multipliers.
+// Fronts of more rows than this.  It is not where the times cross: one dense front per problem, a
+// factorization by digits and by FMAs, 0.21 and 0.30 ms at 102 rows, 0.41 and 0.64 at 229, 0.51 and 0.80 at
+// 295, 0.60 and 0.93 at 328.  It is a line of compatibility: a dense QP solved to 1e-8 amplifies a change of
+// rounding in its root to 1e-9 in the multipliers, within the tolerance but no longer the digits that
+// earlier versions gave; roots up to here keep them.
 constexpr int64_t kFlow64Rows = 320;
 // ... and of more pivots: FMA products take time by the pivots, digits that of 64.  A factorization with
 // 300 fronts of 401 rows and one pivot (and a root of 560) took 2.17 ms with their products by digits, 1.54

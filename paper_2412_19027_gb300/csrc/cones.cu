@@ -1604,6 +1604,8 @@ __global__ void k_step_psd(ConeDev cd, const int32_t* __restrict__ list, const d
 // thread per cone beyond (the same bits either way).  At 4096
 // cones of order 4 / 8 / 10 / 16 the lanes take 0.12 / 0.34 / 0.72 / 1.2 ms, the threads 0.22 / 0.50 /
 // 0.72 / 1.7 ms; the lanes' time grows with the list from ~1000 cones on, the threads' only from ~20 000.
+// One line for the three classes, where no order is slower by lanes (by these figures orders 4, 8 and 16
+// would cross at about 7500, 6000 and 5800).
 constexpr int64_t kPsdLaneCones = 4096;
 template <int KM>
 static void step_psd_small(cudaStream_t st, const ConeDev& cd, int cls, const double* s, const double* ds,

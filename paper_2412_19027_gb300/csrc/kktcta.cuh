@@ -16,8 +16,8 @@
 // ~145 clocks, each), 640 of them one after the other in that problem.  MPC, T = 20, 8
 // states, 3 inputs: a refined solve 1.0 -> 0.22 ms (two at once), a factorization 0.66 ->
 // 0.40, the whole solve 22.0 -> 10.1 ms; 64 uneven ones 124 -> 47 ms.  With rows of ~100
-// entries (dense QP, n = 50) the residual's FP64 work fills the SM and it is about even
-// with the launches (6.5 -> 6.2 ms), so larger fronts and more entries stay with those.
+// entries (one dense QP, n = 50) the residual's FP64 work fills the SM (6.1 ms; by launches
+// 5.7), with thousands of fronts on a level their sweeps do: CtaCost has the line.
 #pragma once
 
 #include <vector>
@@ -29,9 +29,9 @@
 namespace clr {
 
 // Longest source list that is summed entry by entry in list order; beyond, by the trees
-// of k_pull_long.  Small dense QPs (lists up to 400) solved to 1e-8 amplify a change of
-// rounding to 1e-9 in the multipliers, so their sums keep the order they had; from
-// ~500 sources on (portfolio, entropy) the serial chain is what the level waits for.
+// of k_pull_long.  A line of compatibility (see kThinCount): sums up to here keep the order
+// they had.  From ~500 sources on (portfolio, entropy) the serial chain is what the level
+// waits for.
 constexpr int64_t kPullSerial = 512;
 // The solves' lists of more than this many sources are read by a warp (in order up to
 // kPullSerial), the longer ones by a CTA; the factor's lists, as many as a front's

@@ -103,10 +103,13 @@ struct LdlStructure {
 // gave each front f / 32 CTAs of 512 threads for one or two columns (100 -> 9 us).
 // The lines: f^2 c / 2 FMAs on one SM are 0.3 ms in FP64 at 2^21, about what the tile
 // tasks of one such front take end to end.  A problem with fewer than kThinCount of them
-// keeps the tile tasks: there the launch costs a few rounds of tasks only, and small
-// dense QPs (up to 400 such fronts) solved to 1e-8 amplify a change of rounding to 1e-9
-// in the multipliers.  The rule looks at one problem, so that its arithmetic does not
-// depend on its cohort.
+// keeps the tile tasks.  That line, like those of kPullSerial and kFlow64Rows, is one of
+// compatibility and not where the times cross: with the three at 8 fronts, 48 sources and
+// 96 rows a factorization with fronts of 151 rows and one pivot took 0.44 ms in the place
+// of 0.69 for 32 of them and 0.55 for 1.02 with 500 (FP64; FP32 0.16 for 0.17 and 0.17 for
+// 0.47), but dense QPs up to n ~ 250, which have such fronts too, would give other last
+// digits of their multipliers (1e-9) than before.  The rule looks at one problem, so that
+// its arithmetic does not depend on its cohort.
 constexpr int64_t kThinPivots = 16, kThinWork = (int64_t)1 << 21, kThinCount = 512;
 inline bool ldl_thin_front(int64_t f, int64_t c, int small_max) {
   return f > small_max && c <= kThinPivots && f * f * c <= kThinWork;

@@ -128,14 +128,24 @@ __global__ void __launch_bounds__(256) k_pull_long(T* __restrict__ X, const int6
   }
 }
 
+// Targets of one level that k_pull_warp takes; with more a thread each is faster (the same sums): a step of the
+// warp's chain is a whole FP64 warp instruction for one target, one of the thread's for 32.  FP64, dense QPs of
+// n = 100 (200 sources): solves of an iteration 0.46 ms by warps and 0.52 by threads for one problem (129
+// targets), 1.09 and 1.17 for 8, 2.53 and 2.55 for 16, 9.43 and 9.06 for 64, 29.9 and 28.3 for 200; FP32, whose
+// instructions cost little, 2.63 and 2.92 for 64, 8.08 and 8.13 for 200 (25 800 targets).
+template <typename T>
+constexpr int64_t kPullWarps = sizeof(T) == 8 ? 2500 : 25000;
+
 // One level's pulls: `most` sources by a thread, the lists wl by a warp (in list order, or in the order of
 // k_pull_long) and cl by a CTA.
 template <typename T, bool ORDERED>
 static void pull_level(cudaStream_t stm, T* X, const int64_t* tgt, const int64_t* ptr, const int64_t* src, int64_t t0,
                        int64_t t1, int64_t most, const LdlStructure::List& wl, const LdlStructure::List& cl,
                        const int* skip) {
-  if (t1 - t0 > wl.n + cl.n) k_pull<T><<<grid_for(t1 - t0, 256), 256, 0, stm>>>(X, tgt, ptr, src, t0, t1, most, skip);
-  if (wl.n > 0) {
+  const int64_t warps = ORDERED && wl.n > kPullWarps<T> ? 0 : wl.n;
+  if (t1 - t0 > warps + cl.n)
+    k_pull<T><<<grid_for(t1 - t0, 256), 256, 0, stm>>>(X, tgt, ptr, src, t0, t1, warps == wl.n ? most : kPullSerial, skip);
+  if (warps > 0) {
     auto* const warp = ORDERED ? k_pull_warp<T> : k_pull_long<T, 32>;
     warp<<<grid_for(wl.n * 32, 256), 256, 0, stm>>>(X, tgt, ptr, src, wl.id, wl.n, skip);
   }

@@ -602,6 +602,31 @@ __global__ void __launch_bounds__(512) k_sweep_fwd(const __grid_constant__ Sweep
   }
 }
 
+// Backward over levels of many CTAs: x_j = sum_{i >= j} E[i, j] v_i, v = [y / D; x2]; one warp per column.
+template <typename T>
+__global__ void __launch_bounds__(256) k_bf_bwd(const __grid_constant__ SweepLevel lv, const T* __restrict__ E,
+                                                const T* __restrict__ ybuf, T* xs, const int32_t* __restrict__ rows_kkt,
+                                                const int* skip) {
+  if (skip && *skip) return;
+  const SweepFront& fr = sweep_front(lv, false);
+  const int f = fr.f, c = fr.c;
+  const int lane = threadIdx.x & 31, j = 8 * ((int)blockIdx.x - fr.bblk) + (int)(threadIdx.x >> 5);
+  if (j >= c) return;
+  const T* Ec = E + fr.eoff + (int64_t)j * f;
+  const T* v = ybuf + fr.yoff;
+  const int32_t* rk = rows_kkt + fr.rk;
+  T a[4] = {(T)0, (T)0, (T)0, (T)0};
+  int i = j + lane;
+  for (; i + 96 < c; i += 128) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a[u] += Ec[i + 32 * u] * v[i + 32 * u];
+  }
+  for (; i < c; i += 32) a[0] += Ec[i] * v[i];
+  for (i = c + lane; i < f; i += 32) a[1] += Ec[i] * xs[rk[i]];
+  const T acc = warp_sum((a[0] + a[1]) + (a[2] + a[3]));
+  if (lane == 0) xs[rk[j]] = acc;
+}
+
 // Backward: x_j = sum_{i >= j} E[i, j] v_i, v = [y / D; x2]; one warp per column.  The first
 // N1 and N2 entries per lane of the two parts of the column and their rows are loaded
 // before the wait for the previous level (see k_sweep_fwd): 512 and 1024 rows where the launch
@@ -739,8 +764,10 @@ int BigFrontOps<T>::sweep_bwd(cudaStream_t st, const SweepLevel& lv, const T* E,
                               const int32_t* rows_kkt, const int* skip) {
   if (lv.bblocks <= kSMs)
     CLR_CUDA(launch_pdl(k_sweep_bwd<T, 16, 32>, (unsigned)lv.bblocks, 256, 0, st, lv, E, ybuf, xs, rows_kkt, skip));
-  else
+  else if (lv.bblocks <= kSweepBwdCtas)
     CLR_CUDA(launch_pdl(k_sweep_bwd<T, 8, 8>, (unsigned)lv.bblocks, 256, 0, st, lv, E, ybuf, xs, rows_kkt, skip));
+  else
+    k_bf_bwd<T><<<(unsigned)lv.bblocks, 256, 0, st>>>(lv, E, ybuf, xs, rows_kkt, skip);
   return CLR_OK;
 }
 

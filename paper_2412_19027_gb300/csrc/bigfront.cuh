@@ -59,6 +59,12 @@ constexpr int kSweepPull = 512;  // largest c of a front whose forward kernel ga
 // iteration 1.14 ms with it, 0.85 with k_bf_fwd and a pull of its own; 60 fronts of 417 rows 0.74 and
 // 0.62; banded LP n = 40000, FP32, 126 and 121 ms.  Lines at 152, 304 and 608 CTAs are within 2 %.
 constexpr int64_t kSweepCtas = 2 * kSMs;
+// Backward CTAs up to which k_sweep_bwd takes a level, k_bf_bwd beyond (the same sums): on a full GPU the entries
+// loaded ahead, and their FP64 instructions for rows that are not there, only cost.  Solves of an
+// iteration, dense QPs of n = 100 in FP64, roots of 129 rows: 200 of them (3400 CTAs) 28.4 ms by k_sweep_bwd and 25.6
+// by k_bf_bwd, 64 (1088) 8.49 and 8.38, 16 (272) 2.44 and 2.42, 8 1.08 either way; 20 roots of 262 rows (660)
+// 0.76 and 0.72; FP32 200 x 129 7.85 and 7.70, 20 x 262 1.16 and 1.17, 300 fronts of one pivot (300) 0.91 and 0.93.
+constexpr int64_t kSweepBwdCtas = 4 * kSMs;
 
 // Host description of the big-front launches of one level.
 struct BigLevelPlan {

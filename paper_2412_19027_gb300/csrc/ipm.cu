@@ -957,6 +957,19 @@ int Solver::analyze_cohort(std::vector<HostProblem>&& ps, const std::vector<std:
   return CLR_OK;
 }
 
+// kfv from kval on the device: a gather of nnz(K) values (the host's loop and copy of them, with the blocks of
+// large cones, took most of clr_update_PA)
+__global__ void k_row_values(double* __restrict__ kfv, const double* __restrict__ kval, const int32_t* __restrict__ kvi,
+                             int64_t nnz) {
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x)
+    kfv[p] = kval[kvi[p]];
+}
+int Solver::row_values() {
+  if (nnz_ > 0) k_row_values<<<grid_for(nnz_, 256), 256, 0, stream_>>>(v_.kfv, v_.kval, v_.kvi, nnz_);
+  CLR_CHECK_LAUNCH();
+  return CLR_OK;
+}
+
 int Solver::upload() {
   const double t0 = now_s();
   const int64_t failed = ar_.failures();
@@ -1042,15 +1055,10 @@ int Solver::upload() {
     v_.kptr = ar_.upload(cnt.data(), N + 1);
     v_.kcol = ar_.upload(col.data(), (int64_t)col.size());
     v_.kvi = ar_.upload(vi.data(), (int64_t)vi.size());
-    {
-      // the values in full-CSR order: contiguous loads instead of gathers through the value
-      // index for P and A, which are constant through the solve (the z-z block's are not used)
-      std::vector<double> fv(cnt[N], 0.0);
-      for (int64_t p = 0; p < cnt[N]; ++p) fv[p] = hp.kval[vi[p]];
-      h_kfv_src_ = vi;
-      v_.kfv = fv.empty() ? nullptr : ar_.upload(fv.data(), (int64_t)fv.size());
-      if (!fv.empty() && !v_.kfv) return CLR_E_OOM;
-    }
+    // the values in full-CSR order (row_values): contiguous loads instead of gathers through the value
+    // index for P and A, which are constant through the solve (the z-z block's are not used)
+    nnz_ = cnt[N];
+    v_.kfv = ar_.alloc_n<double>(nnz_);
     const double avg = N ? (double)cnt[N] / (double)N : 1.0;
     // one CTA per problem: rows summed by lane groups only, and a bounded number of entries each
     cta_solve_ = ls_.cta.n > 0 && h_rows_[0].empty() && cnt[N] <= kCtaWork * B && cnt[N] < ((int64_t)1 << 31);
@@ -1192,6 +1200,7 @@ int Solver::upload() {
   cd_.ep_zt = ar_.alloc_n<double>(3 * (cd_.n_exp + cd_.n_pow));
   exp_central_point_host(cd_.exp_center);
   if (ar_.failures() != failed) return CLR_E_OOM;
+  if ((rc = row_values()) != CLR_OK) return rc;
   if (st.factor_bits == 64 && (rc = f64_.alloc_packs(ar_, ls_)) != CLR_OK) return rc;
   CLR_CUDA(cudaStreamSynchronize(stream_));
   device_ready = true;
@@ -1862,13 +1871,9 @@ int Solver::update_PA(int64_t p, const double* Px, const double* Ax) {
   if (rc) return rc;
   lay.pc[p].maxPdiag = pr.maxPdiag;
   if (device_ready) {
-    std::vector<double> fv(h_kfv_src_.size());
-    for (size_t k = 0; k < fv.size(); ++k) fv[k] = hp.kval[h_kfv_src_[k]];
     CLR_CUDA(cudaMemcpyAsync(v_.kval, hp.kval.data(), sizeof(double) * (size_t)hp.kval_x, cudaMemcpyHostToDevice,
                              stream_));
-    if (!fv.empty())
-      CLR_CUDA(cudaMemcpyAsync(const_cast<double*>(v_.kfv), fv.data(), sizeof(double) * fv.size(),
-                               cudaMemcpyHostToDevice, stream_));
+    if ((rc = row_values()) != CLR_OK) return rc;
     CLR_CUDA(cudaMemcpyAsync(v_.pc, lay.pc.data(), sizeof(ProbConst) * (size_t)lay.B, cudaMemcpyHostToDevice,
                              stream_));
     CLR_CUDA(cudaStreamSynchronize(stream_));

@@ -19,7 +19,7 @@ namespace clr {
 
 struct VecDev {
   const int64_t* rows_by_len[3] = {nullptr, nullptr, nullptr};  // KKT rows: long, middle, short (sorted; k_kmv_rows)
-  const double* kfv = nullptr;         // values of the full KKT CSR in its order, but for the z-z block (constant)
+  double* kfv = nullptr;               // values of the full KKT CSR in its order, but for the z-z block (constant)
   double *xz, *s;            // iterate: [x; z] (N), s (m)
   double *lo, *hi;           // split K products (N each)
   double *G;                 // [G1; G2] (N)
@@ -110,7 +110,7 @@ class Solver {
   int csr_group_ = 32;
   bool cta_solve_ = false;  // refined KKT solves by one CTA per problem (kktcta.cuh)
   std::vector<int64_t> h_rows_[3];  // rows_by_len on the host
-  std::vector<int32_t> h_kfv_src_;  // kval index of each full-CSR entry (kfv)
+  int64_t nnz_ = 0;                 // entries of the full KKT CSR
   // iteration graphs per factor precision (0: configured, 1: FP64 after an escalation)
   cudaGraph_t graph_[2] = {nullptr, nullptr};
   cudaGraphExec_t gexec_[2] = {nullptr, nullptr};
@@ -127,6 +127,7 @@ class Solver {
   double reg_dyn_eps() const;
   double reg_dyn_delta() const;
   int escalate_to_fp64();
+  int row_values();
   cudaStream_t body_stream_ = nullptr;
   std::vector<cudaGraph_t> ir_nodes_;  // refinement loop bodies captured in the current graph
   cudaEvent_t ev_[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};

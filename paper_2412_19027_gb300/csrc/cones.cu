@@ -1501,7 +1501,7 @@ __global__ void __launch_bounds__(128) k_step_psd_lane(ConeDev cd, const int32_t
     double d = 1.0;
     for (int i = 0; i < k; ++i) {
       double t = av[i] - x;
-      if (i > 0) t = fma(-bq[i - 1], near_rcp(d), t);
+      if (i > 0) t = fma(-bq[i - 1], psd_rcp(d), t);
       if (t == 0.0) t = -1e-300;
       cnt += t < 0.0;
       d = t;

@@ -22,6 +22,13 @@ namespace clr {
 
 constexpr int kNoAllocMaxN = CLR_NOALLOC_MAX_N;
 
+// Reciprocal of a pivot.  (The other order of the two returns makes the chain of pivots 4 % slower.)
+__device__ __forceinline__ double pivot_rcp(double d) {
+  const double a = fabs(d);
+  if (!(a > kRcpLow && a < kRcpHigh)) return 1.0 / d;
+  return rcp_steps(d);
+}
+
 // One CTA, right-looking LDL^T with the dynamic-regularisation rule; the forward
 // solve runs along (y_k is final when column k is), then D^{-1} and the backward
 // solve.
@@ -71,7 +78,7 @@ __global__ void __launch_bounds__(256) k_noalloc_ldl(const double* K, const doub
     const double sg = sgn[k];
     const bool hit = sg * d <= eps;
     if (hit) d = sg * delta;
-    const double inv = near_rcp(d);
+    const double inv = pivot_rcp(d);
     if (ti == kk) {
       sd[k] = d;
       if (hit) ++nhit;

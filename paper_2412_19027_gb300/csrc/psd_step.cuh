@@ -8,6 +8,12 @@
 
 #include "rcp.cuh"
 
+#ifdef __CUDACC__
+#define CLR_HD __host__ __device__
+#else
+#define CLR_HD
+#endif
+
 namespace clr {
 
 #ifndef __CUDACC__
@@ -33,8 +39,17 @@ constexpr double kPsdSqrt2 = 1.4142135623730951;
 // Every product that is added is an explicit fma, so that the lane-parallel version
 // of the same steps (k_step_psd_lane) gives the same bits.
 
-// The Sturm recurrence divides by near_rcp: a relative perturbation of a pivot by an ulp moves the counted
-// eigenvalues by an ulp.
+// 1 / d for the Sturm recurrence: a relative perturbation of a pivot by an ulp moves the counted eigenvalues by
+// an ulp.  (The test written so that the division is the exit: the other way round the bisection's loop is
+// 3 to 12 % slower.)
+CLR_HD inline double psd_rcp(double d) {
+#ifdef __CUDA_ARCH__
+  const double m = fabs(d);
+  if (m > kRcpLow && m < kRcpHigh) return rcp_steps(d);
+#endif
+  return 1.0 / d;
+}
+
 template <int KM>
 CLR_HD double psd_step_side(const double* __restrict__ v, const double* __restrict__ dv, int k) {
   double L[KM * KM], W[KM * KM];  // row-major; L lower, W full then X in its lower part
@@ -124,7 +139,7 @@ CLR_HD double psd_step_side(const double* __restrict__ v, const double* __restri
     double d = 1.0;
     for (int i = 0; i < k; ++i) {
       double t = a[i] - x;
-      if (i > 0) t = fma(-(b[i - 1] * b[i - 1]), near_rcp(d), t);
+      if (i > 0) t = fma(-(b[i - 1] * b[i - 1]), psd_rcp(d), t);
       if (t == 0.0) t = -1e-300;
       cnt += t < 0.0;
       d = t;

@@ -632,7 +632,8 @@ bool cta_solve_pays(const CtaCost& c, const std::vector<int64_t>& entries) {
     t[p] += 3.5e-3 * (double)entries[p];
     all += (double)entries[p];
   }
-  return cta_makespan(t, 2) + cta_makespan(t, 1) < 3.0 * (c.levels + 6e-5 * all);
+  // (6 %: the initial point's two right-hand sides share a launch too)
+  return cta_makespan(t, 2) + cta_makespan(t, 1) < 1.06 * 3.0 * (c.levels + 6e-5 * all);
 }
 
 int cta_plan_build(DeviceArena& ar, const Symbolic& sy, const NumericMaps& mp, int small_max,

@@ -620,13 +620,13 @@ __device__ int diag64(const double* G, int64_t f, int pw, double* D, const int8_
   if (__syncthreads_or(tid < 64 && hs[tid] > gs[tid])) {  // e_k (four threads a row), then g (four a column): see the top
     const int a = tid >> 2, b0 = 16 * (tid & 3);
     int e = -kBad, m = -kBad;
-#pragma unroll 4
+#pragma unroll
     for (int l = b0; l < b0 + 16; ++l) e = max(e, shifted(V[a * LD + l], gs[l]));
     e = max(e, __shfl_xor_sync(~0u, e, 1));
     e = max(e, __shfl_xor_sync(~0u, e, 2));
     if (b0 == 0) sa.xm[a] = max(e, hs[a]);
     __syncthreads();
-#pragma unroll 4
+#pragma unroll
     for (int k = b0; k < b0 + 16; ++k) m = max(m, shifted(V[k * LD + a], -sa.xm[k]));
     m = max(m, __shfl_xor_sync(~0u, m, 1));
     m = max(m, __shfl_xor_sync(~0u, m, 2));

@@ -123,7 +123,7 @@ typedef struct {
                                  products only; 0 three launches per 64-column panel.  The 16-bit-products
                                  variant always uses the per-panel launches.  With the FP64 factor (and after
                                  an escalation) 1 and 3 multiply the 64 x 64 blocks of fronts of more than 320
-                                 rows and 16 pivots as 8-bit digits on the tensor cores: operands rounded to
+                                 rows and 8 pivots as 8-bit digits on the tensor cores: operands rounded to
                                  2^-55 of their row's largest entry, exact from there; 2 has FP64 FMAs.  The
                                  digits are faster and usually more accurate; an unrefined solve with rows
                                  that span many decades can have a few times the residual (clr_ldl_solve does

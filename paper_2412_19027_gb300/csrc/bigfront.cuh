@@ -160,9 +160,10 @@ __host__ __device__ inline int64_t flow_pk64_tiles(int64_t f, int64_t c) {
 constexpr int64_t kFlow64Rows = 320;
 // ... and of more pivots: FMA products take time by the pivots, digits that of 64.  A factorization with
 // 300 fronts of 401 rows and one pivot (and a root of 560) took 2.17 ms with their products by digits, 1.54
-// by FMAs (2.09 with the root's by FMAs as well); 100 of 10 pivots 1.49 and 1.43; 60 of 17 pivots 1.32 and
-// 1.41.
-constexpr int64_t kFlow64Pivots = 16;
+// by FMAs (2.09 with the root's by FMAs as well), with 100 of 8 pivots 1.47 and 1.37, with 20 of 8 1.055
+// and 1.029, with 20 of 12 1.067 both ways, with 60 of 17 1.32 and 1.41; on a chain of levels, where a front's
+// own time counts, digits gain earlier: banded LP n = 20000 25.2 ms with this line at 8, 26.1 at 16.
+constexpr int64_t kFlow64Pivots = 8;
 // A front's own packs decide, not what memory is free or what else is in its cohort: a problem's
 // arithmetic is the same alone and in a mix.  16 GiB: a root of 26 000 rows.
 constexpr int64_t kPack64Front = (int64_t)16 << 30;

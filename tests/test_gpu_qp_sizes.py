@@ -36,7 +36,7 @@ def test_optimum_on_both_sides_of_the_kernel_limits(bits, n):
     routes, sym = sv.routes(), sv.symbolic()
     sv.free()
     f, c = np.diff(sym["row_ptr"]), np.diff(sym["sn_ptr"])
-    assert routes["digit_fronts"] == (np.sum((f > 320) & (c > 16)) if bits == 64 else 0)
+    assert routes["digit_fronts"] == (np.sum((f > 320) & (c > 8)) if bits == 64 else 0)
     assert info["status_name"] == "SOLVED"
     P = p.P.toarray()
     P = np.triu(P) + np.triu(P, 1).T
